@@ -11,6 +11,8 @@
 
 #include "dslash.cuh"
 #include "kernels.h"
+#include "fx.cuh"
+#include "recurrence.cuh"
 
 namespace ov {
 
@@ -612,6 +614,15 @@ static void launch_apply_sweep(const Lat<R>& L, const R* in, R* out, int dagger,
 
 template <typename R>
 void apply_h(const Lat<R>& L, const R* in, R* out, int dagger, cudaStream_t st, int variant, int* err) {
+  if constexpr (std::is_same<R, double>::value) {
+    if (L.fu.e) {
+      fx_encode(in, L.fr, L.nsrc, L.g.V, L.vs, st);
+      fx_apply_h(L, L.fr, in, out, dagger, 0, st, variant);
+    } else {
+      launch_apply<R, 1, 128, 0>(L, in, out, dagger, st);   // no fixed-point links (ov_apply_H_noalloc)
+    }
+    return;
+  } else
   switch (variant) {
     case 12: launch_apply_sweep<R>(L, in, out, dagger, st, err); break;
     case 9: launch_apply_staged<R>(L, in, out, dagger, st, 1, err); break;
@@ -630,55 +641,15 @@ void apply_h(const Lat<R>& L, const R* in, R* out, int dagger, cudaStream_t st, 
 }
 
 // ---------------------------------------------------------------------------
-// helpers for the recurrence scalars
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ bool finite_z(zd a) { return isfinite(a.re) && isfinite(a.im); }
-
-__device__ __forceinline__ void flag_error(SrcScal& sc, int bit, int step) {
-  if (sc.err == 0) sc.err_step = step;
-  sc.err |= bit;
-}
-
-// Sum NV partial slots of this source (fixed block order); thread 0 gets the result.
-template <int NV>
-__device__ __forceinline__ void sum_partials(const zd* part, int nblk, zd (&out)[NV], zd* scratch) {
-  zd v[NV];
-#pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = mk(0.0, 0.0);
-  // each thread takes a contiguous range of blocks, so the order is fixed
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) v[i] = v[i] + ld_cg(part + i * nblk + b);
-  }
-  block_sum<NV>(v, scratch);
-#pragma unroll
-  for (int i = 0; i < NV; ++i) out[i] = v[i];
-}
-
-// omega = s^dag r, rr = r^dag r, ss = s^dag s  ->  delta_{j+1}, beta_{j+1} and the next scales
-template <typename R>
-__device__ void omega_finalize(const Lat<R>& L, int src, int j, zd om, double rr, double ss) {
-  SrcScal& sc = L.sc[src];
-  const double aom = sqrt(om.re * om.re + om.im * om.im);
-  if (!finite_z(om) || !isfinite(rr) || !isfinite(ss)) {
-    flag_error(sc, ERRB_NONFINITE, j + 1);
-    return;
-  }
-  if (aom <= 1e-14 * sqrt(rr * ss)) {
-    flag_error(sc, ERRB_BREAKDOWN, j + 1);
-    return;
-  }
-  const double d = sqrt(aom);
-  const zd bt = mk(om.re / d, om.im / d);
-  L.beta[(int64_t)src * L.k + j + 1] = bt;
-  L.delta[(int64_t)src * L.k + j + 1] = d;
-  sc.sv = mk(1.0 / d, 0.0);
-  sc.sw = zdiv(mk(1.0, 0.0), conj(bt));
-}
-
-// ---------------------------------------------------------------------------
 // TSL forward: initialisation (beta_0 = ||b||)
 // ---------------------------------------------------------------------------
+// the fixed-point copy of a site of an FP64 field (nothing for FP32 fields)
+__device__ __forceinline__ void store_fx(const FxField& f, int src, int64_t vs, int64_t V, int64_t x,
+                                         const Spinor<double>& p) {
+  fx_store(fx_src(f, src, vs, V), V, x, p);
+}
+__device__ __forceinline__ void store_fx(const FxField&, int, int64_t, int64_t, int64_t, const Spinor<float>&) {}
+
 template <typename R>
 __global__ void __launch_bounds__(BS) k_tsl_init(Lat<R> L) {
   __shared__ zd scratch[2 * 32];
@@ -689,10 +660,14 @@ __global__ void __launch_bounds__(BS) k_tsl_init(Lat<R> L) {
     Spinor<R> b;
     load_spinor(L.r + src * L.vs, L.g.V, x, b);
     v[0] = spinor_dot(b, b);
+    store_fx(L.fr, src, L.vs, L.g.V, x, b);
     if (L.block) {
       Spinor<R> a;
       load_spinor(L.s + src * L.vs, L.g.V, x, a);
       v[1] = spinor_dot(a, b);
+      store_fx(L.fs, src, L.vs, L.g.V, x, a);
+    } else {
+      store_fx(L.fs, src, L.vs, L.g.V, x, b);   // s = r
     }
   }
   block_sum<2>(v, scratch);
@@ -878,6 +853,10 @@ static void launch_pair(const Lat<R>& L, int j, int q, cudaStream_t st) {
 template <typename R>
 void tsl_stencil(const Lat<R>& L, int j, bool need_q, cudaStream_t st, int variant) {
   const int q = need_q ? 1 : 0;
+  if constexpr (std::is_same<R, double>::value) {
+    fx_tsl_stencil(L, j, q, st, variant);
+    return;
+  } else {
   if (L.block) {
     k_tsl_stencil_block<R><<<dim3(nblocks(L.gl.V, BS), L.nsrc), BS, 0, st>>>(L, j, q);
     return;
@@ -890,6 +869,7 @@ void tsl_stencil(const Lat<R>& L, int j, bool need_q, cudaStream_t st, int varia
     case 5: launch_pair<R, 1, 256, 1>(L, j, q, st); break;
     case 6: launch_pair<R, 0, 512, 1>(L, j, q, st); break;
     default: launch_pair<R, 1, 128, 0>(L, j, q, st); break;
+  }
   }
 }
 
@@ -926,6 +906,8 @@ __global__ void __launch_bounds__(BS) k_tsl_update(Lat<R> L, int j, int finalize
     store_spinor(L.r + src * L.vs, V, x, r);
     store_spinor(L.s + src * L.vs, V, x, s);
     if (finalize) {
+      store_fx(L.fr, src, L.vs, V, x, r);
+      store_fx(L.fs, src, L.vs, V, x, s);
       v[0] = spinor_dot(s, r);
       v[1] = spinor_dot(r, r);
       v[2] = spinor_dot(s, s);
@@ -1083,7 +1065,9 @@ __global__ void __launch_bounds__(BS) k_proj_update(Lat<R> L, int nb, int mode, 
 #pragma unroll
       for (int c = 0; c < 12; ++c) s.c[c] = s.c[c] - mk<R>((R)cb.c[c].re, (R)cb.c[c].im);
       store_spinor(b + src * ab_stride, V, x, s);
-      if (finalize) {
+      if (finalize) {   // a and b are the recurrence's r and s
+        store_fx(L.fr, src, L.vs, V, x, r);
+        store_fx(L.fs, src, L.vs, V, x, s);
         v[0] = spinor_dot(s, r);
         v[1] = spinor_dot(r, r);
         v[2] = spinor_dot(s, s);
@@ -1445,6 +1429,7 @@ __global__ void __launch_bounds__(BS) k_rev_combine(Lat<R> L, Rev<R> B, int j, i
     for (int c = 0; c < 12; ++c) a.c[c] = ga * e.c[c];
   }
   store_spinor(B.ring(B.gp_ring, slot, src), V, x, a);
+  store_fx(B.fp, src, L.vs, V, x, a);
   const cplx<R> gac = conj(ga);
   load_spinor(L.basis_v(src, j), V, x, e);
   if (carry) {
@@ -1455,7 +1440,11 @@ __global__ void __launch_bounds__(BS) k_rev_combine(Lat<R> L, Rev<R> B, int j, i
 #pragma unroll
     for (int c = 0; c < 12; ++c) a.c[c] = gac * e.c[c];
   }
-  store_spinor(B.hin + src * L.vs, V, x, a);
+  if constexpr (std::is_same<R, double>::value) {
+    if (fx_store(fx_src(B.fh, src, L.vs, V), V, x, a)) store_spinor(B.hin + src * L.vs, V, x, a);
+  } else {
+    store_spinor(B.hin + src * L.vs, V, x, a);
+  }
 }
 template <typename R>
 void rev_combine(const Lat<R>& L, const Rev<R>& B, int j, int slot, cudaStream_t st) {
@@ -1518,8 +1507,11 @@ __global__ void __launch_bounds__(BS) k_rev_stencil(Lat<R> L, Rev<R> B, int j, i
 }
 template <typename R>
 void rev_stencil(const Lat<R>& L, const Rev<R>& B, int j, int slot, int prev_slot, int nrec, cudaStream_t st) {
-  k_rev_stencil<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot,
-                                                                                      prev_slot, nrec);
+  if constexpr (std::is_same<R, double>::value)
+    fx_rev_stencil(L, B, j, slot, prev_slot, nrec, st);
+  else
+    k_rev_stencil<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot,
+                                                                                        prev_slot, nrec);
 }
 
 // ---------------------------------------------------------------------------

@@ -7,6 +7,7 @@
 #include <algorithm>
 #include <atomic>
 #include <thread>
+#include <type_traits>
 #include <cstdio>
 #include <cstring>
 #include <vector>
@@ -22,7 +23,7 @@ enum BufId {
   B_LINKS, B_BV, B_BW, B_P, B_Q, B_R, B_S, B_SC, B_ALPHA, B_BETA, B_DELTA, B_PART, B_CNT, B_COEF, B_CPART,
   B_T, B_X, B_XI, B_XN, B_E, B_EN, B_TMP1, B_TMP2, B_IPIV, B_PROW, B_COL, B_DSTAT, B_DPART, B_DCNT, B_DERR,
   B_Y, B_GY, B_GA, B_GB, B_GD, B_XBAR, B_GV, B_GW, B_GV2, B_GW2, B_GR, B_GS, B_GP, B_EV, B_EW, B_REB,
-  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, NBUF
+  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, B_FXL, B_FXE, B_FXDL, B_FXDE, B_FXR, B_FXRE, B_FXS, B_FXSE, B_FXP, B_FXPE, B_FXH, B_FXHE, NBUF
 };
 
 struct Status {
@@ -325,6 +326,13 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   R* u = wsT<R>(c, B_LINKS, link_reals<R>() * V);
   L.u = u;
   run(c, OV_KIND_LAYOUT, 1, [&] { pack_links<R>(static_cast<const double*>(U), u, V, c->st); });
+  if constexpr (std::is_same<R, double>::value) {
+    int4* fe = wsT<int4>(c, B_FXL, kFxLinkEntries * V);
+    short* fx = wsT<short>(c, B_FXE, 5 * V);
+    L.fu = FxLinks{fe, fx};
+    run(c, OV_KIND_LAYOUT, 1,
+        [&] { pack_links_fx(static_cast<const double*>(U), fe, fx, V, L.ef, L.efinv, c->st); });
+  }
   launch_check();
   if (fm == 2) {
     L.block = 1;
@@ -342,6 +350,10 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   L.q = wsT<R>(c, B_Q, nsrc * L.vs);
   L.r = wsT<R>(c, B_R, nsrc * L.vs);
   L.s = wsT<R>(c, B_S, nsrc * L.vs);
+  if constexpr (std::is_same<R, double>::value) {
+    L.fr = FxField{wsT<int4>(c, B_FXR, nsrc * (L.vs / 2)), wsT<short>(c, B_FXRE, nsrc * Vf)};
+    if (basis) L.fs = FxField{wsT<int4>(c, B_FXS, nsrc * (L.vs / 2)), wsT<short>(c, B_FXSE, nsrc * Vf)};
+  }
   L.sc = wsT<SrcScal>(c, B_SC, nsrc);
   L.alpha = wsT<zd>(c, B_ALPHA, (int64_t)nsrc * k);
   L.beta = wsT<zd>(c, B_BETA, (int64_t)nsrc * k);
@@ -598,6 +610,11 @@ void seg_replay(ov_context* c, Lat<R>& L, const SegPlan& P, const SegStore<R>& K
   // only the forward scalars: the reverse sweep keeps its own in the same structs
   CK(cudaMemcpy2DAsync(L.sc, sizeof(SrcScal), K.sc + t * L.nsrc, sizeof(SrcScal), offsetof(SrcScal, g_alpha),
                        L.nsrc, cudaMemcpyDeviceToDevice, c->st));
+  if constexpr (std::is_same<R, double>::value)
+    run(c, OV_KIND_UPDATE, 2, [&] {
+      fx_encode(L.r, L.fr, L.nsrc, L.g.V, L.vs, c->st);
+      fx_encode(L.s, L.fs, L.nsrc, L.g.V, L.vs, c->st);
+    });
   seg_steps(c, L, j0, P.hi[t], next && P.hi[t] < L.k);
   launch_check();
 }
@@ -1010,6 +1027,15 @@ int block_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, d
     L.ue = ue;
   }
   L.mdir = (R)m_dir;
+  if constexpr (std::is_same<R, double>::value) {
+    int4* fe = wsT<int4>(c, B_FXDL, kFxLinkEntries * V);
+    short* fx = wsT<short>(c, B_FXDE, 5 * V);
+    L.fd = FxLinks{fe, fx};
+    run(c, OV_KIND_LAYOUT, 1, [&] {
+      pack_dh_links_fx(static_cast<const double*>(U), static_cast<const double*>(E), m_dir, fe, fx, V, L.ef, L.efinv,
+                       c->st);
+    });
+  }
   run(c, OV_KIND_LAYOUT, 1, [&] {
     pack_block_start<R>(static_cast<const double*>(top), static_cast<const double*>(bottom), L.r, L.s, nsrc, V,
                         L.vs, c->st);
@@ -1610,6 +1636,10 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
   B.gs_ring = wsT<R>(c, B_GS, (int64_t)m * nsrc * vs);
   B.gp_ring = wsT<R>(c, B_GP, (int64_t)m * nsrc * vs);
   B.hin = wsT<R>(c, B_HIN, (int64_t)nsrc * vs);
+  if constexpr (std::is_same<R, double>::value) {
+    B.fp = FxField{wsT<int4>(c, B_FXP, nsrc * (vs / 2)), wsT<short>(c, B_FXPE, nsrc * V)};
+    B.fh = FxField{wsT<int4>(c, B_FXH, nsrc * (vs / 2)), wsT<short>(c, B_FXHE, nsrc * V)};
+  }
   B.xbar = xb;
   B.y = y;
   B.gaT = gaT;
@@ -2278,7 +2308,12 @@ int apply_h_impl(ov_context* c, const int32_t dims[4], const void* U, double mu,
           [&] { unpack_spinors_il(L.p, static_cast<double*>(out), nsrc, L.g.V, c->st); });
     }
   }
-  if (!std::is_same<R, float>::value || var != APPLY_IL) {
+  if constexpr (std::is_same<R, double>::value) {
+    run(c, OV_KIND_LAYOUT, 1,
+        [&] { fx_pack(static_cast<const double*>(in), L.fr, L.r, nsrc, L.g.V, L.vs, c->st); });
+    run(c, OV_KIND_APPLY_H, 1,
+        [&] { fx_apply_h(L, L.fr, L.r, static_cast<double*>(out), dagger, 1, c->st, var); });
+  } else if (var != APPLY_IL) {
     run(c, OV_KIND_LAYOUT, 1,
         [&] { pack_spinors<R>(static_cast<const double*>(in), L.r, nsrc, L.g.V, L.vs, c->st); });
     run(c, OV_KIND_APPLY_H, 1, [&] { apply_h(L, L.r, L.p, dagger, c->st, var, aerr); });
@@ -2300,6 +2335,10 @@ int autotune_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   CK(cudaMemsetAsync(L.r, 0, sizeof(R) * nsrc * L.vs, c->st));
   CK(cudaMemsetAsync(L.s, 0, sizeof(R) * nsrc * L.vs, c->st));
   CK(cudaMemsetAsync(L.sc, 0, sizeof(SrcScal) * nsrc, c->st));
+  if constexpr (std::is_same<R, double>::value) {
+    fx_encode(L.r, L.fr, nsrc, L.g.V, L.vs, c->st);
+    fx_encode(L.s, L.fs, nsrc, L.g.V, L.vs, c->st);
+  }
   cudaEvent_t e0 = c->ev[6], e1 = c->ev[7];
   auto time_us = [&](auto&& launch) {
     launch();
