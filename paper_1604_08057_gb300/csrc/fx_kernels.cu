@@ -1,7 +1,11 @@
-// FP64 stencil kernels in block fixed point (fx.cuh): ov_apply_H, the two-sided
-// Lanczos step's H / H^dagger pair (plain and Theorem-1 block form) and the
-// reverse sweep's stencil.  Each falls back, site by site, to FP64 arithmetic
-// where the fixed-point form does not hold.
+// FP64 calls in block fixed point (fx.cuh): layout conversion, ov_apply_H, the forward
+// two-sided Lanczos recurrence with its Gram-Schmidt projections, and the reverse sweep
+// with the gauge force.  Every kernel reads and writes fixed-point fields; FP64 is left
+// for the recurrence's scalars and for what goes back to the caller.
+//
+// Two threads (spins sp and 2 + sp) share a site unless a kernel says otherwise; blocks
+// whose two halves treat the two sides of the recurrence (r and s, g_r and g_s) exchange
+// through shared memory.  All reductions are deterministic.
 #include "fx.cuh"
 #include "kernels.h"
 #include "recurrence.cuh"
@@ -9,6 +13,16 @@
 namespace ov {
 
 static inline unsigned nblocks(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
+
+// vector j of a basis
+__device__ __forceinline__ FxField fx_bv(const Lat<double>& L, int src, int j) {
+  const int64_t i = (int64_t)src * L.kcap + (j - L.jbase);
+  return FxField{reinterpret_cast<int4*>(L.bv) + i * (L.vs / 2), L.bve + i * (L.vs / 24)};
+}
+__device__ __forceinline__ FxField fx_bw(const Lat<double>& L, int src, int j) {
+  const int64_t i = (int64_t)src * L.kcap + (j - L.jbase);
+  return FxField{reinterpret_cast<int4*>(L.bw) + i * (L.vs / 2), L.bwe + i * (L.vs / 24)};
+}
 
 // ---------------------------------------------------------------------------
 // links in fixed point
@@ -73,7 +87,7 @@ __global__ void __launch_bounds__(128) k_pack_links_fx(const double* __restrict_
       r = fx_split(4 * fx_conv(hi[2 * q], ee) + __double2ll_rn(f2 * lo[2 * q]));
       i = fx_split(4 * fx_conv(hi[2 * q + 1], ee) + __double2ll_rn(f2 * lo[2 * q + 1]));
     }
-    out[(int64_t)(d * 9 + q) * V + x] = make_int4(r.h, r.l, i.h, i.l);
+    out[fx_link_at(x, d) + q * 32] = make_int4(r.h, r.l, i.h, i.l);
   }
 }
 void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, cudaStream_t st) {
@@ -85,43 +99,111 @@ void pack_dh_links_fx(const double* u, const double* e, double m, int4* out, sho
 }
 
 // ---------------------------------------------------------------------------
-// encoding FP64 fields
+// user fields [src][site][12] (complex128).  A warp's 16 sites are 3 KB in a row there:
+// both directions go through shared memory, so that global accesses are contiguous.
 // ---------------------------------------------------------------------------
-// user spinors [src][site][12] to fixed point; FP64 values (site-major) only where a site
-// is out of the window
-__global__ void __launch_bounds__(128) k_fx_pack(const double* __restrict__ aos, FxField f, double* __restrict__ d,
-                                                 int64_t V, int64_t vs) {
-  const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int src = blockIdx.y;
-  if (x >= V) return;
-  const double2* in = reinterpret_cast<const double2*>(aos) + ((int64_t)src * V + x) * 12;
-  Spinor<double> p;
+constexpr int kStage = 16 * 13;   // double2 per warp, rows padded by one
+__device__ __forceinline__ void aos_load(const double* aos, int64_t src, int64_t V, int64_t x0, double2* st, int sp,
+                                         zd (&p)[6]) {
+  const int lane = threadIdx.x & 31;
+  const int n = (int)min((int64_t)16, V - x0) * 12;
+  const double2* in = reinterpret_cast<const double2*>(aos) + (src * V + x0) * 12;
+  for (int i = lane; i < 192; i += 32) st[i / 12 * 13 + i % 12] = i < n ? in[i] : make_double2(0.0, 0.0);
+  __syncwarp();
 #pragma unroll
-  for (int c = 0; c < 12; ++c) {
-    const double2 t = in[c];
-    p.c[c] = mk(t.x, t.y);
+  for (int i = 0; i < 6; ++i) {
+    const double2 t = st[(lane & 15) * 13 + fx_comp(sp, i)];
+    p[i] = mk(t.x, t.y);
   }
-  if (fx_store(fx_src(f, src, vs, V), V, x, p)) store_spinor(d + src * vs, V, x, p);
+  __syncwarp();
 }
-void fx_pack(const double* aos, const FxField& f, double* d, int nsrc, int64_t V, int64_t vs, cudaStream_t st) {
-  k_fx_pack<<<dim3(nblocks(V, 128), nsrc), 128, 0, st>>>(aos, f, d, V, vs);
+__device__ __forceinline__ void aos_store(double* aos, int64_t src, int64_t V, int64_t x0, double2* st, int sp,
+                                          const zd (&p)[6]) {
+  const int lane = threadIdx.x & 31;
+  const int n = (int)min((int64_t)16, V - x0) * 12;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) st[(lane & 15) * 13 + fx_comp(sp, i)] = make_double2(p[i].re, p[i].im);
+  __syncwarp();
+  double2* o = reinterpret_cast<double2*>(aos) + (src * V + x0) * 12;
+  for (int i = lane; i < n; i += 32) o[i] = st[i / 12 * 13 + i % 12];
+  __syncwarp();
 }
-__global__ void __launch_bounds__(128) k_fx_encode(const double* __restrict__ d, FxField f, int64_t V, int64_t vs) {
-  const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+__device__ __forceinline__ void soa_store(double* f, int64_t V, int64_t s, int sp, const zd (&p)[6]) {
+  double2* q = reinterpret_cast<double2*>(f) + s;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) q[fx_comp(sp, i) * V] = make_double2(p[i].re, p[i].im);
+}
+
+// user spinors to fixed point, in f and (if set) g; marked sites keep FP64 values in d (if
+// set).  top (may be null) with block: the Theorem-1 start, f = (top, bot), g = (top + bot, bot)
+// in fields of 2V sites, bot in aos.
+__global__ void __launch_bounds__(128) k_fx_pack(const double* __restrict__ aos, const double* __restrict__ top,
+                                                 int block, FxField f, FxField g, double* __restrict__ d, int64_t V,
+                                                 int64_t vs) {
+  __shared__ double2 stage[4][kStage];
+  const int sp = fx_spin_of(threadIdx.x), w = threadIdx.x >> 5;
+  const int64_t x0 = blockIdx.x * (int64_t)64 + w * 16, x = x0 + (threadIdx.x & 15);
   const int src = blockIdx.y;
-  if (x >= V) return;
-  Spinor<double> p;
-  load_spinor_ro(d + src * vs, V, x, p);
-  fx_store(fx_src(f, src, vs, V), V, x, p);
+  if (x0 >= V) return;   // whole warps
+  const bool live = x < V;
+  const FxField fs = fx_src(f, src, vs), gs = g.c ? fx_src(g, src, vs) : g;
+  zd p[6];
+  FxH o;
+  aos_load(aos, src, V, x0, stage[w], sp, p);
+  fx_from_double(p, o);
+  if (live) {
+    fx_put(fs, block ? V + x : x, sp, o);
+    if (g.c) fx_put(gs, block ? V + x : x, sp, o);
+    if (d && o.e == FX_BAD) soa_store(d + src * vs, V, x, sp, p);
+  }
+  if (!block) return;
+  zd q[6];
+  if (top) {
+    aos_load(top, src, V, x0, stage[w], sp, q);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) q[i] = mk(0.0, 0.0);
+  }
+  fx_from_double(q, o);
+  if (live) fx_put(fs, x, sp, o);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) q[i] = q[i] + p[i];
+  fx_from_double(q, o);
+  if (live) fx_put(gs, x, sp, o);
+}
+void fx_pack(const double* aos, const FxField& f, const FxField& g, double* d, int nsrc, int64_t V, int64_t vs,
+             cudaStream_t st) {
+  k_fx_pack<<<dim3(nblocks(V, 64), nsrc), 128, 0, st>>>(aos, nullptr, 0, f, g, d, V, vs);
+}
+void fx_pack_block(const double* top, const double* bot, const FxField& f, const FxField& g, int nsrc, int64_t V,
+                   int64_t vs, cudaStream_t st) {
+  k_fx_pack<<<dim3(nblocks(V, 64), nsrc), 128, 0, st>>>(bot, top, 1, f, g, nullptr, V, vs);
+}
+// an FP64 site-major field to fixed point
+__global__ void __launch_bounds__(128) k_fx_encode(const double* __restrict__ d, FxField f, int64_t V, int64_t vs) {
+  const int sp = fx_spin_of(threadIdx.x);
+  const int64_t x = blockIdx.x * (int64_t)64 + fx_site_of(threadIdx.x);
+  const int src = blockIdx.y;
+  const bool live = x < V;
+  const double2* q = reinterpret_cast<const double2*>(d + src * vs);
+  zd p[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const double2 t = live ? q[fx_comp(sp, i) * V + x] : make_double2(0.0, 0.0);
+    p[i] = mk(t.x, t.y);
+  }
+  FxH o;
+  fx_from_double(p, o);
+  if (live) fx_put(fx_src(f, src, vs), x, sp, o);
 }
 void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t vs, cudaStream_t st) {
-  k_fx_encode<<<dim3(nblocks(V, 128), nsrc), 128, 0, st>>>(d, f, V, vs);
+  k_fx_encode<<<dim3(nblocks(V, 64), nsrc), 128, 0, st>>>(d, f, V, vs);
 }
 
 // ---------------------------------------------------------------------------
-// the site's hop sum a with out = psi - kappa a (upper spins), kappa a - psi (lower)
+// ov_apply_H
 // ---------------------------------------------------------------------------
-// FP64 form (out of line: reached only where a site or link is out of its window)
+// FP64 hop sum (out of line: reached only where a site or link is marked)
 __device__ __noinline__ void hops_fp64(const FxLoad& ld, const double* u, const Geom& g, int64_t x, double ft,
                                        double fti, Spinor<double>* a) {
   int c[4];
@@ -134,95 +216,58 @@ __device__ __noinline__ void hops_fp64(const FxLoad& ld, const double* u, const 
   hop_dir<3>(t, ld, u, g, x, c, ft, fti);
   *a = t;
 }
-// dH's hop sum added to a (dh_site_ld's result is -kappa times it on the upper spins)
-__device__ __noinline__ void dh_hops_fp64_add(const FxLoad& ld, const double* ue, const double* u, const Geom& g,
-                                              int64_t x, double ft, double fti, double m, Spinor<double>* a) {
-  Spinor<double> t;
-  dh_site_ld(ld, ue, u, g, x, 1.0, ft, fti, m, t);
-  for (int i = 0; i < 12; ++i) a->c[i] = i < 6 ? a->c[i] - t.c[i] : a->c[i] + t.c[i];
-}
-__device__ __forceinline__ void fx_double(const FxHalf& s, zd (&a)[6]) {
+__device__ __forceinline__ void fx_pick(const Spinor<double>& t, int sp, zd (&p)[6]) {
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    a[i] = mk((double)s.up[i].re, (double)s.up[i].im);
-    a[3 + i] = mk((double)s.lo[i].re, (double)s.lo[i].im);
+    p[i] = sp ? t.c[3 + i] : t.c[i];
+    p[3 + i] = sp ? t.c[9 + i] : t.c[6 + i];
   }
 }
-// the thread's six components of the hop sum of fixed-point field f, in units of the returned
-// power of two (1 from the FP64 form); d: the field's FP64 companion.  Every lane of the warp.
-__device__ __forceinline__ double hop_sum(const Lat<double>& L, const FxField& f, const double* d, int64_t x,
-                                          int dagger, int sp, bool live, zd (&a)[6]) {
-  FxHalf acc;
-  fx_zero(acc);
-  int E = 0;
-  if (live) {
-    const FxSite s(L.g, x);
-    fx_range(E, f, 0, L.fu, L.g, s, dagger);
-    if (E < FX_BAD) fx_hops(acc, E, f, L.g.V, 0, L.fu, L.g, s, dagger, sp);
-  }
-  fx_exchange(acc);
-  if (E >= FX_BAD) {
-    Spinor<double> t;
-    hops_fp64(FxLoad{f, d, L.g.V, 0}, L.u, L.g, x, dagger ? L.efinv : L.ef, dagger ? L.ef : L.efinv, &t);
-    fx_pick(t, sp, a);
-    return 1.0;
-  }
-  fx_double(acc, a);
-  return fx_pow2(E - FX_E_BIAS);
-}
 
-// thread t of a group of 2 n threads: site t / 32 * 16 + t % 16, spin (t / 16) % 2
-__device__ __forceinline__ int fx_site_of(int t) { return (t >> 5) * 16 + (t & 15); }
-__device__ __forceinline__ int fx_spin_of(int t) { return (t >> 4) & 1; }
-
-// ---------------------------------------------------------------------------
-// ov_apply_H: two threads per (site, source); blocks of blockDim.x / 2 sites x blockDim.y
-// sources, whose sources share the link loads through L1.  With aos the output is the
-// user's layout, written through shared memory (a warp's 16 sites are 3 KB in a row).
-// ---------------------------------------------------------------------------
+// Blocks of blockDim.x / 2 sites x blockDim.y sources, whose sources share the link loads
+// through L1.  With aos the output is the user's layout, else site-major.
 __global__ void __launch_bounds__(128, 4) k_fx_apply(const __grid_constant__ Lat<double> L, FxField in,
                                                      const double* __restrict__ din, double* __restrict__ out,
                                                      int dagger, int aos) {
-  __shared__ double2 stage[4][16 * 13];
+  __shared__ double2 stage[4][kStage];
   const int sp = fx_spin_of(threadIdx.x);
-  const int64_t x0 = blockIdx.x * (int64_t)(blockDim.x >> 1) + (threadIdx.x >> 5) * 16, x = x0 + (threadIdx.x & 15);
+  const int64_t x0 = blockIdx.x * (int64_t)(blockDim.x >> 1) + (threadIdx.x >> 5) * 16;
   const int src = blockIdx.y * blockDim.y + threadIdx.y;
   const int64_t V = L.g.V;
   if (src >= L.nsrc || x0 >= V) return;   // whole warps
-  const bool live = x < V;
-  const FxField f = fx_src(in, src, L.vs, V);
+  const bool live = x0 + (threadIdx.x & 15) < V;
+  const int64_t x = min(x0 + (threadIdx.x & 15), V - 1);
+  const FxField f = fx_src(in, src, L.vs);
   const double* d = din + (int64_t)src * L.vs;
+  const FxSite s(L.g, x);
+  FxHalf acc;
+  fx_zero(acc, fx_range(0, f, 0, L.fu, L.g, s, dagger));
+  const bool ok = acc.E < FX_BAD;
+  if (!ok) acc.E = FX_E_BIAS;
+  fx_hops(acc, f, 0, L.fu, L.g, s, dagger, sp);
   zd a[6];
-  const double ks = L.kappa * hop_sum(L, f, d, x, dagger, sp, live, a);
-  if (live) {
-    const int e = f.e[x];
-    const double u = e == FX_BAD ? 1.0 : fx_pow2(e - 1079);
+  if (ok) {
+    fx_double(acc, false, a);
+  } else {
+    Spinor<double> t;
+    hops_fp64(FxLoad{f, d, V, 0}, L.u, L.g, x, dagger ? L.efinv : L.ef, dagger ? L.ef : L.efinv, &t);
+    fx_pick(t, sp, a);
+  }
+  FxH c;
+  fx_load(f, x, sp, c);
+  const double u = fx_pow2(c.e == FX_BAD ? 0 : c.e - 1079);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      const int c = (i < 3 ? sp * 3 + i : (2 + sp) * 3 + i - 3);
-      zd p;
-      if (e == FX_BAD) {
-        const double2 t = reinterpret_cast<const double2*>(d)[c * V + x];
-        p = mk(t.x, t.y);
-      } else {
-        p = u * fx_value(__ldg(f.c + c * V + x));
-      }
-      const zd q = mk(fma(-ks, a[i].re, p.re), fma(-ks, a[i].im, p.im));
-      a[i] = i < 3 ? q : -q;
+  for (int i = 0; i < 6; ++i) {
+    zd p = mk(u * (double)fx_join(c.q[i].x, c.q[i].y), u * (double)fx_join(c.q[i].z, c.q[i].w));
+    if (c.e == FX_BAD) {
+      const double2 t = reinterpret_cast<const double2*>(d)[fx_comp(sp, i) * V + x];
+      p = mk(t.x, t.y);
     }
+    const zd q = mk(fma(-L.kappa, a[i].re, p.re), fma(-L.kappa, a[i].im, p.im));
+    a[i] = i < 3 ? q : -q;
   }
-  if (!aos) {
-    if (live) fx_store_half(out + (int64_t)src * L.vs, V, x, sp, a);
-    return;
-  }
-  double2* st = stage[(threadIdx.y * blockDim.x + threadIdx.x) >> 5];
-  const int lane = threadIdx.x & 31, ns = (int)min((int64_t)16, V - x0);
-#pragma unroll
-  for (int i = 0; i < 6; ++i)
-    st[(lane & 15) * 13 + (i < 3 ? sp * 3 + i : (2 + sp) * 3 + i - 3)] = make_double2(a[i].re, a[i].im);
-  __syncwarp();
-  double2* o = reinterpret_cast<double2*>(out) + ((int64_t)src * V + x0) * 12;
-  for (int i = lane; i < ns * 12; i += 32) o[i] = st[i / 12 * 13 + i % 12];
+  if (aos) aos_store(out, src, V, x0, stage[(threadIdx.y * blockDim.x + threadIdx.x) >> 5], sp, a);
+  else if (live) soa_store(out + (int64_t)src * L.vs, V, x, sp, a);
 }
 void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double* out, int dagger, int aos,
                 cudaStream_t st, int variant) {
@@ -245,12 +290,49 @@ void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double
 }
 
 // ---------------------------------------------------------------------------
-// TSL step j (see k_tsl_stencil): v_j = sv r, w_j = sw s, p = H v_j, q = H^dag w_j,
-// alpha_j = w_j^dag p.  A block of 4 SX threads covers SX (16 or 32) sites; its first
-// half of warps forms v_j and p, the second half w_j and q of the same sites, so the
-// links of both products come from L1 and a small lattice spreads over more warps.
-// w_j crosses to the first half through shared memory for the dot product.
+// forward recurrence
 // ---------------------------------------------------------------------------
+// start: beta_0 = ||r||, scales of v_1 and w_1 (see k_tsl_init)
+__global__ void __launch_bounds__(128) k_fx_init(const __grid_constant__ Lat<double> L) {
+  __shared__ zd scratch[2 * 32];
+  const int sp = fx_spin_of(threadIdx.x);
+  const int64_t x = blockIdx.x * (int64_t)64 + fx_site_of(threadIdx.x);
+  const int src = blockIdx.y;
+  zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
+  if (x < L.g.V) {
+    FxH r, s;
+    fx_load(fx_src(L.fr, src, L.vs), x, sp, r);
+    v[0] = mk(fx_norm2(r), 0.0);
+    if (L.block) {
+      fx_load(fx_src(L.fs, src, L.vs), x, sp, s);
+      v[1] = fx_dot(s, r);
+    }
+  }
+  block_sum<2>(v, scratch);
+  zd* part = L.part + src * L.part_stride;
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = v[0];
+    part[gridDim.x + blockIdx.x] = v[1];
+  }
+  if (arrive_last(L.cnt + src * 16 + 0, gridDim.x)) {
+    zd s[2];
+    sum_partials<2>(part, gridDim.x, s, scratch);
+    if (threadIdx.x == 0) init_finalize(L, src, s[0].re, s[1]);
+  }
+}
+void fx_tsl_init(const Lat<double>& L, cudaStream_t st) {
+  k_fx_init<<<dim3(nblocks(L.g.V, 64), L.nsrc), 128, 0, st>>>(L);
+}
+
+// +-(f + c t) of a thread's components: the lower spins negated (gamma5)
+__device__ __forceinline__ bool h_finish(FxHalf& o, const FxH& f, const FxCoef& c, const FxH& t) {
+  fx_zero(o, 0);
+  bool ok = fx_add(o, f);
+  ok = fx_axpy<1>(o, c, t) && ok;
+#pragma unroll
+  for (int i = 3; i < 6; ++i) o.v[i] = FxZ{-o.v[i].re, -o.v[i].im};
+  return ok;
+}
 __device__ __forceinline__ void alpha_finish(const Lat<double>& L, int src, int j, zd (&v)[1], zd* scratch) {
   block_sum<1>(v, scratch);
   zd* part = L.part + src * L.part_stride;
@@ -265,133 +347,115 @@ __device__ __forceinline__ void alpha_finish(const Lat<double>& L, int src, int 
     }
   }
 }
-// +-(p - kc a): the thread's six components of sc (H psi) from p = sc psi, a the hop sum, kc = kappa sc
-__device__ __forceinline__ void h_finish(zd (&p)[6], const zd (&a)[6], zd kc) {
+
+// Step j: v_j = sv r, w_j = sw s, p = H v_j, q = H^dag w_j, alpha_j = w_j^dag p.  A block of
+// 4 SX threads covers SX (16 or 32) sites; its first half of warps forms v_j and p, the
+// second half w_j and q of the same sites, so the links of both products come from L1 and
+// a small lattice spreads over more warps.  w_j crosses to the first half through shared
+// memory for the dot product.  H v_j = +-(v_j - kappa sv a) from the hop sum a of r.
+struct FxShare {
+  int4 q[6][64];
+  int e[64];
+};
+__device__ __forceinline__ void share_put(FxShare& s, int t, const FxH& f) {
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    zd q = mk(fma(-kc.re, a[i].re, p[i].re), fma(-kc.re, a[i].im, p[i].im));
-    if (kc.im != 0.0) q = mk(fma(kc.im, a[i].im, q.re), fma(-kc.im, a[i].re, q.im));
-    p[i] = i < 3 ? q : -q;
-  }
+  for (int i = 0; i < 6; ++i) s.q[i][t] = f.q[i];
+  s.e[t] = f.e;
+}
+__device__ __forceinline__ void share_get(const FxShare& s, int t, FxH& f) {
+#pragma unroll
+  for (int i = 0; i < 6; ++i) f.q[i] = s.q[i][t];
+  f.e = s.e[t];
 }
 
 __global__ void __launch_bounds__(128, 4) k_fx_tsl(const __grid_constant__ Lat<double> L, int j, int need_q) {
   __shared__ zd scratch[32];
-  __shared__ double2 ws[6][64];
+  __shared__ FxShare ws;
   const int half = blockDim.x >> 1;
   const bool left = threadIdx.x >= half;
   const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
-  const int64_t x = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t);
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
   const int src = blockIdx.y;
-  const int64_t V = L.g.V;
   zd v[1] = {mk(0.0, 0.0)};
-  const bool live = x < V && L.sc[src].err == 0;
-  zd o[6], a[6];
-  const double* d = (left ? L.s : L.r) + src * L.vs;
-  double* bas = left ? L.basis_w(src, j) : L.basis_v(src, j);
-  const zd sc = left ? L.sc[src].sw : L.sc[src].sv;
-  double unit = 0.0;
-  if (!left || need_q)
-    unit = hop_sum(L, fx_src(left ? L.fs : L.fr, src, L.vs, V), d, x, left ? 1 : 0, sp, live, a);
-  if (live) {
-    fx_load_half(d, V, x, sp, o);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      o[c] = sc.im != 0.0 ? sc * o[c] : mk(sc.re * o[c].re, sc.re * o[c].im);
-      if (left) ws[c][t] = make_double2(o[c].re, o[c].im);
-    }
-    fx_store_half(bas, V, x, sp, o);
+  const bool go = L.sc[src].err == 0, live = go && x0 < V;   // go: the whole block
+  FxH o, w;
+  if (go) {
+    const FxField f = fx_src(left ? L.fs : L.fr, src, L.vs);
+    const zd sc = left ? L.sc[src].sw : L.sc[src].sv;
+    FxHalf acc;
+    fx_load(f, x, sp, o);
+    fx_zero(acc, 0);
+    const bool okv = fx_axpy<1>(acc, fx_coef(sc), o);
+    fx_encode(acc, !okv, w);
+    if (live) fx_put(left ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, w);
+    if (left) share_put(ws, t, w);
     if (!left || need_q) {
-      const double ks = L.kappa * unit;
-      h_finish(o, a, mk(ks * sc.re, ks * sc.im));
-      fx_store_half((left ? L.q : L.p) + src * L.vs, V, x, sp, o);
+      const FxSite s(L.g, x);
+      const int dg = left ? 1 : 0;
+      fx_zero(acc, fx_range(0, f, 0, L.fu, L.g, s, dg));
+      const bool ok = acc.E < FX_BAD;
+      if (!ok) acc.E = FX_E_BIAS;
+      fx_hops(acc, f, 0, L.fu, L.g, s, dg, sp);
+      fx_encode(acc, !ok, o);
+      const bool okp = h_finish(acc, w, fx_coef(mk(-L.kappa * sc.re, -L.kappa * sc.im)), o);
+      fx_encode(acc, !okp, o);
+      if (live) fx_put(fx_src(left ? L.fq : L.fp, src, L.vs), x, sp, o);
     }
   }
   __syncthreads();
   if (live && !left) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      const double2 w = ws[c][t];
-      cdotac(v[0], mk(w.x, w.y), o[c]);
-    }
+    share_get(ws, t, w);
+    v[0] = fx_dot(w, o);
   }
   alpha_finish(L, src, j, v, scratch);
 }
 
-// Block step (see k_tsl_stencil_block): four warps of 16 sites,
+// Block step (Theorem 1; fields of 2V sites): four warps of 16 sites,
 //   0: p_u = H v_u + dH v_l   1: p_l = H v_l   2: q_u = H^dag w_u   3: q_l = dH^dag w_u + H^dag w_l
 __global__ void __launch_bounds__(128, 4) k_fx_tsl_block(const __grid_constant__ Lat<double> L, int j, int need_q) {
   __shared__ zd scratch[32];
-  __shared__ double2 ws[2][6][32];
+  __shared__ FxShare ws;
   const int t = threadIdx.x & 31, part_id = threadIdx.x >> 5, sp = fx_spin_of(t);
   const bool left = part_id >= 2, low = part_id & 1;
-  const int64_t x = blockIdx.x * (int64_t)16 + fx_site_of(t);
+  const int64_t V = L.gl.V, x0 = blockIdx.x * (int64_t)16 + fx_site_of(t), x = min(x0, V - 1);
   const int src = blockIdx.y;
-  const int64_t V = L.gl.V, Vf = L.g.V;
   const int off = low ? (int)V : 0, offx = low ? 0 : (int)V;
   const bool cross = part_id == 0 || part_id == 3;   // adds dH of the other half
   zd v[1] = {mk(0.0, 0.0)};
-  const bool live = x < V && L.sc[src].err == 0;
-  zd o[6], a[6];
-  const double* d = (left ? L.s : L.r) + src * L.vs;
-  double* bas = left ? L.basis_w(src, j) : L.basis_v(src, j);
-  const zd sc = left ? L.sc[src].sw : L.sc[src].sv;
-  double unit = 0.0;
-  if (!left || need_q) {
-    const FxField f = fx_src(left ? L.fs : L.fr, src, L.vs, Vf);
-    const int dg = left ? 1 : 0;
+  const bool go = L.sc[src].err == 0, live = go && x0 < V;
+  FxH o, w;
+  if (go) {
+    const FxField f = fx_src(left ? L.fs : L.fr, src, L.vs);
+    const zd sc = left ? L.sc[src].sw : L.sc[src].sv;
     FxHalf acc;
-    fx_zero(acc);
-    int E = 0;
-    if (live) {
-      const FxSite s(L.gl, x);
-      fx_range(E, f, off, L.fu, L.gl, s, dg);
-      if (cross) {
-        fx_range(E, f, offx, L.fd, L.gl, s, dg);
-        ++E;   // sixteen hops
-      }
-      if (E < FX_BAD)
-        for (int h = 0; h < (cross ? 2 : 1); ++h)
-          fx_hops(acc, E, f, Vf, h ? offx : off, h ? L.fd : L.fu, L.gl, s, dg, sp);
-    }
-    fx_exchange(acc);
-    if (E < FX_BAD) {
-      fx_double(acc, a);
-      unit = fx_pow2(E - FX_E_BIAS);
-    } else {
-      const double ft = left ? L.efinv : L.ef, fti = left ? L.ef : L.efinv;
-      Spinor<double> b;
-      hops_fp64(FxLoad{f, d, Vf, off}, L.u, L.gl, x, ft, fti, &b);
-      if (cross) dh_hops_fp64_add(FxLoad{f, d, Vf, offx}, L.ue, L.u, L.gl, x, ft, fti, left ? -L.mdir : L.mdir, &b);
-      fx_pick(b, sp, a);
-      unit = 1.0;
-    }
-  }
-  if (live) {
-    fx_load_half(d, Vf, off + x, sp, o);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      o[c] = sc * o[c];
-      if (left) ws[low][c][t] = make_double2(o[c].re, o[c].im);
-    }
-    fx_store_half(bas, Vf, off + x, sp, o);
+    fx_load(f, off + x, sp, o);
+    fx_zero(acc, 0);
+    const bool okv = fx_axpy<1>(acc, fx_coef(sc), o);
+    fx_encode(acc, !okv, w);
+    if (live) fx_put(left ? fx_bw(L, src, j) : fx_bv(L, src, j), off + x, sp, w);
+    if (left) share_put(ws, low * 32 + t, w);
     if (!left || need_q) {
-      const double ks = L.kappa * unit;
-      h_finish(o, a, mk(ks * sc.re, ks * sc.im));
-      fx_store_half((left ? L.q : L.p) + src * L.vs, Vf, off + x, sp, o);
+      const FxSite s(L.gl, x);
+      const int dg = left ? 1 : 0;
+      int E = fx_range(0, f, off, L.fu, L.gl, s, dg);
+      if (cross) E = fx_range(E, f, offx, L.fd, L.gl, s, dg) + 1;   // sixteen hops
+      const bool ok = E < FX_BAD;
+      fx_zero(acc, ok ? E : FX_E_BIAS);
+      for (int h = 0; h < (cross ? 2 : 1); ++h)
+        fx_hops(acc, f, h ? offx : off, h ? L.fd : L.fu, L.gl, s, dg, sp);
+      fx_encode(acc, !ok, o);
+      const bool okp = h_finish(acc, w, fx_coef(mk(-L.kappa * sc.re, -L.kappa * sc.im)), o);
+      fx_encode(acc, !okp, o);
+      if (live) fx_put(fx_src(left ? L.fq : L.fp, src, L.vs), off + x, sp, o);
     }
   }
   __syncthreads();
   if (live && !left) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      const double2 w = ws[low][c][t];
-      cdotac(v[0], mk(w.x, w.y), o[c]);
-    }
+    share_get(ws, low * 32 + t, w);
+    v[0] = fx_dot(w, o);
   }
   alpha_finish(L, src, j, v, scratch);
 }
-
 void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st, int variant) {
   if (L.block) {
     k_fx_tsl_block<<<dim3(nblocks(L.gl.V, 16), L.nsrc), 128, 0, st>>>(L, j, need_q);
@@ -403,140 +467,747 @@ void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st, in
   k_fx_tsl<<<dim3(nblocks(V, sx), L.nsrc), 4 * sx, 0, st>>>(L, j, need_q);
 }
 
+// r = p - alpha_j v_j - beta_j v_{j-1};  s = q - conj(alpha_j) w_j - delta_j w_{j-1}.  The two
+// halves of a block's threads form r and s of the same SX (16 or 32) sites; s crosses to
+// the first half for s^dag r.
+__device__ __forceinline__ void omega_finish(const Lat<double>& L, int src, int j, int slot, zd (&v)[2], zd* scratch) {
+  block_sum<2>(v, scratch);   // v[0] = s^dag r, v[1] = (|r|^2, |s|^2)
+  zd* part = L.part + src * L.part_stride;
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = v[0];
+    part[gridDim.x + blockIdx.x] = v[1];
+  }
+  if (arrive_last(L.cnt + src * 16 + slot, gridDim.x)) {
+    zd s[2];
+    sum_partials<2>(part, gridDim.x, s, scratch);
+    if (threadIdx.x == 0 && L.sc[src].err == 0) omega_finalize(L, src, j, s[0], s[1].re, s[1].im);
+  }
+}
+__global__ void __launch_bounds__(128, 4) k_fx_update(const __grid_constant__ Lat<double> L, int j, int finalize) {
+  __shared__ zd scratch[2 * 32];
+  __shared__ FxShare ws;
+  __shared__ FxCoef cs[2][2];
+  const int half = blockDim.x >> 1;
+  const int left = threadIdx.x >= half;
+  const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
+  const int src = blockIdx.y;
+  zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
+  const bool go = L.sc[src].err == 0, live = go && x0 < V;
+  if (go && t == 0) {
+    const int64_t o = (int64_t)src * L.k + j;
+    const zd al = L.alpha[o];
+    cs[left][0] = fx_coef(left ? -conj(al) : -al);
+    cs[left][1] = fx_coef(j == 0 ? mk(0.0, 0.0) : left ? mk(-L.delta[o], 0.0) : -L.beta[o]);
+  }
+  __syncthreads();
+  FxH f;
+  if (go) {
+    FxHalf acc;
+    fx_zero(acc, 0);
+    fx_load(fx_src(left ? L.fq : L.fp, src, L.vs), x, sp, f);
+    bool ok = fx_add(acc, f);
+    // what is left of p below 2^-53 of it is its coefficients' rounding: an exact breakdown
+    // (r = 0) stays one
+    const int zero_top = f.e + 1078 - 53;
+    fx_load(left ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, f);
+    ok = fx_axpy<1>(acc, cs[left][0], f) && ok;
+    if (j > 0) {
+      fx_load(left ? fx_bw(L, src, j - 1) : fx_bv(L, src, j - 1), x, sp, f);
+      ok = fx_axpy<1>(acc, cs[left][1], f) && ok;
+    }
+    fx_encode(acc, !ok, f, zero_top);
+    if (live) fx_put(fx_src(left ? L.fs : L.fr, src, L.vs), x, sp, f);
+  }
+  if (!finalize) return;   // uniform across the grid
+  if (left && go) share_put(ws, t, f);
+  __syncthreads();
+  if (live) {
+    if (left) {
+      v[1] = mk(0.0, fx_norm2(f));
+    } else {
+      FxH s;
+      share_get(ws, t, s);
+      v[0] = fx_dot(s, f);
+      v[1] = mk(fx_norm2(f), 0.0);
+    }
+  }
+  omega_finish(L, src, j, 2, v, scratch);
+}
+static inline int two_sided_sites(const Lat<double>& L) { return L.g.V * L.nsrc < 152 * 32 ? 16 : 32; }
+void fx_tsl_update(const Lat<double>& L, int j, int finalize, cudaStream_t st) {
+  const int sx = two_sided_sites(L);
+  k_fx_update<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, j, finalize);
+}
+
 // ---------------------------------------------------------------------------
-// Reverse sweep, gradients of v_j and w_j (see k_rev_stencil):
-//   Gv_j = H^dag g_p  + sum_i c_i f_i,    Gw_j = H h_in + sum_i c'_i f'_i
-// with f over xbar, g_r, the previous g_r and w_{jm+1} of the recorded projections
-// (g_s, previous g_s and v_{jm+1} for Gw).  The sums run in the same fixed-point
-// accumulator as the hops: with c_i / kappa as coefficients,
-//   G = +-(p - kappa [hops -+ sum_i (c_i / kappa) f_i])   (upper / lower spins).
-// One half of a block's warps forms Gv, the other Gw, of the same SX (16 or 32) sites.
-// The coefficients are converted once per block, RT terms at a time.
+// Gram-Schmidt projections (see k_proj_dots for the modes and coefficient layout)
 // ---------------------------------------------------------------------------
-struct RevTerm {
-  const double* f;
-  zd c;           // coefficient in FP64
-  FxCoef k;       // c / kappa
+// conj(b) a over all twelve components of a site: |hh| < 24 2^54, |x| < 48 2^56
+struct FxS {
+  int4 q[12];
+  int e;
 };
-// term i of side (0: Gv, 1: Gw) of step j
-__device__ __forceinline__ void rev_term(const Lat<double>& L, const Rev<double>& B, int src, int side, int j,
-                                         int slot, int prev, int i, RevTerm& t) {
+__device__ __forceinline__ void fx_load_site(const FxField& f, int64_t s, FxS& o) {
+  const int4* p = f.c + fx_at(s);
+#pragma unroll
+  for (int i = 0; i < 12; ++i) o.q[i] = p[i * 32];
+  o.e = f.e[s];
+}
+constexpr int FX_NB = 8;   // basis vectors per block
+// One thread per site (spt sites in turn), one side per block: side 0 dots DA with a, side 1
+// DB with b.  a's integers stay in registers while FX_NB basis vectors stream past; each
+// thread's FP64 sums live in shared memory, so the loop over them stays rolled.
+__global__ void __launch_bounds__(128, 3) k_fx_dots(const __grid_constant__ Lat<double> L, int nb, int mode, FxField a,
+                                                    FxField b, int64_t ab_stride, zd* __restrict__ cpart,
+                                                    int64_t cp_stride, int spt, int ioff, int sides) {
+  __shared__ zd acc[FX_NB][128];
+  __shared__ zd red[4][FX_NB];
+  const int src = blockIdx.z / sides, side = blockIdx.z % sides;
+  const int i0 = blockIdx.y * FX_NB, n = min(FX_NB, nb - i0);
+  const int64_t V = L.g.V;
+  const FxField f = fx_src(side ? b : a, src, ab_stride);
+  const bool usew = (mode == 0) == (side == 0);
+  for (int i = 0; i < n; ++i) acc[i][threadIdx.x] = mk(0.0, 0.0);
+  for (int q = 0; q < spt; ++q) {
+    const int64_t x = (blockIdx.x * (int64_t)spt + q) * 128 + threadIdx.x;
+    if (x >= V) break;
+    FxS u;
+    fx_load_site(f, x, u);
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      FxS w;
+      fx_load_site(usew ? fx_bw(L, src, ioff + i0 + i) : fx_bv(L, src, ioff + i0 + i), x, w);
+      FxAcc t{0, 0, 0, 0};
+#pragma unroll
+      for (int c = 0; c < 12; ++c) fx_cdot(t, w.q[c], u.q[c]);
+      const double un = w.e == FX_BAD || u.e == FX_BAD ? fx_nan() : fx_pow2_wide(w.e + u.e - 2158 + 57);
+      zd s = acc[i][threadIdx.x];
+      s.re = fma(un, (double)((t.hr << 3) + (t.xr >> 27)), s.re);
+      s.im = fma(un, (double)((t.hi << 3) + (t.xi >> 27)), s.im);
+      acc[i][threadIdx.x] = s;
+    }
+  }
+  for (int i = 0; i < n; ++i) {
+    const zd s = warp_sum(acc[i][threadIdx.x]);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][i] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < n) {
+    zd s = red[0][threadIdx.x];
+    for (int w = 1; w < 4; ++w) s = s + red[w][threadIdx.x];
+    cpart[src * cp_stride + (int64_t)(2 * (i0 + threadIdx.x) + side) * gridDim.x + blockIdx.x] = s;
+  }
+}
+// one warp per coefficient: its site blocks' partials in lane-strided order, then a fixed tree
+__global__ void __launch_bounds__(128) k_fx_dots_reduce(const zd* __restrict__ cpart, int64_t cp_stride, int nsb, int nb,
+                                                        zd* __restrict__ coef, int64_t coef_stride, int sides) {
+  const int i = (blockIdx.x * 4 + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
+  const int src = blockIdx.y;
+  if (i >= nb * sides) return;
+  const int t = sides == 2 ? i : 2 * i;
+  const zd* cp = cpart + src * cp_stride + (int64_t)t * nsb;
+  zd s = mk(0.0, 0.0);
+  for (int b = lane; b < nsb; b += 32) s = s + cp[b];
+  s = warp_sum(s);
+  if (lane == 0) coef[src * coef_stride + t] = s;
+}
+void fx_proj_dots(const Lat<double>& L, int j0, int nb, int mode, const FxField& a, const FxField& b,
+                  int64_t ab_stride, zd* coef, zd* cpart, cudaStream_t st) {
+  // four sites per thread once a vector has enough sites for that to leave two blocks per
+  // SM to eight basis vectors (the block's reduction then costs a quarter per site)
+  const int spt = L.g.V >= 32768 ? 4 : 1, sides = b.c ? 2 : 1;
+  const unsigned nsb = nblocks(L.g.V, 128 * spt);
+  const int64_t cp_stride = (int64_t)2 * L.k * nsb;
+  k_fx_dots<<<dim3(nsb, nblocks(nb, FX_NB), L.nsrc * sides), 128, 0, st>>>(L, nb, mode, a, b, ab_stride, cpart,
+                                                                           cp_stride, spt, j0, sides);
+  k_fx_dots_reduce<<<dim3(nblocks(nb * sides, 4), L.nsrc), 128, 0, st>>>(cpart, cp_stride, nsb, nb, coef,
+                                                                         2 * (int64_t)L.k, sides);
+}
+
+// ---------------------------------------------------------------------------
+// reverse sweep (see the k_rev_* kernels of the FP32 form for the equations)
+// ---------------------------------------------------------------------------
+// one of a ring's slots, or a per-source field of the sweep
+__device__ __forceinline__ FxField ring_at(const Lat<double>& L, const FxField& f, int slot, int src) {
+  return fx_src(f, slot * L.nsrc + src, L.vs);
+}
+// D1 = v_j^dag g_r, D2 = w_j^dag g_s, D3 = v_{j-1}^dag g_r, D4 = w_{j-1}^dag g_s -> g_alpha and
+// the carries; g: this thread's g_r (left = 0) or g_s (left = 1)
+__device__ __forceinline__ void rev_alpha_finish(const Lat<double>& L, const Rev<double>& B, int src, int j, int left,
+                                                 bool live, int64_t x, int sp, const FxH& g, int slot, zd* scratch) {
+  zd v[4] = {mk(0.0, 0.0), mk(0.0, 0.0), mk(0.0, 0.0), mk(0.0, 0.0)};
+  if (live) {
+    FxH e;
+    fx_load(left ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, e);
+    const zd d0 = fx_dot(e, g);
+    zd d1 = mk(0.0, 0.0);
+    if (j > 0) {
+      fx_load(left ? fx_bw(L, src, j - 1) : fx_bv(L, src, j - 1), x, sp, e);
+      d1 = fx_dot(e, g);
+    }
+    v[0] = left ? v[0] : d0;
+    v[1] = left ? d0 : v[1];
+    v[2] = left ? v[2] : d1;
+    v[3] = left ? d1 : v[3];
+  }
+  block_sum<4>(v, scratch);
+  zd* part = L.part + src * L.part_stride;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < 4; ++i) part[i * gridDim.x + blockIdx.x] = v[i];
+  if (arrive_last(L.cnt + src * 16 + slot, gridDim.x)) {
+    zd s[4];
+    sum_partials<4>(part, gridDim.x, s, scratch);
+    if (threadIdx.x == 0) alpha_epilogue(L, B, src, j, s);
+  }
+}
+
+// A long sum of coefficient times field, kept as (hh, x) pairs: per term only the products,
+// the coefficient being shifted to the sum's scale.  A term adds less than 2^57 to hh and
+// 2^59.4 to x: x is folded into hh after eight, and hh scaled down when it may pass 2^60.
+struct FxTerms {
+  FxAcc t[6];
+  int E, n;
+  bool ok;
+  __device__ __forceinline__ void init() {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) t[i] = FxAcc{0, 0, 0, 0};
+    E = 0;
+    n = 0;
+    ok = true;
+  }
+  __device__ __forceinline__ void fold() {
+    int m = 0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      t[i].hr += (t[i].xr + (1ll << 29)) >> 30;
+      t[i].hi += (t[i].xi + (1ll << 29)) >> 30;
+      t[i].xr = t[i].xi = 0;
+      m |= fx_top(FxZ{t[i].hr, t[i].hi});
+    }
+    n = 0;
+    if (m >= (1 << 28)) down(2);
+  }
+  __device__ __forceinline__ void down(int sh) {
+    const fxll r = (1ll << sh) >> 1;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      t[i].hr = (t[i].hr + r) >> sh;
+      t[i].hi = (t[i].hi + r) >> sh;
+      t[i].xr = (t[i].xr + r) >> sh;
+      t[i].xi = (t[i].xi + r) >> sh;
+    }
+    E += sh;
+  }
+  __device__ __forceinline__ void add(const FxCoef& c, const FxH& f) {
+    if (f.e == FX_BAD || c.e == FX_BAD) {
+      ok = false;
+      return;
+    }
+    const int et = f.e + c.e;
+    if (et > E) {
+      down(min(et - E, 62));
+      E = et;
+    }
+    const int d = E - et;
+    if (d > 59) return;
+    const fxll half = (1ll << d) >> 1;
+    const FxInt a = fx_split((fx_join(c.c.x, c.c.y) + half) >> d), b = fx_split((fx_join(c.c.z, c.c.w) + half) >> d);
+    const int4 k = make_int4(a.h, a.l, b.h, b.l);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) fx_cmac(t[i], k, f.q[i]);
+    if (++n == 8) fold();
+  }
+  // the sum, below 2^60.6 units
+  __device__ __forceinline__ void value(FxHalf& o) {
+    fold();
+#pragma unroll
+    for (int i = 0; i < 6; ++i) o.v[i] = FxZ{t[i].hr, t[i].hi};
+    o.E = E;
+  }
+};
+// a -= b (a below 2^61, b below 2^60.6 units of their scales)
+__device__ __forceinline__ void fx_subtract(FxHalf& a, FxHalf& b) {
+  if (b.E > a.E) fx_raise(a, b.E);
+  const int sh = min(a.E - b.E, 62);
+  const fxll r = (1ll << sh) >> 1;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    a.v[i].re -= (b.v[i].re + r) >> sh;
+    a.v[i].im -= (b.v[i].im + r) >> sh;
+  }
+}
+
+constexpr int FX_CH = 32;   // coefficients converted at a time per side
+// a -= sum_i coefA_i UA_i by the first half of a block's threads, b -= sum_i coefB_i UB_i by
+// the second, for the same SX sites.  fin 1: omega and the next scales (a = r, b = s); fin 2:
+// the four dots of the reverse step (a = g_r, b = g_s).
+__global__ void __launch_bounds__(128, 3) k_fx_proj_update(const __grid_constant__ Lat<double> L,
+                                                           const __grid_constant__ Rev<double> B, int nb, int mode,
+                                                           FxField a, FxField b, int64_t ab_stride,
+                                                           const zd* __restrict__ coef, int64_t coef_stride, int j,
+                                                           int fin) {
+  __shared__ zd scratch[4 * 32];
+  __shared__ FxShare ws;
+  __shared__ FxCoef cs[2][FX_CH];
+  const int half = blockDim.x >> 1;
+  const int left = threadIdx.x >= half;
+  const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
+  const int src = blockIdx.y;
+  const bool live = x0 < V;
+  const bool usev = (mode == 0) == (left == 0);
+  const zd* cf = coef + src * coef_stride;
+  FxTerms T;
+  T.init();
+  for (int i0 = 0; i0 < nb; i0 += FX_CH) {
+    const int n = min(FX_CH, nb - i0);
+    __syncthreads();
+    for (int i = t; i < n; i += half) cs[left][i] = fx_coef(cf[2 * (i0 + i) + left]);
+    __syncthreads();
+    FxField u = usev ? fx_bv(L, src, i0) : fx_bw(L, src, i0);
+#pragma unroll 2
+    for (int i = 0; i < n; ++i) {
+      FxH f;
+      fx_load(u, x, sp, f);
+      T.add(cs[left][i], f);
+      u.c += L.vs / 2;
+      u.e += L.vs / 24;
+    }
+  }
+  const FxField fa = fx_src(left ? b : a, src, ab_stride);
+  FxH f;
+  {
+    FxHalf acc, s;
+    T.value(s);
+    fx_load(fa, x, sp, f);
+    fx_zero(acc, 0);
+    const bool ok = fx_add(acc, f) && T.ok;
+    fx_subtract(acc, s);
+    fx_encode(acc, !ok, f);
+    if (live) fx_put(fa, x, sp, f);
+  }
+  if (fin == 0) return;
+  if (fin == 1) {
+    zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
+    if (left) share_put(ws, t, f);
+    __syncthreads();
+    if (live) {
+      if (left) {
+        v[1] = mk(0.0, fx_norm2(f));
+      } else {
+        FxH s;
+        share_get(ws, t, s);
+        v[0] = fx_dot(s, f);
+        v[1] = mk(fx_norm2(f), 0.0);
+      }
+    }
+    omega_finish(L, src, j, 3, v, scratch);
+    return;
+  }
+  rev_alpha_finish(L, B, src, j, left, live, x, sp, f, 6, scratch);
+}
+void fx_proj_update(const Lat<double>& L, const Rev<double>* B, int nb, int mode, const FxField& a, const FxField& b,
+                    int64_t ab_stride, const zd* coef, int j, int fin, cudaStream_t st) {
+  const int sx = two_sided_sites(L);
+  k_fx_proj_update<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, B ? *B : Rev<double>{}, nb, mode, a, b,
+                                                                        ab_stride, coef, 2 * (int64_t)L.k, j, fin);
+}
+
+// out[src] (+)= sum_{j0 <= i < j0 + nvec} y_i u_i in the user's layout, u = V (side 0) or W;
+// y at ystride per source, sources src0, src0 + 1, ...
+__global__ void __launch_bounds__(128, 3) k_fx_combine(const __grid_constant__ Lat<double> L, int src0, int side, int j0,
+                                                       int nvec, const zd* __restrict__ y, int64_t ystride,
+                                                       double* __restrict__ out, int accumulate) {
+  __shared__ double2 stage[4][kStage];
+  __shared__ FxCoef cs[64];
+  const int sp = fx_spin_of(threadIdx.x), w = threadIdx.x >> 5;
+  const int64_t V = L.g.V, xw = blockIdx.x * (int64_t)(blockDim.x >> 1) + w * 16;
+  const int64_t x = min(xw + (threadIdx.x & 15), V - 1);
+  FxTerms T;
+  T.init();
+  for (int i0 = 0; i0 < nvec; i0 += 64) {
+    const int n = min(64, nvec - i0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) cs[i] = fx_coef(y[blockIdx.y * ystride + j0 + i0 + i]);
+    __syncthreads();
+    FxField u = side ? fx_bw(L, src0 + blockIdx.y, j0 + i0) : fx_bv(L, src0 + blockIdx.y, j0 + i0);
+#pragma unroll 2
+    for (int i = 0; i < n; ++i) {
+      FxH f;
+      fx_load(u, x, sp, f);
+      T.add(cs[i], f);
+      u.c += L.vs / 2;
+      u.e += L.vs / 24;
+    }
+  }
+  if (xw >= V) return;   // whole warps
+  FxHalf s;
+  T.value(s);
+  zd o[6];
+  fx_double(s, !T.ok, o);
+  if (accumulate) {
+    zd p[6];
+    aos_load(out, blockIdx.y, V, xw, stage[w], sp, p);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) o[i] = p[i] + o[i];
+  }
+  aos_store(out, blockIdx.y, V, xw, stage[w], sp, o);
+}
+void fx_combine(const Lat<double>& L, int src0, int nsrc, int side, int j0, int nvec, const zd* y, int64_t ystride,
+                double* out, int accumulate, cudaStream_t st) {
+  const int bs = L.g.V * nsrc < 152 * 64 ? 32 : 128;
+  k_fx_combine<<<dim3(nblocks(L.g.V, bs / 2), nsrc), bs, 0, st>>>(L, src0, side, j0, nvec, y, ystride, out,
+                                                                  accumulate);
+}
+
+// ---------------------------------------------------------------------------
+// reverse sweep, continued
+// ---------------------------------------------------------------------------
+// g_r = cr1 Gv + cr2 w_{j+1}, g_s = cs1 Gw + cs2 v_{j+1} into the ring slot (first and second
+// half of a block's threads), and with with_dots the four dots for g_alpha
+__global__ void __launch_bounds__(128, 4) k_fx_rev_form(const __grid_constant__ Lat<double> L,
+                                                        const __grid_constant__ Rev<double> B, int j, int slot,
+                                                        int with_dots) {
+  __shared__ zd scratch[4 * 32];
+  __shared__ FxCoef cs[2][2];
+  const int half = blockDim.x >> 1;
+  const int left = threadIdx.x >= half;
+  const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
+  const int src = blockIdx.y;
+  const bool live = x0 < V;
+  if (t < 2) {
+    const SrcScal& sc = L.sc[src];
+    cs[left][t] = fx_coef(left ? (t ? sc.cs2 : sc.cs1) : (t ? sc.cr2 : sc.cr1));
+  }
+  __syncthreads();
+  FxHalf acc;
+  FxH f;
+  fx_zero(acc, 0);
+  fx_load(fx_src(left ? B.fgw : B.fgv, src, L.vs), x, sp, f);
+  bool ok = fx_axpy<1>(acc, cs[left][0], f);
+  fx_load(left ? fx_bv(L, src, j + 1) : fx_bw(L, src, j + 1), x, sp, f);
+  ok = fx_axpy<1>(acc, cs[left][1], f) && ok;
+  fx_encode(acc, !ok, f);
+  if (live) fx_put(ring_at(L, left ? B.fgs : B.fgr, slot, src), x, sp, f);
+  if (!with_dots) return;
+  rev_alpha_finish(L, B, src, j, left, live, x, sp, f, 5, scratch);
+}
+void fx_rev_form(const Lat<double>& L, const Rev<double>& B, int j, int slot, int with_dots, cudaStream_t st) {
+  const int sx = two_sided_sites(L);
+  k_fx_rev_form<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, B, j, slot, with_dots);
+}
+
+// the two stencil inputs of step j: g_p = g_r + g_alpha w_j (first half), h_in = conj(g_alpha)
+// v_j + g_s (second half); g_r and g_s are absent at the last step
+__global__ void __launch_bounds__(128, 4) k_fx_rev_combine(const __grid_constant__ Lat<double> L,
+                                                           const __grid_constant__ Rev<double> B, int j, int slot) {
+  const int half = blockDim.x >> 1;
+  const int left = threadIdx.x >= half;
+  const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
+  const int src = blockIdx.y;
+  const zd ga = L.sc[src].g_alpha;
+  FxHalf acc;
+  FxH f;
+  fx_zero(acc, 0);
+  fx_load(left ? fx_bv(L, src, j) : fx_bw(L, src, j), x, sp, f);
+  bool ok = fx_axpy<1>(acc, fx_coef(left ? conj(ga) : ga), f);
+  if (j < L.k - 1) {
+    fx_load(ring_at(L, left ? B.fgs : B.fgr, slot, src), x, sp, f);
+    ok = fx_add(acc, f) && ok;
+  }
+  fx_encode(acc, !ok, f);
+  if (x0 < V) fx_put(left ? fx_src(B.fh, src, L.vs) : ring_at(L, B.fgp, slot, src), x, sp, f);
+}
+void fx_rev_combine(const Lat<double>& L, const Rev<double>& B, int j, int slot, cudaStream_t st) {
+  const int sx = two_sided_sites(L);
+  k_fx_rev_combine<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, B, j, slot);
+}
+
+// Gradients of v_j and w_j:
+//   Gv_j = H^dag g_p  + sum_i c_i f_i,    Gw_j = H h_in + sum_i c'_i f'_i
+// with f over xbar, g_r, the previous g_r and w_{jm+1} of the recorded projections (g_s,
+// previous g_s and v_{jm+1} for Gw); first and second half of a block's threads.  The sum of
+// the terms, with coefficients c / kappa, joins the hop sum a:
+//   G = +-(p - kappa [a -+ sum_i (c_i / kappa) f_i])   (upper / lower spins).
+// Then, for j > 0, v_j^dag Gv_j and w_j^dag Gw_j give step j - 1 its coefficients.
+__device__ __forceinline__ FxField rev_term(const Lat<double>& L, const Rev<double>& B, int src, int side, int j,
+                                            int slot, int prev, int i, zd* c) {
   const int64_t o = (int64_t)src * L.k + j;
-  const bool carry = j < L.k - 1, pcarry = prev >= 0 && j + 1 < L.k - 1;
   if (side == 0) {
     if (i == 0) {
-      t.f = B.xbar + src * L.vs;
-      t.c = conj(B.y[o]);
-      return;
+      *c = conj(B.y[o]);
+      return fx_src(B.fxb, src, L.vs);
     }
     --i;
   }
-  if (carry) {
+  if (j < L.k - 1) {
     if (i == 0) {
-      t.f = B.ring(side ? B.gs_ring : B.gr_ring, slot, src);
-      t.c = side ? -L.alpha[o] : -conj(L.alpha[o]);
-      return;
+      *c = side ? -L.alpha[o] : -conj(L.alpha[o]);
+      return ring_at(L, side ? B.fgs : B.fgr, slot, src);
     }
     --i;
   }
-  if (pcarry) {
+  if (prev >= 0 && j + 1 < L.k - 1) {
     if (i == 0) {
-      t.f = B.ring(side ? B.gs_ring : B.gr_ring, prev, src);
-      t.c = side ? mk(-L.delta[o + 1], 0.0) : -conj(L.beta[o + 1]);
-      return;
+      *c = side ? mk(-L.delta[o + 1], 0.0) : -conj(L.beta[o + 1]);
+      return ring_at(L, side ? B.fgs : B.fgr, prev, src);
     }
     --i;
   }
   const int jm = B.reb_steps[i];
   const int64_t eo = src * (int64_t)B.nreb_max * L.k + (int64_t)i * L.k + j;
-  t.f = side ? L.basis_v(src, jm + 1) : L.basis_w(src, jm + 1);
-  t.c = side ? B.ew[eo] : B.ev[eo];
+  *c = side ? B.ew[eo] : B.ev[eo];
+  return side ? fx_bv(L, src, jm + 1) : fx_bw(L, src, jm + 1);
 }
-// G of one site and side in FP64 (reached only outside the exponent windows)
-__device__ __noinline__ void rev_site_fp64(const Lat<double>& L, const Rev<double>& B, int src, int side, int j,
-                                           int slot, int prev, int nterms, int64_t x, Spinor<double>* out) {
-  const int64_t V = L.g.V;
-  const FxLoad ld{fx_src(side ? B.fh : B.fp, src, L.vs, V),
-                  side ? B.hin + src * L.vs : B.ring(B.gp_ring, slot, src), V, 0};
-  Spinor<double> h, t;
-  h_site_ld(ld, L.u, L.g, x, L.kappa, side ? L.ef : L.efinv, side ? L.efinv : L.ef, h);
-  for (int i = 0; i < nterms; ++i) {
-    RevTerm r;
-    rev_term(L, B, src, side, j, slot, prev, i, r);
-    load_spinor(r.f, V, x, t);
-    for (int c = 0; c < 12; ++c) cmac(h.c[c], r.c, t.c[c]);
-  }
-  *out = h;
-}
-
+struct RevTerm {
+  FxField f;
+  FxCoef c;
+};
 constexpr int RT = 16;   // terms converted at a time per side
-__global__ void __launch_bounds__(128, 4) k_fx_rev(const __grid_constant__ Lat<double> L,
+__global__ void __launch_bounds__(128, 3) k_fx_rev(const __grid_constant__ Lat<double> L,
                                                    const __grid_constant__ Rev<double> B, int j, int slot, int prev,
                                                    int nrec) {
   __shared__ RevTerm terms[2][RT];
+  __shared__ zd scratch[2 * 32];
   const int half = blockDim.x >> 1;
   const int side = threadIdx.x >= half ? 1 : 0;
   const int t = side ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
-  const int64_t x = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t);
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
   const int src = blockIdx.y;
-  const int64_t V = L.g.V;
+  const bool live = x0 < V;
   const int base = (j < L.k - 1 ? 1 : 0) + (prev >= 0 && j + 1 < L.k - 1 ? 1 : 0) + nrec;
   const int nt = base + (side ? 0 : 1), ntmax = base + 1;
-  const FxField f = fx_src(side ? B.fh : B.fp, src, L.vs, V);
   const double kinv = 1.0 / L.kappa;
   FxHalf acc;
-  fx_zero(acc);
-  int E = FX_BAD, ex = FX_BAD;
-  bool ok = x < V;
-  if (ok) {
-    const FxSite s(L.g, x);
-    ex = f.e[x];
-    E = ex + 1023;
-    fx_range(E, f, 0, L.fu, L.g, s, side ? 0 : 1);
-    ok = E < FX_BAD;
-    if (ok) fx_hops(acc, E, f, V, 0, L.fu, L.g, s, side ? 0 : 1, sp);
-  }
-  fx_exchange(acc);
-  for (int i0 = 0; i0 < ntmax; i0 += RT) {
-    __syncthreads();
-    if (t < RT && i0 + t < nt) {
-      RevTerm r;
-      rev_term(L, B, src, side, j, slot, prev, i0 + t, r);
-      r.k = fx_coef(kinv * r.c.re, kinv * r.c.im);
-      terms[side][t] = r;
-    }
-    __syncthreads();
-    const int n = min(RT, nt - i0);
-    if (ok) fx_headroom(acc, E);
+  bool ok;
+  {
+    FxTerms T;
+    T.init();
+    for (int i0 = 0; i0 < ntmax; i0 += RT) {
+      __syncthreads();
+      for (int i = t; i < RT && i0 + i < nt; i += half) {
+        zd c;
+        terms[side][i].f = rev_term(L, B, src, side, j, slot, prev, i0 + i, &c);
+        terms[side][i].c = fx_coef(kinv * c);
+      }
+      __syncthreads();
+      const int n = min(RT, nt - i0);
 #pragma unroll 1
-    for (int i = 0; i < n && ok; ++i) {
-      const RevTerm& r = terms[side][i];
-      zd p[6];
-      fx_load_half(r.f, V, x, sp, p);
-      ok = r.k.e != FX_BAD && fx_axpy_g5(acc, E, r.k, p);
+      for (int i = 0; i < n; ++i) {
+        FxH f;
+        fx_load(terms[side][i].f, x, sp, f);
+        T.add(terms[side][i].c, f);
+      }
     }
+    T.value(acc);
+    ok = T.ok;
   }
-  if (x >= V) return;
-  zd a[6];
-  if (ok) {
-    const double ks = L.kappa * fx_pow2(E - FX_E_BIAS), us = fx_pow2(ex - 1079);
-    zd h[6];
-    fx_double(acc, h);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) a[i] = us * fx_value(__ldg(f.c + (i < 3 ? sp * 3 + i : (2 + sp) * 3 + i - 3) * V + x));
-    h_finish(a, h, mk(ks, 0.0));
-  } else {
-    Spinor<double> b;
-    rev_site_fp64(L, B, src, side, j, slot, prev, nt, x, &b);
-    fx_pick(b, sp, a);
+  for (int i = 0; i < 3; ++i) acc.v[i] = FxZ{-acc.v[i].re, -acc.v[i].im};
+  const FxField f = side ? fx_src(B.fh, src, L.vs) : ring_at(L, B.fgp, slot, src);
+  const FxSite s(L.g, x);
+  int E = fx_range(0, f, 0, L.fu, L.g, s, side ? 0 : 1);
+  E = max(E, __shfl_xor_sync(0xffffffffu, acc.E, 16));   // one scale for the site's two threads
+  ok = ok && E < FX_BAD;
+  fx_raise(acc, E);
+  // below 2^60 units, so that the hops' 2^62.6 still fit
+  fx_headroom(acc);
+  acc.E = ok ? acc.E : FX_E_BIAS;
+  {
+    const int other = __shfl_xor_sync(0xffffffffu, acc.E, 16);
+    if (other > acc.E) fx_shift(acc, min(other - acc.E, 62));
+    acc.E = max(acc.E, other);
   }
-  fx_store_half((side ? B.gw_new : B.gv_new) + src * L.vs, V, x, sp, a);
+  fx_hops(acc, f, 0, L.fu, L.g, s, side ? 0 : 1, sp);
+  FxH a, p;
+  fx_encode(acc, !ok, a);
+  fx_load(f, x, sp, p);
+  const bool okp = h_finish(acc, p, fx_coef(mk(-L.kappa, 0.0)), a);
+  fx_encode(acc, !okp, p);
+  if (live) fx_put(fx_src(side ? B.fgw : B.fgv, src, L.vs), x, sp, p);
+  if (j == 0) return;
+  zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
+  if (live) {
+    fx_load(side ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, a);
+    const zd d = fx_dot(a, p);
+    v[0] = side ? v[0] : d;
+    v[1] = side ? d : v[1];
+  }
+  block_sum<2>(v, scratch);
+  zd* part = L.part + src * L.part_stride;
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = v[0];
+    part[gridDim.x + blockIdx.x] = v[1];
+  }
+  if (arrive_last(L.cnt + src * 16 + 4, gridDim.x)) {
+    zd q[2];
+    sum_partials<2>(part, gridDim.x, q, scratch);
+    if (threadIdx.x == 0) rev_dots_epilogue(L, B, src, j - 1, q);
+  }
 }
 void fx_rev_stencil(const Lat<double>& L, const Rev<double>& B, int j, int slot, int prev, int nrec,
                     cudaStream_t st) {
-  const int64_t V = L.g.V;
-  const int sx = V * L.nsrc < 152 * 32 ? 16 : 32;
-  k_fx_rev<<<dim3(nblocks(V, sx), L.nsrc), 4 * sx, 0, st>>>(L, B, j, slot, prev, nrec);
+  const int sx = two_sided_sites(L);
+  k_fx_rev<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, B, j, slot, prev, nrec);
+}
+
+// ---------------------------------------------------------------------------
+// Force (see k_force): dU += sum over (source, term) items of the two rank-one terms
+// g_p v_j^dag and w_j g_s^dag, contracted per link on half spinors.  With A = P_-(X(x)),
+// B = P_+(Y(x + nu)):  G_cd += cf sum_s A_s,c conj(B_s,d), (X, Y) = (a, b) for the forward
+// hop and (b, a) for the backward one.  A block covers 16 sites; warp h is hop h of all of
+// them (two threads per site, one spin of the half spinors each), so the fields of a term
+// are read once for all four directions.  A is shifted to the sum's scale (and at least by
+// 2 bits), so a term adds at most 2^55 to hh and 2^58.6 to x: x is folded in after sixteen.
+// ---------------------------------------------------------------------------
+template <int SGN>
+__device__ __forceinline__ int fx_project(const FxField& f, int64_t s, int nu, int sp, int4 (&h)[3]) {
+  const int4* q = f.c + fx_at(s);
+  const int4* qu = q + sp * 96;
+  const int4* qd = q + (nu < 2 ? 3 - sp : 2 + sp) * 96;
+  const int t = SGN * (nu == 0 ? -1 : nu == 3 ? 1 : 2 * sp - 1);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int4 u = __ldg(qu + a * 32), w = __ldg(qd + a * 32);
+    h[a] = (nu & 1) ? make_int4(u.x + t * w.x, u.y + t * w.y, u.z + t * w.z, u.w + t * w.w)
+                    : make_int4(u.x - t * w.z, u.y - t * w.w, u.z + t * w.x, u.w + t * w.y);
+  }
+  return f.e[s];
+}
+struct FxOuter {
+  FxAcc g[9];
+  int E, n;
+  bool ok;
+  __device__ __forceinline__ void down(int sh) {
+    const fxll r = (1ll << sh) >> 1;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      g[i].hr = (g[i].hr + r) >> sh;
+      g[i].hi = (g[i].hi + r) >> sh;
+      g[i].xr = (g[i].xr + r) >> sh;
+      g[i].xi = (g[i].xi + r) >> sh;
+    }
+    E += sh;
+  }
+  __device__ __forceinline__ void fold() {
+    int m = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      g[i].hr += (g[i].xr + (1ll << 29)) >> 30;
+      g[i].hi += (g[i].xi + (1ll << 29)) >> 30;
+      g[i].xr = g[i].xi = 0;
+      m |= fx_top(FxZ{g[i].hr, g[i].hi});
+    }
+    n = 0;
+    if (m >= (1 << 28)) down(2);
+  }
+  __device__ __forceinline__ void add(const FxField& X, int64_t x, const FxField& Y, int64_t y, int nu, int sp) {
+    int4 a[3], b[3];
+    const int ea = fx_project<-1>(X, x, nu, sp, a), eb = fx_project<1>(Y, y, nu, sp, b);
+    if (ea == FX_BAD || eb == FX_BAD) {
+      ok = false;
+      return;
+    }
+    if (ea + eb > E) {
+      down(min(ea + eb - E, 62));
+      E = ea + eb;
+    }
+    const int d = E - (ea + eb) + 2;
+    if (d > 60) return;
+    const fxll half = 1ll << (d - 1);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const FxInt p = fx_split((fx_join(a[c].x, a[c].y) + half) >> d), q = fx_split((fx_join(a[c].z, a[c].w) + half) >> d);
+      a[c] = make_int4(p.h, p.l, q.h, q.l);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int e = 0; e < 3; ++e) fx_cdot(g[c * 3 + e], b[e], a[c]);
+    if (++n == 16) fold();
+  }
+};
+__global__ void __launch_bounds__(256, 2) k_fx_force(const __grid_constant__ Lat<double> L,
+                                                     const __grid_constant__ Rev<double> B, int nterms, int j0,
+                                                     int nsplit, double* parts) {
+  __shared__ double2 bwd[4][9][16];
+  __shared__ zd scratch[32];
+  const int hop = threadIdx.x >> 5, nu = hop >> 1, back = hop & 1, lane = threadIdx.x & 31, sp = lane >> 4;
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)16 + (lane & 15), x = min(x0, V - 1);
+  const bool live = x0 < V;
+  const int split = blockIdx.y, nitems = L.nsrc * nterms;
+  const int i0 = (int)((int64_t)split * nitems / nsplit), i1 = (int)((int64_t)(split + 1) * nitems / nsplit);
+  const int64_t xf = FxSite(L.g, x).neighbour(L.g, 2 * nu);
+  FxOuter G;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) G.g[i] = FxAcc{0, 0, 0, 0};
+  G.E = 0;
+  G.n = 0;
+  G.ok = true;
+#pragma unroll 1
+  for (int i = 2 * i0; i < 2 * i1; ++i) {
+    const int src = (i >> 1) / nterms, t = (i >> 1) - src * nterms, j = j0 - t;
+    const bool second = i & 1;
+    if (second && j == L.k - 1) continue;
+    const FxField a = second ? fx_bw(L, src, j) : ring_at(L, B.fgp, t, src);
+    const FxField b = second ? ring_at(L, B.fgs, t, src) : fx_bv(L, src, j);
+    G.add(back ? b : a, x, back ? a : b, xf, nu, sp);
+  }
+  G.fold();
+  // kappa f with the sign of the hop term; a product's unit is 2^(E + 2 - 2098)
+  const double f = nu < 3 ? 1.0 : back ? L.efinv : L.ef;
+  const double u = G.ok ? -L.kappa * f * fx_pow2_wide(G.E - 2096) : fx_nan();
+  zd o[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    o[i] = mk(u * (double)G.g[i].hr, u * (double)G.g[i].hi);
+    o[i].re += __shfl_xor_sync(0xffffffffu, o[i].re, 16);
+    o[i].im += __shfl_xor_sync(0xffffffffu, o[i].im, 16);
+    if (back && sp == 0) bwd[nu][i][lane] = make_double2(o[i].re, o[i].im);
+  }
+  __syncthreads();
+  zd v[1] = {mk(0.0, 0.0)};
+  if (!back && sp == 0 && live) {
+    double2* dst = reinterpret_cast<double2*>(nsplit > 1 ? parts + (int64_t)split * 72 * V : B.force);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const double2 w = bwd[nu][i][lane];
+      double2* p = dst + (int64_t)(nu * 9 + i) * V + x;
+      double2 s = make_double2(o[i].re + w.x, o[i].im + w.y);
+      if (nsplit == 1) {
+        const double2 old = *p;
+        s.x += old.x;
+        s.y += old.y;
+      }
+      *p = s;
+      if (nu == 3) {   // dmu: Re(conj(G_fwd - G_bwd) U_t)
+        const zd ul = load_link_entry(L.u, V, x, 27 + i);
+        v[0].re += (o[i].re - w.x) * ul.re + (o[i].im - w.y) * ul.im;
+      }
+    }
+  }
+  block_sum<1>(v, scratch);
+  if (threadIdx.x == 0) B.dmu_part[split * gridDim.x + blockIdx.x] = v[0];
+  if (arrive_last(B.dmu_cnt, gridDim.x * gridDim.y)) {
+    zd s[1];
+    sum_partials<1>(B.dmu_part, gridDim.x * gridDim.y, s, scratch);
+    if (threadIdx.x == 0) *B.dmu += s[0].re;
+  }
+}
+int fx_force_splits(int64_t V) {
+  const int64_t blocks = (V + 15) / 16;
+  if (blocks >= 2 * 152) return 1;
+  const int64_t want = (2 * 152 + blocks - 1) / blocks;
+  return (int)(want < kForceSplitMax ? want : kForceSplitMax);
+}
+int fx_force_flush(const Lat<double>& L, const Rev<double>& B, int nterms, int j0, cudaStream_t st) {
+  int nsplit = B.force_parts ? fx_force_splits(L.g.V) : 1;
+  if (nsplit > L.nsrc * nterms) nsplit = L.nsrc * nterms;
+  k_fx_force<<<dim3(nblocks(L.g.V, 16), nsplit), 256, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+  return nsplit;
 }
 
 }  // namespace ov

@@ -24,23 +24,19 @@ struct SrcScal {
   zd cr1, cr2, cs1, cs2; // g_r = cr1 Gv_{j+1} + cr2 w_{j+1};  g_s = cs1 Gw_{j+1} + cs2 v_{j+1}
 };
 
-// Links in fixed point (fx.cuh): five "directions" x, y, z, e^{mu} t, e^{-mu} t; entry e of
-// direction d of site s at (d * 9 + e) * V + s as (re.h, re.l, im.h, im.l), its exponent at
-// ex[d * V + s].
+// FP64 calls hold every lattice field in block fixed point (fx.cuh): vs reals per field as in
+// Lat (a field of Vp sites, a multiple of 32, takes 12 Vp int4 and Vp exponents: vs = 24 Vp).
 struct FxLinks {
   const int4* e;
   const short* ex;
 };
-constexpr int kFxLinkEntries = 45;
-// An FP64 field's copy in fixed point: component c of site s at c * V + s as
-// (re.h, re.l, im.h, im.l), the site's exponent at e[s]; sources at vs reals (sites) apart.
+OV_HD int64_t fx_link_ints(int64_t V) { return (V + 31) / 32 * 1440; }
 struct FxField {
   int4* c;
   short* e;
 };
-OV_HD FxField fx_src(const FxField& f, int src, int64_t vs, int64_t V) {
-  return FxField{f.c + src * (vs / 2), f.e + src * V};
-}
+// field i of an array of fields of vs reals
+OV_HD FxField fx_src(const FxField& f, int64_t i, int64_t vs) { return FxField{f.c + i * (vs / 2), f.e + i * (vs / 24)}; }
 
 // Everything a lattice kernel needs, passed by value.
 template <typename R>
@@ -67,8 +63,11 @@ struct Lat {
   Geom gl;
   const R* ue;               // links of the direction E (internal layout) or null
   R mdir;                    // mu direction
-  FxLinks fu, fd;            // FP64 fields: the links and dH's links in fixed point (fu.e null: FP64 stencil)
-  FxField fr, fs;            // FP64 fields: r and s in fixed point, written by whichever kernel completes them
+  // FP64 calls: links and dH's links (fu.e null: FP64 stencil), the recurrence's fields, and the
+  // exponents of the bases, whose integers are in bv and bw
+  FxLinks fu, fd;
+  FxField fr, fs, fp, fq;
+  short* bve; short* bwe;
   // basis window: vectors jbase .. jbase + kcap - 1 (all k from 0 unless segments are replayed)
   int kcap, jbase;
   OV_HD R* basis_v(int src, int j) const { return bv + ((int64_t)src * kcap + (j - jbase)) * vs; }
@@ -82,8 +81,7 @@ struct Rev {
   R* gv_new; R* gw_new;      // gradients being formed for v_j, w_j
   R* gr_ring; R* gs_ring; R* gp_ring;   // [m][src][vs]
   R* hin;                    // conj(g_alpha) v_j + g_s of the current step: [src][vs]
-  FxField fp, fh;            // FP64 fields: g_p and h_in in fixed point (hin then holds FP64 values only
-                             // at sites out of the fixed-point window)
+  FxField fgv, fgw, fgr, fgs, fgp, fh, fxb;   // FP64 calls: the above (and xbar) in fixed point
   int m;                     // ring length
   const R* xbar;             // [src][vs]
   const zd* y;               // [src][k]
@@ -128,18 +126,37 @@ void apply_h_il(const Lat<float>& L, const float* in, float* out, int dagger, cu
 void pack_spinors_il(const double* aos, float* dst, int nsrc, int64_t V, cudaStream_t st);
 void unpack_spinors_il(const float* f, double* aos, int nsrc, int64_t V, cudaStream_t st);
 
-// fixed-point forms of the FP64 stencils (fx_kernels.cu); reached through apply_h,
-// tsl_stencil and rev_stencil where L.fu is set
+// FP64 calls (fx_kernels.cu); the launchers below dispatch to them
 void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, cudaStream_t st);
 void pack_dh_links_fx(const double* u, const double* e, double m, int4* out, short* ex, int64_t V, double ef,
                       double efinv, cudaStream_t st);
-// in: the field in fixed point, d: its FP64 companion (read where a site is out of the window);
-// aos: out in the user's layout
+// user spinors to f and (if set) g; FP64 values of marked sites to d (if set)
+void fx_pack(const double* aos, const FxField& f, const FxField& g, double* d, int nsrc, int64_t V, int64_t vs,
+             cudaStream_t st);
+void fx_pack_block(const double* top, const double* bot, const FxField& f, const FxField& g, int nsrc, int64_t V,
+                   int64_t vs, cudaStream_t st);
+void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t vs, cudaStream_t st);
+// in: the field in fixed point, d: its FP64 companion (read where a site is marked); aos: out
+// in the user's layout
 void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double* out, int dagger, int aos,
                 cudaStream_t st, int variant);
-void fx_pack(const double* aos, const FxField& f, double* d, int nsrc, int64_t V, int64_t vs, cudaStream_t st);
-void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t vs, cudaStream_t st);
+void fx_tsl_init(const Lat<double>& L, cudaStream_t st);
 void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st, int variant);
+void fx_tsl_update(const Lat<double>& L, int j, int finalize, cudaStream_t st);
+// dots with vectors j0 .. j0 + nb - 1 (modes as proj_dots; b.c null: side A alone)
+void fx_proj_dots(const Lat<double>& L, int j0, int nb, int mode, const FxField& a, const FxField& b,
+                  int64_t ab_stride, zd* coef, zd* cpart, cudaStream_t st);
+// fin 1: omega and the next scales follow; 2: g_alpha and the carries of reverse step j
+void fx_proj_update(const Lat<double>& L, const Rev<double>* B, int nb, int mode, const FxField& a, const FxField& b,
+                    int64_t ab_stride, const zd* coef, int j, int fin, cudaStream_t st);
+void fx_combine(const Lat<double>& L, int src0, int nsrc, int side, int j0, int nvec, const zd* y, int64_t ystride,
+                double* out, int accumulate, cudaStream_t st);
+void fx_rev_form(const Lat<double>& L, const Rev<double>& B, int j, int slot, int with_dots, cudaStream_t st);
+void fx_rev_combine(const Lat<double>& L, const Rev<double>& B, int j, int slot, cudaStream_t st);
+void fx_rev_stencil(const Lat<double>& L, const Rev<double>& B, int j, int slot, int prev_slot, int nrec,
+                    cudaStream_t st);
+int fx_force_splits(int64_t V);
+int fx_force_flush(const Lat<double>& L, const Rev<double>& B, int nterms, int j0, cudaStream_t st);
 
 template <typename R> void tsl_init(const Lat<R>& L, cudaStream_t st);
 template <typename R> void tsl_stencil(const Lat<R>& L, int j, bool need_q, cudaStream_t st, int variant = 0);
@@ -176,8 +193,6 @@ template <typename R> void rev_alpha_dots(const Lat<R>& L, const Rev<R>& B, int 
 template <typename R> void rev_combine(const Lat<R>& L, const Rev<R>& B, int j, int slot, cudaStream_t st);
 template <typename R> void rev_stencil(const Lat<R>& L, const Rev<R>& B, int j, int slot, int prev_slot,
                                        int nrec, cudaStream_t st);
-void fx_rev_stencil(const Lat<double>& L, const Rev<double>& B, int j, int slot, int prev_slot, int nrec,
-                    cudaStream_t st);
 // splits of the force contraction's (source, term) items: 1 unless the lattice has
 // too few sites to fill the GPU, at most kForceSplitMax
 constexpr int kForceSplitMax = 8;

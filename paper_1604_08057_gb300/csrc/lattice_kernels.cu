@@ -11,7 +11,6 @@
 
 #include "dslash.cuh"
 #include "kernels.h"
-#include "fx.cuh"
 #include "recurrence.cuh"
 
 namespace ov {
@@ -643,13 +642,6 @@ void apply_h(const Lat<R>& L, const R* in, R* out, int dagger, cudaStream_t st, 
 // ---------------------------------------------------------------------------
 // TSL forward: initialisation (beta_0 = ||b||)
 // ---------------------------------------------------------------------------
-// the fixed-point copy of a site of an FP64 field (nothing for FP32 fields)
-__device__ __forceinline__ void store_fx(const FxField& f, int src, int64_t vs, int64_t V, int64_t x,
-                                         const Spinor<double>& p) {
-  fx_store(fx_src(f, src, vs, V), V, x, p);
-}
-__device__ __forceinline__ void store_fx(const FxField&, int, int64_t, int64_t, int64_t, const Spinor<float>&) {}
-
 template <typename R>
 __global__ void __launch_bounds__(BS) k_tsl_init(Lat<R> L) {
   __shared__ zd scratch[2 * 32];
@@ -660,14 +652,10 @@ __global__ void __launch_bounds__(BS) k_tsl_init(Lat<R> L) {
     Spinor<R> b;
     load_spinor(L.r + src * L.vs, L.g.V, x, b);
     v[0] = spinor_dot(b, b);
-    store_fx(L.fr, src, L.vs, L.g.V, x, b);
     if (L.block) {
       Spinor<R> a;
       load_spinor(L.s + src * L.vs, L.g.V, x, a);
       v[1] = spinor_dot(a, b);
-      store_fx(L.fs, src, L.vs, L.g.V, x, a);
-    } else {
-      store_fx(L.fs, src, L.vs, L.g.V, x, b);   // s = r
     }
   }
   block_sum<2>(v, scratch);
@@ -680,23 +668,17 @@ __global__ void __launch_bounds__(BS) k_tsl_init(Lat<R> L) {
     zd s[2];
     sum_partials<2>(part, gridDim.x, s, scratch);
     if (threadIdx.x == 0) {
-      SrcScal& sc = L.sc[src];
-      sc.err = 0;
-      sc.err_step = -1;
-      const double b0 = sqrt(s[0].re);
-      sc.beta0 = b0;
-      if (!(b0 > 0.0) || !isfinite(b0)) flag_error(sc, ERRB_NONFINITE, 0);
-      sc.sv = mk(1.0 / b0, 0.0);
-      // w_1 = s sw with w_1^dag v_1 = 1: sw = beta_0 / conj(s^dag r); s = r in plain mode
-      sc.sw = L.block ? zdiv(mk(b0, 0.0), conj(s[1])) : mk(1.0 / b0, 0.0);
-      L.beta[(int64_t)src * L.k] = mk(0.0, 0.0);
-      L.delta[(int64_t)src * L.k] = 0.0;
+      init_finalize(L, src, s[0].re, s[1]);
     }
   }
 }
 template <typename R>
 void tsl_init(const Lat<R>& L, cudaStream_t st) {
-  k_tsl_init<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L);
+  if constexpr (std::is_same<R, double>::value) {
+    fx_tsl_init(L, st);
+  } else {
+    k_tsl_init<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -906,8 +888,6 @@ __global__ void __launch_bounds__(BS) k_tsl_update(Lat<R> L, int j, int finalize
     store_spinor(L.r + src * L.vs, V, x, r);
     store_spinor(L.s + src * L.vs, V, x, s);
     if (finalize) {
-      store_fx(L.fr, src, L.vs, V, x, r);
-      store_fx(L.fs, src, L.vs, V, x, s);
       v[0] = spinor_dot(s, r);
       v[1] = spinor_dot(r, r);
       v[2] = spinor_dot(s, s);
@@ -927,7 +907,11 @@ __global__ void __launch_bounds__(BS) k_tsl_update(Lat<R> L, int j, int finalize
 }
 template <typename R>
 void tsl_update(const Lat<R>& L, int j, bool finalize, cudaStream_t st) {
-  k_tsl_update<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j, finalize ? 1 : 0);
+  if constexpr (std::is_same<R, double>::value) {
+    fx_tsl_update(L, j, finalize ? 1 : 0, st);
+  } else {
+    k_tsl_update<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j, finalize ? 1 : 0);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1065,9 +1049,7 @@ __global__ void __launch_bounds__(BS) k_proj_update(Lat<R> L, int nb, int mode, 
 #pragma unroll
       for (int c = 0; c < 12; ++c) s.c[c] = s.c[c] - mk<R>((R)cb.c[c].re, (R)cb.c[c].im);
       store_spinor(b + src * ab_stride, V, x, s);
-      if (finalize) {   // a and b are the recurrence's r and s
-        store_fx(L.fr, src, L.vs, V, x, r);
-        store_fx(L.fs, src, L.vs, V, x, s);
+      if (finalize) {
         v[0] = spinor_dot(s, r);
         v[1] = spinor_dot(r, r);
         v[2] = spinor_dot(s, s);
@@ -1202,12 +1184,20 @@ __global__ void __launch_bounds__(BS) k_ritz_combine(Lat<R> L, int src, int side
 }
 template <typename R>
 void ritz_combine(const Lat<R>& L, int src, int side, int nvec, const zd* y, double* out, cudaStream_t st) {
-  k_ritz_combine<R><<<nblocks(L.g.V, BS), BS, 0, st>>>(L, src, side, nvec, y, out);
+  if constexpr (std::is_same<R, double>::value) {
+    fx_combine(L, src, 1, side, 0, nvec, y, 0, out, 0, st);
+  } else {
+    k_ritz_combine<R><<<nblocks(L.g.V, BS), BS, 0, st>>>(L, src, side, nvec, y, out);
+  }
 }
 
 template <typename R>
 void combine_range(const Lat<R>& L, int j0, int nvec, const zd* y, double* out, bool acc, cudaStream_t st) {
-  k_combine<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j0, nvec, y, out, acc ? 1 : 0);
+  if constexpr (std::is_same<R, double>::value) {
+    fx_combine(L, 0, L.nsrc, 0, j0, nvec, y, L.k, out, acc ? 1 : 0, st);
+  } else {
+    k_combine<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j0, nvec, y, out, acc ? 1 : 0);
+  }
 }
 template <typename R>
 void combine(const Lat<R>& L, int nvec, const zd* y, double* out, cudaStream_t st) {
@@ -1245,44 +1235,13 @@ __global__ void __launch_bounds__(BS) k_rev_dots(Lat<R> L, Rev<R> B, int j) {
     zd s[2];
     sum_partials<2>(part, gridDim.x, s, scratch);
     if (threadIdx.x == 0) {
-      SrcScal& sc = L.sc[src];
-      const int64_t o = (int64_t)src * L.k + j + 1;
-      const double d = L.delta[o];
-      const zd bt = L.beta[o];
-      const zd om = mk(bt.re * d, bt.im * d);
-      const double aom = d * d;
-      double g_d = B.gdT[o] + sc.carry_delta - s[0].re / d;
-      zd g_b = B.gbT[o] + sc.carry_beta - zdiv(conj(s[1]), conj(bt));
-      zd g_w = mk(g_b.re / d, g_b.im / d);
-      g_d -= (om.re * g_b.re + om.im * g_b.im) / (d * d);      // Re(conj(om) g_b)
-      const double f = g_d / (2.0 * d * aom);
-      g_w = g_w + mk(f * om.re, f * om.im);
-      sc.cr1 = mk(1.0 / d, 0.0);
-      sc.cr2 = conj(bt) * g_w;
-      sc.cs1 = zdiv(mk(1.0, 0.0), bt);
-      sc.cs2 = mk(d * g_w.re, -d * g_w.im);
-      if (!finite_z(sc.cr2) || !finite_z(sc.cs2)) flag_error(sc, ERRB_NONFINITE, j);
+      rev_dots_epilogue(L, B, src, j, s);
     }
   }
 }
 template <typename R>
 void rev_dots(const Lat<R>& L, const Rev<R>& B, int j, cudaStream_t st) {
   k_rev_dots<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j);
-}
-
-// D1 = v_j^dag g_r, D2 = w_j^dag g_s, D3 = v_{j-1}^dag g_r, D4 = w_{j-1}^dag g_s -> g_alpha, carries
-template <typename R>
-__device__ void alpha_epilogue(const Lat<R>& L, const Rev<R>& B, int src, int j, const zd (&s)[4]) {
-  SrcScal& sc = L.sc[src];
-  const int64_t o = (int64_t)src * L.k + j;
-  sc.g_alpha = B.gaT[o] - s[0] - conj(s[1]);
-  if (j > 0) {
-    sc.carry_beta = -s[2];
-    sc.carry_delta = -s[3].re;
-  } else {
-    sc.carry_beta = mk(0.0, 0.0);
-    sc.carry_delta = 0.0;
-  }
 }
 
 template <typename R>
@@ -1339,8 +1298,12 @@ __global__ void __launch_bounds__(BS) k_rev_form(Lat<R> L, Rev<R> B, int j, int 
 }
 template <typename R>
 void rev_form(const Lat<R>& L, const Rev<R>& B, int j, int slot, bool with_dots, cudaStream_t st) {
-  k_rev_form<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot,
-                                                                                   with_dots ? 1 : 0);
+  if constexpr (std::is_same<R, double>::value) {
+    fx_rev_form(L, B, j, slot, with_dots ? 1 : 0, st);
+  } else {
+    k_rev_form<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot,
+                                                                                     with_dots ? 1 : 0);
+  }
 }
 
 // the four dots after the projection adjoint has been applied to g_r, g_s
@@ -1429,7 +1392,6 @@ __global__ void __launch_bounds__(BS) k_rev_combine(Lat<R> L, Rev<R> B, int j, i
     for (int c = 0; c < 12; ++c) a.c[c] = ga * e.c[c];
   }
   store_spinor(B.ring(B.gp_ring, slot, src), V, x, a);
-  store_fx(B.fp, src, L.vs, V, x, a);
   const cplx<R> gac = conj(ga);
   load_spinor(L.basis_v(src, j), V, x, e);
   if (carry) {
@@ -1440,15 +1402,15 @@ __global__ void __launch_bounds__(BS) k_rev_combine(Lat<R> L, Rev<R> B, int j, i
 #pragma unroll
     for (int c = 0; c < 12; ++c) a.c[c] = gac * e.c[c];
   }
-  if constexpr (std::is_same<R, double>::value) {
-    if (fx_store(fx_src(B.fh, src, L.vs, V), V, x, a)) store_spinor(B.hin + src * L.vs, V, x, a);
-  } else {
-    store_spinor(B.hin + src * L.vs, V, x, a);
-  }
+  store_spinor(B.hin + src * L.vs, V, x, a);
 }
 template <typename R>
 void rev_combine(const Lat<R>& L, const Rev<R>& B, int j, int slot, cudaStream_t st) {
-  k_rev_combine<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot);
+  if constexpr (std::is_same<R, double>::value) {
+    fx_rev_combine(L, B, j, slot, st);
+  } else {
+    k_rev_combine<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot);
+  }
 }
 
 // R3b: complete gradients of v_j and w_j
@@ -1635,17 +1597,26 @@ int force_splits(int64_t V) {
 }
 template <typename R>
 void force_flush(const Lat<R>& L, const Rev<R>& B, const int* /*unused*/, int nterms, int j0, cudaStream_t st) {
-  if (nterms <= 0) return;
-  const unsigned nb = nblocks(L.g.V, BS);
-  int nsplit = B.force_parts ? force_splits(L.g.V) : 1;
-  if (nsplit > L.nsrc * nterms) nsplit = L.nsrc * nterms;
-  k_force<0, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
-  k_force<1, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
-  k_force<2, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
-  k_force<3, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
-  if (nsplit > 1) {
-    const int64_t n = 72 * L.g.V;
-    k_force_reduce<<<nblocks(n, 256), 256, 0, st>>>(B.force, B.force_parts, nsplit, n);
+  if constexpr (std::is_same<R, double>::value) {
+    if (nterms <= 0) return;
+    const int nsplit = fx_force_flush(L, B, nterms, j0, st);
+    if (nsplit > 1) {
+      const int64_t n = 72 * L.g.V;
+      k_force_reduce<<<nblocks(n, 256), 256, 0, st>>>(B.force, B.force_parts, nsplit, n);
+    }
+  } else {
+    if (nterms <= 0) return;
+    const unsigned nb = nblocks(L.g.V, BS);
+    int nsplit = B.force_parts ? force_splits(L.g.V) : 1;
+    if (nsplit > L.nsrc * nterms) nsplit = L.nsrc * nterms;
+    k_force<0, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+    k_force<1, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+    k_force<2, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+    k_force<3, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+    if (nsplit > 1) {
+      const int64_t n = 72 * L.g.V;
+      k_force_reduce<<<nblocks(n, 256), 256, 0, st>>>(B.force, B.force_parts, nsplit, n);
+    }
   }
 }
 
@@ -1682,35 +1653,38 @@ void eps_norms(const double* a_top, const double* a_bot, const double* b, int ns
   k_eps_norms<<<nsrc, 512, 0, st>>>(a_top, a_bot, b, n, out);
 }
 
-#define OV_INST(R)                                                                                        \
-  template void ritz_combine<R>(const Lat<R>&, int, int, int, const zd*, double*, cudaStream_t);        \
-  template void apply_dh<R>(const Lat<R>&, const R*, R*, int, cudaStream_t);                             \
-  template void pack_spinors<R>(const double*, R*, int, int64_t, int64_t, cudaStream_t);                 \
-  template void pack_block_start<R>(const double*, const double*, R*, R*, int, int64_t, int64_t,          \
-                                    cudaStream_t);                                                       \
-  template void unpack_spinors<R>(const R*, double*, int, int64_t, int64_t, cudaStream_t);               \
-  template void pack_links<R>(const double*, R*, int64_t, cudaStream_t);                                 \
-  template void apply_h<R>(const Lat<R>&, const R*, R*, int, cudaStream_t, int, int*);                   \
-  template void tsl_init<R>(const Lat<R>&, cudaStream_t);                                                \
-  template void tsl_stencil<R>(const Lat<R>&, int, bool, cudaStream_t, int);                             \
-  template void tsl_update<R>(const Lat<R>&, int, bool, cudaStream_t);                                   \
-  template void proj_dots<R>(const Lat<R>&, int, int, const R*, const R*, int64_t, zd*, zd*, cudaStream_t); \
-  template void proj_update<R>(const Lat<R>&, int, int, R*, R*, int64_t, const zd*, bool, cudaStream_t, \
-                               bool);                                                                   \
-  template void basis_dots<R>(const Lat<R>&, int, const R*, int64_t, zd*, zd*, cudaStream_t);            \
-  template void combine<R>(const Lat<R>&, int, const zd*, double*, cudaStream_t);                        \
-  template void combine_range<R>(const Lat<R>&, int, int, const zd*, double*, bool, cudaStream_t);       \
-  template void basis_dots_range<R>(const Lat<R>&, int, int, const R*, int64_t, zd*, zd*, cudaStream_t); \
-  template void rev_init<R>(const Lat<R>&, const Rev<R>&, cudaStream_t);                                 \
-  template void rev_dots<R>(const Lat<R>&, const Rev<R>&, int, cudaStream_t);                            \
-  template void rev_form<R>(const Lat<R>&, const Rev<R>&, int, int, bool, cudaStream_t);                 \
-  template void rev_proj_record<R>(const Lat<R>&, const Rev<R>&, int, int, const zd*, cudaStream_t);     \
-  template void rev_alpha_dots<R>(const Lat<R>&, const Rev<R>&, int, int, cudaStream_t);                 \
-  template void rev_combine<R>(const Lat<R>&, const Rev<R>&, int, int, cudaStream_t);                    \
-  template void rev_stencil<R>(const Lat<R>&, const Rev<R>&, int, int, int, int, cudaStream_t);          \
+#define OV_INST(R) \
+  template void ritz_combine<R>(const Lat<R>&, int, int, int, const zd*, double*, cudaStream_t); \
+  template void apply_dh<R>(const Lat<R>&, const R*, R*, int, cudaStream_t); \
+  template void pack_spinors<R>(const double*, R*, int, int64_t, int64_t, cudaStream_t); \
+  template void pack_block_start<R>(const double*, const double*, R*, R*, int, int64_t, int64_t, cudaStream_t); \
+  template void unpack_spinors<R>(const R*, double*, int, int64_t, int64_t, cudaStream_t); \
+  template void pack_links<R>(const double*, R*, int64_t, cudaStream_t); \
+  template void apply_h<R>(const Lat<R>&, const R*, R*, int, cudaStream_t, int, int*); \
+  template void tsl_init<R>(const Lat<R>&, cudaStream_t); \
+  template void tsl_stencil<R>(const Lat<R>&, int, bool, cudaStream_t, int); \
+  template void tsl_update<R>(const Lat<R>&, int, bool, cudaStream_t); \
+  template void combine<R>(const Lat<R>&, int, const zd*, double*, cudaStream_t); \
+  template void combine_range<R>(const Lat<R>&, int, int, const zd*, double*, bool, cudaStream_t); \
+  template void rev_init<R>(const Lat<R>&, const Rev<R>&, cudaStream_t); \
+  template void rev_form<R>(const Lat<R>&, const Rev<R>&, int, int, bool, cudaStream_t); \
+  template void rev_proj_record<R>(const Lat<R>&, const Rev<R>&, int, int, const zd*, cudaStream_t); \
+  template void rev_combine<R>(const Lat<R>&, const Rev<R>&, int, int, cudaStream_t); \
+  template void rev_stencil<R>(const Lat<R>&, const Rev<R>&, int, int, int, int, cudaStream_t); \
   template void force_flush<R>(const Lat<R>&, const Rev<R>&, const int*, int, int, cudaStream_t);
 
 OV_INST(double)
 OV_INST(float)
+
+// FP64 calls run these in fixed point (fx_kernels.cu)
+#define OV_INST_FP32(R) \
+  template void proj_dots<R>(const Lat<R>&, int, int, const R*, const R*, int64_t, zd*, zd*, cudaStream_t); \
+  template void proj_update<R>(const Lat<R>&, int, int, R*, R*, int64_t, const zd*, bool, cudaStream_t, bool); \
+  template void basis_dots<R>(const Lat<R>&, int, const R*, int64_t, zd*, zd*, cudaStream_t); \
+  template void basis_dots_range<R>(const Lat<R>&, int, int, const R*, int64_t, zd*, zd*, cudaStream_t); \
+  template void rev_dots<R>(const Lat<R>&, const Rev<R>&, int, cudaStream_t); \
+  template void rev_alpha_dots<R>(const Lat<R>&, const Rev<R>&, int, int, cudaStream_t);
+
+OV_INST_FP32(float)
 
 }  // namespace ov

@@ -23,7 +23,7 @@ enum BufId {
   B_LINKS, B_BV, B_BW, B_P, B_Q, B_R, B_S, B_SC, B_ALPHA, B_BETA, B_DELTA, B_PART, B_CNT, B_COEF, B_CPART,
   B_T, B_X, B_XI, B_XN, B_E, B_EN, B_TMP1, B_TMP2, B_IPIV, B_PROW, B_COL, B_DSTAT, B_DPART, B_DCNT, B_DERR,
   B_Y, B_GY, B_GA, B_GB, B_GD, B_XBAR, B_GV, B_GW, B_GV2, B_GW2, B_GR, B_GS, B_GP, B_EV, B_EW, B_REB,
-  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, B_FXL, B_FXE, B_FXDL, B_FXDE, B_FXR, B_FXRE, B_FXS, B_FXSE, B_FXP, B_FXPE, B_FXH, B_FXHE, NBUF
+  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, B_FXL, B_FXE, B_FXDL, B_FXDE, B_FXR, B_FXRE, B_FXS, B_FXSE, B_FXP, B_FXPE, B_FXQ, B_FXQE, B_BVE, B_BWE, B_CKRE, B_CKSE, B_CKVE, B_CKWE, B_GVE, B_GWE, B_GRE, B_GSE, B_GPE, B_HINE, B_XBE, NBUF
 };
 
 struct Status {
@@ -306,6 +306,29 @@ Geom make_geom(const int32_t dims[4]) {
   return g;
 }
 
+// reals per internal field of V sites
+template <typename R>
+int64_t field_reals(int64_t V) {
+  return std::is_same<R, double>::value ? (V + 31) / 32 * 32 * 24 : ((24 * V + 63) / 64) * 64;
+}
+// n fixed-point fields of vs reals
+FxField fx_fields(ov_context* c, int id, int id_e, int64_t n, int64_t vs) {
+  return FxField{wsT<int4>(c, id, n * (vs / 2)), wsT<short>(c, id_e, n * (vs / 24))};
+}
+// the user's spinors into the recurrence's r and s (equal at the start)
+template <typename R>
+void pack_start(ov_context* c, const Lat<R>& L, const void* b) {
+  const double* bd = static_cast<const double*>(b);
+  if constexpr (std::is_same<R, double>::value) {
+    run(c, OV_KIND_LAYOUT, 1, [&] { fx_pack(bd, L.fr, L.fs, nullptr, L.nsrc, L.g.V, L.vs, c->st); });
+  } else {
+    run(c, OV_KIND_LAYOUT, 2, [&] {
+      pack_spinors<R>(bd, L.r, L.nsrc, L.g.V, L.vs, c->st);
+      pack_spinors<R>(bd, L.s, L.nsrc, L.g.V, L.vs, c->st);
+    });
+  }
+}
+
 // fm = 2 sets up block mode: fields of 2V sites (upper and lower halves)
 template <typename R>
 Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, double m_w, int nsrc, int k,
@@ -322,22 +345,23 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   L.efinv = (R)std::exp(-mu);
   L.nsrc = nsrc;
   L.k = k;
-  L.vs = ((24 * V + 63) / 64) * 64;
+  constexpr bool fx = std::is_same<R, double>::value;   // FP64 calls run in fixed point (fx.cuh)
+  L.vs = field_reals<R>(V);
   R* u = wsT<R>(c, B_LINKS, link_reals<R>() * V);
   L.u = u;
   run(c, OV_KIND_LAYOUT, 1, [&] { pack_links<R>(static_cast<const double*>(U), u, V, c->st); });
-  if constexpr (std::is_same<R, double>::value) {
-    int4* fe = wsT<int4>(c, B_FXL, kFxLinkEntries * V);
-    short* fx = wsT<short>(c, B_FXE, 5 * V);
-    L.fu = FxLinks{fe, fx};
+  if constexpr (fx) {
+    int4* fe = wsT<int4>(c, B_FXL, fx_link_ints(V));
+    short* ex = wsT<short>(c, B_FXE, 5 * V);
+    L.fu = FxLinks{fe, ex};
     run(c, OV_KIND_LAYOUT, 1,
-        [&] { pack_links_fx(static_cast<const double*>(U), fe, fx, V, L.ef, L.efinv, c->st); });
+        [&] { pack_links_fx(static_cast<const double*>(U), fe, ex, V, L.ef, L.efinv, c->st); });
   }
   launch_check();
   if (fm == 2) {
     L.block = 1;
     L.g.V = 2 * V;
-    L.vs = ((48 * V + 63) / 64) * 64;
+    L.vs = field_reals<R>(2 * V);
   }
   const int64_t Vf = L.g.V;
   L.kcap = kcap > 0 ? kcap : k;
@@ -345,14 +369,22 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   if (basis) {
     L.bv = wsT<R>(c, B_BV, (int64_t)nsrc * L.kcap * L.vs);
     L.bw = wsT<R>(c, B_BW, (int64_t)nsrc * L.kcap * L.vs);
+    if constexpr (fx) {
+      L.bve = wsT<short>(c, B_BVE, (int64_t)nsrc * L.kcap * (L.vs / 24));
+      L.bwe = wsT<short>(c, B_BWE, (int64_t)nsrc * L.kcap * (L.vs / 24));
+    }
   }
   L.p = wsT<R>(c, B_P, nsrc * L.vs);
   L.q = wsT<R>(c, B_Q, nsrc * L.vs);
   L.r = wsT<R>(c, B_R, nsrc * L.vs);
   L.s = wsT<R>(c, B_S, nsrc * L.vs);
-  if constexpr (std::is_same<R, double>::value) {
-    L.fr = FxField{wsT<int4>(c, B_FXR, nsrc * (L.vs / 2)), wsT<short>(c, B_FXRE, nsrc * Vf)};
-    if (basis) L.fs = FxField{wsT<int4>(c, B_FXS, nsrc * (L.vs / 2)), wsT<short>(c, B_FXSE, nsrc * Vf)};
+  if constexpr (fx) {
+    L.fr = fx_fields(c, B_FXR, B_FXRE, nsrc, L.vs);
+    if (basis) {
+      L.fs = fx_fields(c, B_FXS, B_FXSE, nsrc, L.vs);
+      L.fp = fx_fields(c, B_FXP, B_FXPE, nsrc, L.vs);
+      L.fq = fx_fields(c, B_FXQ, B_FXQE, nsrc, L.vs);
+    }
   }
   L.sc = wsT<SrcScal>(c, B_SC, nsrc);
   L.alpha = wsT<zd>(c, B_ALPHA, (int64_t)nsrc * k);
@@ -430,9 +462,16 @@ void forward_krylov(ov_context* c, Lat<R>& L) {
       run(c, OV_KIND_UPDATE, 1, [&] { tsl_update(L, j, !reb, c->st); });
       if (reb) {
         for (int ps = 0; ps < c->opt.passes; ++ps) {
-          run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 0, L.r, L.s, L.vs, coef, cpart, c->st); });
-          run(c, OV_KIND_PROJ_UPDATE, 1,
-              [&] { proj_update(L, j, 0, L.r, L.s, L.vs, coef, ps == c->opt.passes - 1, c->st, ps > 0); });
+          const bool last = ps == c->opt.passes - 1;
+          if constexpr (std::is_same<R, double>::value) {
+            run(c, OV_KIND_PROJ_DOTS, 2, [&] { fx_proj_dots(L, 0, j + 1, 0, L.fr, L.fs, L.vs, coef, cpart, c->st); });
+            run(c, OV_KIND_PROJ_UPDATE, 1,
+                [&] { fx_proj_update(L, nullptr, j + 1, 0, L.fr, L.fs, L.vs, coef, j, last ? 1 : 0, c->st); });
+          } else {
+            run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 0, L.r, L.s, L.vs, coef, cpart, c->st); });
+            run(c, OV_KIND_PROJ_UPDATE, 1,
+                [&] { proj_update(L, j, 0, L.r, L.s, L.vs, coef, last, c->st, ps > 0); });
+          }
         }
       }
       inject_after_update(c, L, j);
@@ -457,8 +496,14 @@ int run_diagnostics(ov_context* c, const Lat<R>& L, bool segments, ov_tsl_info* 
     zd* coef = wsT<zd>(c, B_COEF, (int64_t)nsrc * 2 * k);
     zd* cpart = wsT<zd>(c, B_CPART, (int64_t)nsrc * 2 * k * nsb);
     run(c, OV_KIND_PROJ_DOTS, 2, [&] {
-      proj_dots(L, k - 1, 0, L.basis_v(0, k - 1), L.basis_w(0, k - 1), (int64_t)L.kcap * L.vs, coef, cpart,
-                c->st);
+      if constexpr (std::is_same<R, double>::value) {
+        const FxField v{reinterpret_cast<int4*>(L.basis_v(0, k - 1)), L.bve + (int64_t)(k - 1) * (L.vs / 24)};
+        const FxField w{reinterpret_cast<int4*>(L.basis_w(0, k - 1)), L.bwe + (int64_t)(k - 1) * (L.vs / 24)};
+        fx_proj_dots(L, 0, k, 0, v, w, (int64_t)L.kcap * L.vs, coef, cpart, c->st);
+      } else {
+        proj_dots(L, k - 1, 0, L.basis_v(0, k - 1), L.basis_w(0, k - 1), (int64_t)L.kcap * L.vs, coef, cpart,
+                  c->st);
+      }
     });
     launch_check();
     std::vector<zd> h((size_t)nsrc * 2 * k);
@@ -539,27 +584,55 @@ SegPlan seg_plan(int k, int S) {
 
 template <typename R>
 struct SegStore {
-  R *r, *s, *v, *w;   // [segment][src][vs]
-  SrcScal* sc;        // [segment][src]
+  R *r, *s, *v, *w;           // [segment][src][vs]
+  SrcScal* sc;                // [segment][src]
+  short *re, *se, *ve, *we;   // FP64 calls: the exponents of the above
 };
 template <typename R>
 SegStore<R> seg_store(ov_context* c, const Lat<R>& L, int nseg) {
   const int64_t n = (int64_t)nseg * L.nsrc * L.vs;
-  return SegStore<R>{wsT<R>(c, B_CKR, n), wsT<R>(c, B_CKS, n), wsT<R>(c, B_CKV, n), wsT<R>(c, B_CKW, n),
-                     wsT<SrcScal>(c, B_CKSC, (int64_t)nseg * L.nsrc)};
+  SegStore<R> K{wsT<R>(c, B_CKR, n), wsT<R>(c, B_CKS, n), wsT<R>(c, B_CKV, n), wsT<R>(c, B_CKW, n),
+                wsT<SrcScal>(c, B_CKSC, (int64_t)nseg * L.nsrc), nullptr, nullptr, nullptr, nullptr};
+  if constexpr (std::is_same<R, double>::value) {
+    K.re = wsT<short>(c, B_CKRE, n / 24);
+    K.se = wsT<short>(c, B_CKSE, n / 24);
+    K.ve = wsT<short>(c, B_CKVE, n / 24);
+    K.we = wsT<short>(c, B_CKWE, n / 24);
+  }
+  return K;
 }
-// copy the window's first vector (v_{jbase}, w_{jbase}) of every source to or from a checkpoint
+// copy the recurrence's r and s to (or from) the checkpoint of segment t
 template <typename R>
-void window_slot(ov_context* c, const Lat<R>& L, int slot, R* v, R* w, bool to_window) {
-  const size_t pitch = sizeof(R) * L.kcap * L.vs, width = sizeof(R) * L.vs;
-  R* bv = L.bv + (int64_t)slot * L.vs;
-  R* bw = L.bw + (int64_t)slot * L.vs;
-  if (to_window) {
-    CK(cudaMemcpy2DAsync(bv, pitch, v, width, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
-    CK(cudaMemcpy2DAsync(bw, pitch, w, width, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
+void seg_rs(ov_context* c, const Lat<R>& L, const SegStore<R>& K, size_t t, bool restore) {
+  const int64_t fs = (int64_t)L.nsrc * L.vs;
+  auto copy = [&](void* live, void* kept, size_t bytes) {
+    CK(cudaMemcpyAsync(restore ? live : kept, restore ? kept : live, bytes, cudaMemcpyDeviceToDevice, c->st));
+  };
+  if constexpr (std::is_same<R, double>::value) {
+    copy(L.fr.c, K.r + t * fs, sizeof(R) * fs);
+    copy(L.fs.c, K.s + t * fs, sizeof(R) * fs);
+    copy(L.fr.e, K.re + t * (fs / 24), sizeof(short) * (fs / 24));
+    copy(L.fs.e, K.se + t * (fs / 24), sizeof(short) * (fs / 24));
   } else {
-    CK(cudaMemcpy2DAsync(v, width, bv, pitch, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
-    CK(cudaMemcpy2DAsync(w, width, bw, pitch, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
+    copy(L.r, K.r + t * fs, sizeof(R) * fs);
+    copy(L.s, K.s + t * fs, sizeof(R) * fs);
+  }
+}
+// copy a window slot's vectors (v, w of every source) to or from the checkpoint of segment t
+template <typename R>
+void window_slot(ov_context* c, const Lat<R>& L, int slot, const SegStore<R>& K, size_t t, bool to_window) {
+  const int64_t fs = (int64_t)L.nsrc * L.vs;
+  auto copy = [&](void* win, void* kept, size_t elem) {   // vectors of vs reals (or vs / 24 exponents)
+    const size_t n = elem == sizeof(short) ? L.vs / 24 : L.vs, width = elem * n, pitch = width * L.kcap;
+    char* w = static_cast<char*>(win) + slot * width;
+    if (to_window) CK(cudaMemcpy2DAsync(w, pitch, kept, width, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
+    else CK(cudaMemcpy2DAsync(kept, width, w, pitch, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
+  };
+  copy(L.bv, K.v + t * fs, sizeof(R));
+  copy(L.bw, K.w + t * fs, sizeof(R));
+  if constexpr (std::is_same<R, double>::value) {
+    copy(L.bve, K.ve + t * (fs / 24), sizeof(short));
+    copy(L.bwe, K.we + t * (fs / 24), sizeof(short));
   }
 }
 // steps j0 .. j1-1 without re-biorthogonalisation; with `next`, also the stencil of
@@ -579,20 +652,18 @@ void seg_steps(ov_context* c, Lat<R>& L, int j0, int j1, bool next) {
 // pass 1: the recurrence over all segments, checkpointing each segment start
 template <typename R>
 void seg_forward(ov_context* c, Lat<R>& L, const SegPlan& P, const SegStore<R>& K) {
-  const int64_t fs = (int64_t)L.nsrc * L.vs;
   run(c, OV_KIND_UPDATE, 1, [&] { tsl_init(L, c->st); });
   for (size_t t = 0; t < P.lo.size(); ++t) {
     const int j0 = P.lo[t];
     if (t > 0) {
       // v_{j0-1} moves from the end of the previous window to its first slot
-      window_slot(c, L, j0 - L.jbase - 1, K.v + (int64_t)t * fs, K.w + (int64_t)t * fs, false);
+      window_slot(c, L, j0 - L.jbase - 1, K, t, false);
       L.jbase = j0 - 1;
-      window_slot(c, L, 0, K.v + (int64_t)t * fs, K.w + (int64_t)t * fs, true);
+      window_slot(c, L, 0, K, t, true);
     } else {
       L.jbase = j0 - 1;
     }
-    CK(cudaMemcpyAsync(K.r + t * fs, L.r, sizeof(R) * fs, cudaMemcpyDeviceToDevice, c->st));
-    CK(cudaMemcpyAsync(K.s + t * fs, L.s, sizeof(R) * fs, cudaMemcpyDeviceToDevice, c->st));
+    seg_rs(c, L, K, t, false);
     CK(cudaMemcpyAsync(K.sc + t * L.nsrc, L.sc, sizeof(SrcScal) * L.nsrc, cudaMemcpyDeviceToDevice, c->st));
     seg_steps(c, L, j0, P.hi[t], false);
   }
@@ -601,20 +672,13 @@ void seg_forward(ov_context* c, Lat<R>& L, const SegPlan& P, const SegStore<R>& 
 // replay segment t from its checkpoint (with `next`: also v_{j1}, w_{j1})
 template <typename R>
 void seg_replay(ov_context* c, Lat<R>& L, const SegPlan& P, const SegStore<R>& K, int t, bool next) {
-  const int64_t fs = (int64_t)L.nsrc * L.vs;
   const int j0 = P.lo[t];
   L.jbase = j0 - 1;
-  if (t > 0) window_slot(c, L, 0, K.v + (int64_t)t * fs, K.w + (int64_t)t * fs, true);
-  CK(cudaMemcpyAsync(L.r, K.r + t * fs, sizeof(R) * fs, cudaMemcpyDeviceToDevice, c->st));
-  CK(cudaMemcpyAsync(L.s, K.s + t * fs, sizeof(R) * fs, cudaMemcpyDeviceToDevice, c->st));
+  if (t > 0) window_slot(c, L, 0, K, (size_t)t, true);
+  seg_rs(c, L, K, (size_t)t, true);
   // only the forward scalars: the reverse sweep keeps its own in the same structs
   CK(cudaMemcpy2DAsync(L.sc, sizeof(SrcScal), K.sc + t * L.nsrc, sizeof(SrcScal), offsetof(SrcScal, g_alpha),
                        L.nsrc, cudaMemcpyDeviceToDevice, c->st));
-  if constexpr (std::is_same<R, double>::value)
-    run(c, OV_KIND_UPDATE, 2, [&] {
-      fx_encode(L.r, L.fr, L.nsrc, L.g.V, L.vs, c->st);
-      fx_encode(L.s, L.fs, L.nsrc, L.g.V, L.vs, c->st);
-    });
   seg_steps(c, L, j0, P.hi[t], next && P.hi[t] < L.k);
   launch_check();
 }
@@ -947,10 +1011,7 @@ int tsl_sign_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   check_ptr(x);
   const int S = c->opt.segment > 0 && c->opt.segment < k ? c->opt.segment : 0;
   Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0);
-  run(c, OV_KIND_LAYOUT, 2, [&] {
-    pack_spinors<R>(static_cast<const double*>(b), L.r, nsrc, L.g.V, L.vs, c->st);
-    pack_spinors<R>(static_cast<const double*>(b), L.s, nsrc, L.g.V, L.vs, c->st);
-  });
+  pack_start(c, L, b);
   SegPlan P;
   SegStore<R> K{};
   CK(cudaEventRecord(c->ev[0], c->st));
@@ -1028,18 +1089,21 @@ int block_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, d
   }
   L.mdir = (R)m_dir;
   if constexpr (std::is_same<R, double>::value) {
-    int4* fe = wsT<int4>(c, B_FXDL, kFxLinkEntries * V);
-    short* fx = wsT<short>(c, B_FXDE, 5 * V);
-    L.fd = FxLinks{fe, fx};
-    run(c, OV_KIND_LAYOUT, 1, [&] {
-      pack_dh_links_fx(static_cast<const double*>(U), static_cast<const double*>(E), m_dir, fe, fx, V, L.ef, L.efinv,
+    int4* fe = wsT<int4>(c, B_FXDL, fx_link_ints(V));
+    short* ex = wsT<short>(c, B_FXDE, 5 * V);
+    L.fd = FxLinks{fe, ex};
+    run(c, OV_KIND_LAYOUT, 2, [&] {
+      pack_dh_links_fx(static_cast<const double*>(U), static_cast<const double*>(E), m_dir, fe, ex, V, L.ef, L.efinv,
                        c->st);
+      fx_pack_block(static_cast<const double*>(top), static_cast<const double*>(bottom), L.fr, L.fs, nsrc, V, L.vs,
+                    c->st);
+    });
+  } else {
+    run(c, OV_KIND_LAYOUT, 1, [&] {
+      pack_block_start<R>(static_cast<const double*>(top), static_cast<const double*>(bottom), L.r, L.s, nsrc, V,
+                          L.vs, c->st);
     });
   }
-  run(c, OV_KIND_LAYOUT, 1, [&] {
-    pack_block_start<R>(static_cast<const double*>(top), static_cast<const double*>(bottom), L.r, L.s, nsrc, V,
-                        L.vs, c->st);
-  });
   CK(cudaEventRecord(c->ev[0], c->st));
   forward_krylov(c, L);
   CK(cudaEventRecord(c->ev[1], c->st));
@@ -1351,10 +1415,7 @@ int vjp_forward(ov_context* c, const int32_t dims[4], const void* U, double mu, 
   F.L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0);
   Lat<R>& L = F.L;
   const int64_t V = L.g.V, vs = L.vs;
-  run(c, OV_KIND_LAYOUT, 2, [&] {
-    pack_spinors<R>(static_cast<const double*>(b), L.r, nsrc, V, vs, c->st);
-    pack_spinors<R>(static_cast<const double*>(b), L.s, nsrc, V, vs, c->st);
-  });
+  pack_start(c, L, b);
   CK(cudaEventRecord(c->ev[0], c->st));
   if (S > 0) {
     F.P = seg_plan(k, S);
@@ -1431,7 +1492,21 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
   CK(cudaEventRecord(c->ev[2], c->st));
   // g_y = V^dag xbar
   R* xb = wsT<R>(c, B_XBAR, nsrc * vs);
-  run(c, OV_KIND_LAYOUT, 1, [&] { pack_spinors<R>(static_cast<const double*>(xbar), xb, nsrc, V, vs, c->st); });
+  FxField fxb{};
+  if constexpr (std::is_same<R, double>::value) {
+    fxb = FxField{reinterpret_cast<int4*>(xb), wsT<short>(c, B_XBE, nsrc * (vs / 24))};
+    run(c, OV_KIND_LAYOUT, 1,
+        [&] { fx_pack(static_cast<const double*>(xbar), fxb, FxField{}, nullptr, nsrc, V, vs, c->st); });
+  } else {
+    run(c, OV_KIND_LAYOUT, 1, [&] { pack_spinors<R>(static_cast<const double*>(xbar), xb, nsrc, V, vs, c->st); });
+  }
+  // out[src][2 (j - j0)] = v_j^dag xbar
+  auto xbar_dots = [&](int j0, int nvec, zd* out, zd* cpart) {
+    run(c, OV_KIND_COMBINE, 2, [&] {
+      if constexpr (std::is_same<R, double>::value) fx_proj_dots(L, j0, nvec, 1, fxb, FxField{}, vs, out, cpart, c->st);
+      else basis_dots_range(L, j0, nvec, xb, vs, out, cpart, c->st);
+    });
+  };
   const int64_t nsb = (V + 127) / 128;
   zd* gy = wsT<zd>(c, B_GY, (int64_t)nsrc * 2 * k);
   zd* cpart = wsT<zd>(c, B_CPART, (int64_t)nsrc * 2 * k * nsb);
@@ -1439,12 +1514,10 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
     // second pass: g_y one replayed segment at a time
     for (size_t t = 0; t < P.lo.size(); ++t) {
       seg_replay(c, L, P, K, (int)t, false);
-      run(c, OV_KIND_COMBINE, 2, [&] {
-        basis_dots_range(L, P.lo[t], P.hi[t] - P.lo[t], xb, vs, gy + 2 * P.lo[t], cpart, c->st);
-      });
+      xbar_dots(P.lo[t], P.hi[t] - P.lo[t], gy + 2 * P.lo[t], cpart);
     }
   } else {
-    run(c, OV_KIND_COMBINE, 2, [&] { basis_dots(L, k, xb, vs, gy, cpart, c->st); });
+    xbar_dots(0, k, gy, cpart);
   }
   launch_check();
   // G_T = L_sgn(T^dag, beta0 g_y e1^T).  The Theorem-1 block iteration on
@@ -1630,15 +1703,25 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
   B.m = m;
   B.gv = wsT<R>(c, B_GV, nsrc * vs);
   B.gw = wsT<R>(c, B_GW, nsrc * vs);
-  B.gv_new = wsT<R>(c, B_GV2, nsrc * vs);
-  B.gw_new = wsT<R>(c, B_GW2, nsrc * vs);
+  // (the fixed-point sweep replaces its gradients in place)
+  B.gv_new = std::is_same<R, double>::value ? nullptr : wsT<R>(c, B_GV2, nsrc * vs);
+  B.gw_new = std::is_same<R, double>::value ? nullptr : wsT<R>(c, B_GW2, nsrc * vs);
   B.gr_ring = wsT<R>(c, B_GR, (int64_t)m * nsrc * vs);
   B.gs_ring = wsT<R>(c, B_GS, (int64_t)m * nsrc * vs);
   B.gp_ring = wsT<R>(c, B_GP, (int64_t)m * nsrc * vs);
   B.hin = wsT<R>(c, B_HIN, (int64_t)nsrc * vs);
-  if constexpr (std::is_same<R, double>::value) {
-    B.fp = FxField{wsT<int4>(c, B_FXP, nsrc * (vs / 2)), wsT<short>(c, B_FXPE, nsrc * V)};
-    B.fh = FxField{wsT<int4>(c, B_FXH, nsrc * (vs / 2)), wsT<short>(c, B_FXHE, nsrc * V)};
+  constexpr bool fx = std::is_same<R, double>::value;
+  if constexpr (fx) {
+    auto view = [&](R* p, int id, int64_t n) {
+      return FxField{reinterpret_cast<int4*>(p), wsT<short>(c, id, n * (vs / 24))};
+    };
+    B.fgv = view(B.gv, B_GVE, nsrc);
+    B.fgw = view(B.gw, B_GWE, nsrc);
+    B.fgr = view(B.gr_ring, B_GRE, (int64_t)m * nsrc);
+    B.fgs = view(B.gs_ring, B_GSE, (int64_t)m * nsrc);
+    B.fgp = view(B.gp_ring, B_GPE, (int64_t)m * nsrc);
+    B.fh = view(B.hin, B_HINE, nsrc);
+    B.fxb = fxb;
   }
   B.xbar = xb;
   B.y = y;
@@ -1653,23 +1736,27 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
     CK(cudaMemcpyAsync(B.reb_steps, reb.data(), sizeof(int) * reb.size(), cudaMemcpyHostToDevice, c->st));
   B.force = wsT<double>(c, B_FORCE, 72 * V, true);
   {
-    const int ns = force_splits(V);
+    const int ns = fx ? fx_force_splits(V) : force_splits(V);
     B.force_parts = ns > 1 ? wsT<double>(c, B_FPARTS, (int64_t)ns * 72 * V) : nullptr;
   }
   B.dmu = wsT<double>(c, B_DMU, 1, true);
-  B.dmu_part = wsT<zd>(c, B_DMUPART, kForceSplitMax * ((V + 127) / 128) + 64);
+  B.dmu_part = wsT<zd>(c, B_DMUPART, kForceSplitMax * ((V + 15) / 16) + 64);
   B.dmu_cnt = wsT<unsigned>(c, B_DMUCNT, 4);
   zd* coef = wsT<zd>(c, B_COEF, (int64_t)nsrc * 2 * k);
   auto sweep = [&] {
   run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_init(L, B, c->st); });
   run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_combine(L, B, k - 1, 0, c->st); });
   run(c, OV_KIND_REV_STENCIL, 1, [&] { rev_stencil(L, B, k - 1, 0, -1, 0, c->st); });
-  std::swap(B.gv, B.gv_new);
-  std::swap(B.gw, B.gw_new);
+  auto swap_g = [&] {
+    if (fx) return;
+    std::swap(B.gv, B.gv_new);
+    std::swap(B.gw, B.gw_new);
+  };
+  swap_g();
   int slot = 1, j0 = k - 1, nrec = 0;
   for (int j = k - 2; j >= 0; --j) {
     if (slot == m) {
-      run(c, OV_KIND_FORCE, 4, [&] { force_flush(L, B, nullptr, m, j0, c->st); });
+      run(c, OV_KIND_FORCE, fx ? 1 : 4, [&] { force_flush(L, B, nullptr, m, j0, c->st); });
       slot = 0;
       j0 = j;
     }
@@ -1680,27 +1767,34 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
       seg_combine(tcur);
     }
     const int prev = slot == 0 ? m - 1 : slot - 1;
-    run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_dots(L, B, j, c->st); });
+    // (the fixed-point stencil of step j + 1 has formed these dots)
+    if constexpr (!fx) run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_dots(L, B, j, c->st); });
     const int rb = rebiorth_at(j + 1, c->opt.rebiorth);
     run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_form(L, B, j, slot, !rb, c->st); });
     if (rb) {
-      R* grs = B.gr_ring + (int64_t)slot * nsrc * vs;
-      R* gss = B.gs_ring + (int64_t)slot * nsrc * vs;
       for (int ps = 0; ps < c->opt.passes; ++ps) {
-        run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 1, grs, gss, vs, coef, cpart, c->st); });
-        run(c, OV_KIND_PROJ_UPDATE, 1, [&] { proj_update(L, j, 1, grs, gss, vs, coef, false, c->st, ps > 0); });
+        if constexpr (fx) {
+          const FxField gr = fx_src(B.fgr, (int64_t)slot * nsrc, vs), gs = fx_src(B.fgs, (int64_t)slot * nsrc, vs);
+          const int fin = ps == c->opt.passes - 1 ? 2 : 0;
+          run(c, OV_KIND_PROJ_DOTS, 2, [&] { fx_proj_dots(L, 0, j + 1, 1, gr, gs, vs, coef, cpart, c->st); });
+          run(c, OV_KIND_PROJ_UPDATE, 1, [&] { fx_proj_update(L, &B, j + 1, 1, gr, gs, vs, coef, j, fin, c->st); });
+        } else {
+          R* grs = B.gr_ring + (int64_t)slot * nsrc * vs;
+          R* gss = B.gs_ring + (int64_t)slot * nsrc * vs;
+          run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 1, grs, gss, vs, coef, cpart, c->st); });
+          run(c, OV_KIND_PROJ_UPDATE, 1, [&] { proj_update(L, j, 1, grs, gss, vs, coef, false, c->st, ps > 0); });
+        }
         run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_proj_record(L, B, j, nrec, coef, c->st); });
       }
-      run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_alpha_dots(L, B, j, slot, c->st); });
+      if constexpr (!fx) run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_alpha_dots(L, B, j, slot, c->st); });
       ++nrec;
     }
     run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_combine(L, B, j, slot, c->st); });
     run(c, OV_KIND_REV_STENCIL, 1, [&] { rev_stencil(L, B, j, slot, prev, nrec, c->st); });
-    std::swap(B.gv, B.gv_new);
-    std::swap(B.gw, B.gw_new);
+    swap_g();
     ++slot;
   }
-  run(c, OV_KIND_FORCE, 4, [&] { force_flush(L, B, nullptr, slot, j0, c->st); });
+  run(c, OV_KIND_FORCE, fx ? 1 : 4, [&] { force_flush(L, B, nullptr, slot, j0, c->st); });
   };
   if (S > 0) {
     sweep();   // segment replays copy checkpoints between the steps: launched directly
@@ -2310,7 +2404,7 @@ int apply_h_impl(ov_context* c, const int32_t dims[4], const void* U, double mu,
   }
   if constexpr (std::is_same<R, double>::value) {
     run(c, OV_KIND_LAYOUT, 1,
-        [&] { fx_pack(static_cast<const double*>(in), L.fr, L.r, nsrc, L.g.V, L.vs, c->st); });
+        [&] { fx_pack(static_cast<const double*>(in), L.fr, FxField{}, L.r, nsrc, L.g.V, L.vs, c->st); });
     run(c, OV_KIND_APPLY_H, 1,
         [&] { fx_apply_h(L, L.fr, L.r, static_cast<double*>(out), dagger, 1, c->st, var); });
   } else if (var != APPLY_IL) {
