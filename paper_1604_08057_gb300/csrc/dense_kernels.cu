@@ -113,10 +113,6 @@ __device__ __forceinline__ double gj_nrm(zd a) { return fma(a.re, a.re, a.im * a
 __device__ __forceinline__ zd gj_mul(zd a, zd b) {
   return mk(fma(a.re, b.re, -(a.im * b.im)), fma(a.re, b.im, a.im * b.re));
 }
-__device__ __forceinline__ zd gj_recip(zd b) {
-  const double d = gj_nrm(b);
-  return mk(b.re / d, -b.im / d);
-}
 
 __device__ __forceinline__ unsigned long long gj_key(double nrm, int i) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(nrm);
@@ -179,16 +175,19 @@ __global__ void __launch_bounds__(GJ_THREADS, 6) k_gj_step(const zd* __restrict_
   const int p = bad ? kk : cand;
   const zd* pr = xin + (int64_t)p * k;
   const zd piv = pr[kk];
-  // 1/pivot and the row factor m = X[i][kk]/pivot, once per warp
-  zd inv = mk(0.0, 0.0), m = mk(0.0, 0.0);
-  if ((threadIdx.x & 31) == 0) {
-    inv = gj_recip(piv);
-    m = gj_mul(fr, inv);
+  // 1/pivot and the row factor m = X[i][kk]/pivot, once per block, the two divisions in two
+  // lanes (a division of a warp takes the SM's FP64 pipe some 300 cycles)
+  __shared__ zd inv_s, m_s;
+  if (threadIdx.x < 32) {
+    const double q = (threadIdx.x == 0 ? piv.re : -piv.im) / gj_nrm(piv);
+    const zd v = mk(__shfl_sync(0xffffffffu, q, 0), __shfl_sync(0xffffffffu, q, 1));
+    if (threadIdx.x == 0) {
+      inv_s = v;
+      m_s = gj_mul(fr, v);
+    }
   }
-  inv.re = __shfl_sync(0xffffffffu, inv.re, 0);
-  inv.im = __shfl_sync(0xffffffffu, inv.im, 0);
-  m.re = __shfl_sync(0xffffffffu, m.re, 0);
-  m.im = __shfl_sync(0xffffffffu, m.im, 0);
+  __syncthreads();
+  const zd inv = inv_s, m = m_s;
   const bool offer = i != p && !row_used && kk + 1 < k;
   if (JPT > 0) {
     zd pv[JPT > 0 ? JPT : 1];
@@ -381,6 +380,7 @@ __global__ void __launch_bounds__(GJP_THREADS) k_gj_persist(const zd* __restrict
   double* pn = reinterpret_cast<double*>(qs + k);   // |pivot|^2 of each step (block 0, for log|det|)
   zd* pvn = reinterpret_cast<zd*>(pn + k);          // the next step's pivot row, prefetched
   __shared__ zd ms[GJP_RMAX];                 // row factors X[i][kk] / pivot
+  __shared__ zd inv_s;                        // 1 / pivot
   __shared__ int used_s[GJP_RMAX];
   __shared__ unsigned long long best_s, key_s, pre_s;
   const int pb = blockIdx.y;
@@ -448,10 +448,17 @@ __global__ void __launch_bounds__(GJP_THREADS) k_gj_persist(const zd* __restrict
       pvr[q] = j < k ? (pre ? pvn[j] : ld_cg(prg + j)) : mk(0.0, 0.0);
       if (j < k) pv[j] = pvr[q];
     }
-    const zd piv = pre ? pvn[kk] : ld_cg(prg + kk);
-    const zd inv = gj_recip(piv);
     const int lp = p - r0;   // local index of the pivot row (in range only in its owner)
-    if (t < nr) ms[t] = gj_mul(xs[(int64_t)t * k + kk], inv);
+    zd piv = mk(0.0, 0.0);
+    if (t < 32) {
+      // 1/pivot and the row factors by one warp, the two divisions in two lanes: in every
+      // thread they keep the SM's FP64 pipe busy for some 2.5 us per step
+      piv = pre ? pvn[kk] : ld_cg(prg + kk);
+      const double q = (t == 0 ? piv.re : -piv.im) / gj_nrm(piv);
+      const zd inv = mk(__shfl_sync(0xffffffffu, q, 0), __shfl_sync(0xffffffffu, q, 1));
+      if (t == 0) inv_s = inv;
+      if (t < nr) ms[t] = gj_mul(xs[(int64_t)t * k + kk], inv);
+    }
     if (t == 0) {
       prow[kk] = p;
       if (lp >= 0 && lp < nr) used_s[lp] = 1;
@@ -558,7 +565,7 @@ __global__ void __launch_bounds__(GJP_THREADS) k_gj_persist(const zd* __restrict
 #pragma unroll
       for (int q = 0; q < JPT; ++q) {
         const int j = t + q * GJP_THREADS;
-        if (j < k) row[j] = (j == kk) ? inv : gj_mul(pvr[q], inv);
+        if (j < k) row[j] = (j == kk) ? inv_s : gj_mul(pvr[q], inv_s);
       }
     }
     __syncthreads();
@@ -621,29 +628,35 @@ static bool gjp_shape(int k, int nb, int* R_out, int* bp_out, size_t* smem_out) 
   }
   const GjpKernel kern = gjp_kernel(k);
   if (nsm <= 0 || k < 2 || !kern || nb < 1) return false;
-  const int per = std::max(1, nsm / nb);
-  const int R = (k + per - 1) / per;
-  if (R > GJP_RMAX) return false;
-  const int bp = (k + R - 1) / R;
-  if (bp > GJ_KEY_SLOTS) return false;
-  const size_t smem =
-      ((size_t)R * k + 2 * (size_t)k) * sizeof(zd) + 2 * (size_t)k * sizeof(int) + (size_t)k * sizeof(double);
-  if (smem + 2048 > (size_t)smem_optin) return false;
   // one value for every caller (worker threads may race here)
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin - 2048) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GJP_THREADS, smem) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+  // Several problems take two blocks per SM where they fit: one problem's steps fill the
+  // other's waits (four problems at k = 400: 40.1 -> 34.3 ms per sign).  A block has at
+  // least three rows: with fewer, the words to poll cost more than the rows (k = 200: 7.1 ms
+  // per sign with two rows, 6.1 with three, 6.3 with four, 8.7 with eight).
+  for (int occ = nb > 1 ? 2 : 1; occ >= 1; --occ) {
+    const int per = std::max(1, occ * nsm / nb);
+    const int R = std::max((k + per - 1) / per, std::min(k, 3));
+    const int bp = (k + R - 1) / R;
+    if (R > GJP_RMAX || bp > GJ_KEY_SLOTS) continue;
+    const size_t smem =
+        ((size_t)R * k + 2 * (size_t)k) * sizeof(zd) + 2 * (size_t)k * sizeof(int) + (size_t)k * sizeof(double);
+    if (smem + 2048 > (size_t)smem_optin) continue;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GJP_THREADS, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if ((int64_t)per_sm * nsm < (int64_t)bp * nb) continue;
+    *R_out = R;
+    *bp_out = bp;
+    *smem_out = smem;
+    return true;
   }
-  if ((int64_t)per_sm * nsm < (int64_t)bp * nb) return false;
-  *R_out = R;
-  *bp_out = bp;
-  *smem_out = smem;
-  return true;
+  return false;
 }
 
 // Cooperative inversions issued from different streams (the worker contexts of
