@@ -262,6 +262,29 @@ __device__ __forceinline__ zd warp_sum(zd v) {
   return v;
 }
 
+// Sums of N values (a power of two, N <= 32) over the warp's lanes, N values at a time: at
+// each level of the tree half of the values move to the other half of the lanes, so N - 1
+// additions (and one per remaining level) do the work of 5 N.  Every total is formed by the
+// additions of warp_sum's tree, bit for bit; lane l returns value l N / 32.
+template <int N>
+__device__ __forceinline__ double warp_sum_multi(double (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+  int o = 16;
+#pragma unroll
+  for (int n = N / 2; n >= 1; n >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const double keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    o >>= 1;
+  }
+  double s = v[0];
+  for (; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
 // Sum over the block of NV complex values per thread; result valid in thread 0.
 // scratch: shared array of at least NV * 32 zd.  blockDim.x must be a multiple of 32.
 template <int NV>

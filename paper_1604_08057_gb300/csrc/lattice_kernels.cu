@@ -46,15 +46,31 @@ static inline unsigned plane_threads(const Geom& g) { return (unsigned)((g.nx * 
 // ---------------------------------------------------------------------------
 // layout conversion
 // ---------------------------------------------------------------------------
+// The user's spinors are rows of 192 bytes per site: a warp moves its 32 rows (6 KB in a
+// row) through shared memory, so that global accesses on both sides are contiguous (each
+// thread walking its own row: 219 us for the layout of 32 sources at 14x14^3, FP32).
+constexpr int kRow = 13;   // double2 per staged row (padded by one: conflict-free)
 template <typename R>
-__global__ void k_pack_spinors(const double* __restrict__ aos, R* __restrict__ dst, int64_t V, int64_t vs) {
-  const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(BS) k_pack_spinors(const double* __restrict__ aos, R* __restrict__ dst, int64_t V,
+                                                     int64_t vs) {
+  __shared__ double2 rows[BS / 32][32 * kRow];
+  const int lane = threadIdx.x & 31;
+  double2* st = rows[threadIdx.x >> 5];
+  const int64_t x0 = blockIdx.x * (int64_t)BS + (threadIdx.x & ~31), x = x0 + lane;
   const int src = blockIdx.y;
+  if (x0 >= V) return;   // whole warps
+  const int n = (int)min((int64_t)32, V - x0) * 12;
+  const double2* in = reinterpret_cast<const double2*>(aos) + ((int64_t)src * V + x0) * 12;
+#pragma unroll
+  for (int q = 0; q < 12; ++q) {
+    const int i = q * 32 + lane;
+    if (i < n) st[i / 12 * kRow + i % 12] = in[i];
+  }
+  __syncwarp();
   if (x >= V) return;
-  const double2* in = reinterpret_cast<const double2*>(aos) + ((int64_t)src * V + x) * 12;
   Spinor<R> o;
 #pragma unroll
-  for (int c = 0; c < 12; ++c) { double2 t = in[c]; o.c[c] = mk<R>((R)t.x, (R)t.y); }
+  for (int c = 0; c < 12; ++c) { double2 t = st[lane * kRow + c]; o.c[c] = mk<R>((R)t.x, (R)t.y); }
   store_spinor(dst + src * vs, V, x, o);
 }
 
@@ -85,15 +101,28 @@ __global__ void k_pack_block_start(const double* __restrict__ top, const double*
 }
 
 template <typename R>
-__global__ void k_unpack_spinors(const R* __restrict__ f, double* __restrict__ aos, int64_t V, int64_t vs) {
-  const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(BS) k_unpack_spinors(const R* __restrict__ f, double* __restrict__ aos, int64_t V,
+                                                       int64_t vs) {
+  __shared__ double2 rows[BS / 32][32 * kRow];
+  const int lane = threadIdx.x & 31;
+  double2* st = rows[threadIdx.x >> 5];
+  const int64_t x0 = blockIdx.x * (int64_t)BS + (threadIdx.x & ~31), x = x0 + lane;
   const int src = blockIdx.y;
-  if (x >= V) return;
-  Spinor<R> o;
-  load_spinor(f + src * vs, V, x, o);
-  double2* out = reinterpret_cast<double2*>(aos) + ((int64_t)src * V + x) * 12;
+  if (x0 >= V) return;   // whole warps
+  const int n = (int)min((int64_t)32, V - x0) * 12;
+  if (x < V) {
+    Spinor<R> o;
+    load_spinor(f + src * vs, V, x, o);
 #pragma unroll
-  for (int c = 0; c < 12; ++c) out[c] = make_double2((double)o.c[c].re, (double)o.c[c].im);
+    for (int c = 0; c < 12; ++c) st[lane * kRow + c] = make_double2((double)o.c[c].re, (double)o.c[c].im);
+  }
+  __syncwarp();
+  double2* out = reinterpret_cast<double2*>(aos) + ((int64_t)src * V + x0) * 12;
+#pragma unroll
+  for (int q = 0; q < 12; ++q) {
+    const int i = q * 32 + lane;
+    if (i < n) out[i] = st[i / 12 * kRow + i % 12];
+  }
 }
 
 template <typename R>
@@ -927,64 +956,116 @@ void tsl_update(const Lat<R>& L, int j, bool finalize, cudaStream_t st) {
 static inline int proj_spt(int nb) { return nb >= NB ? 4 : 1; }
 
 // Each thread accumulates `spt` sites (strided by the block size, so loads stay
-// coalesced) before the block reduction, which then costs 1/spt per site.
+// coalesced) before the block reduction, which then costs 1/spt per site.  One side per
+// block (blockIdx.z = source * sides + side): both sides' sums and fields in one thread
+// leave two blocks per SM, and the 16 sums cost 160 FP64 additions per warp one by one.
+// The basis vectors come through a ring of three in shared memory, copied two ahead: with
+// the loads in registers the kernel waits for them (9.8 of 13 cycles per instruction).
+// Bound by HBM (each basis vector is read once).  6x18^3, 4 sources, projections every step to
+// k = 80, two passes: 91 ms of dots with both sides in a thread and the loads in registers, 65
+// with one side per block, 47 with the ring.
+constexpr int kDotsRing = 3;
 template <typename R>
 __global__ void __launch_bounds__(BS) k_proj_dots(Lat<R> L, int nb, int mode, const R* __restrict__ a,
                                                    const R* __restrict__ b, int64_t ab_stride,
-                                                   zd* __restrict__ cpart, int64_t cp_stride, int spt, int ioff) {
-  __shared__ zd scratch[2 * NB * 32];
-  const int src = blockIdx.z;
-  const int i0 = blockIdx.y * NB;
+                                                   zd* __restrict__ cpart, int64_t cp_stride, int spt, int ioff,
+                                                   int sides) {
+  constexpr int NC = sizeof(R) == 4 ? 6 : 12;   // 16-byte chunks of a spinor
+  __shared__ float4 ring[kDotsRing][NC][BS];
+  __shared__ double part[BS / 32][2 * NB];
+  const int src = blockIdx.z / sides, side = blockIdx.z - src * sides;
+  const int i0 = blockIdx.y * NB, n = min(NB, nb - i0);
   const int64_t V = L.g.V;
-  SiteDot<R> acc[2 * NB];
+  const R* f = (side ? b : a) + src * ab_stride;
+  const bool usew = (mode == 0) == (side == 0);
+  const float4* bas = reinterpret_cast<const float4*>(usew ? L.basis_w(src, ioff + i0) : L.basis_v(src, ioff + i0));
+  const int64_t vstep = L.vs * (int64_t)sizeof(R) / 16;
+  const int64_t x0 = blockIdx.x * (int64_t)spt * BS + threadIdx.x;
+  SiteDot<R> acc[NB];
 #pragma unroll
-  for (int t = 0; t < 2 * NB; ++t) acc[t].zero();
+  for (int t = 0; t < NB; ++t) acc[t].zero();
+  // the next copy: vector it at site xi
+  int it = 0, slot = 0, nq = 0;
+  int64_t xi = x0;
+  auto issue = [&](int sl) {
+    if (nq < spt && xi < V) {
+      const float4* p = bas + it * vstep + xi;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(&ring[sl][c][threadIdx.x])),
+                     "l"(p + c * V)
+                     : "memory");
+      }
+      if (++it == n) {
+        it = 0;
+        ++nq;
+        xi += BS;
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int u = 0; u < kDotsRing - 1; ++u) issue(u);
   for (int q = 0; q < spt; ++q) {
-    const int64_t x = (blockIdx.x * (int64_t)spt + q) * blockDim.x + threadIdx.x;
+    const int64_t x = x0 + (int64_t)q * BS;
     if (x >= V) break;
-    Spinor<R> va, vb, e;
-    load_spinor(a + src * ab_stride, V, x, va);
-    if (b) load_spinor(b + src * ab_stride, V, x, vb);
+    Spinor<R> v, e;
+    load_spinor(f, V, x, v);
 #pragma unroll
     for (int t = 0; t < NB; ++t) {
-      const int i = i0 + t;
-      if (i < nb) {
-        const R* da = mode == 0 ? L.basis_w(src, ioff + i) : L.basis_v(src, ioff + i);
-        load_spinor(da, V, x, e);
+      if (t < n) {
+        issue(slot == 0 ? kDotsRing - 1 : slot - 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kDotsRing - 1) : "memory");
+        load_spinor(reinterpret_cast<const R*>(&ring[slot][0][0]), BS, threadIdx.x, e);
+        slot = slot == kDotsRing - 1 ? 0 : slot + 1;
 #pragma unroll
-        for (int c = 0; c < 12; ++c) acc[2 * t].add(e.c[c], va.c[c]);
-        if (b) {
-          const R* db = mode == 0 ? L.basis_v(src, ioff + i) : L.basis_w(src, ioff + i);
-          load_spinor(db, V, x, e);
-#pragma unroll
-          for (int c = 0; c < 12; ++c) acc[2 * t + 1].add(e.c[c], vb.c[c]);
-        }
+        for (int c = 0; c < 12; ++c) acc[t].add(e.c[c], v.c[c]);
       }
     }
   }
-  zd v[2 * NB];
+  double v[2 * NB];
 #pragma unroll
-  for (int t = 0; t < 2 * NB; ++t) v[t] = acc[t].value();
-  block_sum<2 * NB>(v, scratch);
-  if (threadIdx.x == 0) {
-    zd* cp = cpart + src * cp_stride;
+  for (int t = 0; t < NB; ++t) {
+    const zd s = acc[t].value();
+    v[2 * t] = s.re;
+    v[2 * t + 1] = s.im;
+  }
+  const double s = warp_sum_multi(v);
+  const int lane = threadIdx.x & 31;
+  if (!(lane & 1)) part[threadIdx.x >> 5][lane >> 1] = s;
+  __syncthreads();
+  if (threadIdx.x < 2 * NB) {
+    double t = part[0][threadIdx.x];
 #pragma unroll
-    for (int t = 0; t < 2 * NB; ++t) {
-      const int i = i0 + t / 2;
-      if (i < nb) cp[(int64_t)(2 * i + (t & 1)) * gridDim.x + blockIdx.x] = v[t];
-    }
+    for (int w = 1; w < BS / 32; ++w) t = t + part[w][threadIdx.x];
+    const int i = i0 + threadIdx.x / 2;
+    double* cp = reinterpret_cast<double*>(cpart + src * cp_stride + (int64_t)(2 * i + side) * gridDim.x + blockIdx.x);
+    if (i < nb) cp[threadIdx.x & 1] = t;
   }
 }
 
-__global__ void k_proj_reduce(const zd* __restrict__ cpart, int64_t cp_stride, int nsb, int nb,
-                              zd* __restrict__ coef, int64_t coef_stride) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;   // 2*i + side
+// coef = the sum of a coefficient's site blocks in block order; 32 coefficients per block,
+// their partials brought in by tiles (a thread that walks its own row alone waits for every
+// load)
+__global__ void __launch_bounds__(128) k_proj_reduce(const zd* __restrict__ cpart, int64_t cp_stride, int nsb, int nb,
+                                                     zd* __restrict__ coef, int64_t coef_stride) {
+  __shared__ double2 tile[32][33];
+  const int t0 = blockIdx.x * 32;   // 2*i + side
   const int src = blockIdx.y;
-  if (t >= 2 * nb) return;
-  const zd* cp = cpart + src * cp_stride + (int64_t)t * nsb;
+  const double2* cp = reinterpret_cast<const double2*>(cpart + src * cp_stride);
   zd s = mk(0.0, 0.0);
-  for (int b = 0; b < nsb; ++b) s = s + cp[b];
-  coef[src * coef_stride + t] = s;
+  for (int b0 = 0; b0 < nsb; b0 += 32) {
+    __syncthreads();
+    for (int q = threadIdx.x; q < 32 * 32; q += 128) {
+      const int t = t0 + q / 32, b = b0 + q % 32;
+      if (t < 2 * nb && b < nsb) tile[q / 32][q % 32] = cp[(int64_t)t * nsb + b];
+    }
+    __syncthreads();
+    if (threadIdx.x < 32)
+      for (int b = 0; b < min(32, nsb - b0); ++b) s = s + mk(tile[threadIdx.x][b].x, tile[threadIdx.x][b].y);
+  }
+  if (threadIdx.x < 32 && t0 + threadIdx.x < 2 * nb) coef[src * coef_stride + t0 + threadIdx.x] = s;
 }
 
 // SMALL: the coefficients are at rounding level relative to a and b (the second
@@ -1076,9 +1157,9 @@ void proj_dots(const Lat<R>& L, int j, int mode, const R* a, const R* b, int64_t
   const int spt = proj_spt(nb);
   const unsigned nsb = nblocks(L.g.V, BS * spt);
   const int64_t cp_stride = (int64_t)2 * L.k * nsb;
-  k_proj_dots<R><<<dim3(nsb, nblocks(nb, NB), L.nsrc), BS, 0, st>>>(L, nb, mode, a, b, ab_stride, cpart,
-                                                                     cp_stride, spt, 0);
-  k_proj_reduce<<<dim3(nblocks(2 * nb, 128), L.nsrc), 128, 0, st>>>(cpart, cp_stride, nsb, nb, coef,
+  k_proj_dots<R><<<dim3(nsb, nblocks(nb, NB), 2 * L.nsrc), BS, 0, st>>>(L, nb, mode, a, b, ab_stride, cpart,
+                                                                         cp_stride, spt, 0, 2);
+  k_proj_reduce<<<dim3(nblocks(2 * nb, 32), L.nsrc), 128, 0, st>>>(cpart, cp_stride, nsb, nb, coef,
                                                                       2 * (int64_t)L.k);
 }
 template <typename R>
@@ -1103,8 +1184,8 @@ void basis_dots_range(const Lat<R>& L, int j0, int nvec, const R* x, int64_t x_s
   const int64_t cp_stride = (int64_t)2 * L.k * nsb;
   // mode 1 makes side A dot the V basis
   k_proj_dots<R><<<dim3(nsb, nblocks(nvec, NB), L.nsrc), BS, 0, st>>>(L, nvec, 1, x, nullptr, x_stride,
-                                                                       cpart, cp_stride, spt, j0);
-  k_proj_reduce<<<dim3(nblocks(2 * nvec, 128), L.nsrc), 128, 0, st>>>(cpart, cp_stride, nsb, nvec, out,
+                                                                       cpart, cp_stride, spt, j0, 1);
+  k_proj_reduce<<<dim3(nblocks(2 * nvec, 32), L.nsrc), 128, 0, st>>>(cpart, cp_stride, nsb, nvec, out,
                                                                         2 * (int64_t)L.k);
 }
 template <typename R>
