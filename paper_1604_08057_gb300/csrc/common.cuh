@@ -309,18 +309,19 @@ __device__ __forceinline__ void block_sum(zd (&v)[NV], zd* scratch) {
 }
 
 // Returns true in every thread of the last block (of `total`) to arrive.
-// The counter is reset by that block.
+// The counter is reset by that block.  One thread fences for the block on both sides of its
+// atomic (the barriers order the others' accesses with it).
 __device__ __forceinline__ bool arrive_last(unsigned* counter, unsigned total) {
   __shared__ bool last;
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
+    __threadfence();
     unsigned t = atomicAdd(counter, 1u);
     last = (t == total - 1);
     if (last) *counter = 0u;
+    __threadfence();
   }
   __syncthreads();
-  if (last) __threadfence();
   return last;
 }
 

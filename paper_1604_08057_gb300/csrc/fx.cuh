@@ -43,6 +43,15 @@ __device__ __forceinline__ FxInt fx_split(fxll x) {
   return r;
 }
 __device__ __forceinline__ fxll fx_join(int h, int l) { return ((fxll)h << 30) + l; }
+// 64-bit shifts by 0 <= n <= 31: two instructions (a shift by any n < 64 takes five)
+__device__ __forceinline__ fxll fx_sar(fxll v, int n) {
+  const int lo = (int)v, hi = (int)(v >> 32);
+  return ((fxll)(hi >> n) << 32) | (unsigned)__funnelshift_r(lo, hi, n);
+}
+__device__ __forceinline__ fxll fx_shl(fxll v, int n) {
+  const int lo = (int)v, hi = (int)(v >> 32);
+  return ((fxll)(int)__funnelshift_l(lo, hi, n) << 32) | ((unsigned)lo << n);
+}
 __device__ __forceinline__ unsigned fx_mag(double d) { return (unsigned)__double2hiint(d) & 0x7fffffffu; }
 // 2^s as an FP64 number, |s| <= 1022
 __device__ __forceinline__ double fx_pow2(int s) { return __hiloint2double((s + 1023) * (1 << 20), 0); }
@@ -129,11 +138,16 @@ struct FxLoad {
   }
 };
 
+// acc += a b as one multiply-add (written out, so that sums are not re-associated into
+// products and separate 64-bit additions)
+__device__ __forceinline__ void fx_wide(fxll& acc, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
+}
 // one real product a b into (hh, x): a b ~ hh 2^60 + x 2^30
 __device__ __forceinline__ void fx_mac(fxll& hh, fxll& x, int ah, int al, int bh, int bl) {
-  hh += (fxll)ah * bh;
-  x += (fxll)ah * bl;
-  x += (fxll)al * bh;
+  fx_wide(hh, ah, bh);
+  fx_wide(x, ah, bl);
+  fx_wide(x, al, bh);
 }
 // acc += a b, acc += conj(a) b (acc as hh and x sums of its two parts)
 struct FxAcc { fxll hr, xr, hi, xi; };
@@ -207,15 +221,26 @@ __device__ __forceinline__ void fx_encode(const FxHalf& a, bool bad, FxH& o, int
   const bool none = top <= zero_top || e < FX_F_MIN;
   if (none && e != FX_BAD) e = FX_F_MIN;
   o.e = e;
-  // to units of 2^(e - 1079) = 2^(top - 57 - FX_E_BIAS): up to 62 bits, then down with rounding
-  const int up = none ? 0 : min(max(62 - (top - a.E), 0), 62);
-  const int dn = none ? 62 : min(max((top - 57) - a.E + up, 0), 62);
-  const fxll r = (1ll << dn) >> 1;
+  // to units of 2^(e - 1079) = 2^(top - 57 - FX_E_BIAS): down by r bits (rounded) or up by -r;
+  // a sum of several terms has r = 0 .. 6
+  const int r = top - 57 - a.E;
+  if (!none && r >= 0 && r < 32) {
+    const fxll h = (1ll << r) >> 1;
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const FxInt x = fx_split(none ? 0 : ((a.v[i].re << up) + r) >> dn);
-    const FxInt y = fx_split(none ? 0 : ((a.v[i].im << up) + r) >> dn);
-    o.q[i] = make_int4(x.h, x.l, y.h, y.l);
+    for (int i = 0; i < 6; ++i) {
+      const FxInt x = fx_split(fx_sar(a.v[i].re + h, r)), y = fx_split(fx_sar(a.v[i].im + h, r));
+      o.q[i] = make_int4(x.h, x.l, y.h, y.l);
+    }
+  } else {
+    const bool zero = none || r >= 62;
+    const int up = min(max(-r, 0), 62), dn = min(max(r, 0), 62);
+    const fxll h = (1ll << dn) >> 1;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const FxInt x = fx_split(zero ? 0 : ((a.v[i].re << up) + h) >> dn);
+      const FxInt y = fx_split(zero ? 0 : ((a.v[i].im << up) + h) >> dn);
+      o.q[i] = make_int4(x.h, x.l, y.h, y.l);
+    }
   }
 }
 // the sum's FP64 values
@@ -260,9 +285,7 @@ __device__ __forceinline__ FxCoef fx_coef(zd z) {
   r.c = make_int4(a.h, a.l, b.h, b.l);
   return r;
 }
-// acc += s c f, s = 1 (SG > 0), or -1 on components 0..2 and +1 on 3..5 (SG = 0: the pattern
-// under which gamma5 (-kappa acc) gains kappa c f).  false when f or c is marked.
-template <int SG>
+// acc += c f; false when f or c is marked
 __device__ __forceinline__ bool fx_axpy(FxHalf& acc, const FxCoef& c, const FxH& f) {
   if (f.e == FX_BAD || c.e == FX_BAD) return false;
   const int et = f.e + c.e;
@@ -274,14 +297,13 @@ __device__ __forceinline__ bool fx_axpy(FxHalf& acc, const FxCoef& c, const FxH&
   for (int i = 0; i < 6; ++i) {
     FxAcc t{half, 1ll << 29, half, 1ll << 29};
     fx_cmac(t, c.c, f.q[i]);
-    const fxll re = (t.hr + (t.xr >> 30)) >> d, im = (t.hi + (t.xi >> 30)) >> d;
-    if (SG == 0 && i < 3) {
-      acc.v[i].re -= re;
-      acc.v[i].im -= im;
-    } else {
-      acc.v[i].re += re;
-      acc.v[i].im += im;
+    fxll re = fx_sar(t.hr + (t.xr >> 30), min(d, 31)), im = fx_sar(t.hi + (t.xi >> 30), min(d, 31));
+    if (d > 31) {
+      re >>= d - 31;
+      im >>= d - 31;
     }
+    acc.v[i].re += re;
+    acc.v[i].im += im;
   }
   return true;
 }
@@ -294,8 +316,14 @@ __device__ __forceinline__ bool fx_add(FxHalf& acc, const FxH& f) {
   const fxll half = (1ll << d) >> 1;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    acc.v[i].re += (fx_join(f.q[i].x, f.q[i].y) + half) >> d;
-    acc.v[i].im += (fx_join(f.q[i].z, f.q[i].w) + half) >> d;
+    fxll re = fx_sar(fx_join(f.q[i].x, f.q[i].y) + half, min(d, 31));
+    fxll im = fx_sar(fx_join(f.q[i].z, f.q[i].w) + half, min(d, 31));
+    if (d > 31) {
+      re >>= d - 31;
+      im >>= d - 31;
+    }
+    acc.v[i].re += re;
+    acc.v[i].im += im;
   }
   return true;
 }
@@ -350,14 +378,23 @@ struct FxSite {
 // link "direction" of a hop: H uses e^{mu} forward and e^{-mu} backward in t, H^dagger the reverse
 __device__ __forceinline__ int fx_link_dir(int hop, int dagger) { return hop < 6 ? hop >> 1 : 3 + ((hop & 1) ^ dagger); }
 
-// E = max(E, exponent of every hop's term); a marked field or link gives at least FX_BAD
-__device__ __forceinline__ int fx_range(int E, const FxField& f, int off, const FxLinks& U, const Geom& g,
+// exponents of the eight hops' terms, 16 bits each: forward hops in f, backward in b
+struct FxExps {
+  unsigned long long f, b;
+};
+// the largest exponent of the hops' terms; a marked field or link gives at least FX_BAD
+__device__ __forceinline__ int fx_range(FxExps& x, const FxField& f, int off, const FxLinks& U, const Geom& g,
                                         const FxSite& s, int dagger) {
   const int V = (int)g.V;
+  int E = 0;
+  x.f = x.b = 0ull;
 #pragma unroll
   for (int hop = 0; hop < 8; ++hop) {
     const int n = s.neighbour(g, hop);
-    E = max(E, (int)f.e[off + n] + (int)U.ex[fx_link_dir(hop, dagger) * V + ((hop & 1) ? n : s.x)]);
+    const int e = (int)f.e[off + n] + (int)U.ex[fx_link_dir(hop, dagger) * V + ((hop & 1) ? n : s.x)];
+    E = max(E, e);
+    if (hop & 1) x.b |= (unsigned long long)(unsigned)e << (hop >> 1) * 16;
+    else x.f |= (unsigned long long)(unsigned)e << (hop >> 1) * 16;
   }
   return E;
 }
@@ -365,38 +402,99 @@ __device__ __forceinline__ int fx_range(int E, const FxField& f, int off, const 
 // (U^dagger h backward), the upper spin gains g and the lower spin +-phase (g_fwd - g_bwd);
 // phase = i for x and z, 1 for y and t; d and that lower spin are the partner's for x and y.
 // g is in units of 2^(E - FX_E_BIAS).
-template <int SGN>
-__device__ __forceinline__ void fx_hop(FxZ (&g)[3], int E, const FxField& f, int off, const FxLinks& U, int V, int n,
-                                       int x, int nu, int dir, int sp, int tau) {
-  const int ls = SGN > 0 ? x : n;
-  const int d = max(0, min(E - (int)f.e[off + n] - (int)U.ex[dir * V + ls], 62));
-  int4 h[3];
-  {
+// The neighbour's six int4 and the link's nine come through shared memory, copied
+// asynchronously one hop ahead: with the loads in registers a warp waits for each hop's
+// data, and 16 warps on an SM do not cover that (67 us per step pair at 14^4; stalls on
+// loads 5.7 cycles out of 11).
+// One such area per warp: everything in it is written and read by that warp's lanes.
+struct FxRow {         // a thread's components of one field, handed to another thread
+  int4 q[6][32];
+  int e[32];
+};
+struct FxSumRow {      // a thread's components of a sum
+  fxll v[12][32];
+  int e[32];
+};
+constexpr int FX_RING = 3;
+union FxStage {
+  struct {
+    int4 q[2][6][32];            // [hop parity][component][lane]
+    int4 u[2][9][16];            // [hop parity][entry][site]
+    int nb[8][16];               // neighbours of the hops
+  };
+  int4 ring[FX_RING][6][32];     // FxStream
+  FxRow row;
+  FxSumRow sum;
+  double2 out[16 * 13];          // rows of the user's layout
+};
+__device__ __forceinline__ void fx_row_put(FxRow& r, const FxH& f) {
+  const int t = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) r.q[i][t] = f.q[i];
+  r.e[t] = f.e;
+}
+__device__ __forceinline__ void fx_row_get(const FxRow& r, FxH& f) {
+  const int t = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) f.q[i] = r.q[i][t];
+  f.e = r.e[t];
+}
+__device__ __forceinline__ void fx_copy16(int4* dst, const int4* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void fx_copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void fx_copy_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void fx_hop_copy(FxStage& S, const FxField& f, int off, const FxLinks& U, int x, int hop,
+                                            int end, int dagger, int sp) {
+  if (hop < end) {
+    const int p = hop & 1, t = threadIdx.x & 31, n = S.nb[hop][t & 15];
     const int4* q = f.c + fx_at(off + n);
     const int4* qu = q + sp * 96;
-    const int4* qd = q + (nu < 2 ? 3 - sp : 2 + sp) * 96;
-    const int t = SGN * tau;
+    const int4* qd = q + (hop < 4 ? 3 - sp : 2 + sp) * 96;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const int4 u = __ldg(qu + a * 32), w = __ldg(qd + a * 32);
-      // |h.h| < 2^28, |h.l| < 2^30: the halves of the split add without carry
-      h[a] = (nu & 1) ? make_int4(u.x + t * w.x, u.y + t * w.y, u.z + t * w.z, u.w + t * w.w)
-                      : make_int4(u.x - t * w.z, u.y - t * w.w, u.z + t * w.x, u.w + t * w.y);
+      fx_copy16(&S.q[p][a][t], qu + a * 32);
+      fx_copy16(&S.q[p][3 + a][t], qd + a * 32);
     }
+    const int4* lk = U.e + fx_link_at(p ? n : x, fx_link_dir(hop, dagger)) + sp * 160;
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+      if (sp == 0 || i < 4) fx_copy16(&S.u[p][sp * 5 + i][t & 15], lk + i * 32);
+  }
+  fx_copy_commit();   // an empty group past the last hop keeps the waits' counts
+}
+template <int SGN>
+__device__ __forceinline__ void fx_hop(FxZ (&g)[3], const FxStage& S, int d, int nu, int sp, int tau) {
+  const int t = threadIdx.x & 31, slot = t & 15, p = SGN > 0 ? 0 : 1;
+  int4 h[3];
+  const int s = SGN * tau;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int4 u = S.q[p][a][t], w = S.q[p][3 + a][t];
+    // |h.h| < 2^28, |h.l| < 2^30: the halves of the split add without carry
+    h[a] = (nu & 1) ? make_int4(u.x + s * w.x, u.y + s * w.y, u.z + s * w.z, u.w + s * w.w)
+                    : make_int4(u.x - s * w.z, u.y - s * w.w, u.z + s * w.x, u.w + s * w.y);
   }
   const fxll half = (1ll << d) >> 1;
-  const int4* lk = U.e + fx_link_at(ls, dir);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     // six real products each: |hh| < 6 2^57, |x| < 6 (2^59 + 2^57)
-    FxAcc t{half, 1ll << 29, half, 1ll << 29};
+    FxAcc c{half, 1ll << 29, half, 1ll << 29};
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      const int4 u = __ldg(lk + (SGN > 0 ? a * 3 + b : b * 3 + a) * 32);
-      if (SGN > 0) fx_cmac(t, u, h[b]);
-      else fx_cdot(t, u, h[b]);
+      const int4 u = S.u[p][SGN > 0 ? a * 3 + b : b * 3 + a][slot];
+      if (SGN > 0) fx_cmac(c, u, h[b]);
+      else fx_cdot(c, u, h[b]);
     }
-    g[a] = FxZ{(t.hr + (t.xr >> 30)) >> d, (t.hi + (t.xi >> 30)) >> d};
+    g[a] = FxZ{fx_sar(c.hr + (c.xr >> 30), min(d, 31)), fx_sar(c.hi + (c.xi >> 30), min(d, 31))};
+  }
+  if (d > 31) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) g[a] = FxZ{g[a].re >> (d - 31), g[a].im >> (d - 31)};
   }
 }
 __device__ __forceinline__ void fx_swap_lower(FxHalf& a) {
@@ -406,31 +504,202 @@ __device__ __forceinline__ void fx_swap_lower(FxHalf& a) {
     a.v[i].im = __shfl_xor_sync(0xffffffffu, a.v[i].im, 16);
   }
 }
-// acc += the eight hops of D_w of field f (sites off + s), at acc's scale; every lane of the
-// warp.  A product is below 2^57 units, so the 48 of eight hops stay below 2^62.6 (for
+// acc += the hops of D_w of field f (sites off + s) in directions nu0 .. nu1 - 1 (all eight by
+// default), at acc's scale; every lane of the warp.  A product is below 2^57 units, so the 48 of eight hops stay below 2^62.6 (for
 // sixteen hops the caller takes E one higher).  The loop is kept rolled: fully unrolled,
 // the code outgrows the instruction cache and instruction fetch sets the pace (144 us per
-// step pair at 14^4 against 72).
+// step pair at 14^4).  Copies in flight and the data read belong to one warp.
 __device__ __forceinline__ void fx_hops(FxHalf& acc, const FxField& f, int off, const FxLinks& U, const Geom& g,
-                                        const FxSite& st, int dagger, int sp) {
-  const int V = (int)g.V;
-  fx_swap_lower(acc);   // x and y feed the partner's lower spin
+                                        const FxSite& st, const FxExps& ex, int dagger, int sp, FxStage& S,
+                                        int nu0 = 0, int nu1 = 4) {
+  __syncwarp();
+  if (sp == 0) {
+#pragma unroll
+    for (int hop = 0; hop < 8; ++hop) S.nb[hop][threadIdx.x & 15] = st.neighbour(g, hop);
+  }
+  __syncwarp();
+  fx_hop_copy(S, f, off, U, st.x, 2 * nu0, 2 * nu1, dagger, sp);
+  fx_hop_copy(S, f, off, U, st.x, 2 * nu0 + 1, 2 * nu1, dagger, sp);
+  if (nu0 < 2) fx_swap_lower(acc);   // x and y feed the partner's lower spin
 #pragma unroll 1
-  for (int nu = 0; nu < 4; ++nu) {
+  for (int nu = nu0; nu < nu1; ++nu) {
     const int tau = nu == 0 ? -1 : nu == 3 ? 1 : 2 * sp - 1;
-    if (nu == 2) fx_swap_lower(acc);
+    if (nu == 2 && nu0 < 2) fx_swap_lower(acc);
     FxZ a[3], b[3];
-    fx_hop<1>(a, acc.E, f, off, U, V, st.neighbour(g, 2 * nu), st.x, nu, fx_link_dir(2 * nu, dagger), sp, tau);
-    fx_hop<-1>(b, acc.E, f, off, U, V, st.neighbour(g, 2 * nu + 1), st.x, nu, fx_link_dir(2 * nu + 1, dagger), sp,
-               tau);
-    const fxll m = (nu == 1 && sp == 0) || (nu == 2 && sp == 1) ? -1 : 0;   // the lower spin's sign
+    fx_copy_wait<1>();
+    __syncwarp();
+    fx_hop<1>(a, S, max(0, min(acc.E - (int)((ex.f >> (16 * nu)) & 0xffff), 62)), nu, sp, tau);
+    __syncwarp();
+    fx_hop_copy(S, f, off, U, st.x, 2 * nu + 2, 2 * nu1, dagger, sp);
+    fx_copy_wait<1>();
+    __syncwarp();
+    fx_hop<-1>(b, S, max(0, min(acc.E - (int)((ex.b >> (16 * nu)) & 0xffff), 62)), nu, sp, tau);
+    __syncwarp();
+    fx_hop_copy(S, f, off, U, st.x, 2 * nu + 3, 2 * nu1, dagger, sp);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       acc.v[i].re += a[i].re + b[i].re;
       acc.v[i].im += a[i].im + b[i].im;
-      const FxZ t{((a[i].re - b[i].re) ^ m) - m, ((a[i].im - b[i].im) ^ m) - m};
-      acc.v[3 + i].re += (nu & 1) ? t.re : -t.im;
-      acc.v[3 + i].im += (nu & 1) ? t.im : t.re;
+      a[i].re -= b[i].re;
+      a[i].im -= b[i].im;
+    }
+    if (nu == 1 || nu == 2) {   // the lower spin's sign: - for (y, spin 0) and (z, spin 1)
+      const fxll m = (nu == 1) == (sp == 0) ? -1 : 0;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        a[i].re = (a[i].re ^ m) - m;
+        a[i].im = (a[i].im ^ m) - m;
+      }
+    }
+    if (nu & 1) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        acc.v[3 + i].re += a[i].re;
+        acc.v[3 + i].im += a[i].im;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        acc.v[3 + i].re -= a[i].im;
+        acc.v[3 + i].im += a[i].re;
+      }
+    }
+  }
+  fx_copy_wait<0>();
+  if (nu0 < 2 && nu1 <= 2) fx_swap_lower(acc);
+}
+
+// The sum of the partial sums that n warps formed for the same sites, in the first of them
+// (n <= 4, each below 2^61.5 units of its own scale; EXACT: all of one scale and their sum
+// below 2^63, as where the warps share the hops of one sum).  st[0 .. n - 1] are the warps'
+// stages, w this warp's place.  Every thread of the block.
+template <bool EXACT>
+__device__ __forceinline__ void fx_join_warps(FxHalf& a, FxStage* st, int w, int n) {
+  const int t = threadIdx.x & 31;
+  __syncthreads();
+  if (w > 0) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      st[w].sum.v[2 * i][t] = a.v[i].re;
+      st[w].sum.v[2 * i + 1][t] = a.v[i].im;
+    }
+    st[w].sum.e[t] = a.E;
+  }
+  __syncthreads();
+  if (w > 0) return;
+  if (!EXACT) {
+    int E = a.E;
+    for (int k = 1; k < n; ++k) E = max(E, st[k].sum.e[t]);
+    fx_shift(a, min(E + 2 - a.E, 62));
+    a.E = E + 2;
+  }
+  for (int k = 1; k < n; ++k) {
+    const int sh = min(a.E - st[k].sum.e[t], 62);
+    const fxll r = (1ll << sh) >> 1;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      a.v[i].re += (st[k].sum.v[2 * i][t] + r) >> sh;
+      a.v[i].im += (st[k].sum.v[2 * i + 1][t] + r) >> sh;
+    }
+  }
+}
+
+// A thread's components of a sequence of fields at one site, copied FX_RING - 1 vectors ahead
+// (integers through shared memory, exponents in registers).  at(i): the i-th field.
+// Every lane of the warp calls next() for i = 0, 1, .. n - 1.
+struct FxStream {
+  int e[FX_RING];
+  template <typename At>
+  __device__ __forceinline__ void issue(FxStage& S, int slot, int i, int n, int64_t s, int sp, const At& at) {
+    if (i < n) {
+      const FxField f = at(i);
+      const int4* p = f.c + fx_at(s) + sp * 96;
+      const int t = threadIdx.x & 31;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        fx_copy16(&S.ring[slot][a][t], p + a * 32);
+        fx_copy16(&S.ring[slot][3 + a][t], p + 192 + a * 32);
+      }
+      e[slot] = f.e[s];
+    }
+    fx_copy_commit();
+  }
+  template <typename At>
+  __device__ __forceinline__ void start(FxStage& S, int n, int64_t s, int sp, const At& at) {
+#pragma unroll
+    for (int i = 0; i < FX_RING - 1; ++i) issue(S, i, i, n, s, sp, at);
+  }
+  // field i of n into o, slot = i % FX_RING (a constant after unrolling)
+  template <typename At>
+  __device__ __forceinline__ void next(FxStage& S, int slot, int i, int n, int64_t s, int sp, const At& at, FxH& o) {
+    issue(S, (slot + FX_RING - 1) % FX_RING, i + FX_RING - 1, n, s, sp, at);
+    fx_copy_wait<FX_RING - 1>();
+    const int t = threadIdx.x & 31;   // each thread reads its own copies
+#pragma unroll
+    for (int a = 0; a < 6; ++a) o.q[a] = S.ring[slot][a][t];
+    o.e = e[slot];
+  }
+};
+
+// ---------------------------------------------------------------------------
+// block sums: one warp per value adds the values of the nw warps that have it (the block's
+// first, or for values 1, 3, .. those from warp `odd` on) and writes the block's partial.  An
+// FP64 addition of a warp, whatever it adds, occupies the SM's FP64 pipe for 19 cycles.
+// Blocks of up to 256 threads
+// ---------------------------------------------------------------------------
+template <int NV, int NT>
+struct FxSumBuf {
+  zd v[NV][NT];
+};
+template <int NV, int NT>
+__device__ __forceinline__ void fx_block_partials(const zd (&v)[NV], FxSumBuf<NV, NT>& buf, zd* part, int nw,
+                                                  int odd = 0) {
+#pragma unroll
+  for (int i = 0; i < NV; ++i) buf.v[i][threadIdx.x] = v[i];
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i < NV; i += blockDim.x >> 5) {
+    const zd* q = &buf.v[i][(i & 1 ? odd * 32 : 0) + lane];
+    zd s = q[0];
+    for (int t = 1; t < nw; ++t) s = s + q[32 * t];
+    s = warp_sum(s);
+    if (lane == 0) part[i * gridDim.x + blockIdx.x] = s;
+  }
+}
+
+// The sums of the n blocks' partials (in block order per thread, then a fixed tree), in every
+// lane of warp 0; every thread of the block calls it.  Eight loads per thread are in flight at
+// a time: one by one they cost a memory latency per 128 blocks.  A warp adds only where it has
+// partials: with 16 blocks the sums of nothing took 1.2 us of FP64 pipe per value.
+template <int NV>
+__device__ __forceinline__ void fx_sum_partials(const zd* part, int n, zd (&out)[NV], zd* scratch) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nw = min((int)blockDim.x >> 5, (n + 31) >> 5);   // warps with partials
+  if (w < nw) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      zd v = mk(0.0, 0.0);
+      for (int b0 = threadIdx.x; b0 - lane < n; b0 += 8 * blockDim.x) {
+        zd t[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int b = b0 + u * blockDim.x;
+          t[u] = b < n ? ld_cg(part + i * n + b) : mk(0.0, 0.0);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (b0 - lane + u * (int)blockDim.x < n) v = v + t[u];
+      }
+      v = warp_sum(v);
+      if (lane == 0) scratch[i * 32 + w] = v;
+    }
+  }
+  __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      out[i] = scratch[i * 32];
+      for (int q = 1; q < nw; ++q) out[i] = out[i] + scratch[i * 32 + q];
     }
   }
 }

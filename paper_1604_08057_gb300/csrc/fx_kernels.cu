@@ -6,6 +6,9 @@
 // Two threads (spins sp and 2 + sp) share a site unless a kernel says otherwise; blocks
 // whose two halves treat the two sides of the recurrence (r and s, g_r and g_s) exchange
 // through shared memory.  All reductions are deterministic.
+#include <algorithm>
+#include <atomic>
+
 #include "fx.cuh"
 #include "kernels.h"
 #include "recurrence.cuh"
@@ -13,6 +16,38 @@
 namespace ov {
 
 static inline unsigned nblocks(int64_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
+
+// Every rule on launch shapes looks at the lattice alone, so that a source's sums have the
+// same order whatever sources run beside it.
+//
+// Blocks of the two-sided kernels cover 32 sites at a time, or 16 where 32 would leave SMs
+// without a block; the elementwise ones take several such groups in turn, so that one wave
+// (four blocks per SM) covers the lattice and a block's reduction serves all its groups.
+static inline int two_sided_sites(const Lat<double>& L) { return L.g.V < 152 * 32 ? 16 : 32; }
+static inline unsigned one_wave(const Lat<double>& L, int sites) {
+  return std::min(nblocks(L.g.V, sites), 4u * 152u);
+}
+// Four warps per 16 sites and side (see k_fx_tsl) where one warp leaves most of an SM idle.
+// In the Lanczos step the split sums are the unsplit ones bit for bit, so its rule may count
+// the sources (8^4 with four sources: 23 ms of stencils with the split, 12
+// without); the sums over terms of the other two are not.
+static inline bool fx_split(const Lat<double>& L) { return L.g.V < 152 * 32; }
+static inline bool fx_split_exact(const Lat<double>& L) { return L.g.V < 152 * 32 && L.g.V * L.nsrc < 152 * 64; }
+
+// a launch with dynamic shared memory, whose limit is raised once per kernel and device
+// (every caller sets the same value)
+template <auto K, typename... A>
+static void fx_launch(dim3 grid, int threads, size_t smem, cudaStream_t st, const A&... a) {
+  static std::atomic<unsigned long long> done{0ull};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (!(done.load() & bit)) {
+    cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+    done.fetch_or(bit);
+  }
+  K<<<grid, threads, smem, st>>>(a...);
+}
 
 // vector j of a basis
 __device__ __forceinline__ FxField fx_bv(const Lat<double>& L, int src, int j) {
@@ -203,17 +238,37 @@ void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t v
 // ---------------------------------------------------------------------------
 // ov_apply_H
 // ---------------------------------------------------------------------------
-// FP64 hop sum (out of line: reached only where a site or link is marked)
+// FP64 hop sum from the user's links [site][direction][3][3] (out of line: reached only where
+// a site or link is marked)
+template <int NU>
+__device__ __forceinline__ void hops_fp64_dir(Spinor<double>& acc, const FxLoad& ld, const double2* u, const Geom& g,
+                                              int64_t x, const int c[4], double ff, double fb) {
+  Spinor<double> nb;
+  Half<double> h, uh;
+  Mat3<double> m;
+  ld(neighbour(g, x, c, NU, +1), nb);
+  for (int e = 0; e < 9; ++e) m.m[e] = mk(u[x * 36 + NU * 9 + e].x, u[x * 36 + NU * 9 + e].y);
+  spin_project<NU, +1>(nb, h);
+  link_mul(m, h, uh);
+  spin_reconstruct_add<NU, +1>(acc, uh, ff);
+  const int64_t xb = neighbour(g, x, c, NU, -1);
+  ld(xb, nb);
+  for (int e = 0; e < 9; ++e) m.m[e] = mk(u[xb * 36 + NU * 9 + e].x, u[xb * 36 + NU * 9 + e].y);
+  spin_project<NU, -1>(nb, h);
+  link_dag_mul(m, h, uh);
+  spin_reconstruct_add<NU, -1>(acc, uh, fb);
+}
 __device__ __noinline__ void hops_fp64(const FxLoad& ld, const double* u, const Geom& g, int64_t x, double ft,
                                        double fti, Spinor<double>* a) {
   int c[4];
   site_coords(g, x, c);
+  const double2* u2 = reinterpret_cast<const double2*>(u);
   Spinor<double> t;
   spinor_zero(t);
-  hop_dir<0>(t, ld, u, g, x, c, ft, fti);
-  hop_dir<1>(t, ld, u, g, x, c, ft, fti);
-  hop_dir<2>(t, ld, u, g, x, c, ft, fti);
-  hop_dir<3>(t, ld, u, g, x, c, ft, fti);
+  hops_fp64_dir<0>(t, ld, u2, g, x, c, 1.0, 1.0);
+  hops_fp64_dir<1>(t, ld, u2, g, x, c, 1.0, 1.0);
+  hops_fp64_dir<2>(t, ld, u2, g, x, c, 1.0, 1.0);
+  hops_fp64_dir<3>(t, ld, u2, g, x, c, ft, fti);
   *a = t;
 }
 __device__ __forceinline__ void fx_pick(const Spinor<double>& t, int sp, zd (&p)[6]) {
@@ -229,7 +284,8 @@ __device__ __forceinline__ void fx_pick(const Spinor<double>& t, int sp, zd (&p)
 __global__ void __launch_bounds__(128, 4) k_fx_apply(const __grid_constant__ Lat<double> L, FxField in,
                                                      const double* __restrict__ din, double* __restrict__ out,
                                                      int dagger, int aos) {
-  __shared__ double2 stage[4][kStage];
+  __shared__ FxStage stage[4];
+  FxStage& S = stage[(threadIdx.y * blockDim.x + threadIdx.x) >> 5];
   const int sp = fx_spin_of(threadIdx.x);
   const int64_t x0 = blockIdx.x * (int64_t)(blockDim.x >> 1) + (threadIdx.x >> 5) * 16;
   const int src = blockIdx.y * blockDim.y + threadIdx.y;
@@ -241,16 +297,17 @@ __global__ void __launch_bounds__(128, 4) k_fx_apply(const __grid_constant__ Lat
   const double* d = din + (int64_t)src * L.vs;
   const FxSite s(L.g, x);
   FxHalf acc;
-  fx_zero(acc, fx_range(0, f, 0, L.fu, L.g, s, dagger));
+  FxExps ex;
+  fx_zero(acc, fx_range(ex, f, 0, L.fu, L.g, s, dagger));
   const bool ok = acc.E < FX_BAD;
   if (!ok) acc.E = FX_E_BIAS;
-  fx_hops(acc, f, 0, L.fu, L.g, s, dagger, sp);
+  fx_hops(acc, f, 0, L.fu, L.g, s, ex, dagger, sp, S);
   zd a[6];
   if (ok) {
     fx_double(acc, false, a);
   } else {
     Spinor<double> t;
-    hops_fp64(FxLoad{f, d, V, 0}, L.u, L.g, x, dagger ? L.efinv : L.ef, dagger ? L.ef : L.efinv, &t);
+    hops_fp64(FxLoad{f, d, V, 0}, L.uaos, L.g, x, dagger ? L.efinv : L.ef, dagger ? L.ef : L.efinv, &t);
     fx_pick(t, sp, a);
   }
   FxH c;
@@ -266,7 +323,8 @@ __global__ void __launch_bounds__(128, 4) k_fx_apply(const __grid_constant__ Lat
     const zd q = mk(fma(-L.kappa, a[i].re, p.re), fma(-L.kappa, a[i].im, p.im));
     a[i] = i < 3 ? q : -q;
   }
-  if (aos) aos_store(out, src, V, x0, stage[(threadIdx.y * blockDim.x + threadIdx.x) >> 5], sp, a);
+  __syncwarp();
+  if (aos) aos_store(out, src, V, x0, S.out, sp, a);
   else if (live) soa_store(out + (int64_t)src * L.vs, V, x, sp, a);
 }
 void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double* out, int dagger, int aos,
@@ -294,6 +352,7 @@ void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double
 // ---------------------------------------------------------------------------
 // start: beta_0 = ||r||, scales of v_1 and w_1 (see k_tsl_init)
 __global__ void __launch_bounds__(128) k_fx_init(const __grid_constant__ Lat<double> L) {
+  __shared__ FxSumBuf<2, 128> sum;
   __shared__ zd scratch[2 * 32];
   const int sp = fx_spin_of(threadIdx.x);
   const int64_t x = blockIdx.x * (int64_t)64 + fx_site_of(threadIdx.x);
@@ -308,15 +367,11 @@ __global__ void __launch_bounds__(128) k_fx_init(const __grid_constant__ Lat<dou
       v[1] = fx_dot(s, r);
     }
   }
-  block_sum<2>(v, scratch);
   zd* part = L.part + src * L.part_stride;
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = v[0];
-    part[gridDim.x + blockIdx.x] = v[1];
-  }
+  fx_block_partials(v, sum, part, blockDim.x >> 5);
   if (arrive_last(L.cnt + src * 16 + 0, gridDim.x)) {
     zd s[2];
-    sum_partials<2>(part, gridDim.x, s, scratch);
+    fx_sum_partials<2>(part, gridDim.x, s, scratch);
     if (threadIdx.x == 0) init_finalize(L, src, s[0].re, s[1]);
   }
 }
@@ -328,18 +383,15 @@ void fx_tsl_init(const Lat<double>& L, cudaStream_t st) {
 __device__ __forceinline__ bool h_finish(FxHalf& o, const FxH& f, const FxCoef& c, const FxH& t) {
   fx_zero(o, 0);
   bool ok = fx_add(o, f);
-  ok = fx_axpy<1>(o, c, t) && ok;
+  ok = fx_axpy(o, c, t) && ok;
 #pragma unroll
   for (int i = 3; i < 6; ++i) o.v[i] = FxZ{-o.v[i].re, -o.v[i].im};
   return ok;
 }
-__device__ __forceinline__ void alpha_finish(const Lat<double>& L, int src, int j, zd (&v)[1], zd* scratch) {
-  block_sum<1>(v, scratch);
-  zd* part = L.part + src * L.part_stride;
-  if (threadIdx.x == 0) part[blockIdx.x] = v[0];
+__device__ __forceinline__ void alpha_finish(const Lat<double>& L, int src, int j, const zd* part, zd* scratch) {
   if (arrive_last(L.cnt + src * 16 + 1, gridDim.x)) {
     zd s[1];
-    sum_partials<1>(part, gridDim.x, s, scratch);
+    fx_sum_partials<1>(part, gridDim.x, s, scratch);
     if (threadIdx.x == 0) {
       SrcScal& sc = L.sc[src];
       if (!finite_z(s[0])) flag_error(sc, ERRB_NONFINITE, j);
@@ -353,68 +405,87 @@ __device__ __forceinline__ void alpha_finish(const Lat<double>& L, int src, int 
 // second half w_j and q of the same sites, so the links of both products come from L1 and
 // a small lattice spreads over more warps.  w_j crosses to the first half through shared
 // memory for the dot product.  H v_j = +-(v_j - kappa sv a) from the hop sum a of r.
-struct FxShare {
-  int4 q[6][64];
-  int e[64];
-};
-__device__ __forceinline__ void share_put(FxShare& s, int t, const FxH& f) {
-#pragma unroll
-  for (int i = 0; i < 6; ++i) s.q[i][t] = f.q[i];
-  s.e[t] = f.e;
-}
-__device__ __forceinline__ void share_get(const FxShare& s, int t, FxH& f) {
-#pragma unroll
-  for (int i = 0; i < 6; ++i) f.q[i] = s.q[i][t];
-  f.e = s.e[t];
-}
-
-__global__ void __launch_bounds__(128, 4) k_fx_tsl(const __grid_constant__ Lat<double> L, int j, int need_q) {
+//
+// SPLIT: on a lattice with too few sites to fill the GPU a step's time is the latency of a
+// thread's chain of hops (22 us at 4^4), so four warps share a side's 16 sites, one
+// direction each, and add their sums through shared memory.
+template <int SPLIT>
+__global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 2 : 4)
+    k_fx_tsl(const __grid_constant__ Lat<double> L, int j, int need_q) {
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  FxStage* stage = reinterpret_cast<FxStage*>(fx_smem);
+  __shared__ FxSumBuf<1, SPLIT ? 256 : 128> sum;
+  __shared__ FxCoef cs[2][2];   // [side]: scale, -kappa scale
   __shared__ zd scratch[32];
-  __shared__ FxShare ws;
-  const int half = blockDim.x >> 1;
+  const int half = blockDim.x >> 1, wid = threadIdx.x >> 5, nw = half >> 5;   // nw warps per side
   const bool left = threadIdx.x >= half;
-  const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
-  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
+  const int w0 = left ? wid - nw : wid;
+  const int t = SPLIT ? (threadIdx.x & 31) : left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(SPLIT ? 16 : half >> 1) + fx_site_of(t), x = min(x0, V - 1);
   const int src = blockIdx.y;
+  FxStage& S = stage[wid];
   zd v[1] = {mk(0.0, 0.0)};
-  const bool go = L.sc[src].err == 0, live = go && x0 < V;   // go: the whole block
+  const bool first = !SPLIT || w0 == 0;
+  const bool go = L.sc[src].err == 0, live = go && x0 < V && first;   // go: the whole block
   FxH o, w;
   if (go) {
     const FxField f = fx_src(left ? L.fs : L.fr, src, L.vs);
     const zd sc = left ? L.sc[src].sw : L.sc[src].sv;
+    if ((threadIdx.x & (half - 1)) < 2) {
+      const double q = (threadIdx.x & 1) ? -L.kappa : 1.0;
+      cs[left][threadIdx.x & 1] = fx_coef(mk(q * sc.re, q * sc.im));
+    }
+    __syncthreads();
     FxHalf acc;
-    fx_load(f, x, sp, o);
+    const FxField bas = left ? fx_bw(L, src, j) : fx_bv(L, src, j);
+    if (first) {
+      fx_load(f, x, sp, o);
+      fx_zero(acc, 0);
+      const bool okv = fx_axpy(acc, cs[left][0], o);
+      fx_encode(acc, !okv, w);
+      if (live) fx_put(bas, x, sp, w);
+    }
+    const bool need = !left || need_q;
+    bool ok = true;
     fx_zero(acc, 0);
-    const bool okv = fx_axpy<1>(acc, fx_coef(sc), o);
-    fx_encode(acc, !okv, w);
-    if (live) fx_put(left ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, w);
-    if (left) share_put(ws, t, w);
-    if (!left || need_q) {
+    if (need) {
       const FxSite s(L.g, x);
       const int dg = left ? 1 : 0;
-      fx_zero(acc, fx_range(0, f, 0, L.fu, L.g, s, dg));
-      const bool ok = acc.E < FX_BAD;
+      FxExps ex;
+      acc.E = fx_range(ex, f, 0, L.fu, L.g, s, dg);
+      ok = acc.E < FX_BAD;
       if (!ok) acc.E = FX_E_BIAS;
-      fx_hops(acc, f, 0, L.fu, L.g, s, dg, sp);
+      fx_hops(acc, f, 0, L.fu, L.g, s, ex, dg, sp, S, SPLIT ? w0 : 0, SPLIT ? w0 + 1 : 4);
+    }
+    if (SPLIT) fx_join_warps<true>(acc, stage + (left ? nw : 0), w0, nw);
+    if (need && first) {
       fx_encode(acc, !ok, o);
-      const bool okp = h_finish(acc, w, fx_coef(mk(-L.kappa * sc.re, -L.kappa * sc.im)), o);
+      // (v_j again from memory: held in registers over the hops it costs a block per SM)
+      __syncwarp();
+      fx_load(bas, x, sp, w);
+      const bool okp = h_finish(acc, w, cs[left][1], o);
       fx_encode(acc, !okp, o);
       if (live) fx_put(fx_src(left ? L.fq : L.fp, src, L.vs), x, sp, o);
     }
+    if (left && first) fx_row_put(S.row, w);
   }
   __syncthreads();
   if (live && !left) {
-    share_get(ws, t, w);
+    fx_row_get(stage[wid + nw].row, w);
     v[0] = fx_dot(w, o);
   }
-  alpha_finish(L, src, j, v, scratch);
+  zd* part = L.part + src * L.part_stride;
+  fx_block_partials(v, sum, part, SPLIT ? 1 : nw);
+  alpha_finish(L, src, j, part, scratch);
 }
 
 // Block step (Theorem 1; fields of 2V sites): four warps of 16 sites,
 //   0: p_u = H v_u + dH v_l   1: p_l = H v_l   2: q_u = H^dag w_u   3: q_l = dH^dag w_u + H^dag w_l
 __global__ void __launch_bounds__(128, 4) k_fx_tsl_block(const __grid_constant__ Lat<double> L, int j, int need_q) {
+  __shared__ FxStage stage[4];
+  __shared__ FxSumBuf<1, 128> sum;
   __shared__ zd scratch[32];
-  __shared__ FxShare ws;
+  FxStage& S = stage[threadIdx.x >> 5];
   const int t = threadIdx.x & 31, part_id = threadIdx.x >> 5, sp = fx_spin_of(t);
   const bool left = part_id >= 2, low = part_id & 1;
   const int64_t V = L.gl.V, x0 = blockIdx.x * (int64_t)16 + fx_site_of(t), x = min(x0, V - 1);
@@ -430,70 +501,75 @@ __global__ void __launch_bounds__(128, 4) k_fx_tsl_block(const __grid_constant__
     FxHalf acc;
     fx_load(f, off + x, sp, o);
     fx_zero(acc, 0);
-    const bool okv = fx_axpy<1>(acc, fx_coef(sc), o);
+    const bool okv = fx_axpy(acc, fx_coef(sc), o);
     fx_encode(acc, !okv, w);
     if (live) fx_put(left ? fx_bw(L, src, j) : fx_bv(L, src, j), off + x, sp, w);
-    if (left) share_put(ws, low * 32 + t, w);
     if (!left || need_q) {
       const FxSite s(L.gl, x);
       const int dg = left ? 1 : 0;
-      int E = fx_range(0, f, off, L.fu, L.gl, s, dg);
-      if (cross) E = fx_range(E, f, offx, L.fd, L.gl, s, dg) + 1;   // sixteen hops
+      FxExps ex, exd;
+      int E = fx_range(ex, f, off, L.fu, L.gl, s, dg);
+      if (cross) E = max(E, fx_range(exd, f, offx, L.fd, L.gl, s, dg)) + 1;   // sixteen hops
       const bool ok = E < FX_BAD;
       fx_zero(acc, ok ? E : FX_E_BIAS);
       for (int h = 0; h < (cross ? 2 : 1); ++h)
-        fx_hops(acc, f, h ? offx : off, h ? L.fd : L.fu, L.gl, s, dg, sp);
+        fx_hops(acc, f, h ? offx : off, h ? L.fd : L.fu, L.gl, s, h ? exd : ex, dg, sp, S);
       fx_encode(acc, !ok, o);
       const bool okp = h_finish(acc, w, fx_coef(mk(-L.kappa * sc.re, -L.kappa * sc.im)), o);
       fx_encode(acc, !okp, o);
       if (live) fx_put(fx_src(left ? L.fq : L.fp, src, L.vs), off + x, sp, o);
     }
+    if (left) fx_row_put(S.row, w);
   }
   __syncthreads();
   if (live && !left) {
-    share_get(ws, low * 32 + t, w);
+    fx_row_get(stage[part_id + 2].row, w);
     v[0] = fx_dot(w, o);
   }
-  alpha_finish(L, src, j, v, scratch);
+  zd* part = L.part + src * L.part_stride;
+  fx_block_partials(v, sum, part, 2);
+  alpha_finish(L, src, j, part, scratch);
 }
 void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st, int variant) {
   if (L.block) {
     k_fx_tsl_block<<<dim3(nblocks(L.gl.V, 16), L.nsrc), 128, 0, st>>>(L, j, need_q);
     return;
   }
-  const int64_t V = L.g.V;
-  // 16 sites per block where 32 would leave SMs without a block
-  const int sx = (variant & 1) || V * L.nsrc < 152 * 32 ? 16 : 32;
-  k_fx_tsl<<<dim3(nblocks(V, sx), L.nsrc), 4 * sx, 0, st>>>(L, j, need_q);
+  if (fx_split_exact(L)) {
+    fx_launch<k_fx_tsl<1>>(dim3(nblocks(L.g.V, 16), L.nsrc), 256, 8 * sizeof(FxStage), st, L, j, need_q);
+    return;
+  }
+  const int sx = (variant & 1) ? 16 : two_sided_sites(L);
+  fx_launch<k_fx_tsl<0>>(dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, (sx / 8) * sizeof(FxStage), st, L, j, need_q);
 }
 
 // r = p - alpha_j v_j - beta_j v_{j-1};  s = q - conj(alpha_j) w_j - delta_j w_{j-1}.  The two
 // halves of a block's threads form r and s of the same SX (16 or 32) sites; s crosses to
 // the first half for s^dag r.
-__device__ __forceinline__ void omega_finish(const Lat<double>& L, int src, int j, int slot, zd (&v)[2], zd* scratch) {
-  block_sum<2>(v, scratch);   // v[0] = s^dag r, v[1] = (|r|^2, |s|^2)
+// v[0] = s^dag r, v[1] = (|r|^2, |s|^2)
+template <int NT>
+__device__ __forceinline__ void omega_finish(const Lat<double>& L, int src, int j, int slot, const zd (&v)[2],
+                                             FxSumBuf<2, NT>& sum, zd* scratch) {
   zd* part = L.part + src * L.part_stride;
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = v[0];
-    part[gridDim.x + blockIdx.x] = v[1];
-  }
+  fx_block_partials(v, sum, part, blockDim.x >> 5);
   if (arrive_last(L.cnt + src * 16 + slot, gridDim.x)) {
     zd s[2];
-    sum_partials<2>(part, gridDim.x, s, scratch);
-    if (threadIdx.x == 0 && L.sc[src].err == 0) omega_finalize(L, src, j, s[0], s[1].re, s[1].im);
+    fx_sum_partials<2>(part, gridDim.x, s, scratch);
+    if (threadIdx.x < 32 && L.sc[src].err == 0) omega_finalize_warp(L, src, j, s[0], s[1].re, s[1].im);
   }
 }
 __global__ void __launch_bounds__(128, 4) k_fx_update(const __grid_constant__ Lat<double> L, int j, int finalize) {
+  __shared__ FxSumBuf<2, 128> sum;
   __shared__ zd scratch[2 * 32];
-  __shared__ FxShare ws;
+  __shared__ FxRow rows[2];
   __shared__ FxCoef cs[2][2];
   const int half = blockDim.x >> 1;
   const int left = threadIdx.x >= half;
   const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
-  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
+  const int64_t V = L.g.V;
   const int src = blockIdx.y;
   zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
-  const bool go = L.sc[src].err == 0, live = go && x0 < V;
+  const bool go = L.sc[src].err == 0;   // the whole block
   if (go && t == 0) {
     const int64_t o = (int64_t)src * L.k + j;
     const zd al = L.alpha[o];
@@ -501,8 +577,10 @@ __global__ void __launch_bounds__(128, 4) k_fx_update(const __grid_constant__ La
     cs[left][1] = fx_coef(j == 0 ? mk(0.0, 0.0) : left ? mk(-L.delta[o], 0.0) : -L.beta[o]);
   }
   __syncthreads();
-  FxH f;
-  if (go) {
+  const int64_t per = half >> 1;
+  for (int64_t b = blockIdx.x; go && b * per < V; b += gridDim.x) {
+    const int64_t x0 = b * per + fx_site_of(t), x = min(x0, V - 1);
+    FxH f;
     FxHalf acc;
     fx_zero(acc, 0);
     fx_load(fx_src(left ? L.fq : L.fp, src, L.vs), x, sp, f);
@@ -511,33 +589,33 @@ __global__ void __launch_bounds__(128, 4) k_fx_update(const __grid_constant__ La
     // (r = 0) stays one
     const int zero_top = f.e + 1078 - 53;
     fx_load(left ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, f);
-    ok = fx_axpy<1>(acc, cs[left][0], f) && ok;
+    ok = fx_axpy(acc, cs[left][0], f) && ok;
     if (j > 0) {
       fx_load(left ? fx_bw(L, src, j - 1) : fx_bv(L, src, j - 1), x, sp, f);
-      ok = fx_axpy<1>(acc, cs[left][1], f) && ok;
+      ok = fx_axpy(acc, cs[left][1], f) && ok;
     }
     fx_encode(acc, !ok, f, zero_top);
-    if (live) fx_put(fx_src(left ? L.fs : L.fr, src, L.vs), x, sp, f);
-  }
-  if (!finalize) return;   // uniform across the grid
-  if (left && go) share_put(ws, t, f);
-  __syncthreads();
-  if (live) {
-    if (left) {
-      v[1] = mk(0.0, fx_norm2(f));
-    } else {
-      FxH s;
-      share_get(ws, t, s);
-      v[0] = fx_dot(s, f);
-      v[1] = mk(fx_norm2(f), 0.0);
+    if (x0 < V) fx_put(fx_src(left ? L.fs : L.fr, src, L.vs), x, sp, f);
+    if (!finalize) continue;
+    if (left) fx_row_put(rows[t >> 5], f);
+    __syncthreads();
+    if (x0 < V) {
+      if (left) {
+        v[1].im += fx_norm2(f);
+      } else {
+        FxH s;
+        fx_row_get(rows[t >> 5], s);
+        v[0] = v[0] + fx_dot(s, f);
+        v[1].re += fx_norm2(f);
+      }
     }
+    __syncthreads();
   }
-  omega_finish(L, src, j, 2, v, scratch);
+  if (finalize) omega_finish(L, src, j, 2, v, sum, scratch);
 }
-static inline int two_sided_sites(const Lat<double>& L) { return L.g.V * L.nsrc < 152 * 32 ? 16 : 32; }
 void fx_tsl_update(const Lat<double>& L, int j, int finalize, cudaStream_t st) {
   const int sx = two_sided_sites(L);
-  k_fx_update<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, j, finalize);
+  k_fx_update<<<dim3(one_wave(L, sx), L.nsrc), 4 * sx, 0, st>>>(L, j, finalize);
 }
 
 // ---------------------------------------------------------------------------
@@ -562,7 +640,7 @@ __global__ void __launch_bounds__(128, 3) k_fx_dots(const __grid_constant__ Lat<
                                                     FxField b, int64_t ab_stride, zd* __restrict__ cpart,
                                                     int64_t cp_stride, int spt, int ioff, int sides) {
   __shared__ zd acc[FX_NB][128];
-  __shared__ zd red[4][FX_NB];
+  __shared__ double red[4][2 * FX_NB];
   const int src = blockIdx.z / sides, side = blockIdx.z % sides;
   const int i0 = blockIdx.y * FX_NB, n = min(FX_NB, nb - i0);
   const int64_t V = L.g.V;
@@ -588,15 +666,22 @@ __global__ void __launch_bounds__(128, 3) k_fx_dots(const __grid_constant__ Lat<
       acc[i][threadIdx.x] = s;
     }
   }
-  for (int i = 0; i < n; ++i) {
-    const zd s = warp_sum(acc[i][threadIdx.x]);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][i] = s;
+  double v[2 * FX_NB];
+#pragma unroll
+  for (int i = 0; i < FX_NB; ++i) {
+    const zd s = i < n ? acc[i][threadIdx.x] : mk(0.0, 0.0);
+    v[2 * i] = s.re;
+    v[2 * i + 1] = s.im;
   }
+  const double s = warp_sum_multi(v);
+  const int lane = threadIdx.x & 31;
+  if (!(lane & 1)) red[threadIdx.x >> 5][lane >> 1] = s;
   __syncthreads();
-  if (threadIdx.x < n) {
-    zd s = red[0][threadIdx.x];
-    for (int w = 1; w < 4; ++w) s = s + red[w][threadIdx.x];
-    cpart[src * cp_stride + (int64_t)(2 * (i0 + threadIdx.x) + side) * gridDim.x + blockIdx.x] = s;
+  if (threadIdx.x < 2 * n) {
+    double r = red[0][threadIdx.x];
+    for (int w = 1; w < 4; ++w) r = r + red[w][threadIdx.x];
+    reinterpret_cast<double*>(cpart + src * cp_stride + (int64_t)(2 * (i0 + threadIdx.x / 2) + side) * gridDim.x +
+                              blockIdx.x)[threadIdx.x & 1] = r;
   }
 }
 // one warp per coefficient: its site blocks' partials in lane-strided order, then a fixed tree
@@ -634,30 +719,26 @@ __device__ __forceinline__ FxField ring_at(const Lat<double>& L, const FxField& 
 }
 // D1 = v_j^dag g_r, D2 = w_j^dag g_s, D3 = v_{j-1}^dag g_r, D4 = w_{j-1}^dag g_s -> g_alpha and
 // the carries; g: this thread's g_r (left = 0) or g_s (left = 1)
-__device__ __forceinline__ void rev_alpha_finish(const Lat<double>& L, const Rev<double>& B, int src, int j, int left,
-                                                 bool live, int64_t x, int sp, const FxH& g, int slot, zd* scratch) {
-  zd v[4] = {mk(0.0, 0.0), mk(0.0, 0.0), mk(0.0, 0.0), mk(0.0, 0.0)};
-  if (live) {
-    FxH e;
-    fx_load(left ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, e);
-    const zd d0 = fx_dot(e, g);
-    zd d1 = mk(0.0, 0.0);
-    if (j > 0) {
-      fx_load(left ? fx_bw(L, src, j - 1) : fx_bv(L, src, j - 1), x, sp, e);
-      d1 = fx_dot(e, g);
-    }
-    v[0] = left ? v[0] : d0;
-    v[1] = left ? d0 : v[1];
-    v[2] = left ? v[2] : d1;
-    v[3] = left ? d1 : v[3];
+__device__ __forceinline__ void rev_alpha_site(const Lat<double>& L, int src, int j, int left, int64_t x, int sp,
+                                               const FxH& g, zd (&d)[2]) {
+  FxH e;
+  fx_load(left ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, e);
+  d[0] = d[0] + fx_dot(e, g);
+  if (j > 0) {
+    fx_load(left ? fx_bw(L, src, j - 1) : fx_bv(L, src, j - 1), x, sp, e);
+    d[1] = d[1] + fx_dot(e, g);
   }
-  block_sum<4>(v, scratch);
+}
+template <int NT>
+__device__ __forceinline__ void rev_alpha_finish(const Lat<double>& L, const Rev<double>& B, int src, int j, int left,
+                                                 const zd (&d)[2], int slot, FxSumBuf<4, NT>& sum, zd* scratch) {
+  const zd z = mk(0.0, 0.0);
+  const zd v[4] = {left ? z : d[0], left ? d[0] : z, left ? z : d[1], left ? d[1] : z};
   zd* part = L.part + src * L.part_stride;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < 4; ++i) part[i * gridDim.x + blockIdx.x] = v[i];
+  fx_block_partials(v, sum, part, blockDim.x >> 6, blockDim.x >> 6);
   if (arrive_last(L.cnt + src * 16 + slot, gridDim.x)) {
     zd s[4];
-    sum_partials<4>(part, gridDim.x, s, scratch);
+    fx_sum_partials<4>(part, gridDim.x, s, scratch);
     if (threadIdx.x == 0) alpha_epilogue(L, B, src, j, s);
   }
 }
@@ -738,80 +819,129 @@ __device__ __forceinline__ void fx_subtract(FxHalf& a, FxHalf& b) {
   }
 }
 
-constexpr int FX_CH = 32;   // coefficients converted at a time per side
+constexpr int FX_CH = 12;   // coefficients converted at a time per side (a multiple of 4 FX_RING)
+// T += sum_i coef[ci + cstep i] u_i(x) over nb vectors; the coefficients are converted by the
+// nt threads of a group (t = 0 .. nt - 1), one chunk ahead of their use, in cs[0] and cs[1].
+// Every thread of the block calls this with the same nb.
+template <typename At>
+__device__ __forceinline__ void sum_vectors(FxTerms& T, FxStage& S, FxCoef (*cs)[FX_CH], const zd* coef, int cstep,
+                                            int nb, int64_t x, int sp, int t, int nt, const At& at0, int w = 0,
+                                            int nw = 1) {
+  FxStream q;
+  // this warp's vectors: i = w, w + nw, ...
+  const int nv = (nb - w + nw - 1) / nw;
+  const auto at = [&](int i) { return at0(w + i * nw); };
+  for (int i = t; i < min(FX_CH, nb); i += nt) cs[0][i] = fx_coef(coef[(int64_t)i * cstep]);
+  q.start(S, nv, x, sp, at);
+  int v0 = 0;   // this warp's first vector of the chunk
+  for (int i0 = 0, c = 0; i0 < nb; i0 += FX_CH, c ^= 1) {
+    __syncthreads();   // this chunk's coefficients are there, and the last chunk's are done with
+    for (int i = i0 + FX_CH + t; i < min(i0 + 2 * FX_CH, nb); i += nt)
+      cs[c ^ 1][i - i0 - FX_CH] = fx_coef(coef[(int64_t)i * cstep]);
+    const int v1 = min((i0 + FX_CH - w + nw - 1) / nw, nv);
+#pragma unroll 1
+    for (int v = v0; v < v1; v += FX_RING) {
+#pragma unroll
+      for (int u = 0; u < FX_RING; ++u) {
+        if (v + u < v1) {
+          FxH f;
+          q.next(S, u, v + u, nv, x, sp, at, f);
+          T.add(cs[c][w + (v + u) * nw - i0], f);
+        }
+      }
+    }
+    v0 = v1;
+  }
+  fx_copy_wait<0>();
+}
+
 // a -= sum_i coefA_i UA_i by the first half of a block's threads, b -= sum_i coefB_i UB_i by
 // the second, for the same SX sites.  fin 1: omega and the next scales (a = r, b = s); fin 2:
 // the four dots of the reverse step (a = g_r, b = g_s).
-__global__ void __launch_bounds__(128, 3) k_fx_proj_update(const __grid_constant__ Lat<double> L,
-                                                           const __grid_constant__ Rev<double> B, int nb, int mode,
-                                                           FxField a, FxField b, int64_t ab_stride,
-                                                           const zd* __restrict__ coef, int64_t coef_stride, int j,
-                                                           int fin) {
+//
+// SPLIT: on a lattice with too few sites to fill the GPU four warps share a side's 16 sites,
+// a quarter of the vectors each (88 us per projection of 100 vectors at 4^4 without).
+template <int SPLIT>
+__global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 1 : 3)
+    k_fx_proj_update(const __grid_constant__ Lat<double> L, const __grid_constant__ Rev<double> B, int nb, int mode,
+                     FxField a, FxField b, int64_t ab_stride, const zd* __restrict__ coef, int64_t coef_stride, int j,
+                     int fin) {
+  constexpr int NT = SPLIT ? 256 : 128;
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  FxStage* stage = reinterpret_cast<FxStage*>(fx_smem);
+  FxSumBuf<2, NT>& sum2 = *reinterpret_cast<FxSumBuf<2, NT>*>(fx_smem);
+  FxSumBuf<4, NT>& sum4 = *reinterpret_cast<FxSumBuf<4, NT>*>(fx_smem);
+  __shared__ FxCoef cs[2][2][FX_CH];
   __shared__ zd scratch[4 * 32];
-  __shared__ FxShare ws;
-  __shared__ FxCoef cs[2][FX_CH];
-  const int half = blockDim.x >> 1;
+  const int half = blockDim.x >> 1, wid = threadIdx.x >> 5, nw = half >> 5;   // nw warps per side
   const int left = threadIdx.x >= half;
-  const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
-  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
+  const int w0 = left ? wid - nw : wid, th = left ? threadIdx.x - half : threadIdx.x;
+  const int t = SPLIT ? (threadIdx.x & 31) : th, sp = fx_spin_of(t);
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(SPLIT ? 16 : half >> 1) + fx_site_of(t), x = min(x0, V - 1);
   const int src = blockIdx.y;
-  const bool live = x0 < V;
+  FxStage& S = stage[wid];
+  const bool first = !SPLIT || w0 == 0;
+  const bool live = x0 < V && first;
   const bool usev = (mode == 0) == (left == 0);
-  const zd* cf = coef + src * coef_stride;
   FxTerms T;
   T.init();
-  for (int i0 = 0; i0 < nb; i0 += FX_CH) {
-    const int n = min(FX_CH, nb - i0);
-    __syncthreads();
-    for (int i = t; i < n; i += half) cs[left][i] = fx_coef(cf[2 * (i0 + i) + left]);
-    __syncthreads();
-    FxField u = usev ? fx_bv(L, src, i0) : fx_bw(L, src, i0);
-#pragma unroll 2
-    for (int i = 0; i < n; ++i) {
-      FxH f;
-      fx_load(u, x, sp, f);
-      T.add(cs[left][i], f);
-      u.c += L.vs / 2;
-      u.e += L.vs / 24;
-    }
-  }
+  const FxField u0 = usev ? fx_bv(L, src, L.jbase) : fx_bw(L, src, L.jbase);
+  sum_vectors(T, S, cs[left], coef + src * coef_stride + left, 2, nb, x, sp, th, half,
+              [&](int i) { return fx_src(u0, i - L.jbase, L.vs); }, SPLIT ? w0 : 0, SPLIT ? 4 : 1);
   const FxField fa = fx_src(left ? b : a, src, ab_stride);
   FxH f;
   {
     FxHalf acc, s;
     T.value(s);
-    fx_load(fa, x, sp, f);
-    fx_zero(acc, 0);
-    const bool ok = fx_add(acc, f) && T.ok;
-    fx_subtract(acc, s);
-    fx_encode(acc, !ok, f);
-    if (live) fx_put(fa, x, sp, f);
+    bool ok = T.ok;
+    if (SPLIT) {
+      if (!ok) s.E = FX_BAD;   // a marked site of any warp's vectors marks the sum
+      fx_join_warps<false>(s, stage + (left ? nw : 0), w0, nw);
+      ok = s.E < FX_BAD;
+    }
+    if (first) {
+      fx_load(fa, x, sp, f);
+      fx_zero(acc, 0);
+      ok = fx_add(acc, f) && ok;
+      fx_subtract(acc, s);
+      fx_encode(acc, !ok, f);
+      if (live) fx_put(fa, x, sp, f);
+    }
   }
   if (fin == 0) return;
+  __syncthreads();   // the stages are done with
   if (fin == 1) {
     zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
-    if (left) share_put(ws, t, f);
+    if (left && first) fx_row_put(S.row, f);
     __syncthreads();
     if (live) {
       if (left) {
         v[1] = mk(0.0, fx_norm2(f));
       } else {
         FxH s;
-        share_get(ws, t, s);
+        fx_row_get(stage[wid + nw].row, s);
         v[0] = fx_dot(s, f);
         v[1] = mk(fx_norm2(f), 0.0);
       }
     }
-    omega_finish(L, src, j, 3, v, scratch);
+    __syncthreads();
+    omega_finish(L, src, j, 3, v, sum2, scratch);
     return;
   }
-  rev_alpha_finish(L, B, src, j, left, live, x, sp, f, 6, scratch);
+  zd d[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
+  if (live) rev_alpha_site(L, src, j, left, x, sp, f, d);
+  rev_alpha_finish(L, B, src, j, left, d, 6, sum4, scratch);
 }
 void fx_proj_update(const Lat<double>& L, const Rev<double>* B, int nb, int mode, const FxField& a, const FxField& b,
                     int64_t ab_stride, const zd* coef, int j, int fin, cudaStream_t st) {
-  const int sx = two_sided_sites(L);
-  k_fx_proj_update<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, B ? *B : Rev<double>{}, nb, mode, a, b,
-                                                                        ab_stride, coef, 2 * (int64_t)L.k, j, fin);
+  const Rev<double> rev = B ? *B : Rev<double>{};
+  if (L.g.V < 152 * 16) {   // fewer than two warps per SM without the split
+    fx_launch<k_fx_proj_update<1>>(dim3(nblocks(L.g.V, 16), L.nsrc), 256, 8 * sizeof(FxStage), st, L, rev, nb, mode, a, b,
+                                   ab_stride, coef, 2 * (int64_t)L.k, j, fin);
+    return;
+  }
+  fx_launch<k_fx_proj_update<0>>(dim3(nblocks(L.g.V, 32), L.nsrc), 128, 4 * sizeof(FxStage), st, L, rev, nb, mode, a, b,
+                                 ab_stride, coef, 2 * (int64_t)L.k, j, fin);
 }
 
 // out[src] (+)= sum_{j0 <= i < j0 + nvec} y_i u_i in the user's layout, u = V (side 0) or W;
@@ -819,44 +949,34 @@ void fx_proj_update(const Lat<double>& L, const Rev<double>* B, int nb, int mode
 __global__ void __launch_bounds__(128, 3) k_fx_combine(const __grid_constant__ Lat<double> L, int src0, int side, int j0,
                                                        int nvec, const zd* __restrict__ y, int64_t ystride,
                                                        double* __restrict__ out, int accumulate) {
-  __shared__ double2 stage[4][kStage];
-  __shared__ FxCoef cs[64];
+  __shared__ FxStage stage[4];
+  __shared__ FxCoef cs[2][FX_CH];
   const int sp = fx_spin_of(threadIdx.x), w = threadIdx.x >> 5;
   const int64_t V = L.g.V, xw = blockIdx.x * (int64_t)(blockDim.x >> 1) + w * 16;
   const int64_t x = min(xw + (threadIdx.x & 15), V - 1);
   FxTerms T;
   T.init();
-  for (int i0 = 0; i0 < nvec; i0 += 64) {
-    const int n = min(64, nvec - i0);
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) cs[i] = fx_coef(y[blockIdx.y * ystride + j0 + i0 + i]);
-    __syncthreads();
-    FxField u = side ? fx_bw(L, src0 + blockIdx.y, j0 + i0) : fx_bv(L, src0 + blockIdx.y, j0 + i0);
-#pragma unroll 2
-    for (int i = 0; i < n; ++i) {
-      FxH f;
-      fx_load(u, x, sp, f);
-      T.add(cs[i], f);
-      u.c += L.vs / 2;
-      u.e += L.vs / 24;
-    }
-  }
+  const int src = src0 + blockIdx.y;
+  const FxField u0 = side ? fx_bw(L, src, j0) : fx_bv(L, src, j0);
+  sum_vectors(T, stage[w], cs, y + blockIdx.y * ystride + j0, 1, nvec, x, sp, threadIdx.x, blockDim.x,
+              [&](int i) { return fx_src(u0, i, L.vs); });
   if (xw >= V) return;   // whole warps
   FxHalf s;
   T.value(s);
   zd o[6];
   fx_double(s, !T.ok, o);
+  __syncwarp();
   if (accumulate) {
     zd p[6];
-    aos_load(out, blockIdx.y, V, xw, stage[w], sp, p);
+    aos_load(out, blockIdx.y, V, xw, stage[w].out, sp, p);
 #pragma unroll
     for (int i = 0; i < 6; ++i) o[i] = p[i] + o[i];
   }
-  aos_store(out, blockIdx.y, V, xw, stage[w], sp, o);
+  aos_store(out, blockIdx.y, V, xw, stage[w].out, sp, o);
 }
 void fx_combine(const Lat<double>& L, int src0, int nsrc, int side, int j0, int nvec, const zd* y, int64_t ystride,
                 double* out, int accumulate, cudaStream_t st) {
-  const int bs = L.g.V * nsrc < 152 * 64 ? 32 : 128;
+  const int bs = L.g.V < 152 * 64 ? 32 : 128;
   k_fx_combine<<<dim3(nblocks(L.g.V, bs / 2), nsrc), bs, 0, st>>>(L, src0, side, j0, nvec, y, ystride, out,
                                                                   accumulate);
 }
@@ -869,34 +989,40 @@ void fx_combine(const Lat<double>& L, int src0, int nsrc, int side, int j0, int 
 __global__ void __launch_bounds__(128, 4) k_fx_rev_form(const __grid_constant__ Lat<double> L,
                                                         const __grid_constant__ Rev<double> B, int j, int slot,
                                                         int with_dots) {
+  __shared__ FxSumBuf<4, 128> sum;
   __shared__ zd scratch[4 * 32];
   __shared__ FxCoef cs[2][2];
   const int half = blockDim.x >> 1;
   const int left = threadIdx.x >= half;
   const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
-  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
+  const int64_t V = L.g.V, per = half >> 1;
   const int src = blockIdx.y;
-  const bool live = x0 < V;
   if (t < 2) {
     const SrcScal& sc = L.sc[src];
     cs[left][t] = fx_coef(left ? (t ? sc.cs2 : sc.cs1) : (t ? sc.cr2 : sc.cr1));
   }
   __syncthreads();
-  FxHalf acc;
-  FxH f;
-  fx_zero(acc, 0);
-  fx_load(fx_src(left ? B.fgw : B.fgv, src, L.vs), x, sp, f);
-  bool ok = fx_axpy<1>(acc, cs[left][0], f);
-  fx_load(left ? fx_bv(L, src, j + 1) : fx_bw(L, src, j + 1), x, sp, f);
-  ok = fx_axpy<1>(acc, cs[left][1], f) && ok;
-  fx_encode(acc, !ok, f);
-  if (live) fx_put(ring_at(L, left ? B.fgs : B.fgr, slot, src), x, sp, f);
-  if (!with_dots) return;
-  rev_alpha_finish(L, B, src, j, left, live, x, sp, f, 5, scratch);
+  zd d[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
+  for (int64_t b = blockIdx.x; b * per < V; b += gridDim.x) {
+    const int64_t x0 = b * per + fx_site_of(t), x = min(x0, V - 1);
+    FxHalf acc;
+    FxH f;
+    fx_zero(acc, 0);
+    fx_load(fx_src(left ? B.fgw : B.fgv, src, L.vs), x, sp, f);
+    bool ok = fx_axpy(acc, cs[left][0], f);
+    fx_load(left ? fx_bv(L, src, j + 1) : fx_bw(L, src, j + 1), x, sp, f);
+    ok = fx_axpy(acc, cs[left][1], f) && ok;
+    fx_encode(acc, !ok, f);
+    if (x0 < V) {
+      fx_put(ring_at(L, left ? B.fgs : B.fgr, slot, src), x, sp, f);
+      if (with_dots) rev_alpha_site(L, src, j, left, x, sp, f, d);
+    }
+  }
+  if (with_dots) rev_alpha_finish(L, B, src, j, left, d, 5, sum, scratch);
 }
 void fx_rev_form(const Lat<double>& L, const Rev<double>& B, int j, int slot, int with_dots, cudaStream_t st) {
   const int sx = two_sided_sites(L);
-  k_fx_rev_form<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, B, j, slot, with_dots);
+  k_fx_rev_form<<<dim3(one_wave(L, sx), L.nsrc), 4 * sx, 0, st>>>(L, B, j, slot, with_dots);
 }
 
 // the two stencil inputs of step j: g_p = g_r + g_alpha w_j (first half), h_in = conj(g_alpha)
@@ -913,7 +1039,7 @@ __global__ void __launch_bounds__(128, 4) k_fx_rev_combine(const __grid_constant
   FxH f;
   fx_zero(acc, 0);
   fx_load(left ? fx_bv(L, src, j) : fx_bw(L, src, j), x, sp, f);
-  bool ok = fx_axpy<1>(acc, fx_coef(left ? conj(ga) : ga), f);
+  bool ok = fx_axpy(acc, fx_coef(left ? conj(ga) : ga), f);
   if (j < L.k - 1) {
     fx_load(ring_at(L, left ? B.fgs : B.fgr, slot, src), x, sp, f);
     ok = fx_add(acc, f) && ok;
@@ -966,21 +1092,29 @@ struct RevTerm {
   FxField f;
   FxCoef c;
 };
-constexpr int RT = 16;   // terms converted at a time per side
-__global__ void __launch_bounds__(128, 3) k_fx_rev(const __grid_constant__ Lat<double> L,
-                                                   const __grid_constant__ Rev<double> B, int j, int slot, int prev,
-                                                   int nrec) {
+constexpr int RT = 30;   // terms converted at a time per side (a multiple of FX_RING)
+template <int SPLIT>
+__global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 1 : 4)
+    k_fx_rev(const __grid_constant__ Lat<double> L, const __grid_constant__ Rev<double> B, int j, int slot, int prev,
+             int nrec) {
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  FxStage* stage = reinterpret_cast<FxStage*>(fx_smem);
+  __shared__ FxSumBuf<2, SPLIT ? 256 : 128> sum;
   __shared__ RevTerm terms[2][RT];
   __shared__ zd scratch[2 * 32];
-  const int half = blockDim.x >> 1;
+  const int half = blockDim.x >> 1, wid = threadIdx.x >> 5, nw = half >> 5;   // nw warps per side
   const int side = threadIdx.x >= half ? 1 : 0;
-  const int t = side ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
-  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
+  const int w0 = side ? wid - nw : wid, th = side ? threadIdx.x - half : threadIdx.x;
+  const int t = SPLIT ? (threadIdx.x & 31) : th, sp = fx_spin_of(t);
+  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(SPLIT ? 16 : half >> 1) + fx_site_of(t), x = min(x0, V - 1);
   const int src = blockIdx.y;
-  const bool live = x0 < V;
+  FxStage& S = stage[wid];
+  const bool first = !SPLIT || w0 == 0;
+  const bool live = x0 < V && first;
   const int base = (j < L.k - 1 ? 1 : 0) + (prev >= 0 && j + 1 < L.k - 1 ? 1 : 0) + nrec;
   const int nt = base + (side ? 0 : 1), ntmax = base + 1;
-  const double kinv = 1.0 / L.kappa;
+  // this warp's terms: all, or (SPLIT) every fourth
+  const int step = SPLIT ? 4 : 1, i1 = SPLIT ? w0 : 0;
   FxHalf acc;
   bool ok;
   {
@@ -988,19 +1122,28 @@ __global__ void __launch_bounds__(128, 3) k_fx_rev(const __grid_constant__ Lat<d
     T.init();
     for (int i0 = 0; i0 < ntmax; i0 += RT) {
       __syncthreads();
-      for (int i = t; i < RT && i0 + i < nt; i += half) {
+      for (int i = th; i < RT && i0 + i < nt; i += half) {
         zd c;
         terms[side][i].f = rev_term(L, B, src, side, j, slot, prev, i0 + i, &c);
-        terms[side][i].c = fx_coef(kinv * c);
+        terms[side][i].c = fx_coef(L.kinv * c);
       }
       __syncthreads();
-      const int n = min(RT, nt - i0);
+      const int n = (min(RT, nt - i0) - i1 + step - 1) / step;
+      const auto at = [&](int i) { return terms[side][i1 + i * step].f; };
+      FxStream q;
+      q.start(S, n, x, sp, at);
 #pragma unroll 1
-      for (int i = 0; i < n; ++i) {
-        FxH f;
-        fx_load(terms[side][i].f, x, sp, f);
-        T.add(terms[side][i].c, f);
+      for (int i = 0; i < n; i += FX_RING) {
+#pragma unroll
+        for (int u = 0; u < FX_RING; ++u) {
+          if (i + u < n) {
+            FxH f;
+            q.next(S, u, i + u, n, x, sp, at, f);
+            T.add(terms[side][i1 + (i + u) * step].c, f);
+          }
+        }
       }
+      fx_copy_wait<0>();
     }
     T.value(acc);
     ok = T.ok;
@@ -1008,26 +1151,34 @@ __global__ void __launch_bounds__(128, 3) k_fx_rev(const __grid_constant__ Lat<d
 #pragma unroll
   for (int i = 0; i < 3; ++i) acc.v[i] = FxZ{-acc.v[i].re, -acc.v[i].im};
   const FxField f = side ? fx_src(B.fh, src, L.vs) : ring_at(L, B.fgp, slot, src);
-  const FxSite s(L.g, x);
-  int E = fx_range(0, f, 0, L.fu, L.g, s, side ? 0 : 1);
-  E = max(E, __shfl_xor_sync(0xffffffffu, acc.E, 16));   // one scale for the site's two threads
-  ok = ok && E < FX_BAD;
-  fx_raise(acc, E);
-  // below 2^60 units, so that the hops' 2^62.6 still fit
-  fx_headroom(acc);
-  acc.E = ok ? acc.E : FX_E_BIAS;
   {
+    const FxSite s(L.g, x);
+    FxExps ex;
+    int E = fx_range(ex, f, 0, L.fu, L.g, s, side ? 0 : 1);
+    E = max(E, __shfl_xor_sync(0xffffffffu, acc.E, 16));   // one scale for the site's two threads
+    ok = ok && E < FX_BAD;
+    fx_raise(acc, E);
+    // below 2^60 units, so that the hops' 2^62.6 still fit
+    fx_headroom(acc);
+    acc.E = ok ? acc.E : FX_E_BIAS;
     const int other = __shfl_xor_sync(0xffffffffu, acc.E, 16);
     if (other > acc.E) fx_shift(acc, min(other - acc.E, 62));
     acc.E = max(acc.E, other);
+    fx_hops(acc, f, 0, L.fu, L.g, s, ex, side ? 0 : 1, sp, S, SPLIT ? w0 : 0, SPLIT ? w0 + 1 : 4);
   }
-  fx_hops(acc, f, 0, L.fu, L.g, s, side ? 0 : 1, sp);
+  if (SPLIT) {
+    if (!ok) acc.E = FX_BAD;   // a marked site of any warp's terms marks the sum
+    fx_join_warps<false>(acc, stage + (side ? nw : 0), w0, nw);
+    ok = acc.E < FX_BAD;
+  }
   FxH a, p;
-  fx_encode(acc, !ok, a);
-  fx_load(f, x, sp, p);
-  const bool okp = h_finish(acc, p, fx_coef(mk(-L.kappa, 0.0)), a);
-  fx_encode(acc, !okp, p);
-  if (live) fx_put(fx_src(side ? B.fgw : B.fgv, src, L.vs), x, sp, p);
+  if (first) {
+    fx_encode(acc, !ok, a);
+    fx_load(f, x, sp, p);
+    const bool okp = h_finish(acc, p, fx_coef(mk(-L.kappa, 0.0)), a);
+    fx_encode(acc, !okp, p);
+    if (live) fx_put(fx_src(side ? B.fgw : B.fgv, src, L.vs), x, sp, p);
+  }
   if (j == 0) return;
   zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
   if (live) {
@@ -1036,22 +1187,23 @@ __global__ void __launch_bounds__(128, 3) k_fx_rev(const __grid_constant__ Lat<d
     v[0] = side ? v[0] : d;
     v[1] = side ? d : v[1];
   }
-  block_sum<2>(v, scratch);
   zd* part = L.part + src * L.part_stride;
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = v[0];
-    part[gridDim.x + blockIdx.x] = v[1];
-  }
+  fx_block_partials(v, sum, part, SPLIT ? 1 : nw, nw);
   if (arrive_last(L.cnt + src * 16 + 4, gridDim.x)) {
     zd q[2];
-    sum_partials<2>(part, gridDim.x, q, scratch);
-    if (threadIdx.x == 0) rev_dots_epilogue(L, B, src, j - 1, q);
+    fx_sum_partials<2>(part, gridDim.x, q, scratch);
+    if (threadIdx.x < 32) rev_dots_epilogue_warp(L, B, src, j - 1, q[0], q[1]);
   }
 }
 void fx_rev_stencil(const Lat<double>& L, const Rev<double>& B, int j, int slot, int prev, int nrec,
                     cudaStream_t st) {
+  if (fx_split(L)) {
+    fx_launch<k_fx_rev<1>>(dim3(nblocks(L.g.V, 16), L.nsrc), 256, 8 * sizeof(FxStage), st, L, B, j, slot, prev, nrec);
+    return;
+  }
   const int sx = two_sided_sites(L);
-  k_fx_rev<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, B, j, slot, prev, nrec);
+  fx_launch<k_fx_rev<0>>(dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, (sx / 8) * sizeof(FxStage), st, L, B, j, slot, prev,
+                         nrec);
 }
 
 // ---------------------------------------------------------------------------
@@ -1063,19 +1215,17 @@ void fx_rev_stencil(const Lat<double>& L, const Rev<double>& B, int j, int slot,
 // are read once for all four directions.  A is shifted to the sum's scale (and at least by
 // 2 bits), so a term adds at most 2^55 to hh and 2^58.6 to x: x is folded in after sixteen.
 // ---------------------------------------------------------------------------
+// the projected half spinor of staged components u (spin sp) and d (the lower spin it meets)
 template <int SGN>
-__device__ __forceinline__ int fx_project(const FxField& f, int64_t s, int nu, int sp, int4 (&h)[3]) {
-  const int4* q = f.c + fx_at(s);
-  const int4* qu = q + sp * 96;
-  const int4* qd = q + (nu < 2 ? 3 - sp : 2 + sp) * 96;
+__device__ __forceinline__ void fx_project(const int4 (*q)[32], int nu, int sp, int4 (&h)[3]) {
+  const int l = threadIdx.x & 31;
   const int t = SGN * (nu == 0 ? -1 : nu == 3 ? 1 : 2 * sp - 1);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const int4 u = __ldg(qu + a * 32), w = __ldg(qd + a * 32);
+    const int4 u = q[a][l], w = q[3 + a][l];
     h[a] = (nu & 1) ? make_int4(u.x + t * w.x, u.y + t * w.y, u.z + t * w.z, u.w + t * w.w)
                     : make_int4(u.x - t * w.z, u.y - t * w.w, u.z + t * w.x, u.w + t * w.y);
   }
-  return f.e[s];
 }
 struct FxOuter {
   FxAcc g[9];
@@ -1104,9 +1254,8 @@ struct FxOuter {
     n = 0;
     if (m >= (1 << 28)) down(2);
   }
-  __device__ __forceinline__ void add(const FxField& X, int64_t x, const FxField& Y, int64_t y, int nu, int sp) {
-    int4 a[3], b[3];
-    const int ea = fx_project<-1>(X, x, nu, sp, a), eb = fx_project<1>(Y, y, nu, sp, b);
+  // a = P_-(X(x)), b = P_+(Y(x + nu)) of exponents ea, eb
+  __device__ __forceinline__ void add(int4 (&a)[3], const int4 (&b)[3], int ea, int eb) {
     if (ea == FX_BAD || eb == FX_BAD) {
       ok = false;
       return;
@@ -1120,7 +1269,12 @@ struct FxOuter {
     const fxll half = 1ll << (d - 1);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const FxInt p = fx_split((fx_join(a[c].x, a[c].y) + half) >> d), q = fx_split((fx_join(a[c].z, a[c].w) + half) >> d);
+      fxll re = fx_sar(fx_join(a[c].x, a[c].y) + half, min(d, 31)), im = fx_sar(fx_join(a[c].z, a[c].w) + half, min(d, 31));
+      if (d > 31) {
+        re >>= d - 31;
+        im >>= d - 31;
+      }
+      const FxInt p = fx_split(re), q = fx_split(im);
       a[c] = make_int4(p.h, p.l, q.h, q.l);
     }
 #pragma unroll
@@ -1147,15 +1301,50 @@ __global__ void __launch_bounds__(256, 2) k_fx_force(const __grid_constant__ Lat
   G.E = 0;
   G.n = 0;
   G.ok = true;
+  // the fields of the next product are copied to shared memory while one is formed
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  int4 (*st)[12][32] = reinterpret_cast<int4 (*)[12][32]>(fx_smem) + hop * 2;
+  int ea[2], eb[2];
+  auto issue = [&](int i, int slot) {
+    if (i < 2 * i1) {
+      const int src = (i >> 1) / nterms, t = (i >> 1) - src * nterms, j = j0 - t;
+      const bool second = i & 1;
+      if (!(second && j == L.k - 1)) {
+        const FxField a = second ? fx_bw(L, src, j) : ring_at(L, B.fgp, t, src);
+        const FxField b = second ? ring_at(L, B.fgs, t, src) : fx_bv(L, src, j);
+        const FxField X = back ? b : a, Y = back ? a : b;
+        const int pd = (nu < 2 ? 3 - sp : 2 + sp) * 96;
+        const int4* qx = X.c + fx_at(x);
+        const int4* qy = Y.c + fx_at(xf);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          fx_copy16(&st[slot][c][lane], qx + sp * 96 + c * 32);
+          fx_copy16(&st[slot][3 + c][lane], qx + pd + c * 32);
+          fx_copy16(&st[slot][6 + c][lane], qy + sp * 96 + c * 32);
+          fx_copy16(&st[slot][9 + c][lane], qy + pd + c * 32);
+        }
+        ea[slot] = X.e[x];
+        eb[slot] = Y.e[xf];
+      }
+    }
+    fx_copy_commit();
+  };
+  issue(2 * i0, 0);
 #pragma unroll 1
-  for (int i = 2 * i0; i < 2 * i1; ++i) {
-    const int src = (i >> 1) / nterms, t = (i >> 1) - src * nterms, j = j0 - t;
-    const bool second = i & 1;
-    if (second && j == L.k - 1) continue;
-    const FxField a = second ? fx_bw(L, src, j) : ring_at(L, B.fgp, t, src);
-    const FxField b = second ? ring_at(L, B.fgs, t, src) : fx_bv(L, src, j);
-    G.add(back ? b : a, x, back ? a : b, xf, nu, sp);
+  for (int i = 2 * i0; i < 2 * i1; i += 2) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      issue(i + s + 1, s ^ 1);
+      fx_copy_wait<1>();
+      // the second product is absent at the recurrence's last step
+      if (s == 1 && j0 - ((i >> 1) % nterms) == L.k - 1) continue;
+      int4 a[3], b[3];
+      fx_project<-1>(&st[s][0], nu, sp, a);
+      fx_project<1>(&st[s][6], nu, sp, b);
+      G.add(a, b, ea[s], eb[s]);
+    }
   }
+  fx_copy_wait<0>();
   G.fold();
   // kappa f with the sign of the hop term; a product's unit is 2^(E + 2 - 2098)
   const double f = nu < 3 ? 1.0 : back ? L.efinv : L.ef;
@@ -1206,7 +1395,8 @@ int fx_force_splits(int64_t V) {
 int fx_force_flush(const Lat<double>& L, const Rev<double>& B, int nterms, int j0, cudaStream_t st) {
   int nsplit = B.force_parts ? fx_force_splits(L.g.V) : 1;
   if (nsplit > L.nsrc * nterms) nsplit = L.nsrc * nterms;
-  k_fx_force<<<dim3(nblocks(L.g.V, 16), nsplit), 256, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+  fx_launch<k_fx_force>(dim3(nblocks(L.g.V, 16), nsplit), 256, 8 * 2 * 12 * 32 * sizeof(int4), st, L, B, nterms, j0,
+                        nsplit, B.force_parts);
   return nsplit;
 }
 

@@ -43,6 +43,7 @@ template <typename R>
 struct Lat {
   Geom g;
   R kappa, ef, efinv;        // kappa, e^{mu}, e^{-mu}
+  R kinv;                    // 1 / kappa = 2 m_w + 8
   const R* u;                // internal links (link_reals<R>() * V reals)
   int nsrc, k;
   int64_t vs;                // reals per lattice vector (padded)
@@ -66,6 +67,7 @@ struct Lat {
   // FP64 calls: links and dH's links (fu.e null: FP64 stencil), the recurrence's fields, and the
   // exponents of the bases, whose integers are in bv and bw
   FxLinks fu, fd;
+  const double* uaos;        // the user's links
   FxField fr, fs, fp, fq;
   short* bve; short* bwe;
   // basis window: vectors jbase .. jbase + kcap - 1 (all k from 0 unless segments are replayed)

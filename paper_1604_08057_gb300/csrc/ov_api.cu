@@ -329,10 +329,11 @@ void pack_start(ov_context* c, const Lat<R>& L, const void* b) {
   }
 }
 
-// fm = 2 sets up block mode: fields of 2V sites (upper and lower halves)
+// fm = 2 sets up block mode: fields of 2V sites (upper and lower halves); links: L.u (FP64
+// calls need it for the force and dH only)
 template <typename R>
 Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, double m_w, int nsrc, int k,
-             bool basis, int fm = 1, int kcap = 0) {
+             bool basis, int fm = 1, int kcap = 0, bool links = true) {
   Lat<R> L{};
   L.g = make_geom(dims);
   L.gl = L.g;
@@ -341,16 +342,20 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   check_ptr(U);
   const int64_t V = L.g.V;
   L.kappa = (R)(1.0 / (2.0 * m_w + 8.0));
+  L.kinv = (R)(2.0 * m_w + 8.0);
   L.ef = (R)std::exp(mu);
   L.efinv = (R)std::exp(-mu);
   L.nsrc = nsrc;
   L.k = k;
   constexpr bool fx = std::is_same<R, double>::value;   // FP64 calls run in fixed point (fx.cuh)
   L.vs = field_reals<R>(V);
-  R* u = wsT<R>(c, B_LINKS, link_reals<R>() * V);
-  L.u = u;
-  run(c, OV_KIND_LAYOUT, 1, [&] { pack_links<R>(static_cast<const double*>(U), u, V, c->st); });
+  if (links) {
+    R* u = wsT<R>(c, B_LINKS, link_reals<R>() * V);
+    L.u = u;
+    run(c, OV_KIND_LAYOUT, 1, [&] { pack_links<R>(static_cast<const double*>(U), u, V, c->st); });
+  }
   if constexpr (fx) {
+    L.uaos = static_cast<const double*>(U);
     int4* fe = wsT<int4>(c, B_FXL, fx_link_ints(V));
     short* ex = wsT<short>(c, B_FXE, 5 * V);
     L.fu = FxLinks{fe, ex};
@@ -445,6 +450,7 @@ void forward_krylov(ov_context* c, Lat<R>& L) {
   const int64_t nsb = (L.g.V + 127) / 128;
   zd* coef = wsT<zd>(c, B_COEF, (int64_t)L.nsrc * 2 * k);
   zd* cpart = wsT<zd>(c, B_CPART, (int64_t)L.nsrc * 2 * k * nsb);
+  L.uaos = nullptr;   // the caller's array: not part of a captured sweep or its key
   std::vector<unsigned char> key;
   key_add(key, L);
   key_add(key, coef);
@@ -1010,7 +1016,8 @@ int tsl_sign_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   check_ptr(b);
   check_ptr(x);
   const int S = c->opt.segment > 0 && c->opt.segment < k ? c->opt.segment : 0;
-  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0);
+  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0,
+                      !std::is_same<R, double>::value);
   pack_start(c, L, b);
   SegPlan P;
   SegStore<R> K{};
@@ -1080,9 +1087,9 @@ int block_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, d
   if (top) check_ptr(top);
   if (E) check_ptr(E);
   if (!std::isfinite(m_dir) || c->opt.segment > 0) throw Status{OV_ERR_INVALID_ARG};
-  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 2);
+  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 2, 0, !std::is_same<R, double>::value);
   const int64_t V = L.gl.V, Vf = L.g.V;
-  if (E) {
+  if (E && !std::is_same<R, double>::value) {
     R* ue = wsT<R>(c, B_ELINKS, link_reals<R>() * V);
     run(c, OV_KIND_LAYOUT, 1, [&] { pack_links<R>(static_cast<const double*>(E), ue, V, c->st); });
     L.ue = ue;
@@ -2390,8 +2397,10 @@ int apply_h_impl(ov_context* c, const int32_t dims[4], const void* U, double mu,
                  const void* in, void* out, int dagger) {
   check_ptr(in);
   check_ptr(out);
-  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, 1, false);
-  int* aerr = wsT<int>(c, B_AERR, 1, true);
+  constexpr bool fx = std::is_same<R, double>::value;
+  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, 1, false, 1, 0, !fx);
+  // (the FP32 staged variants alone have a wait that can run out)
+  int* aerr = fx ? nullptr : wsT<int>(c, B_AERR, 1, true);
   const int var = c->tuned_apply[c->opt.precision];
   if constexpr (std::is_same<R, float>::value) {
     if (var == APPLY_IL) {   // the sources-interleaved form has its own field layout
@@ -2402,7 +2411,7 @@ int apply_h_impl(ov_context* c, const int32_t dims[4], const void* U, double mu,
           [&] { unpack_spinors_il(L.p, static_cast<double*>(out), nsrc, L.g.V, c->st); });
     }
   }
-  if constexpr (std::is_same<R, double>::value) {
+  if constexpr (fx) {
     run(c, OV_KIND_LAYOUT, 1,
         [&] { fx_pack(static_cast<const double*>(in), L.fr, FxField{}, L.r, nsrc, L.g.V, L.vs, c->st); });
     run(c, OV_KIND_APPLY_H, 1,
@@ -2416,7 +2425,7 @@ int apply_h_impl(ov_context* c, const int32_t dims[4], const void* U, double mu,
   }
   launch_check();
   int herr = 0;
-  CK(cudaMemcpyAsync(&herr, aerr, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+  if (aerr) CK(cudaMemcpyAsync(&herr, aerr, sizeof(int), cudaMemcpyDeviceToHost, c->st));
   CK(cudaStreamSynchronize(c->st));
   prof_collect(c);
   return (herr & ERRB_TIMEOUT) ? OV_ERR_TIMEOUT : OV_OK;

@@ -104,4 +104,75 @@ __device__ void alpha_epilogue(const Lat<R>& L, const Rev<R>& B, int src, int j,
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same scalars formed by one warp: the divisions and square roots that do not depend on
+// one another run in different lanes (each takes some 0.5 us at the FP64 rate, and these
+// chains end every step's kernels: 14.9 us per update at 4^4, of which 5 are its fields).
+// Every lane passes the same arguments.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double lane_of(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+
+template <typename R>
+__device__ __forceinline__ void omega_finalize_warp(const Lat<R>& L, int src, int j, zd om, double rr, double ss) {
+  const int lane = threadIdx.x & 31;
+  SrcScal& sc = L.sc[src];
+  const double q = sqrt(lane == 0 ? om.re * om.re + om.im * om.im : rr * ss);
+  const double aom = lane_of(q, 0), rs = lane_of(q, 1);
+  if (!finite_z(om) || !isfinite(rr) || !isfinite(ss)) {
+    if (lane == 0) flag_error(sc, ERRB_NONFINITE, j + 1);
+    return;
+  }
+  if (aom <= 1e-14 * rs) {
+    if (lane == 0) flag_error(sc, ERRB_BREAKDOWN, j + 1);
+    return;
+  }
+  const double d = sqrt(aom);
+  const double y = (lane == 0 ? om.re : lane == 1 ? om.im : 1.0) / d;
+  const zd bt = mk(lane_of(y, 0), lane_of(y, 1));
+  const double sv = lane_of(y, 2);
+  const double w = (lane == 0 ? bt.re : bt.im) / (bt.re * bt.re + bt.im * bt.im);   // 1 / conj(beta)
+  const zd sw = mk(lane_of(w, 0), lane_of(w, 1));
+  if (lane == 0) {
+    L.beta[(int64_t)src * L.k + j + 1] = bt;
+    L.delta[(int64_t)src * L.k + j + 1] = d;
+    sc.sv = mk(sv, 0.0);
+    sc.sw = sw;
+  }
+}
+
+template <typename R>
+__device__ __forceinline__ void rev_dots_epilogue_warp(const Lat<R>& L, const Rev<R>& B, int src, int j, zd s0, zd s1) {
+  const int lane = threadIdx.x & 31;
+  SrcScal& sc = L.sc[src];
+  const int64_t o = (int64_t)src * L.k + j + 1;
+  const double d = L.delta[o];
+  const zd bt = L.beta[o];
+  const zd om = mk(bt.re * d, bt.im * d);
+  const double aom = d * d, b2 = bt.re * bt.re + bt.im * bt.im;
+  // conj(s1) / conj(beta) and 1 / beta over |beta|^2, s0 / d and 1 / d
+  const double num = lane == 0   ? s1.re * bt.re + s1.im * bt.im
+                     : lane == 1 ? s1.re * bt.im - s1.im * bt.re
+                     : lane == 2 ? bt.re
+                     : lane == 3 ? -bt.im
+                     : lane == 4 ? s0.re
+                                 : 1.0;
+  const double a = num / (lane < 4 ? b2 : d);
+  const zd g_b = B.gbT[o] + sc.carry_beta - mk(lane_of(a, 0), lane_of(a, 1));
+  double g_d = B.gdT[o] + sc.carry_delta - lane_of(a, 4);
+  const double b = (lane == 0 ? g_b.re : lane == 1 ? g_b.im : om.re * g_b.re + om.im * g_b.im) / (lane < 2 ? d : d * d);
+  zd g_w = mk(lane_of(b, 0), lane_of(b, 1));
+  g_d -= lane_of(b, 2);                      // Re(conj(om) g_b) / d^2
+  const double f = g_d / (2.0 * d * aom);
+  g_w = g_w + mk(f * om.re, f * om.im);
+  const zd cr2 = conj(bt) * g_w, cs2 = mk(d * g_w.re, -d * g_w.im);
+  const zd cr1 = mk(lane_of(a, 5), 0.0), cs1 = mk(lane_of(a, 2), lane_of(a, 3));
+  if (lane == 0) {
+    sc.cr1 = cr1;
+    sc.cr2 = cr2;
+    sc.cs1 = cs1;
+    sc.cs2 = cs2;
+    if (!finite_z(cr2) || !finite_z(cs2)) flag_error(sc, ERRB_NONFINITE, j);
+  }
+}
+
 }  // namespace ov

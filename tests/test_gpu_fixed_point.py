@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 import torch
 
-from oracle import dirac
+from oracle import dirac, vjp
 from paper_1604_08057_gb300 import binding, inputs
 
 pytestmark = pytest.mark.gpu
@@ -77,3 +77,41 @@ def test_non_finite_values_reach_the_same_sites():
     bad = ~np.isfinite(want).all(axis=(-1, -2))
     assert np.array_equal(bad, ~np.isfinite(got).all(axis=(-1, -2))) and bad.any()
     assert np.abs(got[~bad] - want[~bad]).max() <= 1e-13
+
+
+def rel(a, b):
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+@pytest.mark.parametrize("dims,k,rebiorth,passes", [((1, 3, 2, 5), 20, 1, 2), ((5, 3, 4, 7), 45, 10, 1),
+                                                    ((4, 6, 3, 3), 70, 1, 2)])
+def test_recurrence_and_force_from_a_point_source(dims, k, rebiorth, passes):
+    """b and xbar on one site each: the Krylov vectors start with most sites zero and decay over many
+    binary orders.  m_w = -1, rounding floors of the map ~1e-14: the bars of the parity tests."""
+    rng = np.random.default_rng(21)
+    u = inputs.su3_links(dims, 0.3, rng)
+    b = inputs.gaussian_spinors(dims, 1, rng)[0]
+    xbar = inputs.gaussian_spinors(dims, 1, rng)[0]
+    for f, at in ((b, (0, 0, 0, 0)), (xbar, tuple(n - 1 for n in b.shape[:4]))):
+        keep = f[at].copy()
+        f[...] = 0.0
+        f[at] = keep
+    du_o, dmu_o, fwd = vjp.tsl_vjp(u, b, 0.2, -1.0, k, xbar, rebiorth=rebiorth, passes=passes)
+    t = lambda a: torch.tensor(a, device="cuda")   # noqa: E731
+    du, dmu, x = binding.tsl_sign_vjp(t(u), 0.2, -1.0, t(b), k, t(xbar), rebiorth=rebiorth, passes=passes)
+    assert rel(x.cpu().numpy(), fwd.x) <= 1e-11
+    assert rel(du.cpu().numpy(), du_o) <= 1e-9 and abs(dmu - dmu_o) <= 1e-9 * abs(dmu_o)
+
+
+@pytest.mark.parametrize("dims,nsrc", [((3, 5, 2, 4), 1), ((6, 4, 5, 4), 3)])
+def test_powers_of_two_pass_through_exactly(dims, nsrc):
+    """Scaling the source or the cotangent by a power of two shifts exponents and nothing else."""
+    rng = np.random.default_rng(3)
+    t = lambda a: torch.tensor(a, device="cuda")   # noqa: E731
+    u, b = t(inputs.su3_links(dims, 0.3, rng)), t(inputs.gaussian_spinors(dims, nsrc, rng))
+    xbar = t(inputs.gaussian_spinors(dims, nsrc, rng))
+    du, dmu, x = binding.tsl_sign_vjp(u, 0.3, -1.0, b, 25, xbar, rebiorth=10, passes=1)
+    for sb, sx in ((2.0 ** 90, 1.0), (2.0 ** -130, 1.0), (1.0, 2.0 ** -80), (1.0, 2.0 ** 150)):
+        du2, dmu2, x2 = binding.tsl_sign_vjp(u, 0.3, -1.0, sb * b, 25, sx * xbar, rebiorth=10, passes=1)
+        assert torch.equal(x2, sb * x)
+        assert torch.equal(du2, (sb * sx) * du) and dmu2 == sb * sx * dmu
