@@ -297,6 +297,7 @@ static void gj_launch_all(const zd* a, zd* ainv, zd* w0, zd* w1, int k, int nb, 
 // every problem leaves at its next wait.
 // ---------------------------------------------------------------------------
 constexpr int GJP_THREADS = 256;
+constexpr int GJP_LANES = 4;                       // inversions at once (of a fourth of the SMs each)
 constexpr int GJP_RMAX = 32;                       // rows per block (one warp ranks them)
 constexpr unsigned long long GJP_WAIT_NS = 2000000000ull;
 
@@ -617,7 +618,7 @@ static GjpKernel gjp_kernel(int k) {
   return nullptr;
 }
 
-static bool gjp_shape(int k, int nb, int* R_out, int* bp_out, size_t* smem_out) {
+static bool gjp_shape(int k, int nb, int share, int* nsm_out, int* R_out, int* bp_out, size_t* smem_out) {
   int dev = 0, nsm = 0, smem_optin = 0, coop = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -637,10 +638,16 @@ static bool gjp_shape(int k, int nb, int* R_out, int* bp_out, size_t* smem_out) 
   // other's waits (four problems at k = 400: 40.1 -> 34.3 ms per sign).  A block has at
   // least three rows: with fewer, the words to poll cost more than the rows (k = 200: 7.1 ms
   // per sign with two rows, 6.1 with three, 6.3 with four, 8.7 with eight).
-  for (int occ = nb > 1 ? 2 : 1; occ >= 1; --occ) {
-    const int per = std::max(1, occ * nsm / nb);
+  // A context that shares the GPU with others (a worker of a batch) takes a fourth or half of
+  // the SMs where a step's update (4 R k FMAs per block at two per cycle) stays within the
+  // step's latency of some 3000 cycles, so that four or two inversions run at once (eight
+  // problems of k = 64 to 160 on four workers: 71 ms one inversion at a time, 58 so).
+  const bool shared = share > 1 && nb == 1;
+  for (int occ = nb > 1 ? 2 : shared ? (share > 2 ? GJP_LANES : 2) : 1; occ >= 1; occ >>= 1) {
+    const int per = std::max(1, nb > 1 ? occ * nsm / nb : nsm / occ);
     const int R = std::max((k + per - 1) / per, std::min(k, 3));
     const int bp = (k + R - 1) / R;
+    if (shared && occ > 1 && (int64_t)R * k > 1600) continue;
     if (R > GJP_RMAX || bp > GJ_KEY_SLOTS) continue;
     const size_t smem =
         ((size_t)R * k + 2 * (size_t)k) * sizeof(zd) + 2 * (size_t)k * sizeof(int) + (size_t)k * sizeof(double);
@@ -651,6 +658,7 @@ static bool gjp_shape(int k, int nb, int* R_out, int* bp_out, size_t* smem_out) 
       return false;
     }
     if ((int64_t)per_sm * nsm < (int64_t)bp * nb) continue;
+    *nsm_out = nsm;
     *R_out = R;
     *bp_out = bp;
     *smem_out = smem;
@@ -659,25 +667,42 @@ static bool gjp_shape(int k, int nb, int* R_out, int* bp_out, size_t* smem_out) 
   return false;
 }
 
-// Cooperative inversions issued from different streams (the worker contexts of
-// a batch) are chained through one event per device, so that no two of them
-// are ever partly resident at once, each waiting for blocks that the other
-// holds the room for.
+// Cooperative inversions issued from different streams (the worker contexts of a batch) are
+// ordered by events so that the blocks of those in flight are never more than the SMs: a
+// block that waits for room then finds an SM without such a block, whose other kernels end by
+// themselves, and no two inversions can each hold the room that the other's blocks wait for.
+// Each of the device's lanes stands for a fourth of its SMs; an inversion waits for, and
+// takes, as many lanes as its blocks need (one with more blocks than SMs takes all).
 namespace {
-struct CoopChain {
-  int dev;
-  cudaEvent_t ev;
+struct CoopLanes {
+  int dev, next;
+  cudaEvent_t ev[GJP_LANES];
 };
 std::mutex g_coop_mutex;
-std::vector<CoopChain> g_coop;
+std::vector<CoopLanes> g_coop;
+
+CoopLanes* coop_lanes(int dev) {   // with g_coop_mutex held
+  for (CoopLanes& c : g_coop)
+    if (c.dev == dev) return &c;
+  CoopLanes c{dev, 0, {}};
+  for (int i = 0; i < GJP_LANES; ++i) {
+    if (cudaEventCreateWithFlags(&c.ev[i], cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      while (i-- > 0) cudaEventDestroy(c.ev[i]);
+      return nullptr;
+    }
+  }
+  g_coop.push_back(c);
+  return &g_coop.back();
+}
 }  // namespace
 
 static bool gj_persist_launch(const zd* a, zd* ainv, zd* w0, zd* w1, int k, int nb, const int* act, int* ipiv,
                               int* used, unsigned long long* keys, double* logdet, int ld_stride, int* err,
-                              cudaStream_t st) {
-  int R = 0, bp = 0;
+                              cudaStream_t st, int share) {
+  int R = 0, bp = 0, nsm = 0;
   size_t smem = 0;
-  if (!gjp_shape(k, nb, &R, &bp, &smem)) return false;
+  if (!gjp_shape(k, nb, share, &nsm, &R, &bp, &smem)) return false;
   // the key slots: (k + 1) steps x GJ_KEY_SLOTS words per problem, all zero at the start
   if (cudaMemsetAsync(keys, 0, sizeof(unsigned long long) * (size_t)(k + 1) * GJ_KEY_SLOTS * nb, st) != cudaSuccess)
     return false;
@@ -688,26 +713,23 @@ static bool gj_persist_launch(const zd* a, zd* ainv, zd* w0, zd* w1, int k, int 
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   std::lock_guard<std::mutex> lock(g_coop_mutex);
-  cudaEvent_t ev = nullptr;
-  for (const CoopChain& c : g_coop)
-    if (c.dev == dev) ev = c.ev;
-  if (!ev) {
-    if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
+  CoopLanes* c = coop_lanes(dev);
+  if (!c) return false;
+  const int lane_blocks = std::max(1, nsm / GJP_LANES);
+  const int need = std::min(GJP_LANES, (int)(((int64_t)bp * nb + lane_blocks - 1) / lane_blocks));
+  for (int i = 0; i < need; ++i) {
+    if (cudaStreamWaitEvent(st, c->ev[(c->next + i) % GJP_LANES], 0) != cudaSuccess) {
       cudaGetLastError();
       return false;
     }
-    g_coop.push_back({dev, ev});
-  }
-  if (cudaStreamWaitEvent(st, ev, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
   }
   if (cudaLaunchCooperativeKernel((const void*)gjp_kernel(k), dim3(bp, nb), dim3(GJP_THREADS), args, smem, st) !=
       cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  cudaEventRecord(ev, st);
+  for (int i = 0; i < need; ++i) cudaEventRecord(c->ev[(c->next + i) % GJP_LANES], st);
+  c->next = (c->next + need) % GJP_LANES;
   return true;
 }
 
@@ -725,8 +747,10 @@ std::vector<GjGraph> g_gj_graphs;
 }  // namespace
 
 int dense_inverse(const zd* a, zd* ainv, zd* w0, zd* w1, int k, int nb, const int* act, int* ipiv, int* used,
-                  unsigned long long* keys, double* logdet, int ld_stride, int* err, int mode, cudaStream_t st) {
-  if (mode != GJ_STEPS && gj_persist_launch(a, ainv, w0, w1, k, nb, act, ipiv, used, keys, logdet, ld_stride, err, st))
+                  unsigned long long* keys, double* logdet, int ld_stride, int* err, int mode, cudaStream_t st,
+                  int share) {
+  if (mode != GJ_STEPS &&
+      gj_persist_launch(a, ainv, w0, w1, k, nb, act, ipiv, used, keys, logdet, ld_stride, err, st, share))
     return 1;
   const void* ptrs[11] = {a, ainv, w0, w1, ipiv, used, keys, logdet, err, act, nullptr};
   int dev = 0;

@@ -168,9 +168,8 @@ template <typename R> void tsl_update(const Lat<R>& L, int j, bool finalize, cud
 // mode 1 (adjoint):  e_r = V^dag g_r, e_s = W^dag g_s;  g_r -= W e_r, g_s -= V e_s
 template <typename R> void proj_dots(const Lat<R>& L, int j, int mode, const R* a, const R* b,
                                      int64_t ab_src_stride, zd* coef, zd* cpart, cudaStream_t st);
-// small: the coefficients are at rounding level (a second Gram-Schmidt pass): FP32 accumulation
 template <typename R> void proj_update(const Lat<R>& L, int j, int mode, R* a, R* b, int64_t ab_src_stride,
-                                       const zd* coef, bool finalize_omega, cudaStream_t st, bool small);
+                                       const zd* coef, bool finalize_omega, cudaStream_t st);
 template <typename R> void basis_dots(const Lat<R>& L, int nvec, const R* x, int64_t x_src_stride, zd* out,
                                       zd* cpart, cudaStream_t st);
 // out[src][2 (j - j0)] = v_j^dag x  for j0 <= j < j0 + nvec
@@ -217,12 +216,13 @@ void dense_copy_batch(const zd* A, int64_t sA, zd* B, int64_t sB, int64_t n, int
 // keys: (k + 1) * GJ_KEY_SLOTS words per problem); logdet[p * ld_stride] += log|det A_p|.
 // mode GJ_AUTO: one cooperative launch per inversion where the rows fit in
 // shared memory, else (and with GJ_STEPS) one launch per elimination step,
-// replayed as a CUDA graph.  Both give identical results.  Returns the number
-// of kernels launched.
+// replayed as a CUDA graph.  Both give identical results.  share: contexts that run at the
+// same time (the shape of the cooperative launch).  Returns the number of kernels launched.
 enum : int { GJ_AUTO = 0, GJ_STEPS = 1 };
 constexpr int GJ_KEY_SLOTS = 160;   // pivot-key words per step and problem (>= blocks per problem)
 int dense_inverse(const zd* A, zd* Ainv, zd* w0, zd* w1, int k, int nb, const int* act, int* ipiv, int* used,
-                  unsigned long long* keys, double* logdet, int ld_stride, int* err, int mode, cudaStream_t st);
+                  unsigned long long* keys, double* logdet, int ld_stride, int* err, int mode, cudaStream_t st,
+                  int share = 1);
 // the bounded inter-block wait of the cooperative inversion, made to run out
 void dense_wait_probe(unsigned long long* slot, int* err, int* how, unsigned long long limit_ns, cudaStream_t st);
 void dense_gemm(const zd* A, const zd* B, zd* C, int k, cudaStream_t st);   // C = A B

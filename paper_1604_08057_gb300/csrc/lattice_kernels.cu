@@ -1068,30 +1068,18 @@ __global__ void __launch_bounds__(128) k_proj_reduce(const zd* __restrict__ cpar
   if (threadIdx.x < 32 && t0 + threadIdx.x < 2 * nb) coef[src * coef_stride + t0 + threadIdx.x] = s;
 }
 
-// SMALL: the coefficients are at rounding level relative to a and b (the second
-// Gram-Schmidt pass, whose input is already biorthogonal to working precision),
-// so the correction sum_i c_i u_i is formed in FP32 arithmetic; its rounding is
-// ~6e-8 of a correction that is itself ~1e-12 or less of a, far below FP64
-// rounding of a.  FP64 fields are still read in full.
-template <typename T, typename R> OV_HD void spinor_cast(const Spinor<R>& in, Spinor<T>& out) {
-#pragma unroll
-  for (int c = 0; c < 12; ++c) out.c[c] = mk<T>((T)in.c[c].re, (T)in.c[c].im);
-}
-
-template <typename R, bool SMALL>
+template <typename R>
 __global__ void __launch_bounds__(BS) k_proj_update(Lat<R> L, int nb, int mode, R* __restrict__ a,
                                                      R* __restrict__ b, int64_t ab_stride,
                                                      const zd* __restrict__ coef, int64_t coef_stride,
                                                      int j, int finalize) {
-  using A = typename std::conditional<SMALL, float, R>::type;   // accumulation type
   __shared__ zd cs[2 * 64];
   __shared__ zd scratch[3 * 32];
   const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int src = blockIdx.y;
   const int64_t V = L.g.V;
   const bool active = x < V;
-  Spinor<A> ca, cb;
-  Spinor<R> e;
+  Spinor<R> ca, cb, e;
   spinor_zero(ca);
   spinor_zero(cb);
   const zd* cf = coef + src * coef_stride;
@@ -1104,16 +1092,16 @@ __global__ void __launch_bounds__(BS) k_proj_update(Lat<R> L, int nb, int mode, 
       for (int t = 0; t < n; ++t) {
         const int i = i0 + t;
         const R* ua = mode == 0 ? L.basis_v(src, i) : L.basis_w(src, i);
-        const cplx<A> c0 = cast<A>(cs[2 * t]);
+        const cplx<R> c0 = cast<R>(cs[2 * t]);
         load_spinor(ua, V, x, e);
 #pragma unroll
-        for (int c = 0; c < 12; ++c) cmac(ca.c[c], c0, mk<A>((A)e.c[c].re, (A)e.c[c].im));
+        for (int c = 0; c < 12; ++c) cmac(ca.c[c], c0, e.c[c]);
         if (b) {
           const R* ub = mode == 0 ? L.basis_w(src, i) : L.basis_v(src, i);
-          const cplx<A> c1 = cast<A>(cs[2 * t + 1]);
+          const cplx<R> c1 = cast<R>(cs[2 * t + 1]);
           load_spinor(ub, V, x, e);
 #pragma unroll
-          for (int c = 0; c < 12; ++c) cmac(cb.c[c], c1, mk<A>((A)e.c[c].re, (A)e.c[c].im));
+          for (int c = 0; c < 12; ++c) cmac(cb.c[c], c1, e.c[c]);
         }
       }
     }
@@ -1123,12 +1111,12 @@ __global__ void __launch_bounds__(BS) k_proj_update(Lat<R> L, int nb, int mode, 
     Spinor<R> r, s;
     load_spinor(a + src * ab_stride, V, x, r);
 #pragma unroll
-    for (int c = 0; c < 12; ++c) r.c[c] = r.c[c] - mk<R>((R)ca.c[c].re, (R)ca.c[c].im);
+    for (int c = 0; c < 12; ++c) r.c[c] = r.c[c] - ca.c[c];
     store_spinor(a + src * ab_stride, V, x, r);
     if (b) {
       load_spinor(b + src * ab_stride, V, x, s);
 #pragma unroll
-      for (int c = 0; c < 12; ++c) s.c[c] = s.c[c] - mk<R>((R)cb.c[c].re, (R)cb.c[c].im);
+      for (int c = 0; c < 12; ++c) s.c[c] = s.c[c] - cb.c[c];
       store_spinor(b + src * ab_stride, V, x, s);
       if (finalize) {
         v[0] = spinor_dot(s, r);
@@ -1164,15 +1152,10 @@ void proj_dots(const Lat<R>& L, int j, int mode, const R* a, const R* b, int64_t
 }
 template <typename R>
 void proj_update(const Lat<R>& L, int j, int mode, R* a, R* b, int64_t ab_stride, const zd* coef, bool finalize,
-                 cudaStream_t st, bool small) {
+                 cudaStream_t st) {
   const int bs = site_bs(L.g.V);
   const dim3 grid(nblocks(L.g.V, bs), L.nsrc);
-  if (small && sizeof(R) == 8)
-    k_proj_update<R, true><<<grid, bs, 0, st>>>(L, j + 1, mode, a, b, ab_stride, coef, 2 * (int64_t)L.k, j,
-                                                finalize ? 1 : 0);
-  else
-    k_proj_update<R, false><<<grid, bs, 0, st>>>(L, j + 1, mode, a, b, ab_stride, coef, 2 * (int64_t)L.k, j,
-                                                 finalize ? 1 : 0);
+  k_proj_update<R><<<grid, bs, 0, st>>>(L, j + 1, mode, a, b, ab_stride, coef, 2 * (int64_t)L.k, j, finalize ? 1 : 0);
 }
 
 // out[src][i] = v_i^dag x  for i < nvec (dots of the V basis with one vector per source)
@@ -1593,28 +1576,19 @@ __device__ void force_dir(const Lat<R>& L, const Rev<R>& B, int64_t x, int nterm
   for (int e = 0; e < 9; ++e) acc[e] = accd[e] = mk(0.0, 0.0);
   for (int src = i0 / nterms; src * nterms < i1; ++src) {
     const int t0 = max(i0 - src * nterms, 0), t1 = min(i1 - src * nterms, nterms);
-    if constexpr (sizeof(R) == 8) {
-      // FP64 fields: accumulate straight into the FP64 sums
-      for (int t = t0; t < t1; ++t) {
-        const int j = j0 - t;
-        force_term<NU>(L, x, xf, B.ring(B.gp_ring, t, src), L.basis_v(src, j), acc, accd);
-        if (j < L.k - 1) force_term<NU>(L, x, xf, L.basis_w(src, j), B.ring(B.gs_ring, t, src), acc, accd);
-      }
-    } else {
-      // FP32 fields: FP32 partial sums over one ring of terms, then FP64
-      cplx<R> G[9], Gd[9];
+    // FP32 partial sums over one ring of terms, then FP64
+    cplx<R> G[9], Gd[9];
 #pragma unroll
-      for (int e = 0; e < 9; ++e) G[e] = Gd[e] = czero<R>();
-      for (int t = t0; t < t1; ++t) {
-        const int j = j0 - t;
-        force_term<NU>(L, x, xf, B.ring(B.gp_ring, t, src), L.basis_v(src, j), G, Gd);
-        if (j < L.k - 1) force_term<NU>(L, x, xf, L.basis_w(src, j), B.ring(B.gs_ring, t, src), G, Gd);
-      }
+    for (int e = 0; e < 9; ++e) G[e] = Gd[e] = czero<R>();
+    for (int t = t0; t < t1; ++t) {
+      const int j = j0 - t;
+      force_term<NU>(L, x, xf, B.ring(B.gp_ring, t, src), L.basis_v(src, j), G, Gd);
+      if (j < L.k - 1) force_term<NU>(L, x, xf, L.basis_w(src, j), B.ring(B.gs_ring, t, src), G, Gd);
+    }
 #pragma unroll
-      for (int e = 0; e < 9; ++e) {
-        acc[e] = acc[e] + mk((double)G[e].re, (double)G[e].im);
-        accd[e] = accd[e] + mk((double)Gd[e].re, (double)Gd[e].im);
-      }
+    for (int e = 0; e < 9; ++e) {
+      acc[e] = acc[e] + mk((double)G[e].re, (double)G[e].im);
+      accd[e] = accd[e] + mk((double)Gd[e].re, (double)Gd[e].im);
     }
   }
   if (part) {   // a split of the items: its own partial sum, added in split order later
@@ -1738,7 +1712,6 @@ void eps_norms(const double* a_top, const double* a_bot, const double* b, int ns
   template void ritz_combine<R>(const Lat<R>&, int, int, int, const zd*, double*, cudaStream_t); \
   template void apply_dh<R>(const Lat<R>&, const R*, R*, int, cudaStream_t); \
   template void pack_spinors<R>(const double*, R*, int, int64_t, int64_t, cudaStream_t); \
-  template void pack_block_start<R>(const double*, const double*, R*, R*, int, int64_t, int64_t, cudaStream_t); \
   template void unpack_spinors<R>(const R*, double*, int, int64_t, int64_t, cudaStream_t); \
   template void pack_links<R>(const double*, R*, int64_t, cudaStream_t); \
   template void apply_h<R>(const Lat<R>&, const R*, R*, int, cudaStream_t, int, int*); \
@@ -1759,8 +1732,9 @@ OV_INST(float)
 
 // FP64 calls run these in fixed point (fx_kernels.cu)
 #define OV_INST_FP32(R) \
+  template void pack_block_start<R>(const double*, const double*, R*, R*, int, int64_t, int64_t, cudaStream_t); \
   template void proj_dots<R>(const Lat<R>&, int, int, const R*, const R*, int64_t, zd*, zd*, cudaStream_t); \
-  template void proj_update<R>(const Lat<R>&, int, int, R*, R*, int64_t, const zd*, bool, cudaStream_t, bool); \
+  template void proj_update<R>(const Lat<R>&, int, int, R*, R*, int64_t, const zd*, bool, cudaStream_t); \
   template void basis_dots<R>(const Lat<R>&, int, const R*, int64_t, zd*, zd*, cudaStream_t); \
   template void basis_dots_range<R>(const Lat<R>&, int, int, const R*, int64_t, zd*, zd*, cudaStream_t); \
   template void rev_dots<R>(const Lat<R>&, const Rev<R>&, int, cudaStream_t); \

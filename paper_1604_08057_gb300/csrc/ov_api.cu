@@ -80,6 +80,7 @@ struct ov_context {
   int tuned_apply[2] = {0, 0};  // per precision (OV_FP64, OV_MIXED)
   int tuned_pair[2] = {0, 0};
   bool owns_stream = false;     // worker contexts of ov_tsl_batch own theirs
+  int share = 1;                // contexts at work at the same time (a batch's workers)
   std::vector<ov_context*> workers;
   // captured sweeps (options.graphs): key of the captured call shape, executable graph,
   // kernels it launches; the capture stream and the events ordering it with `st`
@@ -476,7 +477,7 @@ void forward_krylov(ov_context* c, Lat<R>& L) {
           } else {
             run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 0, L.r, L.s, L.vs, coef, cpart, c->st); });
             run(c, OV_KIND_PROJ_UPDATE, 1,
-                [&] { proj_update(L, j, 0, L.r, L.s, L.vs, coef, last, c->st, ps > 0); });
+                [&] { proj_update(L, j, 0, L.r, L.s, L.vs, coef, last, c->st); });
           }
         }
       }
@@ -740,7 +741,8 @@ int newton(ov_context* c, zd* a[2], zd* e[2], int k, int* err_dev, int* which, N
     run(c, OV_KIND_DENSE, 0, [&] {
       // log|det| only where the determinant scaling uses it
       c->launches += dense_inverse(a[cur], ai, w0, w1, k, 1, nullptr, ipiv, used, keys,
-                                   !norm_rules && scaling ? dstat + 2 : nullptr, 0, err_dev, c->opt.dense, c->st);
+                                   !norm_rules && scaling ? dstat + 2 : nullptr, 0, err_dev, c->opt.dense, c->st,
+                                   c->share);
     });
     if (norm_rules && scaling)
       run(c, OV_KIND_DENSE, 1, [&] { dense_norm_scale(a[cur], ai, k, 1, nullptr, dstat + 2, 0, npart, ncnt, c->st); });
@@ -824,7 +826,7 @@ int newton_batch(ov_context* c, zd* a[2], int k, int nb, int* err_dev, std::vect
       // log|det| only where the determinant scaling uses it
       const bool want_ld = !norm_rules && std::find(scaling.begin(), scaling.end(), 1) != scaling.end();
       c->launches += dense_inverse(a[cur], ai, w0, w1, k, nb, act_dev, ipiv, used, keys,
-                                   want_ld ? dstat + 2 : nullptr, 4, err_dev, c->opt.dense, c->st);
+                                   want_ld ? dstat + 2 : nullptr, 4, err_dev, c->opt.dense, c->st, c->share);
     });
     if (norm_rules && std::find(scaling.begin(), scaling.end(), 1) != scaling.end())
       run(c, OV_KIND_DENSE, 1, [&] { dense_norm_scale(a[cur], ai, k, nb, act_dev, dstat + 2, 4, npart, ncnt, c->st); });
@@ -1789,7 +1791,7 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
           R* grs = B.gr_ring + (int64_t)slot * nsrc * vs;
           R* gss = B.gs_ring + (int64_t)slot * nsrc * vs;
           run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 1, grs, gss, vs, coef, cpart, c->st); });
-          run(c, OV_KIND_PROJ_UPDATE, 1, [&] { proj_update(L, j, 1, grs, gss, vs, coef, false, c->st, ps > 0); });
+          run(c, OV_KIND_PROJ_UPDATE, 1, [&] { proj_update(L, j, 1, grs, gss, vs, coef, false, c->st); });
         }
         run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_proj_record(L, B, j, nrec, coef, c->st); });
       }
@@ -2873,6 +2875,7 @@ int ov_tsl_batch(ov_context* c, int32_t nprob, ov_problem* probs, int32_t nworke
   for (int w = 0; w < nw; ++w) {
     ov_context* wc = c->workers[w];
     wc->opt = c->opt;
+    wc->share = nw;
     std::copy(c->tuned_apply, c->tuned_apply + 2, wc->tuned_apply);
     std::copy(c->tuned_pair, c->tuned_pair + 2, wc->tuned_pair);
     cudaStreamWaitEvent(wc->st, start, 0);
