@@ -505,9 +505,9 @@ __device__ __forceinline__ void fx_swap_lower(FxHalf& a) {
   }
 }
 // acc += the hops of D_w of field f (sites off + s) in directions nu0 .. nu1 - 1 (all eight by
-// default), at acc's scale; every lane of the warp.  A product is below 2^57 units, so the 48 of eight hops stay below 2^62.6 (for
-// sixteen hops the caller takes E one higher).  The loop is kept rolled: fully unrolled,
-// the code outgrows the instruction cache and instruction fetch sets the pace (144 us per
+// default), at acc's scale; every lane of the warp.  A product is below 2^57 units, so the 48
+// of eight hops stay below 2^62.6 (for sixteen hops the caller takes E one higher).  The loop
+// is kept rolled: fully unrolled, the code outgrows the instruction cache and instruction fetch sets the pace (144 us per
 // step pair at 14^4).  Copies in flight and the data read belong to one warp.
 __device__ __forceinline__ void fx_hops(FxHalf& acc, const FxField& f, int off, const FxLinks& U, const Geom& g,
                                         const FxSite& st, const FxExps& ex, int dagger, int sp, FxStage& S,
@@ -667,39 +667,42 @@ __device__ __forceinline__ void fx_block_partials(const zd (&v)[NV], FxSumBuf<NV
   }
 }
 
-// The sums of the n blocks' partials (in block order per thread, then a fixed tree), in every
-// lane of warp 0; every thread of the block calls it.  Eight loads per thread are in flight at
-// a time: one by one they cost a memory latency per 128 blocks.  A warp adds only where it has
-// partials: with 16 blocks the sums of nothing took 1.2 us of FP64 pipe per value.
+// The sums of the n blocks' partials (per value in block order per thread, then a fixed tree),
+// in every lane of warp 0; every thread of the block calls it.  The values are spread over the
+// warps, a value over several only where each has partials (trees and sums of nothing cost as
+// much FP64 pipe as others), and eight loads per thread are in flight at a time.  Two values of
+// 608 blocks took 8700 cycles with all warps at one value after the other; a call at 14x14^3,
+// k = 800 402 -> 393 ms, at 4x4^3, k = 200 23.9 -> 22.7 ms.
 template <int NV>
 __device__ __forceinline__ void fx_sum_partials(const zd* part, int n, zd (&out)[NV], zd* scratch) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int nw = min((int)blockDim.x >> 5, (n + 31) >> 5);   // warps with partials
-  if (w < nw) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int per = max(1, min(nw / NV, (n + 31) >> 5));   // warps per value
+  const int h = w % per;
+  for (int i = w / per; i < NV && w < nw / per * per; i += nw / per) {
+    const zd* p = part + (int64_t)i * n;
+    zd v = mk(0.0, 0.0), v1 = mk(0.0, 0.0);   // two chains: an addition's latency is long
+    for (int b0 = h * 32; b0 < n; b0 += 8 * 32 * per) {
+      zd t[8];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      zd v = mk(0.0, 0.0);
-      for (int b0 = threadIdx.x; b0 - lane < n; b0 += 8 * blockDim.x) {
-        zd t[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int b = b0 + u * blockDim.x;
-          t[u] = b < n ? ld_cg(part + i * n + b) : mk(0.0, 0.0);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (b0 - lane + u * (int)blockDim.x < n) v = v + t[u];
+      for (int u = 0; u < 8; ++u) {
+        const int b = b0 + u * 32 * per + lane;
+        t[u] = b < n ? ld_cg(p + b) : mk(0.0, 0.0);
       }
-      v = warp_sum(v);
-      if (lane == 0) scratch[i * 32 + w] = v;
+#pragma unroll
+      for (int u = 0; u < 8; u += 2) {
+        if (b0 + u * 32 * per < n) v = v + t[u];
+        if (b0 + (u + 1) * 32 * per < n) v1 = v1 + t[u + 1];
+      }
     }
+    v = warp_sum(n > 32 * per ? v + v1 : v);
+    if (lane == 0) scratch[i * 32 + h] = v;
   }
   __syncthreads();
   if (w == 0) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
       out[i] = scratch[i * 32];
-      for (int q = 1; q < nw; ++q) out[i] = out[i] + scratch[i * 32 + q];
+      for (int q = 1; q < per; ++q) out[i] = out[i] + scratch[i * 32 + q];
     }
   }
 }

@@ -405,10 +405,12 @@ __device__ __forceinline__ void alpha_finish(const Lat<double>& L, int src, int 
 // second half w_j and q of the same sites, so the links of both products come from L1 and
 // a small lattice spreads over more warps.  w_j crosses to the first half through shared
 // memory for the dot product.  H v_j = +-(v_j - kappa sv a) from the hop sum a of r.
+// Bound by instruction issue and latency (some 5500 instructions per warp; its bytes take 10
+// us at 14x14^3): 57 us there, 149 in FP64, whose products the FP64 units alone took 120 for.
 //
 // SPLIT: on a lattice with too few sites to fill the GPU a step's time is the latency of a
 // thread's chain of hops (22 us at 4^4), so four warps share a side's 16 sites, one
-// direction each, and add their sums through shared memory.
+// direction each, and add their sums through shared memory (14 us).
 template <int SPLIT>
 __global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 2 : 4)
     k_fx_tsl(const __grid_constant__ Lat<double> L, int j, int need_q) {
@@ -546,6 +548,8 @@ void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st, in
 // r = p - alpha_j v_j - beta_j v_{j-1};  s = q - conj(alpha_j) w_j - delta_j w_{j-1}.  The two
 // halves of a block's threads form r and s of the same SX (16 or 32) sites; s crosses to
 // the first half for s^dag r.
+// Bound by the latency of its loads and of the closing sums: 26 us at 14x14^3 (40 in FP64),
+// of which its bytes take 9 and the sums and scalars 8.
 // v[0] = s^dag r, v[1] = (|r|^2, |s|^2)
 template <int NT>
 __device__ __forceinline__ void omega_finish(const Lat<double>& L, int src, int j, int slot, const zd (&v)[2],
@@ -635,7 +639,9 @@ __device__ __forceinline__ void fx_load_site(const FxField& f, int64_t s, FxS& o
 constexpr int FX_NB = 8;   // basis vectors per block
 // One thread per site (spt sites in turn), one side per block: side 0 dots DA with a, side 1
 // DB with b.  a's integers stay in registers while FX_NB basis vectors stream past; each
-// thread's FP64 sums live in shared memory, so the loop over them stays rolled.
+// thread's FP64 sums live in shared memory, so the loop over them stays rolled.  Bound by HBM:
+// 56 ms of dots per call at 14x14^3, k = 800 (148 in FP64, at 87% of its units' rate; the
+// basis vectors' bytes take 48.5).
 __global__ void __launch_bounds__(128, 3) k_fx_dots(const __grid_constant__ Lat<double> L, int nb, int mode, FxField a,
                                                     FxField b, int64_t ab_stride, zd* __restrict__ cpart,
                                                     int64_t cp_stride, int spt, int ioff, int sides) {
@@ -860,7 +866,9 @@ __device__ __forceinline__ void sum_vectors(FxTerms& T, FxStage& S, FxCoef (*cs)
 // the four dots of the reverse step (a = g_r, b = g_s).
 //
 // SPLIT: on a lattice with too few sites to fill the GPU four warps share a side's 16 sites,
-// a quarter of the vectors each (88 us per projection of 100 vectors at 4^4 without).
+// a quarter of the vectors each (88 us per projection of 100 vectors at 4^4 without, 36 with).
+// Above 16 sites per SM the joins cost more than they give (6x12^3: 95 ms per call, 114 split).
+// Bound by HBM: 58 ms per call at 14x14^3, k = 800 (146 in FP64; the bytes take 48.5).
 template <int SPLIT>
 __global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 1 : 3)
     k_fx_proj_update(const __grid_constant__ Lat<double> L, const __grid_constant__ Rev<double> B, int nb, int mode,
@@ -1092,6 +1100,8 @@ struct RevTerm {
   FxField f;
   FxCoef c;
 };
+// Bound by instruction issue (the terms' products and the two hop sums), then by HBM: 122 us on
+// average at 14x14^3, k = 800 (234 in FP64; the bytes take 37).
 constexpr int RT = 30;   // terms converted at a time per side (a multiple of FX_RING)
 template <int SPLIT>
 __global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 1 : 4)
