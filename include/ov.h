@@ -54,7 +54,9 @@ extern "C" {
                                      diagnostics, or ov_overlap_solve within maxit */
 
 /* Precision of lattice vectors, links and stencil arithmetic.
- * OV_FP64 : everything in FP64.
+ * OV_FP64 : FP64 accuracy throughout.  Lattice vectors and links are held as 57- and
+ *           59-bit integers with an exponent per site or link (their products and sums
+ *           run on the integer units), scalars and k x k matrices in FP64.
  * OV_MIXED: links, basis vectors and stencils in FP32; dot products accumulated
  *           with compensated (Dot2) FP32 arithmetic per thread and FP64 across
  *           threads; recurrence coefficients, re-biorthogonalisation
