@@ -63,50 +63,24 @@ __device__ __forceinline__ FxField fx_bw(const Lat<double>& L, int src, int j) {
 // links in fixed point
 // ---------------------------------------------------------------------------
 // Direction d = blockIdx.y: the links (d < 3 spatial, 3: ef U_t, 4: efinv U_t) of the
-// user's array u, or with dh the combinations of the directional derivative dH:
-// d < 3: E, 3: ef (E_t + m U_t), 4: efinv (E_t - m U_t), E (may be null: zero) in e.
-// The products are formed with their FP64 rounding errors, so each entry carries the
-// fixed-point error alone.
-__global__ void __launch_bounds__(128) k_pack_links_fx(const double* __restrict__ u, const double* __restrict__ e,
-                                                       int dh, double m, double ef, double efinv,
+// user's array u.  The products are formed with their FP64 rounding errors, so each entry
+// carries the fixed-point error alone.
+__global__ void __launch_bounds__(128) k_pack_links_fx(const double* __restrict__ u, double ef, double efinv,
                                                        int4* __restrict__ out, short* __restrict__ ex, int64_t V) {
   const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (x >= V) return;
   const int d = blockIdx.y, nu = d < 3 ? d : 3;
   const double f = d < 3 ? 1.0 : (d == 3 ? ef : efinv);
   const double2* iu = reinterpret_cast<const double2*>(u) + x * 36 + nu * 9;
-  const double2* ie = e ? reinterpret_cast<const double2*>(e) + x * 36 + nu * 9 : nullptr;
-  const double mm = d == 3 ? m : -m;
   double hi[18], lo[18];
   unsigned mag = 0u;
 #pragma unroll
   for (int q = 0; q < 9; ++q) {
-    double2 a, al = make_double2(0.0, 0.0);
-    if (!dh) {
-      a = iu[q];
-    } else {
-      a = ie ? ie[q] : make_double2(0.0, 0.0);
-      if (d >= 3) {   // E + mm U, as a sum and its rounding error
-        const double2 t = iu[q];
-        const double pr = mm * t.x, pi = mm * t.y;
-        const double er = fma(mm, t.x, -pr), ei = fma(mm, t.y, -pi);
-        const double sr = a.x + pr, si = a.y + pi;
-        const double zr = sr - a.x, zi = si - a.y;
-        al.x = ((a.x - (sr - zr)) + (pr - zr)) + er;
-        al.y = ((a.y - (si - zi)) + (pi - zi)) + ei;
-        a = make_double2(sr, si);
-      }
-    }
-    if (d < 3) {
-      hi[2 * q] = a.x;
-      hi[2 * q + 1] = a.y;
-      lo[2 * q] = lo[2 * q + 1] = 0.0;
-    } else {
-      hi[2 * q] = f * a.x;
-      hi[2 * q + 1] = f * a.y;
-      lo[2 * q] = fma(f, a.x, -hi[2 * q]) + f * al.x;
-      lo[2 * q + 1] = fma(f, a.y, -hi[2 * q + 1]) + f * al.y;
-    }
+    const double2 a = iu[q];
+    hi[2 * q] = f * a.x;
+    hi[2 * q + 1] = f * a.y;
+    lo[2 * q] = d < 3 ? 0.0 : fma(f, a.x, -hi[2 * q]);
+    lo[2 * q + 1] = d < 3 ? 0.0 : fma(f, a.y, -hi[2 * q + 1]);
     mag = max(mag, max(fx_mag(hi[2 * q]), fx_mag(hi[2 * q + 1])));
   }
   const int eb = (int)(mag >> 20);
@@ -126,11 +100,7 @@ __global__ void __launch_bounds__(128) k_pack_links_fx(const double* __restrict_
   }
 }
 void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, cudaStream_t st) {
-  k_pack_links_fx<<<dim3(nblocks(V, 128), 5), 128, 0, st>>>(u, nullptr, 0, 0.0, ef, efinv, out, ex, V);
-}
-void pack_dh_links_fx(const double* u, const double* e, double m, int4* out, short* ex, int64_t V, double ef,
-                      double efinv, cudaStream_t st) {
-  k_pack_links_fx<<<dim3(nblocks(V, 128), 5), 128, 0, st>>>(u, e, 1, m, ef, efinv, out, ex, V);
+  k_pack_links_fx<<<dim3(nblocks(V, 128), 5), 128, 0, st>>>(u, ef, efinv, out, ex, V);
 }
 
 // ---------------------------------------------------------------------------
@@ -170,49 +140,27 @@ __device__ __forceinline__ void soa_store(double* f, int64_t V, int64_t s, int s
 }
 
 // user spinors to fixed point, in f and (if set) g; marked sites keep FP64 values in d (if
-// set).  top (may be null) with block: the Theorem-1 start, f = (top, bot), g = (top + bot, bot)
-// in fields of 2V sites, bot in aos.
-__global__ void __launch_bounds__(128) k_fx_pack(const double* __restrict__ aos, const double* __restrict__ top,
-                                                 int block, FxField f, FxField g, double* __restrict__ d, int64_t V,
-                                                 int64_t vs) {
+// set)
+__global__ void __launch_bounds__(128) k_fx_pack(const double* __restrict__ aos, FxField f, FxField g,
+                                                 double* __restrict__ d, int64_t V, int64_t vs) {
   __shared__ double2 stage[4][kStage];
   const int sp = fx_spin_of(threadIdx.x), w = threadIdx.x >> 5;
   const int64_t x0 = blockIdx.x * (int64_t)64 + w * 16, x = x0 + (threadIdx.x & 15);
   const int src = blockIdx.y;
   if (x0 >= V) return;   // whole warps
   const bool live = x < V;
-  const FxField fs = fx_src(f, src, vs), gs = g.c ? fx_src(g, src, vs) : g;
   zd p[6];
   FxH o;
   aos_load(aos, src, V, x0, stage[w], sp, p);
   fx_from_double(p, o);
-  if (live) {
-    fx_put(fs, block ? V + x : x, sp, o);
-    if (g.c) fx_put(gs, block ? V + x : x, sp, o);
-    if (d && o.e == FX_BAD) soa_store(d + src * vs, V, x, sp, p);
-  }
-  if (!block) return;
-  zd q[6];
-  if (top) {
-    aos_load(top, src, V, x0, stage[w], sp, q);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) q[i] = mk(0.0, 0.0);
-  }
-  fx_from_double(q, o);
-  if (live) fx_put(fs, x, sp, o);
-#pragma unroll
-  for (int i = 0; i < 6; ++i) q[i] = q[i] + p[i];
-  fx_from_double(q, o);
-  if (live) fx_put(gs, x, sp, o);
+  if (!live) return;
+  fx_put(fx_src(f, src, vs), x, sp, o);
+  if (g.c) fx_put(fx_src(g, src, vs), x, sp, o);
+  if (d && o.e == FX_BAD) soa_store(d + src * vs, V, x, sp, p);
 }
 void fx_pack(const double* aos, const FxField& f, const FxField& g, double* d, int nsrc, int64_t V, int64_t vs,
              cudaStream_t st) {
-  k_fx_pack<<<dim3(nblocks(V, 64), nsrc), 128, 0, st>>>(aos, nullptr, 0, f, g, d, V, vs);
-}
-void fx_pack_block(const double* top, const double* bot, const FxField& f, const FxField& g, int nsrc, int64_t V,
-                   int64_t vs, cudaStream_t st) {
-  k_fx_pack<<<dim3(nblocks(V, 64), nsrc), 128, 0, st>>>(bot, top, 1, f, g, nullptr, V, vs);
+  k_fx_pack<<<dim3(nblocks(V, 64), nsrc), 128, 0, st>>>(aos, f, g, d, V, vs);
 }
 // an FP64 site-major field to fixed point
 __global__ void __launch_bounds__(128) k_fx_encode(const double* __restrict__ d, FxField f, int64_t V, int64_t vs) {
@@ -359,13 +307,9 @@ __global__ void __launch_bounds__(128) k_fx_init(const __grid_constant__ Lat<dou
   const int src = blockIdx.y;
   zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
   if (x < L.g.V) {
-    FxH r, s;
+    FxH r;
     fx_load(fx_src(L.fr, src, L.vs), x, sp, r);
     v[0] = mk(fx_norm2(r), 0.0);
-    if (L.block) {
-      fx_load(fx_src(L.fs, src, L.vs), x, sp, s);
-      v[1] = fx_dot(s, r);
-    }
   }
   zd* part = L.part + src * L.part_stride;
   fx_block_partials(v, sum, part, blockDim.x >> 5);
@@ -481,67 +425,12 @@ __global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 2 : 4)
   alpha_finish(L, src, j, part, scratch);
 }
 
-// Block step (Theorem 1; fields of 2V sites): four warps of 16 sites,
-//   0: p_u = H v_u + dH v_l   1: p_l = H v_l   2: q_u = H^dag w_u   3: q_l = dH^dag w_u + H^dag w_l
-__global__ void __launch_bounds__(128, 4) k_fx_tsl_block(const __grid_constant__ Lat<double> L, int j, int need_q) {
-  __shared__ FxStage stage[4];
-  __shared__ FxSumBuf<1, 128> sum;
-  __shared__ zd scratch[32];
-  FxStage& S = stage[threadIdx.x >> 5];
-  const int t = threadIdx.x & 31, part_id = threadIdx.x >> 5, sp = fx_spin_of(t);
-  const bool left = part_id >= 2, low = part_id & 1;
-  const int64_t V = L.gl.V, x0 = blockIdx.x * (int64_t)16 + fx_site_of(t), x = min(x0, V - 1);
-  const int src = blockIdx.y;
-  const int off = low ? (int)V : 0, offx = low ? 0 : (int)V;
-  const bool cross = part_id == 0 || part_id == 3;   // adds dH of the other half
-  zd v[1] = {mk(0.0, 0.0)};
-  const bool go = L.sc[src].err == 0, live = go && x0 < V;
-  FxH o, w;
-  if (go) {
-    const FxField f = fx_src(left ? L.fs : L.fr, src, L.vs);
-    const zd sc = left ? L.sc[src].sw : L.sc[src].sv;
-    FxHalf acc;
-    fx_load(f, off + x, sp, o);
-    fx_zero(acc, 0);
-    const bool okv = fx_axpy(acc, fx_coef(sc), o);
-    fx_encode(acc, !okv, w);
-    if (live) fx_put(left ? fx_bw(L, src, j) : fx_bv(L, src, j), off + x, sp, w);
-    if (!left || need_q) {
-      const FxSite s(L.gl, x);
-      const int dg = left ? 1 : 0;
-      FxExps ex, exd;
-      int E = fx_range(ex, f, off, L.fu, L.gl, s, dg);
-      if (cross) E = max(E, fx_range(exd, f, offx, L.fd, L.gl, s, dg)) + 1;   // sixteen hops
-      const bool ok = E < FX_BAD;
-      fx_zero(acc, ok ? E : FX_E_BIAS);
-      for (int h = 0; h < (cross ? 2 : 1); ++h)
-        fx_hops(acc, f, h ? offx : off, h ? L.fd : L.fu, L.gl, s, h ? exd : ex, dg, sp, S);
-      fx_encode(acc, !ok, o);
-      const bool okp = h_finish(acc, w, fx_coef(mk(-L.kappa * sc.re, -L.kappa * sc.im)), o);
-      fx_encode(acc, !okp, o);
-      if (live) fx_put(fx_src(left ? L.fq : L.fp, src, L.vs), off + x, sp, o);
-    }
-    if (left) fx_row_put(S.row, w);
-  }
-  __syncthreads();
-  if (live && !left) {
-    fx_row_get(stage[part_id + 2].row, w);
-    v[0] = fx_dot(w, o);
-  }
-  zd* part = L.part + src * L.part_stride;
-  fx_block_partials(v, sum, part, 2);
-  alpha_finish(L, src, j, part, scratch);
-}
-void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st, int variant) {
-  if (L.block) {
-    k_fx_tsl_block<<<dim3(nblocks(L.gl.V, 16), L.nsrc), 128, 0, st>>>(L, j, need_q);
-    return;
-  }
+void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st) {
   if (fx_split_exact(L)) {
     fx_launch<k_fx_tsl<1>>(dim3(nblocks(L.g.V, 16), L.nsrc), 256, 8 * sizeof(FxStage), st, L, j, need_q);
     return;
   }
-  const int sx = (variant & 1) ? 16 : two_sided_sites(L);
+  const int sx = two_sided_sites(L);
   fx_launch<k_fx_tsl<0>>(dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, (sx / 8) * sizeof(FxStage), st, L, j, need_q);
 }
 

@@ -24,8 +24,9 @@ struct SrcScal {
   zd cr1, cr2, cs1, cs2; // g_r = cr1 Gv_{j+1} + cr2 w_{j+1};  g_s = cs1 Gw_{j+1} + cs2 v_{j+1}
 };
 
-// FP64 calls hold every lattice field in block fixed point (fx.cuh): vs reals per field as in
-// Lat (a field of Vp sites, a multiple of 32, takes 12 Vp int4 and Vp exponents: vs = 24 Vp).
+// Fields in block fixed point (fx.cuh; which FP64 calls use them: struct Lat): vs reals per
+// field as in Lat (a field of Vp sites, a multiple of 32, takes 12 Vp int4 and Vp exponents:
+// vs = 24 Vp).
 struct FxLinks {
   const int4* e;
   const short* ex;
@@ -64,12 +65,13 @@ struct Lat {
   Geom gl;
   const R* ue;               // links of the direction E (internal layout) or null
   R mdir;                    // mu direction
-  // FP64 calls: links and dH's links (fu.e null: FP64 stencil), the recurrence's fields, and the
-  // exponents of the bases, whose integers are in bv and bw
-  FxLinks fu, fd;
+  // FP64 calls: fixed-point links (fu.e null: FP64 stencil), the fields of a fixed-point
+  // recurrence, and the exponents of fixed-point bases, whose integers are in bv and bw
+  FxLinks fu;
   const double* uaos;        // the user's links
   FxField fr, fs, fp, fq;
   short* bve; short* bwe;
+  OV_HD bool fx() const { return fs.c != nullptr; }   // the recurrence runs in fixed point
   // basis window: vectors jbase .. jbase + kcap - 1 (all k from 0 unless segments are replayed)
   int kcap, jbase;
   OV_HD R* basis_v(int src, int j) const { return bv + ((int64_t)src * kcap + (j - jbase)) * vs; }
@@ -130,20 +132,16 @@ void unpack_spinors_il(const float* f, double* aos, int nsrc, int64_t V, cudaStr
 
 // FP64 calls (fx_kernels.cu); the launchers below dispatch to them
 void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, cudaStream_t st);
-void pack_dh_links_fx(const double* u, const double* e, double m, int4* out, short* ex, int64_t V, double ef,
-                      double efinv, cudaStream_t st);
 // user spinors to f and (if set) g; FP64 values of marked sites to d (if set)
 void fx_pack(const double* aos, const FxField& f, const FxField& g, double* d, int nsrc, int64_t V, int64_t vs,
              cudaStream_t st);
-void fx_pack_block(const double* top, const double* bot, const FxField& f, const FxField& g, int nsrc, int64_t V,
-                   int64_t vs, cudaStream_t st);
 void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t vs, cudaStream_t st);
 // in: the field in fixed point, d: its FP64 companion (read where a site is marked); aos: out
 // in the user's layout
 void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double* out, int dagger, int aos,
                 cudaStream_t st, int variant);
 void fx_tsl_init(const Lat<double>& L, cudaStream_t st);
-void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st, int variant);
+void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st);
 void fx_tsl_update(const Lat<double>& L, int j, int finalize, cudaStream_t st);
 // dots with vectors j0 .. j0 + nb - 1 (modes as proj_dots; b.c null: side A alone)
 void fx_proj_dots(const Lat<double>& L, int j0, int nb, int mode, const FxField& a, const FxField& b,
@@ -168,8 +166,9 @@ template <typename R> void tsl_update(const Lat<R>& L, int j, bool finalize, cud
 // mode 1 (adjoint):  e_r = V^dag g_r, e_s = W^dag g_s;  g_r -= W e_r, g_s -= V e_s
 template <typename R> void proj_dots(const Lat<R>& L, int j, int mode, const R* a, const R* b,
                                      int64_t ab_src_stride, zd* coef, zd* cpart, cudaStream_t st);
+// small: the coefficients are at rounding level (a second Gram-Schmidt pass): FP32 accumulation
 template <typename R> void proj_update(const Lat<R>& L, int j, int mode, R* a, R* b, int64_t ab_src_stride,
-                                       const zd* coef, bool finalize_omega, cudaStream_t st);
+                                       const zd* coef, bool finalize_omega, cudaStream_t st, bool small);
 template <typename R> void basis_dots(const Lat<R>& L, int nvec, const R* x, int64_t x_src_stride, zd* out,
                                       zd* cpart, cudaStream_t st);
 // out[src][2 (j - j0)] = v_j^dag x  for j0 <= j < j0 + nvec

@@ -703,11 +703,9 @@ __global__ void __launch_bounds__(BS) k_tsl_init(Lat<R> L) {
 }
 template <typename R>
 void tsl_init(const Lat<R>& L, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value) {
-    fx_tsl_init(L, st);
-  } else {
-    k_tsl_init<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L);
-  }
+  if constexpr (std::is_same<R, double>::value)
+    if (L.fx()) return fx_tsl_init(L, st);
+  k_tsl_init<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L);
 }
 
 // ---------------------------------------------------------------------------
@@ -864,10 +862,8 @@ static void launch_pair(const Lat<R>& L, int j, int q, cudaStream_t st) {
 template <typename R>
 void tsl_stencil(const Lat<R>& L, int j, bool need_q, cudaStream_t st, int variant) {
   const int q = need_q ? 1 : 0;
-  if constexpr (std::is_same<R, double>::value) {
-    fx_tsl_stencil(L, j, q, st, variant);
-    return;
-  } else {
+  if constexpr (std::is_same<R, double>::value)
+    if (L.fx()) return fx_tsl_stencil(L, j, q, st);
   if (L.block) {
     k_tsl_stencil_block<R><<<dim3(nblocks(L.gl.V, BS), L.nsrc), BS, 0, st>>>(L, j, q);
     return;
@@ -880,7 +876,6 @@ void tsl_stencil(const Lat<R>& L, int j, bool need_q, cudaStream_t st, int varia
     case 5: launch_pair<R, 1, 256, 1>(L, j, q, st); break;
     case 6: launch_pair<R, 0, 512, 1>(L, j, q, st); break;
     default: launch_pair<R, 1, 128, 0>(L, j, q, st); break;
-  }
   }
 }
 
@@ -936,11 +931,9 @@ __global__ void __launch_bounds__(BS) k_tsl_update(Lat<R> L, int j, int finalize
 }
 template <typename R>
 void tsl_update(const Lat<R>& L, int j, bool finalize, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value) {
-    fx_tsl_update(L, j, finalize ? 1 : 0, st);
-  } else {
-    k_tsl_update<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j, finalize ? 1 : 0);
-  }
+  if constexpr (std::is_same<R, double>::value)
+    if (L.fx()) return fx_tsl_update(L, j, finalize ? 1 : 0, st);
+  k_tsl_update<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j, finalize ? 1 : 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -959,9 +952,10 @@ static inline int proj_spt(int nb) { return nb >= NB ? 4 : 1; }
 // coalesced) before the block reduction, which then costs 1/spt per site.  One side per
 // block (blockIdx.z = source * sides + side): both sides' sums and fields in one thread
 // leave two blocks per SM, and the 16 sums cost 160 FP64 additions per warp one by one.
-// The basis vectors come through a ring of three in shared memory, copied two ahead: with
-// the loads in registers the kernel waits for them (9.8 of 13 cycles per instruction).
-// Bound by HBM (each basis vector is read once).  6x18^3, 4 sources, projections every step to
+// FP32 basis vectors come through a ring of three in shared memory, copied two ahead: with
+// the loads in registers the kernel waits for them (9.8 of 13 cycles per instruction).  FP64
+// ones are loaded into registers: their sums keep the FP64 units busy, not the loads.
+// FP32 is bound by HBM (each basis vector is read once).  6x18^3, 4 sources, projections every step to
 // k = 80, two passes: 91 ms of dots with both sides in a thread and the loads in registers, 65
 // with one side per block, 47 with the ring.
 constexpr int kDotsRing = 3;
@@ -970,8 +964,9 @@ __global__ void __launch_bounds__(BS) k_proj_dots(Lat<R> L, int nb, int mode, co
                                                    const R* __restrict__ b, int64_t ab_stride,
                                                    zd* __restrict__ cpart, int64_t cp_stride, int spt, int ioff,
                                                    int sides) {
-  constexpr int NC = sizeof(R) == 4 ? 6 : 12;   // 16-byte chunks of a spinor
-  __shared__ float4 ring[kDotsRing][NC][BS];
+  constexpr bool RING = sizeof(R) == 4;
+  constexpr int NC = 6;   // 16-byte chunks of an FP32 spinor
+  __shared__ float4 ring[RING ? kDotsRing : 1][RING ? NC : 1][RING ? BS : 1];
   __shared__ double part[BS / 32][2 * NB];
   const int src = blockIdx.z / sides, side = blockIdx.z - src * sides;
   const int i0 = blockIdx.y * NB, n = min(NB, nb - i0);
@@ -1006,7 +1001,7 @@ __global__ void __launch_bounds__(BS) k_proj_dots(Lat<R> L, int nb, int mode, co
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
 #pragma unroll
-  for (int u = 0; u < kDotsRing - 1; ++u) issue(u);
+  for (int u = 0; RING && u < kDotsRing - 1; ++u) issue(u);
   for (int q = 0; q < spt; ++q) {
     const int64_t x = x0 + (int64_t)q * BS;
     if (x >= V) break;
@@ -1015,10 +1010,14 @@ __global__ void __launch_bounds__(BS) k_proj_dots(Lat<R> L, int nb, int mode, co
 #pragma unroll
     for (int t = 0; t < NB; ++t) {
       if (t < n) {
-        issue(slot == 0 ? kDotsRing - 1 : slot - 1);
-        asm volatile("cp.async.wait_group %0;" ::"n"(kDotsRing - 1) : "memory");
-        load_spinor(reinterpret_cast<const R*>(&ring[slot][0][0]), BS, threadIdx.x, e);
-        slot = slot == kDotsRing - 1 ? 0 : slot + 1;
+        if constexpr (RING) {
+          issue(slot == 0 ? kDotsRing - 1 : slot - 1);
+          asm volatile("cp.async.wait_group %0;" ::"n"(kDotsRing - 1) : "memory");
+          load_spinor(reinterpret_cast<const R*>(&ring[slot][0][0]), BS, threadIdx.x, e);
+          slot = slot == kDotsRing - 1 ? 0 : slot + 1;
+        } else {
+          load_spinor(usew ? L.basis_w(src, ioff + i0 + t) : L.basis_v(src, ioff + i0 + t), V, x, e);
+        }
 #pragma unroll
         for (int c = 0; c < 12; ++c) acc[t].add(e.c[c], v.c[c]);
       }
@@ -1068,18 +1067,25 @@ __global__ void __launch_bounds__(128) k_proj_reduce(const zd* __restrict__ cpar
   if (threadIdx.x < 32 && t0 + threadIdx.x < 2 * nb) coef[src * coef_stride + t0 + threadIdx.x] = s;
 }
 
-template <typename R>
+// SMALL: the coefficients are at rounding level relative to a and b (the second
+// Gram-Schmidt pass, whose input is already biorthogonal to working precision),
+// so the correction sum_i c_i u_i is formed in FP32 arithmetic; its rounding is
+// ~6e-8 of a correction that is itself ~1e-12 or less of a, far below FP64
+// rounding of a.  FP64 fields are still read in full.
+template <typename R, bool SMALL>
 __global__ void __launch_bounds__(BS) k_proj_update(Lat<R> L, int nb, int mode, R* __restrict__ a,
                                                      R* __restrict__ b, int64_t ab_stride,
                                                      const zd* __restrict__ coef, int64_t coef_stride,
                                                      int j, int finalize) {
+  using A = typename std::conditional<SMALL, float, R>::type;   // accumulation type
   __shared__ zd cs[2 * 64];
   __shared__ zd scratch[3 * 32];
   const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int src = blockIdx.y;
   const int64_t V = L.g.V;
   const bool active = x < V;
-  Spinor<R> ca, cb, e;
+  Spinor<A> ca, cb;
+  Spinor<R> e;
   spinor_zero(ca);
   spinor_zero(cb);
   const zd* cf = coef + src * coef_stride;
@@ -1092,16 +1098,16 @@ __global__ void __launch_bounds__(BS) k_proj_update(Lat<R> L, int nb, int mode, 
       for (int t = 0; t < n; ++t) {
         const int i = i0 + t;
         const R* ua = mode == 0 ? L.basis_v(src, i) : L.basis_w(src, i);
-        const cplx<R> c0 = cast<R>(cs[2 * t]);
+        const cplx<A> c0 = cast<A>(cs[2 * t]);
         load_spinor(ua, V, x, e);
 #pragma unroll
-        for (int c = 0; c < 12; ++c) cmac(ca.c[c], c0, e.c[c]);
+        for (int c = 0; c < 12; ++c) cmac(ca.c[c], c0, mk<A>((A)e.c[c].re, (A)e.c[c].im));
         if (b) {
           const R* ub = mode == 0 ? L.basis_w(src, i) : L.basis_v(src, i);
-          const cplx<R> c1 = cast<R>(cs[2 * t + 1]);
+          const cplx<A> c1 = cast<A>(cs[2 * t + 1]);
           load_spinor(ub, V, x, e);
 #pragma unroll
-          for (int c = 0; c < 12; ++c) cmac(cb.c[c], c1, e.c[c]);
+          for (int c = 0; c < 12; ++c) cmac(cb.c[c], c1, mk<A>((A)e.c[c].re, (A)e.c[c].im));
         }
       }
     }
@@ -1111,12 +1117,12 @@ __global__ void __launch_bounds__(BS) k_proj_update(Lat<R> L, int nb, int mode, 
     Spinor<R> r, s;
     load_spinor(a + src * ab_stride, V, x, r);
 #pragma unroll
-    for (int c = 0; c < 12; ++c) r.c[c] = r.c[c] - ca.c[c];
+    for (int c = 0; c < 12; ++c) r.c[c] = r.c[c] - mk<R>((R)ca.c[c].re, (R)ca.c[c].im);
     store_spinor(a + src * ab_stride, V, x, r);
     if (b) {
       load_spinor(b + src * ab_stride, V, x, s);
 #pragma unroll
-      for (int c = 0; c < 12; ++c) s.c[c] = s.c[c] - cb.c[c];
+      for (int c = 0; c < 12; ++c) s.c[c] = s.c[c] - mk<R>((R)cb.c[c].re, (R)cb.c[c].im);
       store_spinor(b + src * ab_stride, V, x, s);
       if (finalize) {
         v[0] = spinor_dot(s, r);
@@ -1152,10 +1158,15 @@ void proj_dots(const Lat<R>& L, int j, int mode, const R* a, const R* b, int64_t
 }
 template <typename R>
 void proj_update(const Lat<R>& L, int j, int mode, R* a, R* b, int64_t ab_stride, const zd* coef, bool finalize,
-                 cudaStream_t st) {
+                 cudaStream_t st, bool small) {
   const int bs = site_bs(L.g.V);
   const dim3 grid(nblocks(L.g.V, bs), L.nsrc);
-  k_proj_update<R><<<grid, bs, 0, st>>>(L, j + 1, mode, a, b, ab_stride, coef, 2 * (int64_t)L.k, j, finalize ? 1 : 0);
+  if (small && sizeof(R) == 8)
+    k_proj_update<R, true><<<grid, bs, 0, st>>>(L, j + 1, mode, a, b, ab_stride, coef, 2 * (int64_t)L.k, j,
+                                                finalize ? 1 : 0);
+  else
+    k_proj_update<R, false><<<grid, bs, 0, st>>>(L, j + 1, mode, a, b, ab_stride, coef, 2 * (int64_t)L.k, j,
+                                                 finalize ? 1 : 0);
 }
 
 // out[src][i] = v_i^dag x  for i < nvec (dots of the V basis with one vector per source)
@@ -1248,20 +1259,16 @@ __global__ void __launch_bounds__(BS) k_ritz_combine(Lat<R> L, int src, int side
 }
 template <typename R>
 void ritz_combine(const Lat<R>& L, int src, int side, int nvec, const zd* y, double* out, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value) {
-    fx_combine(L, src, 1, side, 0, nvec, y, 0, out, 0, st);
-  } else {
-    k_ritz_combine<R><<<nblocks(L.g.V, BS), BS, 0, st>>>(L, src, side, nvec, y, out);
-  }
+  if constexpr (std::is_same<R, double>::value)
+    if (L.bve) return fx_combine(L, src, 1, side, 0, nvec, y, 0, out, 0, st);   // bases in fixed point
+  k_ritz_combine<R><<<nblocks(L.g.V, BS), BS, 0, st>>>(L, src, side, nvec, y, out);
 }
 
 template <typename R>
 void combine_range(const Lat<R>& L, int j0, int nvec, const zd* y, double* out, bool acc, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value) {
-    fx_combine(L, 0, L.nsrc, 0, j0, nvec, y, L.k, out, acc ? 1 : 0, st);
-  } else {
-    k_combine<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j0, nvec, y, out, acc ? 1 : 0);
-  }
+  if constexpr (std::is_same<R, double>::value)
+    if (L.fx()) return fx_combine(L, 0, L.nsrc, 0, j0, nvec, y, L.k, out, acc ? 1 : 0, st);
+  k_combine<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j0, nvec, y, out, acc ? 1 : 0);
 }
 template <typename R>
 void combine(const Lat<R>& L, int nvec, const zd* y, double* out, cudaStream_t st) {
@@ -1712,12 +1719,15 @@ void eps_norms(const double* a_top, const double* a_bot, const double* b, int ns
   template void ritz_combine<R>(const Lat<R>&, int, int, int, const zd*, double*, cudaStream_t); \
   template void apply_dh<R>(const Lat<R>&, const R*, R*, int, cudaStream_t); \
   template void pack_spinors<R>(const double*, R*, int, int64_t, int64_t, cudaStream_t); \
+  template void pack_block_start<R>(const double*, const double*, R*, R*, int, int64_t, int64_t, cudaStream_t); \
   template void unpack_spinors<R>(const R*, double*, int, int64_t, int64_t, cudaStream_t); \
   template void pack_links<R>(const double*, R*, int64_t, cudaStream_t); \
   template void apply_h<R>(const Lat<R>&, const R*, R*, int, cudaStream_t, int, int*); \
   template void tsl_init<R>(const Lat<R>&, cudaStream_t); \
   template void tsl_stencil<R>(const Lat<R>&, int, bool, cudaStream_t, int); \
   template void tsl_update<R>(const Lat<R>&, int, bool, cudaStream_t); \
+  template void proj_dots<R>(const Lat<R>&, int, int, const R*, const R*, int64_t, zd*, zd*, cudaStream_t); \
+  template void proj_update<R>(const Lat<R>&, int, int, R*, R*, int64_t, const zd*, bool, cudaStream_t, bool); \
   template void combine<R>(const Lat<R>&, int, const zd*, double*, cudaStream_t); \
   template void combine_range<R>(const Lat<R>&, int, int, const zd*, double*, bool, cudaStream_t); \
   template void rev_init<R>(const Lat<R>&, const Rev<R>&, cudaStream_t); \
@@ -1730,11 +1740,8 @@ void eps_norms(const double* a_top, const double* a_bot, const double* b, int ns
 OV_INST(double)
 OV_INST(float)
 
-// FP64 calls run these in fixed point (fx_kernels.cu)
+// FP64 calls run the reverse sweep in fixed point (fx_kernels.cu)
 #define OV_INST_FP32(R) \
-  template void pack_block_start<R>(const double*, const double*, R*, R*, int, int64_t, int64_t, cudaStream_t); \
-  template void proj_dots<R>(const Lat<R>&, int, int, const R*, const R*, int64_t, zd*, zd*, cudaStream_t); \
-  template void proj_update<R>(const Lat<R>&, int, int, R*, R*, int64_t, const zd*, bool, cudaStream_t); \
   template void basis_dots<R>(const Lat<R>&, int, const R*, int64_t, zd*, zd*, cudaStream_t); \
   template void basis_dots_range<R>(const Lat<R>&, int, int, const R*, int64_t, zd*, zd*, cudaStream_t); \
   template void rev_dots<R>(const Lat<R>&, const Rev<R>&, int, cudaStream_t); \

@@ -23,7 +23,7 @@ enum BufId {
   B_LINKS, B_BV, B_BW, B_P, B_Q, B_R, B_S, B_SC, B_ALPHA, B_BETA, B_DELTA, B_PART, B_CNT, B_COEF, B_CPART,
   B_T, B_X, B_XI, B_XN, B_E, B_EN, B_TMP1, B_TMP2, B_IPIV, B_PROW, B_COL, B_DSTAT, B_DPART, B_DCNT, B_DERR,
   B_Y, B_GY, B_GA, B_GB, B_GD, B_XBAR, B_GV, B_GW, B_GV2, B_GW2, B_GR, B_GS, B_GP, B_EV, B_EW, B_REB,
-  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, B_FXL, B_FXE, B_FXDL, B_FXDE, B_FXR, B_FXRE, B_FXS, B_FXSE, B_FXP, B_FXPE, B_FXQ, B_FXQE, B_BVE, B_BWE, B_CKRE, B_CKSE, B_CKVE, B_CKWE, B_GVE, B_GWE, B_GRE, B_GSE, B_GPE, B_HINE, B_XBE, NBUF
+  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, B_FXL, B_FXE, B_FXR, B_FXRE, B_FXS, B_FXSE, B_FXP, B_FXPE, B_FXQ, B_FXQE, B_BVE, B_BWE, B_CKRE, B_CKSE, B_CKVE, B_CKWE, B_GVE, B_GWE, B_GRE, B_GSE, B_GPE, B_HINE, B_XBE, NBUF
 };
 
 struct Status {
@@ -73,6 +73,7 @@ struct ov_context {
   int last_k = 0, last_nsrc = 0;
   // shape of the last forward pass whose bases stay in B_BV / B_BW (for ov_tsl_ritz_triples)
   int last_block = 0, last_seg = 0, last_prec = -1;
+  bool last_fx = false;   // the last forward pass left its bases in fixed point
   int32_t last_dims[4] = {0, 0, 0, 0};
   cudaEvent_t ev[8] = {};
   Prof* prof = nullptr;
@@ -321,20 +322,40 @@ template <typename R>
 void pack_start(ov_context* c, const Lat<R>& L, const void* b) {
   const double* bd = static_cast<const double*>(b);
   if constexpr (std::is_same<R, double>::value) {
-    run(c, OV_KIND_LAYOUT, 1, [&] { fx_pack(bd, L.fr, L.fs, nullptr, L.nsrc, L.g.V, L.vs, c->st); });
-  } else {
-    run(c, OV_KIND_LAYOUT, 2, [&] {
-      pack_spinors<R>(bd, L.r, L.nsrc, L.g.V, L.vs, c->st);
-      pack_spinors<R>(bd, L.s, L.nsrc, L.g.V, L.vs, c->st);
-    });
+    if (L.fx()) {
+      run(c, OV_KIND_LAYOUT, 1, [&] { fx_pack(bd, L.fr, L.fs, nullptr, L.nsrc, L.g.V, L.vs, c->st); });
+      return;
+    }
   }
+  run(c, OV_KIND_LAYOUT, 2, [&] {
+    pack_spinors<R>(bd, L.r, L.nsrc, L.g.V, L.vs, c->st);
+    pack_spinors<R>(bd, L.s, L.nsrc, L.g.V, L.vs, c->st);
+  });
 }
 
-// fm = 2 sets up block mode: fields of 2V sites (upper and lower halves); links: L.u (FP64
-// calls need it for the force and dH only)
+// What a call's Lat holds beside the scalars: links and p, q, r, s in R, or (FP64 calls) in
+// fixed point (fx.cuh), as the call's kernels read them.
+//   The operator: fixed-point links and input; marked sites and their neighbours in FP64.
+//   sgn(H) b and its gradient: the recurrence (and the reverse sweep) in fixed point.
+//   Theorem-1 calls: FP64.  The two halves of a block vector meet in one sum, whose
+//   fixed-point scale is the larger half's: dH along a small direction is lost in its rounding
+//   (dx to 1.5e-9 at a direction of 1e-8, to nothing at 1e-18).
+enum : int {
+  LAT_LINKS = 1,      // u
+  LAT_FIELDS = 2,     // p, q, r, s
+  LAT_FX_LINKS = 4,   // fu
+  LAT_FX_IN = 8,      // fr
+  LAT_FX_STEP = 16,   // fr, fs, fp, fq and the bases' exponents: the recurrence in fixed point
+  LAT_FX_BASES = 32,  // the bases' exponents
+  LAT_PLAIN = LAT_LINKS | LAT_FIELDS,
+  LAT_OPERATOR = LAT_FIELDS | LAT_FX_LINKS | LAT_FX_IN,
+  LAT_FX_SIGN = LAT_FX_LINKS | LAT_FX_STEP
+};
+// fm = 2 sets up block mode: fields of 2V sites (upper and lower halves).  parts: of FP64
+// calls (FP32 ones have LAT_PLAIN)
 template <typename R>
 Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, double m_w, int nsrc, int k,
-             bool basis, int fm = 1, int kcap = 0, bool links = true) {
+             bool basis, int fm = 1, int kcap = 0, int parts = LAT_PLAIN) {
   Lat<R> L{};
   L.g = make_geom(dims);
   L.gl = L.g;
@@ -348,14 +369,14 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   L.efinv = (R)std::exp(-mu);
   L.nsrc = nsrc;
   L.k = k;
-  constexpr bool fx = std::is_same<R, double>::value;   // FP64 calls run in fixed point (fx.cuh)
+  if (!std::is_same<R, double>::value) parts = LAT_PLAIN;
   L.vs = field_reals<R>(V);
-  if (links) {
+  if (parts & LAT_LINKS) {
     R* u = wsT<R>(c, B_LINKS, link_reals<R>() * V);
     L.u = u;
     run(c, OV_KIND_LAYOUT, 1, [&] { pack_links<R>(static_cast<const double*>(U), u, V, c->st); });
   }
-  if constexpr (fx) {
+  if (parts & LAT_FX_LINKS) {
     L.uaos = static_cast<const double*>(U);
     int4* fe = wsT<int4>(c, B_FXL, fx_link_ints(V));
     short* ex = wsT<short>(c, B_FXE, 5 * V);
@@ -375,22 +396,22 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   if (basis) {
     L.bv = wsT<R>(c, B_BV, (int64_t)nsrc * L.kcap * L.vs);
     L.bw = wsT<R>(c, B_BW, (int64_t)nsrc * L.kcap * L.vs);
-    if constexpr (fx) {
+    if (parts & (LAT_FX_STEP | LAT_FX_BASES)) {
       L.bve = wsT<short>(c, B_BVE, (int64_t)nsrc * L.kcap * (L.vs / 24));
       L.bwe = wsT<short>(c, B_BWE, (int64_t)nsrc * L.kcap * (L.vs / 24));
     }
   }
-  L.p = wsT<R>(c, B_P, nsrc * L.vs);
-  L.q = wsT<R>(c, B_Q, nsrc * L.vs);
-  L.r = wsT<R>(c, B_R, nsrc * L.vs);
-  L.s = wsT<R>(c, B_S, nsrc * L.vs);
-  if constexpr (fx) {
-    L.fr = fx_fields(c, B_FXR, B_FXRE, nsrc, L.vs);
-    if (basis) {
-      L.fs = fx_fields(c, B_FXS, B_FXSE, nsrc, L.vs);
-      L.fp = fx_fields(c, B_FXP, B_FXPE, nsrc, L.vs);
-      L.fq = fx_fields(c, B_FXQ, B_FXQE, nsrc, L.vs);
-    }
+  if (parts & LAT_FIELDS) {
+    L.p = wsT<R>(c, B_P, nsrc * L.vs);
+    L.q = wsT<R>(c, B_Q, nsrc * L.vs);
+    L.r = wsT<R>(c, B_R, nsrc * L.vs);
+    L.s = wsT<R>(c, B_S, nsrc * L.vs);
+  }
+  if (parts & (LAT_FX_IN | LAT_FX_STEP)) L.fr = fx_fields(c, B_FXR, B_FXRE, nsrc, L.vs);
+  if (parts & LAT_FX_STEP) {
+    L.fs = fx_fields(c, B_FXS, B_FXSE, nsrc, L.vs);
+    L.fp = fx_fields(c, B_FXP, B_FXPE, nsrc, L.vs);
+    L.fq = fx_fields(c, B_FXQ, B_FXQE, nsrc, L.vs);
   }
   L.sc = wsT<SrcScal>(c, B_SC, nsrc);
   L.alpha = wsT<zd>(c, B_ALPHA, (int64_t)nsrc * k);
@@ -471,14 +492,16 @@ void forward_krylov(ov_context* c, Lat<R>& L) {
         for (int ps = 0; ps < c->opt.passes; ++ps) {
           const bool last = ps == c->opt.passes - 1;
           if constexpr (std::is_same<R, double>::value) {
-            run(c, OV_KIND_PROJ_DOTS, 2, [&] { fx_proj_dots(L, 0, j + 1, 0, L.fr, L.fs, L.vs, coef, cpart, c->st); });
-            run(c, OV_KIND_PROJ_UPDATE, 1,
-                [&] { fx_proj_update(L, nullptr, j + 1, 0, L.fr, L.fs, L.vs, coef, j, last ? 1 : 0, c->st); });
-          } else {
-            run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 0, L.r, L.s, L.vs, coef, cpart, c->st); });
-            run(c, OV_KIND_PROJ_UPDATE, 1,
-                [&] { proj_update(L, j, 0, L.r, L.s, L.vs, coef, last, c->st); });
+            if (L.fx()) {
+              run(c, OV_KIND_PROJ_DOTS, 2, [&] { fx_proj_dots(L, 0, j + 1, 0, L.fr, L.fs, L.vs, coef, cpart, c->st); });
+              run(c, OV_KIND_PROJ_UPDATE, 1,
+                  [&] { fx_proj_update(L, nullptr, j + 1, 0, L.fr, L.fs, L.vs, coef, j, last ? 1 : 0, c->st); });
+              continue;
+            }
           }
+          run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 0, L.r, L.s, L.vs, coef, cpart, c->st); });
+          run(c, OV_KIND_PROJ_UPDATE, 1,
+              [&] { proj_update(L, j, 0, L.r, L.s, L.vs, coef, last, c->st, ps > 0); });
         }
       }
       inject_after_update(c, L, j);
@@ -504,13 +527,13 @@ int run_diagnostics(ov_context* c, const Lat<R>& L, bool segments, ov_tsl_info* 
     zd* cpart = wsT<zd>(c, B_CPART, (int64_t)nsrc * 2 * k * nsb);
     run(c, OV_KIND_PROJ_DOTS, 2, [&] {
       if constexpr (std::is_same<R, double>::value) {
-        const FxField v{reinterpret_cast<int4*>(L.basis_v(0, k - 1)), L.bve + (int64_t)(k - 1) * (L.vs / 24)};
-        const FxField w{reinterpret_cast<int4*>(L.basis_w(0, k - 1)), L.bwe + (int64_t)(k - 1) * (L.vs / 24)};
-        fx_proj_dots(L, 0, k, 0, v, w, (int64_t)L.kcap * L.vs, coef, cpart, c->st);
-      } else {
-        proj_dots(L, k - 1, 0, L.basis_v(0, k - 1), L.basis_w(0, k - 1), (int64_t)L.kcap * L.vs, coef, cpart,
-                  c->st);
+        if (L.fx()) {
+          const FxField v{reinterpret_cast<int4*>(L.basis_v(0, k - 1)), L.bve + (int64_t)(k - 1) * (L.vs / 24)};
+          const FxField w{reinterpret_cast<int4*>(L.basis_w(0, k - 1)), L.bwe + (int64_t)(k - 1) * (L.vs / 24)};
+          return fx_proj_dots(L, 0, k, 0, v, w, (int64_t)L.kcap * L.vs, coef, cpart, c->st);
+        }
       }
+      proj_dots(L, k - 1, 0, L.basis_v(0, k - 1), L.basis_w(0, k - 1), (int64_t)L.kcap * L.vs, coef, cpart, c->st);
     });
     launch_check();
     std::vector<zd> h((size_t)nsrc * 2 * k);
@@ -593,14 +616,14 @@ template <typename R>
 struct SegStore {
   R *r, *s, *v, *w;           // [segment][src][vs]
   SrcScal* sc;                // [segment][src]
-  short *re, *se, *ve, *we;   // FP64 calls: the exponents of the above
+  short *re, *se, *ve, *we;   // fixed-point recurrence: the exponents of the above
 };
 template <typename R>
 SegStore<R> seg_store(ov_context* c, const Lat<R>& L, int nseg) {
   const int64_t n = (int64_t)nseg * L.nsrc * L.vs;
   SegStore<R> K{wsT<R>(c, B_CKR, n), wsT<R>(c, B_CKS, n), wsT<R>(c, B_CKV, n), wsT<R>(c, B_CKW, n),
                 wsT<SrcScal>(c, B_CKSC, (int64_t)nseg * L.nsrc), nullptr, nullptr, nullptr, nullptr};
-  if constexpr (std::is_same<R, double>::value) {
+  if (L.fx()) {
     K.re = wsT<short>(c, B_CKRE, n / 24);
     K.se = wsT<short>(c, B_CKSE, n / 24);
     K.ve = wsT<short>(c, B_CKVE, n / 24);
@@ -615,7 +638,7 @@ void seg_rs(ov_context* c, const Lat<R>& L, const SegStore<R>& K, size_t t, bool
   auto copy = [&](void* live, void* kept, size_t bytes) {
     CK(cudaMemcpyAsync(restore ? live : kept, restore ? kept : live, bytes, cudaMemcpyDeviceToDevice, c->st));
   };
-  if constexpr (std::is_same<R, double>::value) {
+  if (L.fx()) {
     copy(L.fr.c, K.r + t * fs, sizeof(R) * fs);
     copy(L.fs.c, K.s + t * fs, sizeof(R) * fs);
     copy(L.fr.e, K.re + t * (fs / 24), sizeof(short) * (fs / 24));
@@ -637,7 +660,7 @@ void window_slot(ov_context* c, const Lat<R>& L, int slot, const SegStore<R>& K,
   };
   copy(L.bv, K.v + t * fs, sizeof(R));
   copy(L.bw, K.w + t * fs, sizeof(R));
-  if constexpr (std::is_same<R, double>::value) {
+  if (L.fx()) {
     copy(L.bve, K.ve + t * (fs / 24), sizeof(short));
     copy(L.bwe, K.we + t * (fs / 24), sizeof(short));
   }
@@ -1019,7 +1042,7 @@ int tsl_sign_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   check_ptr(x);
   const int S = c->opt.segment > 0 && c->opt.segment < k ? c->opt.segment : 0;
   Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0,
-                      !std::is_same<R, double>::value);
+                      LAT_FX_SIGN);
   pack_start(c, L, b);
   SegPlan P;
   SegStore<R> K{};
@@ -1040,6 +1063,7 @@ int tsl_sign_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   c->last_block = 0;
   c->last_seg = S > 0 ? 1 : 0;
   c->last_prec = c->opt.precision;
+  c->last_fx = L.fx();
   std::copy(dims, dims + 4, c->last_dims);
   if (info) info->k_reached = kr;
   if (st != OV_OK) return st;
@@ -1089,30 +1113,18 @@ int block_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, d
   if (top) check_ptr(top);
   if (E) check_ptr(E);
   if (!std::isfinite(m_dir) || c->opt.segment > 0) throw Status{OV_ERR_INVALID_ARG};
-  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 2, 0, !std::is_same<R, double>::value);
+  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 2);
   const int64_t V = L.gl.V, Vf = L.g.V;
-  if (E && !std::is_same<R, double>::value) {
+  if (E) {
     R* ue = wsT<R>(c, B_ELINKS, link_reals<R>() * V);
     run(c, OV_KIND_LAYOUT, 1, [&] { pack_links<R>(static_cast<const double*>(E), ue, V, c->st); });
     L.ue = ue;
   }
   L.mdir = (R)m_dir;
-  if constexpr (std::is_same<R, double>::value) {
-    int4* fe = wsT<int4>(c, B_FXDL, fx_link_ints(V));
-    short* ex = wsT<short>(c, B_FXDE, 5 * V);
-    L.fd = FxLinks{fe, ex};
-    run(c, OV_KIND_LAYOUT, 2, [&] {
-      pack_dh_links_fx(static_cast<const double*>(U), static_cast<const double*>(E), m_dir, fe, ex, V, L.ef, L.efinv,
-                       c->st);
-      fx_pack_block(static_cast<const double*>(top), static_cast<const double*>(bottom), L.fr, L.fs, nsrc, V, L.vs,
-                    c->st);
-    });
-  } else {
-    run(c, OV_KIND_LAYOUT, 1, [&] {
-      pack_block_start<R>(static_cast<const double*>(top), static_cast<const double*>(bottom), L.r, L.s, nsrc, V,
-                          L.vs, c->st);
-    });
-  }
+  run(c, OV_KIND_LAYOUT, 1, [&] {
+    pack_block_start<R>(static_cast<const double*>(top), static_cast<const double*>(bottom), L.r, L.s, nsrc, V,
+                        L.vs, c->st);
+  });
   CK(cudaEventRecord(c->ev[0], c->st));
   forward_krylov(c, L);
   CK(cudaEventRecord(c->ev[1], c->st));
@@ -1124,6 +1136,7 @@ int block_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, d
   c->last_block = 1;
   c->last_seg = 0;
   c->last_prec = c->opt.precision;
+  c->last_fx = L.fx();
   std::copy(dims, dims + 4, c->last_dims);
   if (info) info->k_reached = kr;
   if (st != OV_OK) return st;
@@ -1178,7 +1191,8 @@ int ritz_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, do
               double tol, int32_t* l_out, double* lam, void* Rv, void* Lv, double* resid) {
   check_ptr(Rv);
   check_ptr(Lv);
-  Lat<R> L = setup<R>(c, dims, U, mu, m_w, c->last_nsrc, k, true);
+  Lat<R> L = setup<R>(c, dims, U, mu, m_w, c->last_nsrc, k, true, 1, 0,
+                      LAT_OPERATOR | (c->last_fx ? LAT_FX_BASES : 0));
   const int64_t V = L.g.V, n = 12 * V, fd = 24 * V;
   std::vector<double> al(2 * k), be(2 * k), de(k), th(2 * k);
   CK(cudaMemcpyAsync(al.data(), L.alpha + (int64_t)src * k, sizeof(zd) * k, cudaMemcpyDeviceToHost, c->st));
@@ -1421,7 +1435,7 @@ int vjp_forward(ov_context* c, const int32_t dims[4], const void* U, double mu, 
   F.S = S;
   F.k = k;
   F.nsrc = nsrc;
-  F.L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0);
+  F.L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0, LAT_FX_SIGN | LAT_LINKS);
   Lat<R>& L = F.L;
   const int64_t V = L.g.V, vs = L.vs;
   pack_start(c, L, b);
@@ -1442,6 +1456,7 @@ int vjp_forward(ov_context* c, const int32_t dims[4], const void* U, double mu, 
   c->last_block = 0;
   c->last_seg = S > 0 ? 1 : 0;
   c->last_prec = c->opt.precision;
+  c->last_fx = L.fx();
   std::copy(dims, dims + 4, c->last_dims);
   if (info) info->k_reached = kr;
   if (st != OV_OK) return st;
@@ -1791,7 +1806,7 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
           R* grs = B.gr_ring + (int64_t)slot * nsrc * vs;
           R* gss = B.gs_ring + (int64_t)slot * nsrc * vs;
           run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 1, grs, gss, vs, coef, cpart, c->st); });
-          run(c, OV_KIND_PROJ_UPDATE, 1, [&] { proj_update(L, j, 1, grs, gss, vs, coef, false, c->st); });
+          run(c, OV_KIND_PROJ_UPDATE, 1, [&] { proj_update(L, j, 1, grs, gss, vs, coef, false, c->st, ps > 0); });
         }
         run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_proj_record(L, B, j, nrec, coef, c->st); });
       }
@@ -2082,7 +2097,7 @@ int eigderiv_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   check_ptr(dLf);
   if (E) check_ptr(E);
   if (!(tol > 0.0) || maxit < 1 || !std::isfinite(m_dir)) throw Status{OV_ERR_INVALID_ARG};
-  Lat<double> L1 = setup<double>(c, dims, U, mu, m_w, 1, 2, false);
+  Lat<double> L1 = setup<double>(c, dims, U, mu, m_w, 1, 2, false, 1, 0, LAT_OPERATOR | LAT_LINKS);
   const int64_t V = L1.g.V, n = 12 * V, fd = 24 * V;
   if (E) {
     double* ue = wsT<double>(c, B_ELINKS, link_reals<double>() * V);
@@ -2181,7 +2196,7 @@ int eigsmall_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   check_ptr(Rf);
   check_ptr(Lf);
   if (!(tol > 0.0) || maxit < 1 || m < l || m > 1024) throw Status{OV_ERR_INVALID_ARG};
-  Lat<double> L1 = setup<double>(c, dims, U, mu, m_w, 1, 2, false);
+  Lat<double> L1 = setup<double>(c, dims, U, mu, m_w, 1, 2, false, 1, 0, LAT_OPERATOR);
   const int64_t V = L1.g.V, n = 12 * V, fd = 24 * V;
   double* Q = wsT<double>(c, B_SIQ, (int64_t)(m + 1) * fd);
   double* lt = wsT<double>(c, B_SILT, (int64_t)l * fd);
@@ -2400,7 +2415,7 @@ int apply_h_impl(ov_context* c, const int32_t dims[4], const void* U, double mu,
   check_ptr(in);
   check_ptr(out);
   constexpr bool fx = std::is_same<R, double>::value;
-  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, 1, false, 1, 0, !fx);
+  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, 1, false, 1, 0, LAT_OPERATOR);
   // (the FP32 staged variants alone have a wait that can run out)
   int* aerr = fx ? nullptr : wsT<int>(c, B_AERR, 1, true);
   const int var = c->tuned_apply[c->opt.precision];
@@ -2436,13 +2451,12 @@ int apply_h_impl(ov_context* c, const int32_t dims[4], const void* U, double mu,
 template <typename R>
 int autotune_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, double m_w, int nsrc,
                   ov_tune_report* rep) {
-  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, 2, true);
+  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, 2, true, 1, 0, LAT_PLAIN | LAT_OPERATOR);
   CK(cudaMemsetAsync(L.r, 0, sizeof(R) * nsrc * L.vs, c->st));
   CK(cudaMemsetAsync(L.s, 0, sizeof(R) * nsrc * L.vs, c->st));
   CK(cudaMemsetAsync(L.sc, 0, sizeof(SrcScal) * nsrc, c->st));
   if constexpr (std::is_same<R, double>::value) {
     fx_encode(L.r, L.fr, nsrc, L.g.V, L.vs, c->st);
-    fx_encode(L.s, L.fs, nsrc, L.g.V, L.vs, c->st);
   }
   cudaEvent_t e0 = c->ev[6], e1 = c->ev[7];
   auto time_us = [&](auto&& launch) {
