@@ -196,14 +196,6 @@ __device__ __forceinline__ int fx_top(FxZ a) {
   const int x = (int)(a.re >> 32), y = (int)(a.im >> 32);
   return (x ^ (x >> 31)) | (y ^ (y >> 31));
 }
-// Room for 16 more terms (each below 2^57 units): a sum that may pass 2^60 is shifted down
-// by two bits (rounded), which leaves it below 2^60.6.
-__device__ __forceinline__ void fx_headroom(FxHalf& a) {
-  int m = 0;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) m |= fx_top(a.v[i]);
-  if (m >= (1 << 28)) fx_shift(a, 2);
-}
 // Encode the sum: 57 bits below its largest component (of the site's two threads: every lane
 // of the warp).  bad marks the site; a site below 2^(zero_top - FX_E_BIAS) becomes zero.
 __device__ __forceinline__ void fx_encode(const FxHalf& a, bool bad, FxH& o, int zero_top = 0) {
@@ -506,7 +498,7 @@ __device__ __forceinline__ void fx_swap_lower(FxHalf& a) {
 }
 // acc += the hops of D_w of field f (sites off + s) in directions nu0 .. nu1 - 1 (all eight by
 // default), at acc's scale; every lane of the warp.  A product is below 2^57 units, so the 48
-// of eight hops stay below 2^62.6 (for sixteen hops the caller takes E one higher).  The loop
+// of eight hops stay below 2^62.6.  The loop
 // is kept rolled: fully unrolled, the code outgrows the instruction cache and instruction fetch sets the pace (144 us per
 // step pair at 14^4).  Copies in flight and the data read belong to one warp.
 __device__ __forceinline__ void fx_hops(FxHalf& acc, const FxField& f, int off, const FxLinks& U, const Geom& g,
@@ -643,7 +635,7 @@ struct FxStream {
 
 // ---------------------------------------------------------------------------
 // block sums: one warp per value adds the values of the nw warps that have it (the block's
-// first, or for values 1, 3, .. those from warp `odd` on) and writes the block's partial.  An
+// first) and writes the block's partial.  An
 // FP64 addition of a warp, whatever it adds, occupies the SM's FP64 pipe for 19 cycles.
 // Blocks of up to 256 threads
 // ---------------------------------------------------------------------------
@@ -652,14 +644,13 @@ struct FxSumBuf {
   zd v[NV][NT];
 };
 template <int NV, int NT>
-__device__ __forceinline__ void fx_block_partials(const zd (&v)[NV], FxSumBuf<NV, NT>& buf, zd* part, int nw,
-                                                  int odd = 0) {
+__device__ __forceinline__ void fx_block_partials(const zd (&v)[NV], FxSumBuf<NV, NT>& buf, zd* part, int nw) {
 #pragma unroll
   for (int i = 0; i < NV; ++i) buf.v[i][threadIdx.x] = v[i];
   __syncthreads();
   const int lane = threadIdx.x & 31;
   for (int i = threadIdx.x >> 5; i < NV; i += blockDim.x >> 5) {
-    const zd* q = &buf.v[i][(i & 1 ? odd * 32 : 0) + lane];
+    const zd* q = &buf.v[i][lane];
     zd s = q[0];
     for (int t = 1; t < nw; ++t) s = s + q[32 * t];
     s = warp_sum(s);

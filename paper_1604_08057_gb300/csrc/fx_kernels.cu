@@ -1,11 +1,11 @@
-// FP64 calls in block fixed point (fx.cuh): layout conversion, ov_apply_H, the forward
-// two-sided Lanczos recurrence with its Gram-Schmidt projections, and the reverse sweep
-// with the gauge force.  Every kernel reads and writes fixed-point fields; FP64 is left
-// for the recurrence's scalars and for what goes back to the caller.
+// FP64 calls in block fixed point (fx.cuh): layout conversion, ov_apply_H, and the two-sided
+// Lanczos recurrence with its Gram-Schmidt projections where x alone is wanted (see LAT_* in
+// ov_api.cu).  Every kernel reads and writes fixed-point fields; FP64 is left for the
+// recurrence's scalars and for what goes back to the caller.
 //
 // Two threads (spins sp and 2 + sp) share a site unless a kernel says otherwise; blocks
-// whose two halves treat the two sides of the recurrence (r and s, g_r and g_s) exchange
-// through shared memory.  All reductions are deterministic.
+// whose two halves treat the two sides of the recurrence (r and s) exchange through shared
+// memory.  All reductions are deterministic.
 #include <algorithm>
 #include <atomic>
 
@@ -31,7 +31,6 @@ static inline unsigned one_wave(const Lat<double>& L, int sites) {
 // In the Lanczos step the split sums are the unsplit ones bit for bit, so its rule may count
 // the sources (8^4 with four sources: 23 ms of stencils with the split, 12
 // without); the sums over terms of the other two are not.
-static inline bool fx_split(const Lat<double>& L) { return L.g.V < 152 * 32; }
 static inline bool fx_split_exact(const Lat<double>& L) { return L.g.V < 152 * 32 && L.g.V * L.nsrc < 152 * 64; }
 
 // a launch with dynamic shared memory, whose limit is raised once per kernel and device
@@ -512,7 +511,7 @@ void fx_tsl_update(const Lat<double>& L, int j, int finalize, cudaStream_t st) {
 }
 
 // ---------------------------------------------------------------------------
-// Gram-Schmidt projections (see k_proj_dots for the modes and coefficient layout)
+// Gram-Schmidt projections
 // ---------------------------------------------------------------------------
 // conj(b) a over all twelve components of a site: |hh| < 24 2^54, |x| < 48 2^56
 struct FxS {
@@ -526,21 +525,20 @@ __device__ __forceinline__ void fx_load_site(const FxField& f, int64_t s, FxS& o
   o.e = f.e[s];
 }
 constexpr int FX_NB = 8;   // basis vectors per block
-// One thread per site (spt sites in turn), one side per block: side 0 dots DA with a, side 1
-// DB with b.  a's integers stay in registers while FX_NB basis vectors stream past; each
+// One thread per site (spt sites in turn), one side per block: side 0 dots W with a, side 1
+// V with b.  a's integers stay in registers while FX_NB basis vectors stream past; each
 // thread's FP64 sums live in shared memory, so the loop over them stays rolled.  Bound by HBM:
 // 56 ms of dots per call at 14x14^3, k = 800 (148 in FP64, at 87% of its units' rate; the
 // basis vectors' bytes take 48.5).
-__global__ void __launch_bounds__(128, 3) k_fx_dots(const __grid_constant__ Lat<double> L, int nb, int mode, FxField a,
-                                                    FxField b, int64_t ab_stride, zd* __restrict__ cpart,
-                                                    int64_t cp_stride, int spt, int ioff, int sides) {
+__global__ void __launch_bounds__(128, 3) k_fx_dots(const __grid_constant__ Lat<double> L, int nb, FxField a, FxField b,
+                                                    int64_t ab_stride, zd* __restrict__ cpart, int64_t cp_stride,
+                                                    int spt) {
   __shared__ zd acc[FX_NB][128];
   __shared__ double red[4][2 * FX_NB];
-  const int src = blockIdx.z / sides, side = blockIdx.z % sides;
+  const int src = blockIdx.z >> 1, side = blockIdx.z & 1;
   const int i0 = blockIdx.y * FX_NB, n = min(FX_NB, nb - i0);
   const int64_t V = L.g.V;
   const FxField f = fx_src(side ? b : a, src, ab_stride);
-  const bool usew = (mode == 0) == (side == 0);
   for (int i = 0; i < n; ++i) acc[i][threadIdx.x] = mk(0.0, 0.0);
   for (int q = 0; q < spt; ++q) {
     const int64_t x = (blockIdx.x * (int64_t)spt + q) * 128 + threadIdx.x;
@@ -550,7 +548,7 @@ __global__ void __launch_bounds__(128, 3) k_fx_dots(const __grid_constant__ Lat<
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
       FxS w;
-      fx_load_site(usew ? fx_bw(L, src, ioff + i0 + i) : fx_bv(L, src, ioff + i0 + i), x, w);
+      fx_load_site(side ? fx_bv(L, src, i0 + i) : fx_bw(L, src, i0 + i), x, w);
       FxAcc t{0, 0, 0, 0};
 #pragma unroll
       for (int c = 0; c < 12; ++c) fx_cdot(t, w.q[c], u.q[c]);
@@ -581,61 +579,24 @@ __global__ void __launch_bounds__(128, 3) k_fx_dots(const __grid_constant__ Lat<
 }
 // one warp per coefficient: its site blocks' partials in lane-strided order, then a fixed tree
 __global__ void __launch_bounds__(128) k_fx_dots_reduce(const zd* __restrict__ cpart, int64_t cp_stride, int nsb, int nb,
-                                                        zd* __restrict__ coef, int64_t coef_stride, int sides) {
+                                                        zd* __restrict__ coef, int64_t coef_stride) {
   const int i = (blockIdx.x * 4 + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
   const int src = blockIdx.y;
-  if (i >= nb * sides) return;
-  const int t = sides == 2 ? i : 2 * i;
-  const zd* cp = cpart + src * cp_stride + (int64_t)t * nsb;
+  if (i >= 2 * nb) return;
+  const zd* cp = cpart + src * cp_stride + (int64_t)i * nsb;
   zd s = mk(0.0, 0.0);
   for (int b = lane; b < nsb; b += 32) s = s + cp[b];
   s = warp_sum(s);
-  if (lane == 0) coef[src * coef_stride + t] = s;
+  if (lane == 0) coef[src * coef_stride + i] = s;
 }
-void fx_proj_dots(const Lat<double>& L, int j0, int nb, int mode, const FxField& a, const FxField& b,
-                  int64_t ab_stride, zd* coef, zd* cpart, cudaStream_t st) {
-  // four sites per thread once a vector has enough sites for that to leave two blocks per
-  // SM to eight basis vectors (the block's reduction then costs a quarter per site)
-  const int spt = L.g.V >= 32768 ? 4 : 1, sides = b.c ? 2 : 1;
+void fx_proj_dots(const Lat<double>& L, int nb, const FxField& a, const FxField& b, int64_t ab_stride, zd* coef,
+                  zd* cpart, cudaStream_t st) {
+  // four sites per thread from V = 32768 on (the block's reduction then costs a quarter per site)
+  const int spt = L.g.V >= 32768 ? 4 : 1;
   const unsigned nsb = nblocks(L.g.V, 128 * spt);
   const int64_t cp_stride = (int64_t)2 * L.k * nsb;
-  k_fx_dots<<<dim3(nsb, nblocks(nb, FX_NB), L.nsrc * sides), 128, 0, st>>>(L, nb, mode, a, b, ab_stride, cpart,
-                                                                           cp_stride, spt, j0, sides);
-  k_fx_dots_reduce<<<dim3(nblocks(nb * sides, 4), L.nsrc), 128, 0, st>>>(cpart, cp_stride, nsb, nb, coef,
-                                                                         2 * (int64_t)L.k, sides);
-}
-
-// ---------------------------------------------------------------------------
-// reverse sweep (see the k_rev_* kernels of the FP32 form for the equations)
-// ---------------------------------------------------------------------------
-// one of a ring's slots, or a per-source field of the sweep
-__device__ __forceinline__ FxField ring_at(const Lat<double>& L, const FxField& f, int slot, int src) {
-  return fx_src(f, slot * L.nsrc + src, L.vs);
-}
-// D1 = v_j^dag g_r, D2 = w_j^dag g_s, D3 = v_{j-1}^dag g_r, D4 = w_{j-1}^dag g_s -> g_alpha and
-// the carries; g: this thread's g_r (left = 0) or g_s (left = 1)
-__device__ __forceinline__ void rev_alpha_site(const Lat<double>& L, int src, int j, int left, int64_t x, int sp,
-                                               const FxH& g, zd (&d)[2]) {
-  FxH e;
-  fx_load(left ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, e);
-  d[0] = d[0] + fx_dot(e, g);
-  if (j > 0) {
-    fx_load(left ? fx_bw(L, src, j - 1) : fx_bv(L, src, j - 1), x, sp, e);
-    d[1] = d[1] + fx_dot(e, g);
-  }
-}
-template <int NT>
-__device__ __forceinline__ void rev_alpha_finish(const Lat<double>& L, const Rev<double>& B, int src, int j, int left,
-                                                 const zd (&d)[2], int slot, FxSumBuf<4, NT>& sum, zd* scratch) {
-  const zd z = mk(0.0, 0.0);
-  const zd v[4] = {left ? z : d[0], left ? d[0] : z, left ? z : d[1], left ? d[1] : z};
-  zd* part = L.part + src * L.part_stride;
-  fx_block_partials(v, sum, part, blockDim.x >> 6, blockDim.x >> 6);
-  if (arrive_last(L.cnt + src * 16 + slot, gridDim.x)) {
-    zd s[4];
-    fx_sum_partials<4>(part, gridDim.x, s, scratch);
-    if (threadIdx.x == 0) alpha_epilogue(L, B, src, j, s);
-  }
+  k_fx_dots<<<dim3(nsb, nblocks(nb, FX_NB), 2 * L.nsrc), 128, 0, st>>>(L, nb, a, b, ab_stride, cpart, cp_stride, spt);
+  k_fx_dots_reduce<<<dim3(nblocks(2 * nb, 4), L.nsrc), 128, 0, st>>>(cpart, cp_stride, nsb, nb, coef, 2 * (int64_t)L.k);
 }
 
 // A long sum of coefficient times field, kept as (hh, x) pairs: per term only the products,
@@ -750,9 +711,8 @@ __device__ __forceinline__ void sum_vectors(FxTerms& T, FxStage& S, FxCoef (*cs)
   fx_copy_wait<0>();
 }
 
-// a -= sum_i coefA_i UA_i by the first half of a block's threads, b -= sum_i coefB_i UB_i by
-// the second, for the same SX sites.  fin 1: omega and the next scales (a = r, b = s); fin 2:
-// the four dots of the reverse step (a = g_r, b = g_s).
+// a -= sum_i coefA_i v_i by the first half of a block's threads, b -= sum_i coefB_i w_i by
+// the second, for the same SX sites.  fin: omega and the next scales (a = r, b = s).
 //
 // SPLIT: on a lattice with too few sites to fill the GPU four warps share a side's 16 sites,
 // a quarter of the vectors each (88 us per projection of 100 vectors at 4^4 without, 36 with).
@@ -760,16 +720,14 @@ __device__ __forceinline__ void sum_vectors(FxTerms& T, FxStage& S, FxCoef (*cs)
 // Bound by HBM: 58 ms per call at 14x14^3, k = 800 (146 in FP64; the bytes take 48.5).
 template <int SPLIT>
 __global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 1 : 3)
-    k_fx_proj_update(const __grid_constant__ Lat<double> L, const __grid_constant__ Rev<double> B, int nb, int mode,
-                     FxField a, FxField b, int64_t ab_stride, const zd* __restrict__ coef, int64_t coef_stride, int j,
-                     int fin) {
+    k_fx_proj_update(const __grid_constant__ Lat<double> L, int nb, FxField a, FxField b, int64_t ab_stride,
+                     const zd* __restrict__ coef, int64_t coef_stride, int j, int fin) {
   constexpr int NT = SPLIT ? 256 : 128;
   extern __shared__ __align__(16) unsigned char fx_smem[];
   FxStage* stage = reinterpret_cast<FxStage*>(fx_smem);
   FxSumBuf<2, NT>& sum2 = *reinterpret_cast<FxSumBuf<2, NT>*>(fx_smem);
-  FxSumBuf<4, NT>& sum4 = *reinterpret_cast<FxSumBuf<4, NT>*>(fx_smem);
   __shared__ FxCoef cs[2][2][FX_CH];
-  __shared__ zd scratch[4 * 32];
+  __shared__ zd scratch[2 * 32];
   const int half = blockDim.x >> 1, wid = threadIdx.x >> 5, nw = half >> 5;   // nw warps per side
   const int left = threadIdx.x >= half;
   const int w0 = left ? wid - nw : wid, th = left ? threadIdx.x - half : threadIdx.x;
@@ -779,10 +737,9 @@ __global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 1 : 3)
   FxStage& S = stage[wid];
   const bool first = !SPLIT || w0 == 0;
   const bool live = x0 < V && first;
-  const bool usev = (mode == 0) == (left == 0);
   FxTerms T;
   T.init();
-  const FxField u0 = usev ? fx_bv(L, src, L.jbase) : fx_bw(L, src, L.jbase);
+  const FxField u0 = left ? fx_bw(L, src, L.jbase) : fx_bv(L, src, L.jbase);
   sum_vectors(T, S, cs[left], coef + src * coef_stride + left, 2, nb, x, sp, th, half,
               [&](int i) { return fx_src(u0, i - L.jbase, L.vs); }, SPLIT ? w0 : 0, SPLIT ? 4 : 1);
   const FxField fa = fx_src(left ? b : a, src, ab_stride);
@@ -805,40 +762,34 @@ __global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 1 : 3)
       if (live) fx_put(fa, x, sp, f);
     }
   }
-  if (fin == 0) return;
+  if (!fin) return;
   __syncthreads();   // the stages are done with
-  if (fin == 1) {
-    zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
-    if (left && first) fx_row_put(S.row, f);
-    __syncthreads();
-    if (live) {
-      if (left) {
-        v[1] = mk(0.0, fx_norm2(f));
-      } else {
-        FxH s;
-        fx_row_get(stage[wid + nw].row, s);
-        v[0] = fx_dot(s, f);
-        v[1] = mk(fx_norm2(f), 0.0);
-      }
+  zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
+  if (left && first) fx_row_put(S.row, f);
+  __syncthreads();
+  if (live) {
+    if (left) {
+      v[1] = mk(0.0, fx_norm2(f));
+    } else {
+      FxH s;
+      fx_row_get(stage[wid + nw].row, s);
+      v[0] = fx_dot(s, f);
+      v[1] = mk(fx_norm2(f), 0.0);
     }
-    __syncthreads();
-    omega_finish(L, src, j, 3, v, sum2, scratch);
-    return;
   }
-  zd d[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
-  if (live) rev_alpha_site(L, src, j, left, x, sp, f, d);
-  rev_alpha_finish(L, B, src, j, left, d, 6, sum4, scratch);
+  __syncthreads();
+  omega_finish(L, src, j, 3, v, sum2, scratch);
 }
-void fx_proj_update(const Lat<double>& L, const Rev<double>* B, int nb, int mode, const FxField& a, const FxField& b,
-                    int64_t ab_stride, const zd* coef, int j, int fin, cudaStream_t st) {
-  const Rev<double> rev = B ? *B : Rev<double>{};
+void fx_proj_update(const Lat<double>& L, int nb, const FxField& a, const FxField& b, int64_t ab_stride, const zd* coef,
+                    int j, int fin, cudaStream_t st) {
+  const int64_t cs = 2 * (int64_t)L.k;
   if (L.g.V < 152 * 16) {   // fewer than two warps per SM without the split
-    fx_launch<k_fx_proj_update<1>>(dim3(nblocks(L.g.V, 16), L.nsrc), 256, 8 * sizeof(FxStage), st, L, rev, nb, mode, a, b,
-                                   ab_stride, coef, 2 * (int64_t)L.k, j, fin);
+    fx_launch<k_fx_proj_update<1>>(dim3(nblocks(L.g.V, 16), L.nsrc), 256, 8 * sizeof(FxStage), st, L, nb, a, b, ab_stride,
+                                   coef, cs, j, fin);
     return;
   }
-  fx_launch<k_fx_proj_update<0>>(dim3(nblocks(L.g.V, 32), L.nsrc), 128, 4 * sizeof(FxStage), st, L, rev, nb, mode, a, b,
-                                 ab_stride, coef, 2 * (int64_t)L.k, j, fin);
+  fx_launch<k_fx_proj_update<0>>(dim3(nblocks(L.g.V, 32), L.nsrc), 128, 4 * sizeof(FxStage), st, L, nb, a, b, ab_stride,
+                                 coef, cs, j, fin);
 }
 
 // out[src] (+)= sum_{j0 <= i < j0 + nvec} y_i u_i in the user's layout, u = V (side 0) or W;
@@ -876,427 +827,6 @@ void fx_combine(const Lat<double>& L, int src0, int nsrc, int side, int j0, int 
   const int bs = L.g.V < 152 * 64 ? 32 : 128;
   k_fx_combine<<<dim3(nblocks(L.g.V, bs / 2), nsrc), bs, 0, st>>>(L, src0, side, j0, nvec, y, ystride, out,
                                                                   accumulate);
-}
-
-// ---------------------------------------------------------------------------
-// reverse sweep, continued
-// ---------------------------------------------------------------------------
-// g_r = cr1 Gv + cr2 w_{j+1}, g_s = cs1 Gw + cs2 v_{j+1} into the ring slot (first and second
-// half of a block's threads), and with with_dots the four dots for g_alpha
-__global__ void __launch_bounds__(128, 4) k_fx_rev_form(const __grid_constant__ Lat<double> L,
-                                                        const __grid_constant__ Rev<double> B, int j, int slot,
-                                                        int with_dots) {
-  __shared__ FxSumBuf<4, 128> sum;
-  __shared__ zd scratch[4 * 32];
-  __shared__ FxCoef cs[2][2];
-  const int half = blockDim.x >> 1;
-  const int left = threadIdx.x >= half;
-  const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
-  const int64_t V = L.g.V, per = half >> 1;
-  const int src = blockIdx.y;
-  if (t < 2) {
-    const SrcScal& sc = L.sc[src];
-    cs[left][t] = fx_coef(left ? (t ? sc.cs2 : sc.cs1) : (t ? sc.cr2 : sc.cr1));
-  }
-  __syncthreads();
-  zd d[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
-  for (int64_t b = blockIdx.x; b * per < V; b += gridDim.x) {
-    const int64_t x0 = b * per + fx_site_of(t), x = min(x0, V - 1);
-    FxHalf acc;
-    FxH f;
-    fx_zero(acc, 0);
-    fx_load(fx_src(left ? B.fgw : B.fgv, src, L.vs), x, sp, f);
-    bool ok = fx_axpy(acc, cs[left][0], f);
-    fx_load(left ? fx_bv(L, src, j + 1) : fx_bw(L, src, j + 1), x, sp, f);
-    ok = fx_axpy(acc, cs[left][1], f) && ok;
-    fx_encode(acc, !ok, f);
-    if (x0 < V) {
-      fx_put(ring_at(L, left ? B.fgs : B.fgr, slot, src), x, sp, f);
-      if (with_dots) rev_alpha_site(L, src, j, left, x, sp, f, d);
-    }
-  }
-  if (with_dots) rev_alpha_finish(L, B, src, j, left, d, 5, sum, scratch);
-}
-void fx_rev_form(const Lat<double>& L, const Rev<double>& B, int j, int slot, int with_dots, cudaStream_t st) {
-  const int sx = two_sided_sites(L);
-  k_fx_rev_form<<<dim3(one_wave(L, sx), L.nsrc), 4 * sx, 0, st>>>(L, B, j, slot, with_dots);
-}
-
-// the two stencil inputs of step j: g_p = g_r + g_alpha w_j (first half), h_in = conj(g_alpha)
-// v_j + g_s (second half); g_r and g_s are absent at the last step
-__global__ void __launch_bounds__(128, 4) k_fx_rev_combine(const __grid_constant__ Lat<double> L,
-                                                           const __grid_constant__ Rev<double> B, int j, int slot) {
-  const int half = blockDim.x >> 1;
-  const int left = threadIdx.x >= half;
-  const int t = left ? threadIdx.x - half : threadIdx.x, sp = fx_spin_of(t);
-  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(half >> 1) + fx_site_of(t), x = min(x0, V - 1);
-  const int src = blockIdx.y;
-  const zd ga = L.sc[src].g_alpha;
-  FxHalf acc;
-  FxH f;
-  fx_zero(acc, 0);
-  fx_load(left ? fx_bv(L, src, j) : fx_bw(L, src, j), x, sp, f);
-  bool ok = fx_axpy(acc, fx_coef(left ? conj(ga) : ga), f);
-  if (j < L.k - 1) {
-    fx_load(ring_at(L, left ? B.fgs : B.fgr, slot, src), x, sp, f);
-    ok = fx_add(acc, f) && ok;
-  }
-  fx_encode(acc, !ok, f);
-  if (x0 < V) fx_put(left ? fx_src(B.fh, src, L.vs) : ring_at(L, B.fgp, slot, src), x, sp, f);
-}
-void fx_rev_combine(const Lat<double>& L, const Rev<double>& B, int j, int slot, cudaStream_t st) {
-  const int sx = two_sided_sites(L);
-  k_fx_rev_combine<<<dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, 0, st>>>(L, B, j, slot);
-}
-
-// Gradients of v_j and w_j:
-//   Gv_j = H^dag g_p  + sum_i c_i f_i,    Gw_j = H h_in + sum_i c'_i f'_i
-// with f over xbar, g_r, the previous g_r and w_{jm+1} of the recorded projections (g_s,
-// previous g_s and v_{jm+1} for Gw); first and second half of a block's threads.  The sum of
-// the terms, with coefficients c / kappa, joins the hop sum a:
-//   G = +-(p - kappa [a -+ sum_i (c_i / kappa) f_i])   (upper / lower spins).
-// Then, for j > 0, v_j^dag Gv_j and w_j^dag Gw_j give step j - 1 its coefficients.
-__device__ __forceinline__ FxField rev_term(const Lat<double>& L, const Rev<double>& B, int src, int side, int j,
-                                            int slot, int prev, int i, zd* c) {
-  const int64_t o = (int64_t)src * L.k + j;
-  if (side == 0) {
-    if (i == 0) {
-      *c = conj(B.y[o]);
-      return fx_src(B.fxb, src, L.vs);
-    }
-    --i;
-  }
-  if (j < L.k - 1) {
-    if (i == 0) {
-      *c = side ? -L.alpha[o] : -conj(L.alpha[o]);
-      return ring_at(L, side ? B.fgs : B.fgr, slot, src);
-    }
-    --i;
-  }
-  if (prev >= 0 && j + 1 < L.k - 1) {
-    if (i == 0) {
-      *c = side ? mk(-L.delta[o + 1], 0.0) : -conj(L.beta[o + 1]);
-      return ring_at(L, side ? B.fgs : B.fgr, prev, src);
-    }
-    --i;
-  }
-  const int jm = B.reb_steps[i];
-  const int64_t eo = src * (int64_t)B.nreb_max * L.k + (int64_t)i * L.k + j;
-  *c = side ? B.ew[eo] : B.ev[eo];
-  return side ? fx_bv(L, src, jm + 1) : fx_bw(L, src, jm + 1);
-}
-struct RevTerm {
-  FxField f;
-  FxCoef c;
-};
-// Bound by instruction issue (the terms' products and the two hop sums), then by HBM: 122 us on
-// average at 14x14^3, k = 800 (234 in FP64; the bytes take 37).
-constexpr int RT = 30;   // terms converted at a time per side (a multiple of FX_RING)
-template <int SPLIT>
-__global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 1 : 4)
-    k_fx_rev(const __grid_constant__ Lat<double> L, const __grid_constant__ Rev<double> B, int j, int slot, int prev,
-             int nrec) {
-  extern __shared__ __align__(16) unsigned char fx_smem[];
-  FxStage* stage = reinterpret_cast<FxStage*>(fx_smem);
-  __shared__ FxSumBuf<2, SPLIT ? 256 : 128> sum;
-  __shared__ RevTerm terms[2][RT];
-  __shared__ zd scratch[2 * 32];
-  const int half = blockDim.x >> 1, wid = threadIdx.x >> 5, nw = half >> 5;   // nw warps per side
-  const int side = threadIdx.x >= half ? 1 : 0;
-  const int w0 = side ? wid - nw : wid, th = side ? threadIdx.x - half : threadIdx.x;
-  const int t = SPLIT ? (threadIdx.x & 31) : th, sp = fx_spin_of(t);
-  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)(SPLIT ? 16 : half >> 1) + fx_site_of(t), x = min(x0, V - 1);
-  const int src = blockIdx.y;
-  FxStage& S = stage[wid];
-  const bool first = !SPLIT || w0 == 0;
-  const bool live = x0 < V && first;
-  const int base = (j < L.k - 1 ? 1 : 0) + (prev >= 0 && j + 1 < L.k - 1 ? 1 : 0) + nrec;
-  const int nt = base + (side ? 0 : 1), ntmax = base + 1;
-  // this warp's terms: all, or (SPLIT) every fourth
-  const int step = SPLIT ? 4 : 1, i1 = SPLIT ? w0 : 0;
-  FxHalf acc;
-  bool ok;
-  {
-    FxTerms T;
-    T.init();
-    for (int i0 = 0; i0 < ntmax; i0 += RT) {
-      __syncthreads();
-      for (int i = th; i < RT && i0 + i < nt; i += half) {
-        zd c;
-        terms[side][i].f = rev_term(L, B, src, side, j, slot, prev, i0 + i, &c);
-        terms[side][i].c = fx_coef(L.kinv * c);
-      }
-      __syncthreads();
-      const int n = (min(RT, nt - i0) - i1 + step - 1) / step;
-      const auto at = [&](int i) { return terms[side][i1 + i * step].f; };
-      FxStream q;
-      q.start(S, n, x, sp, at);
-#pragma unroll 1
-      for (int i = 0; i < n; i += FX_RING) {
-#pragma unroll
-        for (int u = 0; u < FX_RING; ++u) {
-          if (i + u < n) {
-            FxH f;
-            q.next(S, u, i + u, n, x, sp, at, f);
-            T.add(terms[side][i1 + (i + u) * step].c, f);
-          }
-        }
-      }
-      fx_copy_wait<0>();
-    }
-    T.value(acc);
-    ok = T.ok;
-  }
-#pragma unroll
-  for (int i = 0; i < 3; ++i) acc.v[i] = FxZ{-acc.v[i].re, -acc.v[i].im};
-  const FxField f = side ? fx_src(B.fh, src, L.vs) : ring_at(L, B.fgp, slot, src);
-  {
-    const FxSite s(L.g, x);
-    FxExps ex;
-    int E = fx_range(ex, f, 0, L.fu, L.g, s, side ? 0 : 1);
-    E = max(E, __shfl_xor_sync(0xffffffffu, acc.E, 16));   // one scale for the site's two threads
-    ok = ok && E < FX_BAD;
-    fx_raise(acc, E);
-    // below 2^60 units, so that the hops' 2^62.6 still fit
-    fx_headroom(acc);
-    acc.E = ok ? acc.E : FX_E_BIAS;
-    const int other = __shfl_xor_sync(0xffffffffu, acc.E, 16);
-    if (other > acc.E) fx_shift(acc, min(other - acc.E, 62));
-    acc.E = max(acc.E, other);
-    fx_hops(acc, f, 0, L.fu, L.g, s, ex, side ? 0 : 1, sp, S, SPLIT ? w0 : 0, SPLIT ? w0 + 1 : 4);
-  }
-  if (SPLIT) {
-    if (!ok) acc.E = FX_BAD;   // a marked site of any warp's terms marks the sum
-    fx_join_warps<false>(acc, stage + (side ? nw : 0), w0, nw);
-    ok = acc.E < FX_BAD;
-  }
-  FxH a, p;
-  if (first) {
-    fx_encode(acc, !ok, a);
-    fx_load(f, x, sp, p);
-    const bool okp = h_finish(acc, p, fx_coef(mk(-L.kappa, 0.0)), a);
-    fx_encode(acc, !okp, p);
-    if (live) fx_put(fx_src(side ? B.fgw : B.fgv, src, L.vs), x, sp, p);
-  }
-  if (j == 0) return;
-  zd v[2] = {mk(0.0, 0.0), mk(0.0, 0.0)};
-  if (live) {
-    fx_load(side ? fx_bw(L, src, j) : fx_bv(L, src, j), x, sp, a);
-    const zd d = fx_dot(a, p);
-    v[0] = side ? v[0] : d;
-    v[1] = side ? d : v[1];
-  }
-  zd* part = L.part + src * L.part_stride;
-  fx_block_partials(v, sum, part, SPLIT ? 1 : nw, nw);
-  if (arrive_last(L.cnt + src * 16 + 4, gridDim.x)) {
-    zd q[2];
-    fx_sum_partials<2>(part, gridDim.x, q, scratch);
-    if (threadIdx.x < 32) rev_dots_epilogue_warp(L, B, src, j - 1, q[0], q[1]);
-  }
-}
-void fx_rev_stencil(const Lat<double>& L, const Rev<double>& B, int j, int slot, int prev, int nrec,
-                    cudaStream_t st) {
-  if (fx_split(L)) {
-    fx_launch<k_fx_rev<1>>(dim3(nblocks(L.g.V, 16), L.nsrc), 256, 8 * sizeof(FxStage), st, L, B, j, slot, prev, nrec);
-    return;
-  }
-  const int sx = two_sided_sites(L);
-  fx_launch<k_fx_rev<0>>(dim3(nblocks(L.g.V, sx), L.nsrc), 4 * sx, (sx / 8) * sizeof(FxStage), st, L, B, j, slot, prev,
-                         nrec);
-}
-
-// ---------------------------------------------------------------------------
-// Force (see k_force): dU += sum over (source, term) items of the two rank-one terms
-// g_p v_j^dag and w_j g_s^dag, contracted per link on half spinors.  With A = P_-(X(x)),
-// B = P_+(Y(x + nu)):  G_cd += cf sum_s A_s,c conj(B_s,d), (X, Y) = (a, b) for the forward
-// hop and (b, a) for the backward one.  A block covers 16 sites; warp h is hop h of all of
-// them (two threads per site, one spin of the half spinors each), so the fields of a term
-// are read once for all four directions.  A is shifted to the sum's scale (and at least by
-// 2 bits), so a term adds at most 2^55 to hh and 2^58.6 to x: x is folded in after sixteen.
-// ---------------------------------------------------------------------------
-// the projected half spinor of staged components u (spin sp) and d (the lower spin it meets)
-template <int SGN>
-__device__ __forceinline__ void fx_project(const int4 (*q)[32], int nu, int sp, int4 (&h)[3]) {
-  const int l = threadIdx.x & 31;
-  const int t = SGN * (nu == 0 ? -1 : nu == 3 ? 1 : 2 * sp - 1);
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int4 u = q[a][l], w = q[3 + a][l];
-    h[a] = (nu & 1) ? make_int4(u.x + t * w.x, u.y + t * w.y, u.z + t * w.z, u.w + t * w.w)
-                    : make_int4(u.x - t * w.z, u.y - t * w.w, u.z + t * w.x, u.w + t * w.y);
-  }
-}
-struct FxOuter {
-  FxAcc g[9];
-  int E, n;
-  bool ok;
-  __device__ __forceinline__ void down(int sh) {
-    const fxll r = (1ll << sh) >> 1;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      g[i].hr = (g[i].hr + r) >> sh;
-      g[i].hi = (g[i].hi + r) >> sh;
-      g[i].xr = (g[i].xr + r) >> sh;
-      g[i].xi = (g[i].xi + r) >> sh;
-    }
-    E += sh;
-  }
-  __device__ __forceinline__ void fold() {
-    int m = 0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      g[i].hr += (g[i].xr + (1ll << 29)) >> 30;
-      g[i].hi += (g[i].xi + (1ll << 29)) >> 30;
-      g[i].xr = g[i].xi = 0;
-      m |= fx_top(FxZ{g[i].hr, g[i].hi});
-    }
-    n = 0;
-    if (m >= (1 << 28)) down(2);
-  }
-  // a = P_-(X(x)), b = P_+(Y(x + nu)) of exponents ea, eb
-  __device__ __forceinline__ void add(int4 (&a)[3], const int4 (&b)[3], int ea, int eb) {
-    if (ea == FX_BAD || eb == FX_BAD) {
-      ok = false;
-      return;
-    }
-    if (ea + eb > E) {
-      down(min(ea + eb - E, 62));
-      E = ea + eb;
-    }
-    const int d = E - (ea + eb) + 2;
-    if (d > 60) return;
-    const fxll half = 1ll << (d - 1);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      fxll re = fx_sar(fx_join(a[c].x, a[c].y) + half, min(d, 31)), im = fx_sar(fx_join(a[c].z, a[c].w) + half, min(d, 31));
-      if (d > 31) {
-        re >>= d - 31;
-        im >>= d - 31;
-      }
-      const FxInt p = fx_split(re), q = fx_split(im);
-      a[c] = make_int4(p.h, p.l, q.h, q.l);
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int e = 0; e < 3; ++e) fx_cdot(g[c * 3 + e], b[e], a[c]);
-    if (++n == 16) fold();
-  }
-};
-__global__ void __launch_bounds__(256, 2) k_fx_force(const __grid_constant__ Lat<double> L,
-                                                     const __grid_constant__ Rev<double> B, int nterms, int j0,
-                                                     int nsplit, double* parts) {
-  __shared__ double2 bwd[4][9][16];
-  __shared__ zd scratch[32];
-  const int hop = threadIdx.x >> 5, nu = hop >> 1, back = hop & 1, lane = threadIdx.x & 31, sp = lane >> 4;
-  const int64_t V = L.g.V, x0 = blockIdx.x * (int64_t)16 + (lane & 15), x = min(x0, V - 1);
-  const bool live = x0 < V;
-  const int split = blockIdx.y, nitems = L.nsrc * nterms;
-  const int i0 = (int)((int64_t)split * nitems / nsplit), i1 = (int)((int64_t)(split + 1) * nitems / nsplit);
-  const int64_t xf = FxSite(L.g, x).neighbour(L.g, 2 * nu);
-  FxOuter G;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) G.g[i] = FxAcc{0, 0, 0, 0};
-  G.E = 0;
-  G.n = 0;
-  G.ok = true;
-  // the fields of the next product are copied to shared memory while one is formed
-  extern __shared__ __align__(16) unsigned char fx_smem[];
-  int4 (*st)[12][32] = reinterpret_cast<int4 (*)[12][32]>(fx_smem) + hop * 2;
-  int ea[2], eb[2];
-  auto issue = [&](int i, int slot) {
-    if (i < 2 * i1) {
-      const int src = (i >> 1) / nterms, t = (i >> 1) - src * nterms, j = j0 - t;
-      const bool second = i & 1;
-      if (!(second && j == L.k - 1)) {
-        const FxField a = second ? fx_bw(L, src, j) : ring_at(L, B.fgp, t, src);
-        const FxField b = second ? ring_at(L, B.fgs, t, src) : fx_bv(L, src, j);
-        const FxField X = back ? b : a, Y = back ? a : b;
-        const int pd = (nu < 2 ? 3 - sp : 2 + sp) * 96;
-        const int4* qx = X.c + fx_at(x);
-        const int4* qy = Y.c + fx_at(xf);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          fx_copy16(&st[slot][c][lane], qx + sp * 96 + c * 32);
-          fx_copy16(&st[slot][3 + c][lane], qx + pd + c * 32);
-          fx_copy16(&st[slot][6 + c][lane], qy + sp * 96 + c * 32);
-          fx_copy16(&st[slot][9 + c][lane], qy + pd + c * 32);
-        }
-        ea[slot] = X.e[x];
-        eb[slot] = Y.e[xf];
-      }
-    }
-    fx_copy_commit();
-  };
-  issue(2 * i0, 0);
-#pragma unroll 1
-  for (int i = 2 * i0; i < 2 * i1; i += 2) {
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      issue(i + s + 1, s ^ 1);
-      fx_copy_wait<1>();
-      // the second product is absent at the recurrence's last step
-      if (s == 1 && j0 - ((i >> 1) % nterms) == L.k - 1) continue;
-      int4 a[3], b[3];
-      fx_project<-1>(&st[s][0], nu, sp, a);
-      fx_project<1>(&st[s][6], nu, sp, b);
-      G.add(a, b, ea[s], eb[s]);
-    }
-  }
-  fx_copy_wait<0>();
-  G.fold();
-  // kappa f with the sign of the hop term; a product's unit is 2^(E + 2 - 2098)
-  const double f = nu < 3 ? 1.0 : back ? L.efinv : L.ef;
-  const double u = G.ok ? -L.kappa * f * fx_pow2_wide(G.E - 2096) : fx_nan();
-  zd o[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    o[i] = mk(u * (double)G.g[i].hr, u * (double)G.g[i].hi);
-    o[i].re += __shfl_xor_sync(0xffffffffu, o[i].re, 16);
-    o[i].im += __shfl_xor_sync(0xffffffffu, o[i].im, 16);
-    if (back && sp == 0) bwd[nu][i][lane] = make_double2(o[i].re, o[i].im);
-  }
-  __syncthreads();
-  zd v[1] = {mk(0.0, 0.0)};
-  if (!back && sp == 0 && live) {
-    double2* dst = reinterpret_cast<double2*>(nsplit > 1 ? parts + (int64_t)split * 72 * V : B.force);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const double2 w = bwd[nu][i][lane];
-      double2* p = dst + (int64_t)(nu * 9 + i) * V + x;
-      double2 s = make_double2(o[i].re + w.x, o[i].im + w.y);
-      if (nsplit == 1) {
-        const double2 old = *p;
-        s.x += old.x;
-        s.y += old.y;
-      }
-      *p = s;
-      if (nu == 3) {   // dmu: Re(conj(G_fwd - G_bwd) U_t)
-        const zd ul = load_link_entry(L.u, V, x, 27 + i);
-        v[0].re += (o[i].re - w.x) * ul.re + (o[i].im - w.y) * ul.im;
-      }
-    }
-  }
-  block_sum<1>(v, scratch);
-  if (threadIdx.x == 0) B.dmu_part[split * gridDim.x + blockIdx.x] = v[0];
-  if (arrive_last(B.dmu_cnt, gridDim.x * gridDim.y)) {
-    zd s[1];
-    sum_partials<1>(B.dmu_part, gridDim.x * gridDim.y, s, scratch);
-    if (threadIdx.x == 0) *B.dmu += s[0].re;
-  }
-}
-int fx_force_splits(int64_t V) {
-  const int64_t blocks = (V + 15) / 16;
-  if (blocks >= 2 * 152) return 1;
-  const int64_t want = (2 * 152 + blocks - 1) / blocks;
-  return (int)(want < kForceSplitMax ? want : kForceSplitMax);
-}
-int fx_force_flush(const Lat<double>& L, const Rev<double>& B, int nterms, int j0, cudaStream_t st) {
-  int nsplit = B.force_parts ? fx_force_splits(L.g.V) : 1;
-  if (nsplit > L.nsrc * nterms) nsplit = L.nsrc * nterms;
-  fx_launch<k_fx_force>(dim3(nblocks(L.g.V, 16), nsplit), 256, 8 * 2 * 12 * 32 * sizeof(int4), st, L, B, nterms, j0,
-                        nsplit, B.force_parts);
-  return nsplit;
 }
 
 }  // namespace ov

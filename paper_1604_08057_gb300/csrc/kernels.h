@@ -44,7 +44,6 @@ template <typename R>
 struct Lat {
   Geom g;
   R kappa, ef, efinv;        // kappa, e^{mu}, e^{-mu}
-  R kinv;                    // 1 / kappa = 2 m_w + 8
   const R* u;                // internal links (link_reals<R>() * V reals)
   int nsrc, k;
   int64_t vs;                // reals per lattice vector (padded)
@@ -85,7 +84,6 @@ struct Rev {
   R* gv_new; R* gw_new;      // gradients being formed for v_j, w_j
   R* gr_ring; R* gs_ring; R* gp_ring;   // [m][src][vs]
   R* hin;                    // conj(g_alpha) v_j + g_s of the current step: [src][vs]
-  FxField fgv, fgw, fgr, fgs, fgp, fh, fxb;   // FP64 calls: the above (and xbar) in fixed point
   int m;                     // ring length
   const R* xbar;             // [src][vs]
   const zd* y;               // [src][k]
@@ -143,20 +141,14 @@ void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double
 void fx_tsl_init(const Lat<double>& L, cudaStream_t st);
 void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st);
 void fx_tsl_update(const Lat<double>& L, int j, int finalize, cudaStream_t st);
-// dots with vectors j0 .. j0 + nb - 1 (modes as proj_dots; b.c null: side A alone)
-void fx_proj_dots(const Lat<double>& L, int j0, int nb, int mode, const FxField& a, const FxField& b,
-                  int64_t ab_stride, zd* coef, zd* cpart, cudaStream_t st);
-// fin 1: omega and the next scales follow; 2: g_alpha and the carries of reverse step j
-void fx_proj_update(const Lat<double>& L, const Rev<double>* B, int nb, int mode, const FxField& a, const FxField& b,
-                    int64_t ab_stride, const zd* coef, int j, int fin, cudaStream_t st);
+// dots with vectors 0 .. nb - 1: out[2 i] = w_i^dag a, out[2 i + 1] = v_i^dag b
+void fx_proj_dots(const Lat<double>& L, int nb, const FxField& a, const FxField& b, int64_t ab_stride, zd* coef,
+                  zd* cpart, cudaStream_t st);
+// fin: omega and the next scales follow
+void fx_proj_update(const Lat<double>& L, int nb, const FxField& a, const FxField& b, int64_t ab_stride, const zd* coef,
+                    int j, int fin, cudaStream_t st);
 void fx_combine(const Lat<double>& L, int src0, int nsrc, int side, int j0, int nvec, const zd* y, int64_t ystride,
                 double* out, int accumulate, cudaStream_t st);
-void fx_rev_form(const Lat<double>& L, const Rev<double>& B, int j, int slot, int with_dots, cudaStream_t st);
-void fx_rev_combine(const Lat<double>& L, const Rev<double>& B, int j, int slot, cudaStream_t st);
-void fx_rev_stencil(const Lat<double>& L, const Rev<double>& B, int j, int slot, int prev_slot, int nrec,
-                    cudaStream_t st);
-int fx_force_splits(int64_t V);
-int fx_force_flush(const Lat<double>& L, const Rev<double>& B, int nterms, int j0, cudaStream_t st);
 
 template <typename R> void tsl_init(const Lat<R>& L, cudaStream_t st);
 template <typename R> void tsl_stencil(const Lat<R>& L, int j, bool need_q, cudaStream_t st, int variant = 0);

@@ -1369,12 +1369,8 @@ __global__ void __launch_bounds__(BS) k_rev_form(Lat<R> L, Rev<R> B, int j, int 
 }
 template <typename R>
 void rev_form(const Lat<R>& L, const Rev<R>& B, int j, int slot, bool with_dots, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value) {
-    fx_rev_form(L, B, j, slot, with_dots ? 1 : 0, st);
-  } else {
-    k_rev_form<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot,
-                                                                                     with_dots ? 1 : 0);
-  }
+  k_rev_form<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot,
+                                                                                   with_dots ? 1 : 0);
 }
 
 // the four dots after the projection adjoint has been applied to g_r, g_s
@@ -1477,11 +1473,7 @@ __global__ void __launch_bounds__(BS) k_rev_combine(Lat<R> L, Rev<R> B, int j, i
 }
 template <typename R>
 void rev_combine(const Lat<R>& L, const Rev<R>& B, int j, int slot, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value) {
-    fx_rev_combine(L, B, j, slot, st);
-  } else {
-    k_rev_combine<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot);
-  }
+  k_rev_combine<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot);
 }
 
 // R3b: complete gradients of v_j and w_j
@@ -1540,11 +1532,8 @@ __global__ void __launch_bounds__(BS) k_rev_stencil(Lat<R> L, Rev<R> B, int j, i
 }
 template <typename R>
 void rev_stencil(const Lat<R>& L, const Rev<R>& B, int j, int slot, int prev_slot, int nrec, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value)
-    fx_rev_stencil(L, B, j, slot, prev_slot, nrec, st);
-  else
-    k_rev_stencil<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot,
-                                                                                        prev_slot, nrec);
+  k_rev_stencil<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j, slot,
+                                                                                      prev_slot, nrec);
 }
 
 // ---------------------------------------------------------------------------
@@ -1583,19 +1572,28 @@ __device__ void force_dir(const Lat<R>& L, const Rev<R>& B, int64_t x, int nterm
   for (int e = 0; e < 9; ++e) acc[e] = accd[e] = mk(0.0, 0.0);
   for (int src = i0 / nterms; src * nterms < i1; ++src) {
     const int t0 = max(i0 - src * nterms, 0), t1 = min(i1 - src * nterms, nterms);
-    // FP32 partial sums over one ring of terms, then FP64
-    cplx<R> G[9], Gd[9];
+    if constexpr (sizeof(R) == 8) {
+      // FP64 fields: accumulate straight into the FP64 sums
+      for (int t = t0; t < t1; ++t) {
+        const int j = j0 - t;
+        force_term<NU>(L, x, xf, B.ring(B.gp_ring, t, src), L.basis_v(src, j), acc, accd);
+        if (j < L.k - 1) force_term<NU>(L, x, xf, L.basis_w(src, j), B.ring(B.gs_ring, t, src), acc, accd);
+      }
+    } else {
+      // FP32 fields: FP32 partial sums over one ring of terms, then FP64
+      cplx<R> G[9], Gd[9];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) G[e] = Gd[e] = czero<R>();
-    for (int t = t0; t < t1; ++t) {
-      const int j = j0 - t;
-      force_term<NU>(L, x, xf, B.ring(B.gp_ring, t, src), L.basis_v(src, j), G, Gd);
-      if (j < L.k - 1) force_term<NU>(L, x, xf, L.basis_w(src, j), B.ring(B.gs_ring, t, src), G, Gd);
-    }
+      for (int e = 0; e < 9; ++e) G[e] = Gd[e] = czero<R>();
+      for (int t = t0; t < t1; ++t) {
+        const int j = j0 - t;
+        force_term<NU>(L, x, xf, B.ring(B.gp_ring, t, src), L.basis_v(src, j), G, Gd);
+        if (j < L.k - 1) force_term<NU>(L, x, xf, L.basis_w(src, j), B.ring(B.gs_ring, t, src), G, Gd);
+      }
 #pragma unroll
-    for (int e = 0; e < 9; ++e) {
-      acc[e] = acc[e] + mk((double)G[e].re, (double)G[e].im);
-      accd[e] = accd[e] + mk((double)Gd[e].re, (double)Gd[e].im);
+      for (int e = 0; e < 9; ++e) {
+        acc[e] = acc[e] + mk((double)G[e].re, (double)G[e].im);
+        accd[e] = accd[e] + mk((double)Gd[e].re, (double)Gd[e].im);
+      }
     }
   }
   if (part) {   // a split of the items: its own partial sum, added in split order later
@@ -1659,26 +1657,17 @@ int force_splits(int64_t V) {
 }
 template <typename R>
 void force_flush(const Lat<R>& L, const Rev<R>& B, const int* /*unused*/, int nterms, int j0, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value) {
-    if (nterms <= 0) return;
-    const int nsplit = fx_force_flush(L, B, nterms, j0, st);
-    if (nsplit > 1) {
-      const int64_t n = 72 * L.g.V;
-      k_force_reduce<<<nblocks(n, 256), 256, 0, st>>>(B.force, B.force_parts, nsplit, n);
-    }
-  } else {
-    if (nterms <= 0) return;
-    const unsigned nb = nblocks(L.g.V, BS);
-    int nsplit = B.force_parts ? force_splits(L.g.V) : 1;
-    if (nsplit > L.nsrc * nterms) nsplit = L.nsrc * nterms;
-    k_force<0, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
-    k_force<1, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
-    k_force<2, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
-    k_force<3, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
-    if (nsplit > 1) {
-      const int64_t n = 72 * L.g.V;
-      k_force_reduce<<<nblocks(n, 256), 256, 0, st>>>(B.force, B.force_parts, nsplit, n);
-    }
+  if (nterms <= 0) return;
+  const unsigned nb = nblocks(L.g.V, BS);
+  int nsplit = B.force_parts ? force_splits(L.g.V) : 1;
+  if (nsplit > L.nsrc * nterms) nsplit = L.nsrc * nterms;
+  k_force<0, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+  k_force<1, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+  k_force<2, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+  k_force<3, R><<<dim3(nb, nsplit), BS, 0, st>>>(L, B, nterms, j0, nsplit, B.force_parts);
+  if (nsplit > 1) {
+    const int64_t n = 72 * L.g.V;
+    k_force_reduce<<<nblocks(n, 256), 256, 0, st>>>(B.force, B.force_parts, nsplit, n);
   }
 }
 
@@ -1715,38 +1704,33 @@ void eps_norms(const double* a_top, const double* a_bot, const double* b, int ns
   k_eps_norms<<<nsrc, 512, 0, st>>>(a_top, a_bot, b, n, out);
 }
 
-#define OV_INST(R) \
-  template void ritz_combine<R>(const Lat<R>&, int, int, int, const zd*, double*, cudaStream_t); \
-  template void apply_dh<R>(const Lat<R>&, const R*, R*, int, cudaStream_t); \
-  template void pack_spinors<R>(const double*, R*, int, int64_t, int64_t, cudaStream_t); \
-  template void pack_block_start<R>(const double*, const double*, R*, R*, int, int64_t, int64_t, cudaStream_t); \
-  template void unpack_spinors<R>(const R*, double*, int, int64_t, int64_t, cudaStream_t); \
-  template void pack_links<R>(const double*, R*, int64_t, cudaStream_t); \
-  template void apply_h<R>(const Lat<R>&, const R*, R*, int, cudaStream_t, int, int*); \
-  template void tsl_init<R>(const Lat<R>&, cudaStream_t); \
-  template void tsl_stencil<R>(const Lat<R>&, int, bool, cudaStream_t, int); \
-  template void tsl_update<R>(const Lat<R>&, int, bool, cudaStream_t); \
-  template void proj_dots<R>(const Lat<R>&, int, int, const R*, const R*, int64_t, zd*, zd*, cudaStream_t); \
-  template void proj_update<R>(const Lat<R>&, int, int, R*, R*, int64_t, const zd*, bool, cudaStream_t, bool); \
-  template void combine<R>(const Lat<R>&, int, const zd*, double*, cudaStream_t); \
-  template void combine_range<R>(const Lat<R>&, int, int, const zd*, double*, bool, cudaStream_t); \
-  template void rev_init<R>(const Lat<R>&, const Rev<R>&, cudaStream_t); \
-  template void rev_form<R>(const Lat<R>&, const Rev<R>&, int, int, bool, cudaStream_t); \
-  template void rev_proj_record<R>(const Lat<R>&, const Rev<R>&, int, int, const zd*, cudaStream_t); \
-  template void rev_combine<R>(const Lat<R>&, const Rev<R>&, int, int, cudaStream_t); \
-  template void rev_stencil<R>(const Lat<R>&, const Rev<R>&, int, int, int, int, cudaStream_t); \
+#define OV_INST(R)                                                                                                \
+  template void ritz_combine<R>(const Lat<R>&, int, int, int, const zd*, double*, cudaStream_t);                  \
+  template void apply_dh<R>(const Lat<R>&, const R*, R*, int, cudaStream_t);                                      \
+  template void pack_spinors<R>(const double*, R*, int, int64_t, int64_t, cudaStream_t);                          \
+  template void pack_block_start<R>(const double*, const double*, R*, R*, int, int64_t, int64_t, cudaStream_t);   \
+  template void unpack_spinors<R>(const R*, double*, int, int64_t, int64_t, cudaStream_t);                        \
+  template void pack_links<R>(const double*, R*, int64_t, cudaStream_t);                                          \
+  template void apply_h<R>(const Lat<R>&, const R*, R*, int, cudaStream_t, int, int*);                            \
+  template void tsl_init<R>(const Lat<R>&, cudaStream_t);                                                         \
+  template void tsl_stencil<R>(const Lat<R>&, int, bool, cudaStream_t, int);                                      \
+  template void tsl_update<R>(const Lat<R>&, int, bool, cudaStream_t);                                            \
+  template void proj_dots<R>(const Lat<R>&, int, int, const R*, const R*, int64_t, zd*, zd*, cudaStream_t);       \
+  template void proj_update<R>(const Lat<R>&, int, int, R*, R*, int64_t, const zd*, bool, cudaStream_t, bool);    \
+  template void basis_dots<R>(const Lat<R>&, int, const R*, int64_t, zd*, zd*, cudaStream_t);                     \
+  template void combine<R>(const Lat<R>&, int, const zd*, double*, cudaStream_t);                                 \
+  template void combine_range<R>(const Lat<R>&, int, int, const zd*, double*, bool, cudaStream_t);                \
+  template void basis_dots_range<R>(const Lat<R>&, int, int, const R*, int64_t, zd*, zd*, cudaStream_t);          \
+  template void rev_init<R>(const Lat<R>&, const Rev<R>&, cudaStream_t);                                          \
+  template void rev_dots<R>(const Lat<R>&, const Rev<R>&, int, cudaStream_t);                                     \
+  template void rev_form<R>(const Lat<R>&, const Rev<R>&, int, int, bool, cudaStream_t);                          \
+  template void rev_proj_record<R>(const Lat<R>&, const Rev<R>&, int, int, const zd*, cudaStream_t);              \
+  template void rev_alpha_dots<R>(const Lat<R>&, const Rev<R>&, int, int, cudaStream_t);                          \
+  template void rev_combine<R>(const Lat<R>&, const Rev<R>&, int, int, cudaStream_t);                             \
+  template void rev_stencil<R>(const Lat<R>&, const Rev<R>&, int, int, int, int, cudaStream_t);                   \
   template void force_flush<R>(const Lat<R>&, const Rev<R>&, const int*, int, int, cudaStream_t);
 
 OV_INST(double)
 OV_INST(float)
-
-// FP64 calls run the reverse sweep in fixed point (fx_kernels.cu)
-#define OV_INST_FP32(R) \
-  template void basis_dots<R>(const Lat<R>&, int, const R*, int64_t, zd*, zd*, cudaStream_t); \
-  template void basis_dots_range<R>(const Lat<R>&, int, int, const R*, int64_t, zd*, zd*, cudaStream_t); \
-  template void rev_dots<R>(const Lat<R>&, const Rev<R>&, int, cudaStream_t); \
-  template void rev_alpha_dots<R>(const Lat<R>&, const Rev<R>&, int, int, cudaStream_t);
-
-OV_INST_FP32(float)
 
 }  // namespace ov

@@ -23,7 +23,7 @@ enum BufId {
   B_LINKS, B_BV, B_BW, B_P, B_Q, B_R, B_S, B_SC, B_ALPHA, B_BETA, B_DELTA, B_PART, B_CNT, B_COEF, B_CPART,
   B_T, B_X, B_XI, B_XN, B_E, B_EN, B_TMP1, B_TMP2, B_IPIV, B_PROW, B_COL, B_DSTAT, B_DPART, B_DCNT, B_DERR,
   B_Y, B_GY, B_GA, B_GB, B_GD, B_XBAR, B_GV, B_GW, B_GV2, B_GW2, B_GR, B_GS, B_GP, B_EV, B_EW, B_REB,
-  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, B_FXL, B_FXE, B_FXR, B_FXRE, B_FXS, B_FXSE, B_FXP, B_FXPE, B_FXQ, B_FXQE, B_BVE, B_BWE, B_CKRE, B_CKSE, B_CKVE, B_CKWE, B_GVE, B_GWE, B_GRE, B_GSE, B_GPE, B_HINE, B_XBE, NBUF
+  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, B_FXL, B_FXE, B_FXR, B_FXRE, B_FXS, B_FXSE, B_FXP, B_FXPE, B_FXQ, B_FXQE, B_BVE, B_BWE, B_CKRE, B_CKSE, B_CKVE, B_CKWE, NBUF
 };
 
 struct Status {
@@ -336,10 +336,13 @@ void pack_start(ov_context* c, const Lat<R>& L, const void* b) {
 // What a call's Lat holds beside the scalars: links and p, q, r, s in R, or (FP64 calls) in
 // fixed point (fx.cuh), as the call's kernels read them.
 //   The operator: fixed-point links and input; marked sites and their neighbours in FP64.
-//   sgn(H) b and its gradient: the recurrence (and the reverse sweep) in fixed point.
-//   Theorem-1 calls: FP64.  The two halves of a block vector meet in one sum, whose
-//   fixed-point scale is the larger half's: dH along a small direction is lost in its rounding
-//   (dx to 1.5e-9 at a direction of 1e-8, to nothing at 1e-18).
+//   sgn(H) b where the result is x alone (the nested k x k stage, the overlap operator,
+//   eps_A): the recurrence in fixed point.
+//   ov_tsl_sign, its derivatives and tapes: FP64.  The derivative of sgn at T_k grows without
+//   bound as a Ritz value comes near Re z = 0, and with it what a change of rounding in the
+//   recurrence or in the reverse sweep does to dU and dmu (from FP64 to fixed point and back:
+//   up to 3e-7 at mu = 0.3 and 0.5, on lattices of every size, where x moves by less than
+//   1e-12 and the error of either is as large).  ov_tsl_sign's x is the tape's, bit for bit.
 enum : int {
   LAT_LINKS = 1,      // u
   LAT_FIELDS = 2,     // p, q, r, s
@@ -364,7 +367,6 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   check_ptr(U);
   const int64_t V = L.g.V;
   L.kappa = (R)(1.0 / (2.0 * m_w + 8.0));
-  L.kinv = (R)(2.0 * m_w + 8.0);
   L.ef = (R)std::exp(mu);
   L.efinv = (R)std::exp(-mu);
   L.nsrc = nsrc;
@@ -493,9 +495,9 @@ void forward_krylov(ov_context* c, Lat<R>& L) {
           const bool last = ps == c->opt.passes - 1;
           if constexpr (std::is_same<R, double>::value) {
             if (L.fx()) {
-              run(c, OV_KIND_PROJ_DOTS, 2, [&] { fx_proj_dots(L, 0, j + 1, 0, L.fr, L.fs, L.vs, coef, cpart, c->st); });
+              run(c, OV_KIND_PROJ_DOTS, 2, [&] { fx_proj_dots(L, j + 1, L.fr, L.fs, L.vs, coef, cpart, c->st); });
               run(c, OV_KIND_PROJ_UPDATE, 1,
-                  [&] { fx_proj_update(L, nullptr, j + 1, 0, L.fr, L.fs, L.vs, coef, j, last ? 1 : 0, c->st); });
+                  [&] { fx_proj_update(L, j + 1, L.fr, L.fs, L.vs, coef, j, last, c->st); });
               continue;
             }
           }
@@ -530,7 +532,7 @@ int run_diagnostics(ov_context* c, const Lat<R>& L, bool segments, ov_tsl_info* 
         if (L.fx()) {
           const FxField v{reinterpret_cast<int4*>(L.basis_v(0, k - 1)), L.bve + (int64_t)(k - 1) * (L.vs / 24)};
           const FxField w{reinterpret_cast<int4*>(L.basis_w(0, k - 1)), L.bwe + (int64_t)(k - 1) * (L.vs / 24)};
-          return fx_proj_dots(L, 0, k, 0, v, w, (int64_t)L.kcap * L.vs, coef, cpart, c->st);
+          return fx_proj_dots(L, k, v, w, (int64_t)L.kcap * L.vs, coef, cpart, c->st);
         }
       }
       proj_dots(L, k - 1, 0, L.basis_v(0, k - 1), L.basis_w(0, k - 1), (int64_t)L.kcap * L.vs, coef, cpart, c->st);
@@ -1035,14 +1037,15 @@ float elapsed(cudaEvent_t a, cudaEvent_t b) {
   return ms;
 }
 
+// alone: no derivative of this x is taken and none has to equal it
 template <typename R>
 int tsl_sign_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, double m_w, int nsrc,
-                  const void* b, int k, void* x, ov_tsl_info* info) {
+                  const void* b, int k, void* x, ov_tsl_info* info, bool alone) {
   check_ptr(b);
   check_ptr(x);
   const int S = c->opt.segment > 0 && c->opt.segment < k ? c->opt.segment : 0;
   Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0,
-                      LAT_FX_SIGN);
+                      alone || c->opt.nested > 0 ? LAT_FX_SIGN : LAT_PLAIN);
   pack_start(c, L, b);
   SegPlan P;
   SegStore<R> K{};
@@ -1342,7 +1345,7 @@ int deflated_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   }
   launch_check();
   const int st = block ? block_impl<R>(c, dims, U, mu, m_w, nsrc, top, bot, k, E, m_dir, dx, x, info)
-                       : tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, bot, k, x, info);
+                       : tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, bot, k, x, info, false);
   if (st != OV_OK) return st;
   if (l > 0) {
     double* xd = static_cast<double*>(x);
@@ -1385,11 +1388,11 @@ int eps_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
     one = ov_tsl_info{};
     st = block_impl<R>(c, dims, U, mu, m_w, nsrc, t1, b1, k, E, m_dir, t2, b2, &one);
   } else {
-    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b, k, b1, &one);
+    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b, k, b1, &one, true);
     merge_info(info, one);
     if (st != OV_OK) return st;
     one = ov_tsl_info{};
-    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b1, k, b2, &one);
+    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b1, k, b2, &one, true);
   }
   merge_info(info, one);
   if (st != OV_OK) return st;
@@ -1435,7 +1438,7 @@ int vjp_forward(ov_context* c, const int32_t dims[4], const void* U, double mu, 
   F.S = S;
   F.k = k;
   F.nsrc = nsrc;
-  F.L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0, LAT_FX_SIGN | LAT_LINKS);
+  F.L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0);
   Lat<R>& L = F.L;
   const int64_t V = L.g.V, vs = L.vs;
   pack_start(c, L, b);
@@ -1516,21 +1519,7 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
   CK(cudaEventRecord(c->ev[2], c->st));
   // g_y = V^dag xbar
   R* xb = wsT<R>(c, B_XBAR, nsrc * vs);
-  FxField fxb{};
-  if constexpr (std::is_same<R, double>::value) {
-    fxb = FxField{reinterpret_cast<int4*>(xb), wsT<short>(c, B_XBE, nsrc * (vs / 24))};
-    run(c, OV_KIND_LAYOUT, 1,
-        [&] { fx_pack(static_cast<const double*>(xbar), fxb, FxField{}, nullptr, nsrc, V, vs, c->st); });
-  } else {
-    run(c, OV_KIND_LAYOUT, 1, [&] { pack_spinors<R>(static_cast<const double*>(xbar), xb, nsrc, V, vs, c->st); });
-  }
-  // out[src][2 (j - j0)] = v_j^dag xbar
-  auto xbar_dots = [&](int j0, int nvec, zd* out, zd* cpart) {
-    run(c, OV_KIND_COMBINE, 2, [&] {
-      if constexpr (std::is_same<R, double>::value) fx_proj_dots(L, j0, nvec, 1, fxb, FxField{}, vs, out, cpart, c->st);
-      else basis_dots_range(L, j0, nvec, xb, vs, out, cpart, c->st);
-    });
-  };
+  run(c, OV_KIND_LAYOUT, 1, [&] { pack_spinors<R>(static_cast<const double*>(xbar), xb, nsrc, V, vs, c->st); });
   const int64_t nsb = (V + 127) / 128;
   zd* gy = wsT<zd>(c, B_GY, (int64_t)nsrc * 2 * k);
   zd* cpart = wsT<zd>(c, B_CPART, (int64_t)nsrc * 2 * k * nsb);
@@ -1538,10 +1527,12 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
     // second pass: g_y one replayed segment at a time
     for (size_t t = 0; t < P.lo.size(); ++t) {
       seg_replay(c, L, P, K, (int)t, false);
-      xbar_dots(P.lo[t], P.hi[t] - P.lo[t], gy + 2 * P.lo[t], cpart);
+      run(c, OV_KIND_COMBINE, 2, [&] {
+        basis_dots_range(L, P.lo[t], P.hi[t] - P.lo[t], xb, vs, gy + 2 * P.lo[t], cpart, c->st);
+      });
     }
   } else {
-    xbar_dots(0, k, gy, cpart);
+    run(c, OV_KIND_COMBINE, 2, [&] { basis_dots(L, k, xb, vs, gy, cpart, c->st); });
   }
   launch_check();
   // G_T = L_sgn(T^dag, beta0 g_y e1^T).  The Theorem-1 block iteration on
@@ -1727,26 +1718,12 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
   B.m = m;
   B.gv = wsT<R>(c, B_GV, nsrc * vs);
   B.gw = wsT<R>(c, B_GW, nsrc * vs);
-  // (the fixed-point sweep replaces its gradients in place)
-  B.gv_new = std::is_same<R, double>::value ? nullptr : wsT<R>(c, B_GV2, nsrc * vs);
-  B.gw_new = std::is_same<R, double>::value ? nullptr : wsT<R>(c, B_GW2, nsrc * vs);
+  B.gv_new = wsT<R>(c, B_GV2, nsrc * vs);
+  B.gw_new = wsT<R>(c, B_GW2, nsrc * vs);
   B.gr_ring = wsT<R>(c, B_GR, (int64_t)m * nsrc * vs);
   B.gs_ring = wsT<R>(c, B_GS, (int64_t)m * nsrc * vs);
   B.gp_ring = wsT<R>(c, B_GP, (int64_t)m * nsrc * vs);
   B.hin = wsT<R>(c, B_HIN, (int64_t)nsrc * vs);
-  constexpr bool fx = std::is_same<R, double>::value;
-  if constexpr (fx) {
-    auto view = [&](R* p, int id, int64_t n) {
-      return FxField{reinterpret_cast<int4*>(p), wsT<short>(c, id, n * (vs / 24))};
-    };
-    B.fgv = view(B.gv, B_GVE, nsrc);
-    B.fgw = view(B.gw, B_GWE, nsrc);
-    B.fgr = view(B.gr_ring, B_GRE, (int64_t)m * nsrc);
-    B.fgs = view(B.gs_ring, B_GSE, (int64_t)m * nsrc);
-    B.fgp = view(B.gp_ring, B_GPE, (int64_t)m * nsrc);
-    B.fh = view(B.hin, B_HINE, nsrc);
-    B.fxb = fxb;
-  }
   B.xbar = xb;
   B.y = y;
   B.gaT = gaT;
@@ -1760,27 +1737,23 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
     CK(cudaMemcpyAsync(B.reb_steps, reb.data(), sizeof(int) * reb.size(), cudaMemcpyHostToDevice, c->st));
   B.force = wsT<double>(c, B_FORCE, 72 * V, true);
   {
-    const int ns = fx ? fx_force_splits(V) : force_splits(V);
+    const int ns = force_splits(V);
     B.force_parts = ns > 1 ? wsT<double>(c, B_FPARTS, (int64_t)ns * 72 * V) : nullptr;
   }
   B.dmu = wsT<double>(c, B_DMU, 1, true);
-  B.dmu_part = wsT<zd>(c, B_DMUPART, kForceSplitMax * ((V + 15) / 16) + 64);
+  B.dmu_part = wsT<zd>(c, B_DMUPART, kForceSplitMax * ((V + 127) / 128) + 64);
   B.dmu_cnt = wsT<unsigned>(c, B_DMUCNT, 4);
   zd* coef = wsT<zd>(c, B_COEF, (int64_t)nsrc * 2 * k);
   auto sweep = [&] {
   run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_init(L, B, c->st); });
   run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_combine(L, B, k - 1, 0, c->st); });
   run(c, OV_KIND_REV_STENCIL, 1, [&] { rev_stencil(L, B, k - 1, 0, -1, 0, c->st); });
-  auto swap_g = [&] {
-    if (fx) return;
-    std::swap(B.gv, B.gv_new);
-    std::swap(B.gw, B.gw_new);
-  };
-  swap_g();
+  std::swap(B.gv, B.gv_new);
+  std::swap(B.gw, B.gw_new);
   int slot = 1, j0 = k - 1, nrec = 0;
   for (int j = k - 2; j >= 0; --j) {
     if (slot == m) {
-      run(c, OV_KIND_FORCE, fx ? 1 : 4, [&] { force_flush(L, B, nullptr, m, j0, c->st); });
+      run(c, OV_KIND_FORCE, 4, [&] { force_flush(L, B, nullptr, m, j0, c->st); });
       slot = 0;
       j0 = j;
     }
@@ -1791,34 +1764,27 @@ int vjp_reverse(ov_context* c, FwdState<R>& F, const void* xbar, void* x, void* 
       seg_combine(tcur);
     }
     const int prev = slot == 0 ? m - 1 : slot - 1;
-    // (the fixed-point stencil of step j + 1 has formed these dots)
-    if constexpr (!fx) run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_dots(L, B, j, c->st); });
+    run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_dots(L, B, j, c->st); });
     const int rb = rebiorth_at(j + 1, c->opt.rebiorth);
     run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_form(L, B, j, slot, !rb, c->st); });
     if (rb) {
+      R* grs = B.gr_ring + (int64_t)slot * nsrc * vs;
+      R* gss = B.gs_ring + (int64_t)slot * nsrc * vs;
       for (int ps = 0; ps < c->opt.passes; ++ps) {
-        if constexpr (fx) {
-          const FxField gr = fx_src(B.fgr, (int64_t)slot * nsrc, vs), gs = fx_src(B.fgs, (int64_t)slot * nsrc, vs);
-          const int fin = ps == c->opt.passes - 1 ? 2 : 0;
-          run(c, OV_KIND_PROJ_DOTS, 2, [&] { fx_proj_dots(L, 0, j + 1, 1, gr, gs, vs, coef, cpart, c->st); });
-          run(c, OV_KIND_PROJ_UPDATE, 1, [&] { fx_proj_update(L, &B, j + 1, 1, gr, gs, vs, coef, j, fin, c->st); });
-        } else {
-          R* grs = B.gr_ring + (int64_t)slot * nsrc * vs;
-          R* gss = B.gs_ring + (int64_t)slot * nsrc * vs;
-          run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 1, grs, gss, vs, coef, cpart, c->st); });
-          run(c, OV_KIND_PROJ_UPDATE, 1, [&] { proj_update(L, j, 1, grs, gss, vs, coef, false, c->st, ps > 0); });
-        }
+        run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 1, grs, gss, vs, coef, cpart, c->st); });
+        run(c, OV_KIND_PROJ_UPDATE, 1, [&] { proj_update(L, j, 1, grs, gss, vs, coef, false, c->st, ps > 0); });
         run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_proj_record(L, B, j, nrec, coef, c->st); });
       }
-      if constexpr (!fx) run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_alpha_dots(L, B, j, slot, c->st); });
+      run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_alpha_dots(L, B, j, slot, c->st); });
       ++nrec;
     }
     run(c, OV_KIND_REV_SCALAR, 1, [&] { rev_combine(L, B, j, slot, c->st); });
     run(c, OV_KIND_REV_STENCIL, 1, [&] { rev_stencil(L, B, j, slot, prev, nrec, c->st); });
-    swap_g();
+    std::swap(B.gv, B.gv_new);
+    std::swap(B.gw, B.gw_new);
     ++slot;
   }
-  run(c, OV_KIND_FORCE, fx ? 1 : 4, [&] { force_flush(L, B, nullptr, slot, j0, c->st); });
+  run(c, OV_KIND_FORCE, 4, [&] { force_flush(L, B, nullptr, slot, j0, c->st); });
   };
   if (S > 0) {
     sweep();   // segment replays copy checkpoints between the steps: launched directly
@@ -1883,13 +1849,13 @@ int overlap_apply_impl(ov_context* c, const int32_t dims[4], const void* U, doub
   double* xs = wsT<double>(c, B_OVX, 2 * n);
   int st;
   if (!dagger) {
-    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b, k, xs, info);
+    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b, k, xs, info, true);
     if (st != OV_OK) return st;
     run(c, OV_KIND_COMBINE, 1, [&] { ov_combine(bd, xs, od, n, 1, c->st); });
   } else {
     double* g5b = wsT<double>(c, B_OVB, 2 * n);
     run(c, OV_KIND_COMBINE, 1, [&] { gamma5_scale(bd, g5b, n, 1.0, 0.0, c->st); });
-    st = tsl_sign_impl<R>(c, dims, U, -mu, m_w, nsrc, g5b, k, xs, info);
+    st = tsl_sign_impl<R>(c, dims, U, -mu, m_w, nsrc, g5b, k, xs, info, true);
     if (st != OV_OK) return st;
     run(c, OV_KIND_COMBINE, 1, [&] { ov_combine(bd, xs, od, n, 0, c->st); });
   }
@@ -2704,8 +2670,8 @@ int ov_tsl_sign(ov_context* c, const int32_t dims[4], const void* U, double mu, 
   if (!c || k < 2 || k > 4096) return OV_ERR_INVALID_ARG;
   if (info) std::memset(info, 0, sizeof(*info));
   return guarded([&] {
-    return c->opt.precision == OV_MIXED ? tsl_sign_impl<float>(c, dims, U, mu, m_w, nsrc, b, k, x, info)
-                                        : tsl_sign_impl<double>(c, dims, U, mu, m_w, nsrc, b, k, x, info);
+    return c->opt.precision == OV_MIXED ? tsl_sign_impl<float>(c, dims, U, mu, m_w, nsrc, b, k, x, info, false)
+                                        : tsl_sign_impl<double>(c, dims, U, mu, m_w, nsrc, b, k, x, info, false);
   });
 }
 

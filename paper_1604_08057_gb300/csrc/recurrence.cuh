@@ -140,39 +140,4 @@ __device__ __forceinline__ void omega_finalize_warp(const Lat<R>& L, int src, in
   }
 }
 
-template <typename R>
-__device__ __forceinline__ void rev_dots_epilogue_warp(const Lat<R>& L, const Rev<R>& B, int src, int j, zd s0, zd s1) {
-  const int lane = threadIdx.x & 31;
-  SrcScal& sc = L.sc[src];
-  const int64_t o = (int64_t)src * L.k + j + 1;
-  const double d = L.delta[o];
-  const zd bt = L.beta[o];
-  const zd om = mk(bt.re * d, bt.im * d);
-  const double aom = d * d, b2 = bt.re * bt.re + bt.im * bt.im;
-  // conj(s1) / conj(beta) and 1 / beta over |beta|^2, s0 / d and 1 / d
-  const double num = lane == 0   ? s1.re * bt.re + s1.im * bt.im
-                     : lane == 1 ? s1.re * bt.im - s1.im * bt.re
-                     : lane == 2 ? bt.re
-                     : lane == 3 ? -bt.im
-                     : lane == 4 ? s0.re
-                                 : 1.0;
-  const double a = num / (lane < 4 ? b2 : d);
-  const zd g_b = B.gbT[o] + sc.carry_beta - mk(lane_of(a, 0), lane_of(a, 1));
-  double g_d = B.gdT[o] + sc.carry_delta - lane_of(a, 4);
-  const double b = (lane == 0 ? g_b.re : lane == 1 ? g_b.im : om.re * g_b.re + om.im * g_b.im) / (lane < 2 ? d : d * d);
-  zd g_w = mk(lane_of(b, 0), lane_of(b, 1));
-  g_d -= lane_of(b, 2);                      // Re(conj(om) g_b) / d^2
-  const double f = g_d / (2.0 * d * aom);
-  g_w = g_w + mk(f * om.re, f * om.im);
-  const zd cr2 = conj(bt) * g_w, cs2 = mk(d * g_w.re, -d * g_w.im);
-  const zd cr1 = mk(lane_of(a, 5), 0.0), cs1 = mk(lane_of(a, 2), lane_of(a, 3));
-  if (lane == 0) {
-    sc.cr1 = cr1;
-    sc.cr2 = cr2;
-    sc.cs1 = cs1;
-    sc.cs2 = cs2;
-    if (!finite_z(cr2) || !finite_z(cs2)) flag_error(sc, ERRB_NONFINITE, j);
-  }
-}
-
 }  // namespace ov
