@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(128) k_pack_links_fx(const double* __restrict_
   }
   const int eb = (int)(mag >> 20);
   const bool bad = mag != 0u && (eb < FX_U_MIN || eb > FX_U_MAX);
-  const int ee = mag == 0u ? 1022 : eb;
+  const int ee = mag == 0u ? FX_U_MIN : eb;   // (a zero link does not raise a sum's scale)
   ex[(int64_t)d * V + x] = (short)(bad ? FX_BAD : ee);
   // u 2^(1081 - e): 59 bits; the error terms are at most 2^-53 of the largest entry
   const double f2 = fx_pow2(1081 - (bad ? 1022 : ee));
