@@ -15,9 +15,10 @@
 // with their own scale E: units of 2^(E - 2100), kept to some 2^-56 of the largest
 // contribution to the site, against 2^-53 per operation in FP64 arithmetic.
 // Infinities, NaN and magnitudes outside the window below mark a site (FX_BAD);
-// the operator's own entry points then use FP64 for every sum that meets it, and
-// in the Lanczos recurrence it is what a NaN was: it reaches the next dot product
-// and stops the source with a non-finite error.
+// the operator's own entry points then use FP64 for every sum that meets it.  In
+// the Lanczos recurrence a site (or link) below the window is zero, and a marked
+// one is what a NaN is in FP64: it reaches the next dot product and stops the
+// source with a non-finite error (above the window the norm overflows in FP64 too).
 #pragma once
 #include "dslash.cuh"
 #include "kernels.h"
@@ -241,13 +242,14 @@ __device__ __forceinline__ void fx_double(const FxHalf& a, bool bad, zd (&o)[6])
 #pragma unroll
   for (int i = 0; i < 6; ++i) o[i] = mk(u * (double)a.v[i].re, u * (double)a.v[i].im);
 }
-// six FP64 components encoded (every lane)
-__device__ __forceinline__ void fx_from_double(const zd (&p)[6], FxH& o) {
+// six FP64 components encoded (every lane); flush: a site below the window is encoded with the
+// window's smallest exponent, to zero or to the bits above 2^-880, instead of marked
+__device__ __forceinline__ void fx_from_double(const zd (&p)[6], FxH& o, bool flush = false) {
   unsigned m = 0u;
 #pragma unroll
   for (int i = 0; i < 6; ++i) m = max(m, max(fx_mag(p[i].re), fx_mag(p[i].im)));
   m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
-  const int e = fx_field_exp(m);
+  const int e = flush && (int)(m >> 20) < FX_F_MIN ? FX_F_MIN : fx_field_exp(m);
   o.e = e;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {

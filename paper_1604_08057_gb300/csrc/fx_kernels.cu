@@ -63,9 +63,11 @@ __device__ __forceinline__ FxField fx_bw(const Lat<double>& L, int src, int j) {
 // ---------------------------------------------------------------------------
 // Direction d = blockIdx.y: the links (d < 3 spatial, 3: ef U_t, 4: efinv U_t) of the
 // user's array u.  The products are formed with their FP64 rounding errors, so each entry
-// carries the fixed-point error alone.
+// carries the fixed-point error alone.  flush: a link below the window is encoded with the
+// smallest exponent instead of marked (the callers that never use the links in FP64).
 __global__ void __launch_bounds__(128) k_pack_links_fx(const double* __restrict__ u, double ef, double efinv,
-                                                       int4* __restrict__ out, short* __restrict__ ex, int64_t V) {
+                                                       int4* __restrict__ out, short* __restrict__ ex, int64_t V,
+                                                       int flush) {
   const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (x >= V) return;
   const int d = blockIdx.y, nu = d < 3 ? d : 3;
@@ -83,8 +85,9 @@ __global__ void __launch_bounds__(128) k_pack_links_fx(const double* __restrict_
     mag = max(mag, max(fx_mag(hi[2 * q]), fx_mag(hi[2 * q + 1])));
   }
   const int eb = (int)(mag >> 20);
-  const bool bad = mag != 0u && (eb < FX_U_MIN || eb > FX_U_MAX);
-  const int ee = mag == 0u ? FX_U_MIN : eb;   // (a zero link does not raise a sum's scale)
+  const bool low = mag == 0u || (flush && eb < FX_U_MIN);
+  const bool bad = !low && (eb < FX_U_MIN || eb > FX_U_MAX);
+  const int ee = low ? FX_U_MIN : eb;   // (a zero link does not raise a sum's scale)
   ex[(int64_t)d * V + x] = (short)(bad ? FX_BAD : ee);
   // u 2^(1081 - e): 59 bits; the error terms are at most 2^-53 of the largest entry
   const double f2 = fx_pow2(1081 - (bad ? 1022 : ee));
@@ -98,8 +101,9 @@ __global__ void __launch_bounds__(128) k_pack_links_fx(const double* __restrict_
     out[fx_link_at(x, d) + q * 32] = make_int4(r.h, r.l, i.h, i.l);
   }
 }
-void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, cudaStream_t st) {
-  k_pack_links_fx<<<dim3(nblocks(V, 128), 5), 128, 0, st>>>(u, ef, efinv, out, ex, V);
+void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, bool flush,
+                   cudaStream_t st) {
+  k_pack_links_fx<<<dim3(nblocks(V, 128), 5), 128, 0, st>>>(u, ef, efinv, out, ex, V, flush ? 1 : 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -138,8 +142,8 @@ __device__ __forceinline__ void soa_store(double* f, int64_t V, int64_t s, int s
   for (int i = 0; i < 6; ++i) q[fx_comp(sp, i) * V] = make_double2(p[i].re, p[i].im);
 }
 
-// user spinors to fixed point, in f and (if set) g; marked sites keep FP64 values in d (if
-// set)
+// user spinors to fixed point, in f and (if set) g.  With d marked sites keep their FP64 values
+// there; without it sites below the window are zero: nothing reads them in FP64
 __global__ void __launch_bounds__(128) k_fx_pack(const double* __restrict__ aos, FxField f, FxField g,
                                                  double* __restrict__ d, int64_t V, int64_t vs) {
   __shared__ double2 stage[4][kStage];
@@ -151,7 +155,7 @@ __global__ void __launch_bounds__(128) k_fx_pack(const double* __restrict__ aos,
   zd p[6];
   FxH o;
   aos_load(aos, src, V, x0, stage[w], sp, p);
-  fx_from_double(p, o);
+  fx_from_double(p, o, !d);
   if (!live) return;
   fx_put(fx_src(f, src, vs), x, sp, o);
   if (g.c) fx_put(fx_src(g, src, vs), x, sp, o);

@@ -129,8 +129,11 @@ void pack_spinors_il(const double* aos, float* dst, int nsrc, int64_t V, cudaStr
 void unpack_spinors_il(const float* f, double* aos, int nsrc, int64_t V, cudaStream_t st);
 
 // FP64 calls (fx_kernels.cu); the launchers below dispatch to them
-void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, cudaStream_t st);
-// user spinors to f and (if set) g; FP64 values of marked sites to d (if set)
+// flush: links below the window to zero (else marked)
+void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, bool flush,
+                   cudaStream_t st);
+// user spinors to f and (if set) g; FP64 values of marked sites to d, or (d null) sites below the
+// window to zero
 void fx_pack(const double* aos, const FxField& f, const FxField& g, double* d, int nsrc, int64_t V, int64_t vs,
              cudaStream_t st);
 void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t vs, cudaStream_t st);

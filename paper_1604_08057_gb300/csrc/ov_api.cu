@@ -384,7 +384,7 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
     short* ex = wsT<short>(c, B_FXE, 5 * V);
     L.fu = FxLinks{fe, ex};
     run(c, OV_KIND_LAYOUT, 1,
-        [&] { pack_links_fx(static_cast<const double*>(U), fe, ex, V, L.ef, L.efinv, c->st); });
+        [&] { pack_links_fx(static_cast<const double*>(U), fe, ex, V, L.ef, L.efinv, !(parts & LAT_FX_IN), c->st); });
   }
   launch_check();
   if (fm == 2) {

@@ -11,7 +11,7 @@ import numpy as np
 import pytest
 import torch
 
-from oracle import dirac
+from oracle import dirac, nested, overlap, tsl, vjp
 from paper_1604_08057_gb300 import binding, inputs
 
 pytestmark = pytest.mark.gpu
@@ -36,14 +36,14 @@ def local_magnitude(u, psi):
     return m
 
 
-def check_operator(u, psi):
+def check_operator(u, psi, units=8):
     ul, pl = u.astype(np.clongdouble), psi.astype(np.clongdouble)
     m = local_magnitude(u, psi)
     for dagger in (False, True):
         got = binding.apply_H(T(u), MU, M_W, T(psi), dagger=dagger).cpu().numpy()
         want = (dirac.apply_h_dagger if dagger else dirac.apply_h)(ul, pl, MU, M_W)
         err = np.abs(got - want).max(axis=(-1, -2)).astype(np.float64)
-        assert np.all(err <= 8 * 2.0 ** -53 * m), (dagger, float((err / np.where(m > 0, m, 1)).max() * 2.0 ** 53))
+        assert np.all(err <= units * 2.0 ** -53 * m), (dagger, float((err / np.where(m > 0, m, 1)).max() * 2.0 ** 53))
 
 
 def ragged(rng, psi, lo, hi):
@@ -64,3 +64,54 @@ def test_operator_against_extended_precision(dims, links):
     if links != "su3":
         psi = ragged(rng, psi, -60, 60)
     check_operator(u, psi)
+
+
+def tails(rng, dims):
+    """A Gaussian field whose last planes fall to 1e-260 and to the smallest subnormal."""
+    f = inputs.gaussian_spinors(dims, 1, rng)[0]
+    f[-1] *= 1e-260
+    f[0, -1] = 5e-324
+    return f
+
+
+# b (and the cotangent) far below the fixed-point window on some sites, a link there too.  x and the
+# gradients are the oracle's to the bars of the parity tests at m_w = -1
+@pytest.mark.parametrize("rebiorth,passes", [(1, 2), (10, 1)])
+def test_sites_and_links_below_the_window(rebiorth, passes):
+    dims, k = (3, 4, 3, 5), 30
+    rng = np.random.default_rng(43)
+    u = inputs.su3_links(dims, 0.3, rng)
+    u[2, 1, 0, 1, 2] *= 1e-290
+    b, xbar = tails(rng, dims), tails(rng, dims)
+    opts = dict(rebiorth=rebiorth, passes=passes)
+    du_o, dmu_o, f = vjp.tsl_vjp(u, b, 0.2, -1.0, k, xbar, **opts)
+    assert rel(binding.tsl_sign(T(u), 0.2, -1.0, T(b), k, **opts).cpu().numpy(), f.x) <= 1e-11
+    du, dmu, x = binding.tsl_sign_vjp(T(u), 0.2, -1.0, T(b), k, T(xbar), **opts)
+    assert rel(x.cpu().numpy(), f.x) <= 1e-11
+    assert rel(du.cpu().numpy(), du_o) <= 1e-9 and abs(dmu - dmu_o) <= 1e-9 * abs(dmu_o)
+    dx_o, x_o, _ = tsl.block_tsl(u, b, 0.2, -1.0, k, None, 0.7, **opts)
+    dx, xj = binding.tsl_sign_jvp(T(u), 0.2, -1.0, T(b), k, None, 0.7, **opts)
+    assert rel(dx.cpu().numpy(), dx_o) <= 1e-10 and rel(xj.cpu().numpy(), x_o) <= 1e-10
+    want, _, _ = nested.nested_tsl(u, b, 0.2, -1.0, k, 15, **opts)
+    binding.nested_sign(15, **opts)
+    try:
+        xn = binding.tsl_sign(T(u), 0.2, -1.0, T(b), k, **opts)
+    finally:
+        binding.nested_sign(0, **opts)
+    assert rel(xn.cpu().numpy(), want) <= 1e-10
+    eps = binding.tsl_eps(T(u), 0.2, -1.0, T(b), k, **opts)
+    assert abs(eps - tsl.eps_a(u, b, 0.2, -1.0, k, **opts)) <= 1e-6 * eps
+    do = binding.overlap_apply(T(u), 0.2, -1.0, T(b), k, **opts)
+    assert rel(do.cpu().numpy(), overlap.apply_dov(u, b, 0.2, -1.0, k, **opts)) <= 1e-10
+
+
+def test_operator_below_the_window():
+    """The same values through the operator: at the sites that meet them FP64 sums of up to 6 m with
+    some ten roundings each, 64 units of m."""
+    rng = np.random.default_rng(44)
+    dims = (3, 4, 3, 5)
+    u = inputs.su3_links(dims, 0.3, rng)
+    u[2, 1, 0, 1, 2] *= 1e-290
+    psi = tails(rng, dims)
+    psi[0, -1] = 1e-280     # (a subnormal site's sums round to the subnormals' own unit)
+    check_operator(u, psi, 64)
