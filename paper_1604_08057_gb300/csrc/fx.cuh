@@ -661,14 +661,15 @@ __device__ __forceinline__ void fx_block_partials(const zd (&v)[NV], FxSumBuf<NV
 }
 
 // The sums of the n blocks' partials (per value in block order per thread, then a fixed tree),
-// in every lane of warp 0; every thread of the block calls it.  The values are spread over the
+// in every lane of warp 0; every thread of the block calls it.  The order depends on n and on
+// the number nw of warps that take part.  The values are spread over the
 // warps, a value over several only where each has partials (trees and sums of nothing cost as
 // much FP64 pipe as others), and eight loads per thread are in flight at a time.  Two values of
 // 608 blocks took 8700 cycles with all warps at one value after the other; a call at 14x14^3,
 // k = 800 402 -> 393 ms, at 4x4^3, k = 200 23.9 -> 22.7 ms.
 template <int NV>
-__device__ __forceinline__ void fx_sum_partials(const zd* part, int n, zd (&out)[NV], zd* scratch) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+__device__ __forceinline__ void fx_sum_partials(const zd* part, int n, zd (&out)[NV], zd* scratch, int nw) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int per = max(1, min(nw / NV, (n + 31) >> 5));   // warps per value
   const int h = w % per;
   for (int i = w / per; i < NV && w < nw / per * per; i += nw / per) {

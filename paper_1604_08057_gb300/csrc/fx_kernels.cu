@@ -28,9 +28,9 @@ static inline unsigned one_wave(const Lat<double>& L, int sites) {
   return std::min(nblocks(L.g.V, sites), 4u * 152u);
 }
 // Four warps per 16 sites and side (see k_fx_tsl) where one warp leaves most of an SM idle.
-// In the Lanczos step the split sums are the unsplit ones bit for bit, so its rule may count
-// the sources (8^4 with four sources: 23 ms of stencils with the split, 12
-// without); the sums over terms of the other two are not.
+// In the Lanczos step the split sums are the unsplit ones bit for bit (alpha's partials are
+// added by two warps in both), so its rule may count the sources (8^4 with four sources: 23 ms
+// of stencils with the split, 12 without); the projection's sums over terms are not.
 static inline bool fx_split_exact(const Lat<double>& L) { return L.g.V < 152 * 32 && L.g.V * L.nsrc < 152 * 64; }
 
 // a launch with dynamic shared memory, whose limit is raised once per kernel and device
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(128) k_fx_init(const __grid_constant__ Lat<dou
   fx_block_partials(v, sum, part, blockDim.x >> 5);
   if (arrive_last(L.cnt + src * 16 + 0, gridDim.x)) {
     zd s[2];
-    fx_sum_partials<2>(part, gridDim.x, s, scratch);
+    fx_sum_partials<2>(part, gridDim.x, s, scratch, blockDim.x >> 5);
     if (threadIdx.x == 0) init_finalize(L, src, s[0].re, s[1]);
   }
 }
@@ -335,10 +335,10 @@ __device__ __forceinline__ bool h_finish(FxHalf& o, const FxH& f, const FxCoef& 
   for (int i = 3; i < 6; ++i) o.v[i] = FxZ{-o.v[i].re, -o.v[i].im};
   return ok;
 }
-__device__ __forceinline__ void alpha_finish(const Lat<double>& L, int src, int j, const zd* part, zd* scratch) {
+__device__ __forceinline__ void alpha_finish(const Lat<double>& L, int src, int j, const zd* part, zd* scratch, int nw) {
   if (arrive_last(L.cnt + src * 16 + 1, gridDim.x)) {
     zd s[1];
-    fx_sum_partials<1>(part, gridDim.x, s, scratch);
+    fx_sum_partials<1>(part, gridDim.x, s, scratch, nw);
     if (threadIdx.x == 0) {
       SrcScal& sc = L.sc[src];
       if (!finite_z(s[0])) flag_error(sc, ERRB_NONFINITE, j);
@@ -425,7 +425,8 @@ __global__ void __launch_bounds__(SPLIT ? 256 : 128, SPLIT ? 2 : 4)
   }
   zd* part = L.part + src * L.part_stride;
   fx_block_partials(v, sum, part, SPLIT ? 1 : nw);
-  alpha_finish(L, src, j, part, scratch);
+  // (two warps: the block of the unsplit form on the lattices that may be split)
+  alpha_finish(L, src, j, part, scratch, SPLIT ? 2 : blockDim.x >> 5);
 }
 
 void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st) {
@@ -450,7 +451,7 @@ __device__ __forceinline__ void omega_finish(const Lat<double>& L, int src, int 
   fx_block_partials(v, sum, part, blockDim.x >> 5);
   if (arrive_last(L.cnt + src * 16 + slot, gridDim.x)) {
     zd s[2];
-    fx_sum_partials<2>(part, gridDim.x, s, scratch);
+    fx_sum_partials<2>(part, gridDim.x, s, scratch, blockDim.x >> 5);
     if (threadIdx.x < 32 && L.sc[src].err == 0) omega_finalize_warp(L, src, j, s[0], s[1].re, s[1].im);
   }
 }

@@ -115,3 +115,21 @@ def test_operator_below_the_window():
     psi = tails(rng, dims)
     psi[0, -1] = 1e-280     # (a subnormal site's sums round to the subnormals' own unit)
     check_operator(u, psi, 64)
+
+
+# on either side of the rule that splits a small lattice's sites over warps, which counts the sources
+@pytest.mark.parametrize("dims,nsrc", [((8, 8, 8, 8), 4), ((6, 6, 6, 6), 8), ((6, 8, 4, 6), 9)])
+def test_a_source_does_not_depend_on_those_beside_it(dims, nsrc):
+    rng = np.random.default_rng(45)
+    k, opts = 40, dict(rebiorth=20, passes=1)
+    u, b = T(inputs.su3_links(dims, 0.25, rng)), T(inputs.gaussian_spinors(dims, nsrc, rng))
+    binding.nested_sign(20, **opts)
+    try:
+        x = binding.tsl_sign(u, 0.2, -1.0, b, k, **opts)
+        co = [binding.tsl_coefficients(k, s, **opts) for s in range(nsrc)]
+        for s in (0, 1, nsrc - 1):
+            assert torch.equal(binding.tsl_sign(u, 0.2, -1.0, b[s], k, **opts), x[s]), s
+            for one, all_ in zip(binding.tsl_coefficients(k, 0, **opts), co[s]):
+                assert np.array_equal(one, all_), s
+    finally:
+        binding.nested_sign(0, **opts)
