@@ -231,10 +231,11 @@ __device__ __forceinline__ void fx_pick(const Spinor<double>& t, int sp, zd (&p)
 }
 
 // Blocks of blockDim.x / 2 sites x blockDim.y sources, whose sources share the link loads
-// through L1.  With aos the output is the user's layout, else site-major.
+// through L1.  psi's own term is read in FP64: from aos, the user's array, where the output has
+// its layout too, else (aos null) from the site-major din.
 __global__ void __launch_bounds__(128, 4) k_fx_apply(const __grid_constant__ Lat<double> L, FxField in,
-                                                     const double* __restrict__ din, double* __restrict__ out,
-                                                     int dagger, int aos) {
+                                                     const double* __restrict__ din, const double* __restrict__ aos,
+                                                     double* __restrict__ out, int dagger) {
   __shared__ FxStage stage[4];
   FxStage& S = stage[(threadIdx.y * blockDim.x + threadIdx.x) >> 5];
   const int sp = fx_spin_of(threadIdx.x);
@@ -261,24 +262,26 @@ __global__ void __launch_bounds__(128, 4) k_fx_apply(const __grid_constant__ Lat
     hops_fp64(FxLoad{f, d, V, 0}, L.uaos, L.g, x, dagger ? L.efinv : L.ef, dagger ? L.ef : L.efinv, &t);
     fx_pick(t, sp, a);
   }
-  FxH c;
-  fx_load(f, x, sp, c);
-  const double u = fx_pow2(c.e == FX_BAD ? 0 : c.e - 1079);
+  zd p[6];
+  __syncwarp();
+  if (aos) {
+    aos_load(aos, src, V, x0, S.out, sp, p);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const double2 t = reinterpret_cast<const double2*>(d)[fx_comp(sp, i) * V + x];
+      p[i] = mk(t.x, t.y);
+    }
+  }
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    zd p = mk(u * (double)fx_join(c.q[i].x, c.q[i].y), u * (double)fx_join(c.q[i].z, c.q[i].w));
-    if (c.e == FX_BAD) {
-      const double2 t = reinterpret_cast<const double2*>(d)[fx_comp(sp, i) * V + x];
-      p = mk(t.x, t.y);
-    }
-    const zd q = mk(fma(-L.kappa, a[i].re, p.re), fma(-L.kappa, a[i].im, p.im));
+    const zd q = mk(fma(-L.kappa, a[i].re, p[i].re), fma(-L.kappa, a[i].im, p[i].im));
     a[i] = i < 3 ? q : -q;
   }
-  __syncwarp();
   if (aos) aos_store(out, src, V, x0, S.out, sp, a);
   else if (live) soa_store(out + (int64_t)src * L.vs, V, x, sp, a);
 }
-void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double* out, int dagger, int aos,
+void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, const double* aos, double* out, int dagger,
                 cudaStream_t st, int variant) {
   // threads per block in x (two per site) and sources per block: variant v > 0 takes shape v
   // of this table (modulo its length), 0 the rule below
@@ -295,7 +298,7 @@ void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double
     sy = L.nsrc >= 4 ? 4 : L.nsrc >= 2 ? 2 : 1;
     sx = 128 / sy;
   }
-  k_fx_apply<<<dim3(nblocks(L.g.V, sx / 2), nblocks(L.nsrc, sy)), dim3(sx, sy), 0, st>>>(L, in, d, out, dagger, aos);
+  k_fx_apply<<<dim3(nblocks(L.g.V, sx / 2), nblocks(L.nsrc, sy)), dim3(sx, sy), 0, st>>>(L, in, d, aos, out, dagger);
 }
 
 // ---------------------------------------------------------------------------

@@ -137,9 +137,10 @@ void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, 
 void fx_pack(const double* aos, const FxField& f, const FxField& g, double* d, int nsrc, int64_t V, int64_t vs,
              cudaStream_t st);
 void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t vs, cudaStream_t st);
-// in: the field in fixed point, d: its FP64 companion (read where a site is marked); aos: out
-// in the user's layout
-void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, double* out, int dagger, int aos,
+// in: the field in fixed point, d: its FP64 companion, site-major (read where a site is marked);
+// aos: the field as the user's array, with out in the same layout, or null: out site-major and all
+// of d set
+void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, const double* aos, double* out, int dagger,
                 cudaStream_t st, int variant);
 void fx_tsl_init(const Lat<double>& L, cudaStream_t st);
 void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st);

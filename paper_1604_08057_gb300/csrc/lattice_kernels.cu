@@ -645,7 +645,7 @@ void apply_h(const Lat<R>& L, const R* in, R* out, int dagger, cudaStream_t st, 
   if constexpr (std::is_same<R, double>::value) {
     if (L.fu.e) {
       fx_encode(in, L.fr, L.nsrc, L.g.V, L.vs, st);
-      fx_apply_h(L, L.fr, in, out, dagger, 0, st, variant);
+      fx_apply_h(L, L.fr, in, nullptr, out, dagger, st, variant);
     } else {
       launch_apply<R, 1, 128, 0>(L, in, out, dagger, st);   // no fixed-point links (ov_apply_H_noalloc)
     }

@@ -2398,7 +2398,9 @@ int apply_h_impl(ov_context* c, const int32_t dims[4], const void* U, double mu,
     run(c, OV_KIND_LAYOUT, 1,
         [&] { fx_pack(static_cast<const double*>(in), L.fr, FxField{}, L.r, nsrc, L.g.V, L.vs, c->st); });
     run(c, OV_KIND_APPLY_H, 1,
-        [&] { fx_apply_h(L, L.fr, L.r, static_cast<double*>(out), dagger, 1, c->st, var); });
+        [&] {
+          fx_apply_h(L, L.fr, L.r, static_cast<const double*>(in), static_cast<double*>(out), dagger, c->st, var);
+        });
   } else if (var != APPLY_IL) {
     run(c, OV_KIND_LAYOUT, 1,
         [&] { pack_spinors<R>(static_cast<const double*>(in), L.r, nsrc, L.g.V, L.vs, c->st); });

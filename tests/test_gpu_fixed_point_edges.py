@@ -133,3 +133,16 @@ def test_a_source_does_not_depend_on_those_beside_it(dims, nsrc):
                 assert np.array_equal(one, all_), s
     finally:
         binding.nested_sign(0, **opts)
+
+
+@pytest.mark.parametrize("dims,nsrc", [((1, 2, 3, 2), 1), ((3, 5, 2, 4), 3), ((5, 3, 3, 3), 5)])
+def test_operator_returns_its_own_term_as_it_is(dims, nsrc):
+    """Without links H is gamma5: bit for bit, components of 2^-100 of their site's largest among them."""
+    rng = np.random.default_rng(46)
+    psi = inputs.gaussian_spinors(dims, nsrc, rng)
+    psi *= 2.0 ** rng.integers(-100, 0, size=psi.shape, endpoint=True)
+    u = np.zeros(inputs.lattice_shape(dims) + (4, 3, 3), dtype=np.complex128)
+    for dagger in (False, True):
+        got = binding.apply_H(T(u), MU, M_W, T(psi), dagger=dagger).cpu().numpy()
+        for s in range(nsrc):
+            assert np.array_equal(got[s], dirac.apply_gamma5(psi[s]))
