@@ -24,9 +24,8 @@ struct SrcScal {
   zd cr1, cr2, cs1, cs2; // g_r = cr1 Gv_{j+1} + cr2 w_{j+1};  g_s = cs1 Gw_{j+1} + cs2 v_{j+1}
 };
 
-// Fields in block fixed point (fx.cuh; which FP64 calls use them: struct Lat): vs reals per
-// field as in Lat (a field of Vp sites, a multiple of 32, takes 12 Vp int4 and Vp exponents:
-// vs = 24 Vp).
+// The FP64 operator's input and links in block fixed point (fx.cuh): a field of Vp sites (a
+// multiple of 32) takes 12 Vp int4 and Vp exponents, vs = 24 Vp reals as in Lat.
 struct FxLinks {
   const int4* e;
   const short* ex;
@@ -64,13 +63,10 @@ struct Lat {
   Geom gl;
   const R* ue;               // links of the direction E (internal layout) or null
   R mdir;                    // mu direction
-  // FP64 calls: fixed-point links (fu.e null: FP64 stencil), the fields of a fixed-point
-  // recurrence, and the exponents of fixed-point bases, whose integers are in bv and bw
+  // the FP64 operator: fixed-point links (fu.e null: FP64 stencil) and input, the user's links
   FxLinks fu;
-  const double* uaos;        // the user's links
-  FxField fr, fs, fp, fq;
-  short* bve; short* bwe;
-  OV_HD bool fx() const { return fs.c != nullptr; }   // the recurrence runs in fixed point
+  const double* uaos;
+  FxField fr;
   // basis window: vectors jbase .. jbase + kcap - 1 (all k from 0 unless segments are replayed)
   int kcap, jbase;
   OV_HD R* basis_v(int src, int j) const { return bv + ((int64_t)src * kcap + (j - jbase)) * vs; }
@@ -128,31 +124,17 @@ void apply_h_il(const Lat<float>& L, const float* in, float* out, int dagger, cu
 void pack_spinors_il(const double* aos, float* dst, int nsrc, int64_t V, cudaStream_t st);
 void unpack_spinors_il(const float* f, double* aos, int nsrc, int64_t V, cudaStream_t st);
 
-// FP64 calls (fx_kernels.cu); the launchers below dispatch to them
-// flush: links below the window to zero (else marked)
-void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, bool flush,
-                   cudaStream_t st);
-// user spinors to f and (if set) g; FP64 values of marked sites to d, or (d null) sites below the
-// window to zero
-void fx_pack(const double* aos, const FxField& f, const FxField& g, double* d, int nsrc, int64_t V, int64_t vs,
-             cudaStream_t st);
+// the FP64 operator in fixed point (fx_kernels.cu)
+void pack_links_fx(const double* u, int4* out, short* ex, int64_t V, double ef, double efinv, cudaStream_t st);
+// user spinors to f; FP64 values of marked sites to d, site-major
+void fx_pack(const double* aos, const FxField& f, double* d, int nsrc, int64_t V, int64_t vs, cudaStream_t st);
+// a site-major FP64 field to f
 void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t vs, cudaStream_t st);
 // in: the field in fixed point, d: its FP64 companion, site-major (read where a site is marked);
 // aos: the field as the user's array, with out in the same layout, or null: out site-major and all
 // of d set
 void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, const double* aos, double* out, int dagger,
                 cudaStream_t st, int variant);
-void fx_tsl_init(const Lat<double>& L, cudaStream_t st);
-void fx_tsl_stencil(const Lat<double>& L, int j, int need_q, cudaStream_t st);
-void fx_tsl_update(const Lat<double>& L, int j, int finalize, cudaStream_t st);
-// dots with vectors 0 .. nb - 1: out[2 i] = w_i^dag a, out[2 i + 1] = v_i^dag b
-void fx_proj_dots(const Lat<double>& L, int nb, const FxField& a, const FxField& b, int64_t ab_stride, zd* coef,
-                  zd* cpart, cudaStream_t st);
-// fin: omega and the next scales follow
-void fx_proj_update(const Lat<double>& L, int nb, const FxField& a, const FxField& b, int64_t ab_stride, const zd* coef,
-                    int j, int fin, cudaStream_t st);
-void fx_combine(const Lat<double>& L, int src0, int nsrc, int side, int j0, int nvec, const zd* y, int64_t ystride,
-                double* out, int accumulate, cudaStream_t st);
 
 template <typename R> void tsl_init(const Lat<R>& L, cudaStream_t st);
 template <typename R> void tsl_stencil(const Lat<R>& L, int j, bool need_q, cudaStream_t st, int variant = 0);

@@ -11,7 +11,6 @@
 
 #include "dslash.cuh"
 #include "kernels.h"
-#include "recurrence.cuh"
 
 namespace ov {
 
@@ -669,6 +668,53 @@ void apply_h(const Lat<R>& L, const R* in, R* out, int dagger, cudaStream_t st, 
 }
 
 // ---------------------------------------------------------------------------
+// helpers for the recurrence scalars
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ bool finite_z(zd a) { return isfinite(a.re) && isfinite(a.im); }
+
+__device__ __forceinline__ void flag_error(SrcScal& sc, int bit, int step) {
+  if (sc.err == 0) sc.err_step = step;
+  sc.err |= bit;
+}
+
+// Sum NV partial slots of this source (fixed block order); thread 0 gets the result.
+template <int NV>
+__device__ __forceinline__ void sum_partials(const zd* part, int nblk, zd (&out)[NV], zd* scratch) {
+  zd v[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) v[i] = mk(0.0, 0.0);
+  // each thread takes a contiguous range of blocks, so the order is fixed
+  for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = v[i] + ld_cg(part + i * nblk + b);
+  }
+  block_sum<NV>(v, scratch);
+#pragma unroll
+  for (int i = 0; i < NV; ++i) out[i] = v[i];
+}
+
+// omega = s^dag r, rr = r^dag r, ss = s^dag s  ->  delta_{j+1}, beta_{j+1} and the next scales
+template <typename R>
+__device__ void omega_finalize(const Lat<R>& L, int src, int j, zd om, double rr, double ss) {
+  SrcScal& sc = L.sc[src];
+  const double aom = sqrt(om.re * om.re + om.im * om.im);
+  if (!finite_z(om) || !isfinite(rr) || !isfinite(ss)) {
+    flag_error(sc, ERRB_NONFINITE, j + 1);
+    return;
+  }
+  if (aom <= 1e-14 * sqrt(rr * ss)) {
+    flag_error(sc, ERRB_BREAKDOWN, j + 1);
+    return;
+  }
+  const double d = sqrt(aom);
+  const zd bt = mk(om.re / d, om.im / d);
+  L.beta[(int64_t)src * L.k + j + 1] = bt;
+  L.delta[(int64_t)src * L.k + j + 1] = d;
+  sc.sv = mk(1.0 / d, 0.0);
+  sc.sw = zdiv(mk(1.0, 0.0), conj(bt));
+}
+
+// ---------------------------------------------------------------------------
 // TSL forward: initialisation (beta_0 = ||b||)
 // ---------------------------------------------------------------------------
 template <typename R>
@@ -697,14 +743,22 @@ __global__ void __launch_bounds__(BS) k_tsl_init(Lat<R> L) {
     zd s[2];
     sum_partials<2>(part, gridDim.x, s, scratch);
     if (threadIdx.x == 0) {
-      init_finalize(L, src, s[0].re, s[1]);
+      SrcScal& sc = L.sc[src];
+      sc.err = 0;
+      sc.err_step = -1;
+      const double b0 = sqrt(s[0].re);
+      sc.beta0 = b0;
+      if (!(b0 > 0.0) || !isfinite(b0)) flag_error(sc, ERRB_NONFINITE, 0);
+      sc.sv = mk(1.0 / b0, 0.0);
+      // w_1 = s sw with w_1^dag v_1 = 1: sw = beta_0 / conj(s^dag r); s = r in plain mode
+      sc.sw = L.block ? zdiv(mk(b0, 0.0), conj(s[1])) : mk(1.0 / b0, 0.0);
+      L.beta[(int64_t)src * L.k] = mk(0.0, 0.0);
+      L.delta[(int64_t)src * L.k] = 0.0;
     }
   }
 }
 template <typename R>
 void tsl_init(const Lat<R>& L, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value)
-    if (L.fx()) return fx_tsl_init(L, st);
   k_tsl_init<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L);
 }
 
@@ -862,8 +916,6 @@ static void launch_pair(const Lat<R>& L, int j, int q, cudaStream_t st) {
 template <typename R>
 void tsl_stencil(const Lat<R>& L, int j, bool need_q, cudaStream_t st, int variant) {
   const int q = need_q ? 1 : 0;
-  if constexpr (std::is_same<R, double>::value)
-    if (L.fx()) return fx_tsl_stencil(L, j, q, st);
   if (L.block) {
     k_tsl_stencil_block<R><<<dim3(nblocks(L.gl.V, BS), L.nsrc), BS, 0, st>>>(L, j, q);
     return;
@@ -931,8 +983,6 @@ __global__ void __launch_bounds__(BS) k_tsl_update(Lat<R> L, int j, int finalize
 }
 template <typename R>
 void tsl_update(const Lat<R>& L, int j, bool finalize, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value)
-    if (L.fx()) return fx_tsl_update(L, j, finalize ? 1 : 0, st);
   k_tsl_update<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j, finalize ? 1 : 0);
 }
 
@@ -1259,15 +1309,11 @@ __global__ void __launch_bounds__(BS) k_ritz_combine(Lat<R> L, int src, int side
 }
 template <typename R>
 void ritz_combine(const Lat<R>& L, int src, int side, int nvec, const zd* y, double* out, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value)
-    if (L.bve) return fx_combine(L, src, 1, side, 0, nvec, y, 0, out, 0, st);   // bases in fixed point
   k_ritz_combine<R><<<nblocks(L.g.V, BS), BS, 0, st>>>(L, src, side, nvec, y, out);
 }
 
 template <typename R>
 void combine_range(const Lat<R>& L, int j0, int nvec, const zd* y, double* out, bool acc, cudaStream_t st) {
-  if constexpr (std::is_same<R, double>::value)
-    if (L.fx()) return fx_combine(L, 0, L.nsrc, 0, j0, nvec, y, L.k, out, acc ? 1 : 0, st);
   k_combine<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, j0, nvec, y, out, acc ? 1 : 0);
 }
 template <typename R>
@@ -1306,13 +1352,44 @@ __global__ void __launch_bounds__(BS) k_rev_dots(Lat<R> L, Rev<R> B, int j) {
     zd s[2];
     sum_partials<2>(part, gridDim.x, s, scratch);
     if (threadIdx.x == 0) {
-      rev_dots_epilogue(L, B, src, j, s);
+      SrcScal& sc = L.sc[src];
+      const int64_t o = (int64_t)src * L.k + j + 1;
+      const double d = L.delta[o];
+      const zd bt = L.beta[o];
+      const zd om = mk(bt.re * d, bt.im * d);
+      const double aom = d * d;
+      double g_d = B.gdT[o] + sc.carry_delta - s[0].re / d;
+      zd g_b = B.gbT[o] + sc.carry_beta - zdiv(conj(s[1]), conj(bt));
+      zd g_w = mk(g_b.re / d, g_b.im / d);
+      g_d -= (om.re * g_b.re + om.im * g_b.im) / (d * d);      // Re(conj(om) g_b)
+      const double f = g_d / (2.0 * d * aom);
+      g_w = g_w + mk(f * om.re, f * om.im);
+      sc.cr1 = mk(1.0 / d, 0.0);
+      sc.cr2 = conj(bt) * g_w;
+      sc.cs1 = zdiv(mk(1.0, 0.0), bt);
+      sc.cs2 = mk(d * g_w.re, -d * g_w.im);
+      if (!finite_z(sc.cr2) || !finite_z(sc.cs2)) flag_error(sc, ERRB_NONFINITE, j);
     }
   }
 }
 template <typename R>
 void rev_dots(const Lat<R>& L, const Rev<R>& B, int j, cudaStream_t st) {
   k_rev_dots<R><<<dim3(nblocks(L.g.V, site_bs(L.g.V)), L.nsrc), site_bs(L.g.V), 0, st>>>(L, B, j);
+}
+
+// D1 = v_j^dag g_r, D2 = w_j^dag g_s, D3 = v_{j-1}^dag g_r, D4 = w_{j-1}^dag g_s -> g_alpha, carries
+template <typename R>
+__device__ void alpha_epilogue(const Lat<R>& L, const Rev<R>& B, int src, int j, const zd (&s)[4]) {
+  SrcScal& sc = L.sc[src];
+  const int64_t o = (int64_t)src * L.k + j;
+  sc.g_alpha = B.gaT[o] - s[0] - conj(s[1]);
+  if (j > 0) {
+    sc.carry_beta = -s[2];
+    sc.carry_delta = -s[3].re;
+  } else {
+    sc.carry_beta = mk(0.0, 0.0);
+    sc.carry_delta = 0.0;
+  }
 }
 
 template <typename R>

@@ -23,7 +23,7 @@ enum BufId {
   B_LINKS, B_BV, B_BW, B_P, B_Q, B_R, B_S, B_SC, B_ALPHA, B_BETA, B_DELTA, B_PART, B_CNT, B_COEF, B_CPART,
   B_T, B_X, B_XI, B_XN, B_E, B_EN, B_TMP1, B_TMP2, B_IPIV, B_PROW, B_COL, B_DSTAT, B_DPART, B_DCNT, B_DERR,
   B_Y, B_GY, B_GA, B_GB, B_GD, B_XBAR, B_GV, B_GW, B_GV2, B_GW2, B_GR, B_GS, B_GP, B_EV, B_EW, B_REB,
-  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, B_FXL, B_FXE, B_FXR, B_FXRE, B_FXS, B_FXSE, B_FXP, B_FXPE, B_FXQ, B_FXQE, B_BVE, B_BWE, B_CKRE, B_CKSE, B_CKVE, B_CKWE, NBUF
+  B_FORCE, B_DMU, B_DMUPART, B_DMUCNT, B_W0, B_W1, B_REC, B_RECLD, B_ELINKS, B_BLOCKOUT, B_HIN, B_CKR, B_CKS, B_CKV, B_CKW, B_CKSC, B_FSIGN, B_ACT, B_SCAL, B_RSCAL, B_FPARTS, B_LRA, B_LRB, B_BETA0, B_EPS1T, B_EPS1B, B_EPS2T, B_EPS2B, B_EPSN, B_NSPART, B_NSCNT, B_OVX, B_OVB, B_GMV, B_GMW, B_GMR, B_GMH, B_GMP, B_CHI, B_CURX1, B_CURX2, B_CURG1, B_CURG2, B_AERR, B_OZ, B_DFA, B_DFC, B_DFSA, B_DFSC, B_DFPART, B_DFTOP, B_DFBOT, B_DFSG, B_RZY, B_RZF, B_RZH, B_RZD, B_EDT1, B_EDT2, B_EDX, B_EDC, B_CGY, B_CGR, B_CGP, B_CGQ, B_CGT, B_CGC, B_SIQ, B_SILT, B_SIT1, B_SIC, B_SIP, B_NLU, B_NPIV, B_NS, B_NQ, B_NW, B_NH, B_NHN, B_NMEFF, B_NHC, B_NHCN, B_NTA, B_NTB, B_NTD, B_NTY, B_NHB, B_NWN, B_FXL, B_FXE, B_FXR, B_FXRE, NBUF
 };
 
 struct Status {
@@ -73,7 +73,6 @@ struct ov_context {
   int last_k = 0, last_nsrc = 0;
   // shape of the last forward pass whose bases stay in B_BV / B_BW (for ov_tsl_ritz_triples)
   int last_block = 0, last_seg = 0, last_prec = -1;
-  bool last_fx = false;   // the last forward pass left its bases in fixed point
   int32_t last_dims[4] = {0, 0, 0, 0};
   cudaEvent_t ev[8] = {};
   Prof* prof = nullptr;
@@ -313,46 +312,19 @@ template <typename R>
 int64_t field_reals(int64_t V) {
   return std::is_same<R, double>::value ? (V + 31) / 32 * 32 * 24 : ((24 * V + 63) / 64) * 64;
 }
-// n fixed-point fields of vs reals
-FxField fx_fields(ov_context* c, int id, int id_e, int64_t n, int64_t vs) {
-  return FxField{wsT<int4>(c, id, n * (vs / 2)), wsT<short>(c, id_e, n * (vs / 24))};
-}
-// the user's spinors into the recurrence's r and s (equal at the start)
-template <typename R>
-void pack_start(ov_context* c, const Lat<R>& L, const void* b) {
-  const double* bd = static_cast<const double*>(b);
-  if constexpr (std::is_same<R, double>::value) {
-    if (L.fx()) {
-      run(c, OV_KIND_LAYOUT, 1, [&] { fx_pack(bd, L.fr, L.fs, nullptr, L.nsrc, L.g.V, L.vs, c->st); });
-      return;
-    }
-  }
-  run(c, OV_KIND_LAYOUT, 2, [&] {
-    pack_spinors<R>(bd, L.r, L.nsrc, L.g.V, L.vs, c->st);
-    pack_spinors<R>(bd, L.s, L.nsrc, L.g.V, L.vs, c->st);
-  });
-}
 
-// What a call's Lat holds beside the scalars: links and p, q, r, s in R, or (FP64 calls) in
-// fixed point (fx.cuh), as the call's kernels read them.
-//   The operator: fixed-point links and input; marked sites and their neighbours in FP64.
-//   sgn(H) b where the result is x alone (the nested k x k stage, the overlap operator,
-//   eps_A): the recurrence in fixed point.
-//   ov_tsl_sign, its derivatives and tapes: FP64.  The derivative of sgn at T_k grows without
-//   bound as a Ritz value comes near Re z = 0, and with it what a change of rounding in the
-//   recurrence or in the reverse sweep does to dU and dmu (from FP64 to fixed point and back:
-//   up to 3e-7 at mu = 0.3 and 0.5, on lattices of every size, where x moves by less than
-//   1e-12 and the error of either is as large).  ov_tsl_sign's x is the tape's, bit for bit.
+// What a call's Lat holds beside the scalars.  The FP64 operator runs in fixed point (fx.cuh).
+// Every sgn(H) b and its derivatives run in FP64.  A fixed-point recurrence gives T_k to half
+// the FP64 one's error, but the derivative of sgn at T_k grows without bound as a Ritz value
+// comes near Re z = 0, and with it what a change of rounding in the recurrence or the reverse
+// sweep does to dU and dmu (up to 3e-7 at mu = 0.3 and 0.5, on lattices of every size, where x
+// moves by less than 1e-12 at m_w = -1 and 1e-9 at -2).  All of them share one recurrence, so
+// that the x of a tape, of the nested stage and of the plain sign stay one x.
 enum : int {
   LAT_LINKS = 1,      // u
   LAT_FIELDS = 2,     // p, q, r, s
-  LAT_FX_LINKS = 4,   // fu
-  LAT_FX_IN = 8,      // fr
-  LAT_FX_STEP = 16,   // fr, fs, fp, fq and the bases' exponents: the recurrence in fixed point
-  LAT_FX_BASES = 32,  // the bases' exponents
-  LAT_PLAIN = LAT_LINKS | LAT_FIELDS,
-  LAT_OPERATOR = LAT_FIELDS | LAT_FX_LINKS | LAT_FX_IN,
-  LAT_FX_SIGN = LAT_FX_LINKS | LAT_FX_STEP
+  LAT_OPERATOR = 4,   // p, r, and of FP64 calls fu, fr
+  LAT_PLAIN = LAT_LINKS | LAT_FIELDS
 };
 // fm = 2 sets up block mode: fields of 2V sites (upper and lower halves).  parts: of FP64
 // calls (FP32 ones have LAT_PLAIN)
@@ -371,20 +343,20 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   L.efinv = (R)std::exp(-mu);
   L.nsrc = nsrc;
   L.k = k;
-  if (!std::is_same<R, double>::value) parts = LAT_PLAIN;
+  if (!std::is_same<R, double>::value) parts = LAT_PLAIN;   // (the FP32 operator: any of its forms)
   L.vs = field_reals<R>(V);
   if (parts & LAT_LINKS) {
     R* u = wsT<R>(c, B_LINKS, link_reals<R>() * V);
     L.u = u;
     run(c, OV_KIND_LAYOUT, 1, [&] { pack_links<R>(static_cast<const double*>(U), u, V, c->st); });
   }
-  if (parts & LAT_FX_LINKS) {
+  if (parts & LAT_OPERATOR) {
     L.uaos = static_cast<const double*>(U);
     int4* fe = wsT<int4>(c, B_FXL, fx_link_ints(V));
     short* ex = wsT<short>(c, B_FXE, 5 * V);
     L.fu = FxLinks{fe, ex};
     run(c, OV_KIND_LAYOUT, 1,
-        [&] { pack_links_fx(static_cast<const double*>(U), fe, ex, V, L.ef, L.efinv, !(parts & LAT_FX_IN), c->st); });
+        [&] { pack_links_fx(static_cast<const double*>(U), fe, ex, V, L.ef, L.efinv, c->st); });
   }
   launch_check();
   if (fm == 2) {
@@ -398,23 +370,15 @@ Lat<R> setup(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
   if (basis) {
     L.bv = wsT<R>(c, B_BV, (int64_t)nsrc * L.kcap * L.vs);
     L.bw = wsT<R>(c, B_BW, (int64_t)nsrc * L.kcap * L.vs);
-    if (parts & (LAT_FX_STEP | LAT_FX_BASES)) {
-      L.bve = wsT<short>(c, B_BVE, (int64_t)nsrc * L.kcap * (L.vs / 24));
-      L.bwe = wsT<short>(c, B_BWE, (int64_t)nsrc * L.kcap * (L.vs / 24));
-    }
   }
+  L.p = wsT<R>(c, B_P, nsrc * L.vs);
+  L.r = wsT<R>(c, B_R, nsrc * L.vs);
   if (parts & LAT_FIELDS) {
-    L.p = wsT<R>(c, B_P, nsrc * L.vs);
     L.q = wsT<R>(c, B_Q, nsrc * L.vs);
-    L.r = wsT<R>(c, B_R, nsrc * L.vs);
     L.s = wsT<R>(c, B_S, nsrc * L.vs);
   }
-  if (parts & (LAT_FX_IN | LAT_FX_STEP)) L.fr = fx_fields(c, B_FXR, B_FXRE, nsrc, L.vs);
-  if (parts & LAT_FX_STEP) {
-    L.fs = fx_fields(c, B_FXS, B_FXSE, nsrc, L.vs);
-    L.fp = fx_fields(c, B_FXP, B_FXPE, nsrc, L.vs);
-    L.fq = fx_fields(c, B_FXQ, B_FXQE, nsrc, L.vs);
-  }
+  if (parts & LAT_OPERATOR)
+    L.fr = FxField{wsT<int4>(c, B_FXR, nsrc * (L.vs / 2)), wsT<short>(c, B_FXRE, nsrc * (L.vs / 24))};
   L.sc = wsT<SrcScal>(c, B_SC, nsrc);
   L.alpha = wsT<zd>(c, B_ALPHA, (int64_t)nsrc * k);
   L.beta = wsT<zd>(c, B_BETA, (int64_t)nsrc * k);
@@ -474,7 +438,6 @@ void forward_krylov(ov_context* c, Lat<R>& L) {
   const int64_t nsb = (L.g.V + 127) / 128;
   zd* coef = wsT<zd>(c, B_COEF, (int64_t)L.nsrc * 2 * k);
   zd* cpart = wsT<zd>(c, B_CPART, (int64_t)L.nsrc * 2 * k * nsb);
-  L.uaos = nullptr;   // the caller's array: not part of a captured sweep or its key
   std::vector<unsigned char> key;
   key_add(key, L);
   key_add(key, coef);
@@ -492,18 +455,9 @@ void forward_krylov(ov_context* c, Lat<R>& L) {
       run(c, OV_KIND_UPDATE, 1, [&] { tsl_update(L, j, !reb, c->st); });
       if (reb) {
         for (int ps = 0; ps < c->opt.passes; ++ps) {
-          const bool last = ps == c->opt.passes - 1;
-          if constexpr (std::is_same<R, double>::value) {
-            if (L.fx()) {
-              run(c, OV_KIND_PROJ_DOTS, 2, [&] { fx_proj_dots(L, j + 1, L.fr, L.fs, L.vs, coef, cpart, c->st); });
-              run(c, OV_KIND_PROJ_UPDATE, 1,
-                  [&] { fx_proj_update(L, j + 1, L.fr, L.fs, L.vs, coef, j, last, c->st); });
-              continue;
-            }
-          }
           run(c, OV_KIND_PROJ_DOTS, 2, [&] { proj_dots(L, j, 0, L.r, L.s, L.vs, coef, cpart, c->st); });
           run(c, OV_KIND_PROJ_UPDATE, 1,
-              [&] { proj_update(L, j, 0, L.r, L.s, L.vs, coef, last, c->st, ps > 0); });
+              [&] { proj_update(L, j, 0, L.r, L.s, L.vs, coef, ps == c->opt.passes - 1, c->st, ps > 0); });
         }
       }
       inject_after_update(c, L, j);
@@ -528,14 +482,8 @@ int run_diagnostics(ov_context* c, const Lat<R>& L, bool segments, ov_tsl_info* 
     zd* coef = wsT<zd>(c, B_COEF, (int64_t)nsrc * 2 * k);
     zd* cpart = wsT<zd>(c, B_CPART, (int64_t)nsrc * 2 * k * nsb);
     run(c, OV_KIND_PROJ_DOTS, 2, [&] {
-      if constexpr (std::is_same<R, double>::value) {
-        if (L.fx()) {
-          const FxField v{reinterpret_cast<int4*>(L.basis_v(0, k - 1)), L.bve + (int64_t)(k - 1) * (L.vs / 24)};
-          const FxField w{reinterpret_cast<int4*>(L.basis_w(0, k - 1)), L.bwe + (int64_t)(k - 1) * (L.vs / 24)};
-          return fx_proj_dots(L, k, v, w, (int64_t)L.kcap * L.vs, coef, cpart, c->st);
-        }
-      }
-      proj_dots(L, k - 1, 0, L.basis_v(0, k - 1), L.basis_w(0, k - 1), (int64_t)L.kcap * L.vs, coef, cpart, c->st);
+      proj_dots(L, k - 1, 0, L.basis_v(0, k - 1), L.basis_w(0, k - 1), (int64_t)L.kcap * L.vs, coef, cpart,
+                c->st);
     });
     launch_check();
     std::vector<zd> h((size_t)nsrc * 2 * k);
@@ -616,55 +564,27 @@ SegPlan seg_plan(int k, int S) {
 
 template <typename R>
 struct SegStore {
-  R *r, *s, *v, *w;           // [segment][src][vs]
-  SrcScal* sc;                // [segment][src]
-  short *re, *se, *ve, *we;   // fixed-point recurrence: the exponents of the above
+  R *r, *s, *v, *w;   // [segment][src][vs]
+  SrcScal* sc;        // [segment][src]
 };
 template <typename R>
 SegStore<R> seg_store(ov_context* c, const Lat<R>& L, int nseg) {
   const int64_t n = (int64_t)nseg * L.nsrc * L.vs;
-  SegStore<R> K{wsT<R>(c, B_CKR, n), wsT<R>(c, B_CKS, n), wsT<R>(c, B_CKV, n), wsT<R>(c, B_CKW, n),
-                wsT<SrcScal>(c, B_CKSC, (int64_t)nseg * L.nsrc), nullptr, nullptr, nullptr, nullptr};
-  if (L.fx()) {
-    K.re = wsT<short>(c, B_CKRE, n / 24);
-    K.se = wsT<short>(c, B_CKSE, n / 24);
-    K.ve = wsT<short>(c, B_CKVE, n / 24);
-    K.we = wsT<short>(c, B_CKWE, n / 24);
-  }
-  return K;
+  return SegStore<R>{wsT<R>(c, B_CKR, n), wsT<R>(c, B_CKS, n), wsT<R>(c, B_CKV, n), wsT<R>(c, B_CKW, n),
+                     wsT<SrcScal>(c, B_CKSC, (int64_t)nseg * L.nsrc)};
 }
-// copy the recurrence's r and s to (or from) the checkpoint of segment t
+// copy the window's first vector (v_{jbase}, w_{jbase}) of every source to or from a checkpoint
 template <typename R>
-void seg_rs(ov_context* c, const Lat<R>& L, const SegStore<R>& K, size_t t, bool restore) {
-  const int64_t fs = (int64_t)L.nsrc * L.vs;
-  auto copy = [&](void* live, void* kept, size_t bytes) {
-    CK(cudaMemcpyAsync(restore ? live : kept, restore ? kept : live, bytes, cudaMemcpyDeviceToDevice, c->st));
-  };
-  if (L.fx()) {
-    copy(L.fr.c, K.r + t * fs, sizeof(R) * fs);
-    copy(L.fs.c, K.s + t * fs, sizeof(R) * fs);
-    copy(L.fr.e, K.re + t * (fs / 24), sizeof(short) * (fs / 24));
-    copy(L.fs.e, K.se + t * (fs / 24), sizeof(short) * (fs / 24));
+void window_slot(ov_context* c, const Lat<R>& L, int slot, R* v, R* w, bool to_window) {
+  const size_t pitch = sizeof(R) * L.kcap * L.vs, width = sizeof(R) * L.vs;
+  R* bv = L.bv + (int64_t)slot * L.vs;
+  R* bw = L.bw + (int64_t)slot * L.vs;
+  if (to_window) {
+    CK(cudaMemcpy2DAsync(bv, pitch, v, width, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
+    CK(cudaMemcpy2DAsync(bw, pitch, w, width, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
   } else {
-    copy(L.r, K.r + t * fs, sizeof(R) * fs);
-    copy(L.s, K.s + t * fs, sizeof(R) * fs);
-  }
-}
-// copy a window slot's vectors (v, w of every source) to or from the checkpoint of segment t
-template <typename R>
-void window_slot(ov_context* c, const Lat<R>& L, int slot, const SegStore<R>& K, size_t t, bool to_window) {
-  const int64_t fs = (int64_t)L.nsrc * L.vs;
-  auto copy = [&](void* win, void* kept, size_t elem) {   // vectors of vs reals (or vs / 24 exponents)
-    const size_t n = elem == sizeof(short) ? L.vs / 24 : L.vs, width = elem * n, pitch = width * L.kcap;
-    char* w = static_cast<char*>(win) + slot * width;
-    if (to_window) CK(cudaMemcpy2DAsync(w, pitch, kept, width, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
-    else CK(cudaMemcpy2DAsync(kept, width, w, pitch, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
-  };
-  copy(L.bv, K.v + t * fs, sizeof(R));
-  copy(L.bw, K.w + t * fs, sizeof(R));
-  if (L.fx()) {
-    copy(L.bve, K.ve + t * (fs / 24), sizeof(short));
-    copy(L.bwe, K.we + t * (fs / 24), sizeof(short));
+    CK(cudaMemcpy2DAsync(v, width, bv, pitch, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
+    CK(cudaMemcpy2DAsync(w, width, bw, pitch, width, L.nsrc, cudaMemcpyDeviceToDevice, c->st));
   }
 }
 // steps j0 .. j1-1 without re-biorthogonalisation; with `next`, also the stencil of
@@ -684,18 +604,20 @@ void seg_steps(ov_context* c, Lat<R>& L, int j0, int j1, bool next) {
 // pass 1: the recurrence over all segments, checkpointing each segment start
 template <typename R>
 void seg_forward(ov_context* c, Lat<R>& L, const SegPlan& P, const SegStore<R>& K) {
+  const int64_t fs = (int64_t)L.nsrc * L.vs;
   run(c, OV_KIND_UPDATE, 1, [&] { tsl_init(L, c->st); });
   for (size_t t = 0; t < P.lo.size(); ++t) {
     const int j0 = P.lo[t];
     if (t > 0) {
       // v_{j0-1} moves from the end of the previous window to its first slot
-      window_slot(c, L, j0 - L.jbase - 1, K, t, false);
+      window_slot(c, L, j0 - L.jbase - 1, K.v + (int64_t)t * fs, K.w + (int64_t)t * fs, false);
       L.jbase = j0 - 1;
-      window_slot(c, L, 0, K, t, true);
+      window_slot(c, L, 0, K.v + (int64_t)t * fs, K.w + (int64_t)t * fs, true);
     } else {
       L.jbase = j0 - 1;
     }
-    seg_rs(c, L, K, t, false);
+    CK(cudaMemcpyAsync(K.r + t * fs, L.r, sizeof(R) * fs, cudaMemcpyDeviceToDevice, c->st));
+    CK(cudaMemcpyAsync(K.s + t * fs, L.s, sizeof(R) * fs, cudaMemcpyDeviceToDevice, c->st));
     CK(cudaMemcpyAsync(K.sc + t * L.nsrc, L.sc, sizeof(SrcScal) * L.nsrc, cudaMemcpyDeviceToDevice, c->st));
     seg_steps(c, L, j0, P.hi[t], false);
   }
@@ -704,10 +626,12 @@ void seg_forward(ov_context* c, Lat<R>& L, const SegPlan& P, const SegStore<R>& 
 // replay segment t from its checkpoint (with `next`: also v_{j1}, w_{j1})
 template <typename R>
 void seg_replay(ov_context* c, Lat<R>& L, const SegPlan& P, const SegStore<R>& K, int t, bool next) {
+  const int64_t fs = (int64_t)L.nsrc * L.vs;
   const int j0 = P.lo[t];
   L.jbase = j0 - 1;
-  if (t > 0) window_slot(c, L, 0, K, (size_t)t, true);
-  seg_rs(c, L, K, (size_t)t, true);
+  if (t > 0) window_slot(c, L, 0, K.v + (int64_t)t * fs, K.w + (int64_t)t * fs, true);
+  CK(cudaMemcpyAsync(L.r, K.r + t * fs, sizeof(R) * fs, cudaMemcpyDeviceToDevice, c->st));
+  CK(cudaMemcpyAsync(L.s, K.s + t * fs, sizeof(R) * fs, cudaMemcpyDeviceToDevice, c->st));
   // only the forward scalars: the reverse sweep keeps its own in the same structs
   CK(cudaMemcpy2DAsync(L.sc, sizeof(SrcScal), K.sc + t * L.nsrc, sizeof(SrcScal), offsetof(SrcScal, g_alpha),
                        L.nsrc, cudaMemcpyDeviceToDevice, c->st));
@@ -1037,16 +961,17 @@ float elapsed(cudaEvent_t a, cudaEvent_t b) {
   return ms;
 }
 
-// alone: no derivative of this x is taken and none has to equal it
 template <typename R>
 int tsl_sign_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, double m_w, int nsrc,
-                  const void* b, int k, void* x, ov_tsl_info* info, bool alone) {
+                  const void* b, int k, void* x, ov_tsl_info* info) {
   check_ptr(b);
   check_ptr(x);
   const int S = c->opt.segment > 0 && c->opt.segment < k ? c->opt.segment : 0;
-  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0,
-                      alone || c->opt.nested > 0 ? LAT_FX_SIGN : LAT_PLAIN);
-  pack_start(c, L, b);
+  Lat<R> L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0);
+  run(c, OV_KIND_LAYOUT, 2, [&] {
+    pack_spinors<R>(static_cast<const double*>(b), L.r, nsrc, L.g.V, L.vs, c->st);
+    pack_spinors<R>(static_cast<const double*>(b), L.s, nsrc, L.g.V, L.vs, c->st);
+  });
   SegPlan P;
   SegStore<R> K{};
   CK(cudaEventRecord(c->ev[0], c->st));
@@ -1066,7 +991,6 @@ int tsl_sign_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   c->last_block = 0;
   c->last_seg = S > 0 ? 1 : 0;
   c->last_prec = c->opt.precision;
-  c->last_fx = L.fx();
   std::copy(dims, dims + 4, c->last_dims);
   if (info) info->k_reached = kr;
   if (st != OV_OK) return st;
@@ -1139,7 +1063,6 @@ int block_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, d
   c->last_block = 1;
   c->last_seg = 0;
   c->last_prec = c->opt.precision;
-  c->last_fx = L.fx();
   std::copy(dims, dims + 4, c->last_dims);
   if (info) info->k_reached = kr;
   if (st != OV_OK) return st;
@@ -1194,8 +1117,7 @@ int ritz_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, do
               double tol, int32_t* l_out, double* lam, void* Rv, void* Lv, double* resid) {
   check_ptr(Rv);
   check_ptr(Lv);
-  Lat<R> L = setup<R>(c, dims, U, mu, m_w, c->last_nsrc, k, true, 1, 0,
-                      LAT_OPERATOR | (c->last_fx ? LAT_FX_BASES : 0));
+  Lat<R> L = setup<R>(c, dims, U, mu, m_w, c->last_nsrc, k, true, 1, 0, LAT_OPERATOR);
   const int64_t V = L.g.V, n = 12 * V, fd = 24 * V;
   std::vector<double> al(2 * k), be(2 * k), de(k), th(2 * k);
   CK(cudaMemcpyAsync(al.data(), L.alpha + (int64_t)src * k, sizeof(zd) * k, cudaMemcpyDeviceToHost, c->st));
@@ -1345,7 +1267,7 @@ int deflated_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   }
   launch_check();
   const int st = block ? block_impl<R>(c, dims, U, mu, m_w, nsrc, top, bot, k, E, m_dir, dx, x, info)
-                       : tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, bot, k, x, info, false);
+                       : tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, bot, k, x, info);
   if (st != OV_OK) return st;
   if (l > 0) {
     double* xd = static_cast<double*>(x);
@@ -1388,11 +1310,11 @@ int eps_impl(ov_context* c, const int32_t dims[4], const void* U, double mu, dou
     one = ov_tsl_info{};
     st = block_impl<R>(c, dims, U, mu, m_w, nsrc, t1, b1, k, E, m_dir, t2, b2, &one);
   } else {
-    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b, k, b1, &one, true);
+    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b, k, b1, &one);
     merge_info(info, one);
     if (st != OV_OK) return st;
     one = ov_tsl_info{};
-    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b1, k, b2, &one, true);
+    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b1, k, b2, &one);
   }
   merge_info(info, one);
   if (st != OV_OK) return st;
@@ -1441,7 +1363,10 @@ int vjp_forward(ov_context* c, const int32_t dims[4], const void* U, double mu, 
   F.L = setup<R>(c, dims, U, mu, m_w, nsrc, k, true, 1, S > 0 ? S + 2 : 0);
   Lat<R>& L = F.L;
   const int64_t V = L.g.V, vs = L.vs;
-  pack_start(c, L, b);
+  run(c, OV_KIND_LAYOUT, 2, [&] {
+    pack_spinors<R>(static_cast<const double*>(b), L.r, nsrc, V, vs, c->st);
+    pack_spinors<R>(static_cast<const double*>(b), L.s, nsrc, V, vs, c->st);
+  });
   CK(cudaEventRecord(c->ev[0], c->st));
   if (S > 0) {
     F.P = seg_plan(k, S);
@@ -1459,7 +1384,6 @@ int vjp_forward(ov_context* c, const int32_t dims[4], const void* U, double mu, 
   c->last_block = 0;
   c->last_seg = S > 0 ? 1 : 0;
   c->last_prec = c->opt.precision;
-  c->last_fx = L.fx();
   std::copy(dims, dims + 4, c->last_dims);
   if (info) info->k_reached = kr;
   if (st != OV_OK) return st;
@@ -1849,13 +1773,13 @@ int overlap_apply_impl(ov_context* c, const int32_t dims[4], const void* U, doub
   double* xs = wsT<double>(c, B_OVX, 2 * n);
   int st;
   if (!dagger) {
-    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b, k, xs, info, true);
+    st = tsl_sign_impl<R>(c, dims, U, mu, m_w, nsrc, b, k, xs, info);
     if (st != OV_OK) return st;
     run(c, OV_KIND_COMBINE, 1, [&] { ov_combine(bd, xs, od, n, 1, c->st); });
   } else {
     double* g5b = wsT<double>(c, B_OVB, 2 * n);
     run(c, OV_KIND_COMBINE, 1, [&] { gamma5_scale(bd, g5b, n, 1.0, 0.0, c->st); });
-    st = tsl_sign_impl<R>(c, dims, U, -mu, m_w, nsrc, g5b, k, xs, info, true);
+    st = tsl_sign_impl<R>(c, dims, U, -mu, m_w, nsrc, g5b, k, xs, info);
     if (st != OV_OK) return st;
     run(c, OV_KIND_COMBINE, 1, [&] { ov_combine(bd, xs, od, n, 0, c->st); });
   }
@@ -2396,11 +2320,10 @@ int apply_h_impl(ov_context* c, const int32_t dims[4], const void* U, double mu,
   }
   if constexpr (fx) {
     run(c, OV_KIND_LAYOUT, 1,
-        [&] { fx_pack(static_cast<const double*>(in), L.fr, FxField{}, L.r, nsrc, L.g.V, L.vs, c->st); });
-    run(c, OV_KIND_APPLY_H, 1,
-        [&] {
-          fx_apply_h(L, L.fr, L.r, static_cast<const double*>(in), static_cast<double*>(out), dagger, c->st, var);
-        });
+        [&] { fx_pack(static_cast<const double*>(in), L.fr, L.r, nsrc, L.g.V, L.vs, c->st); });
+    run(c, OV_KIND_APPLY_H, 1, [&] {
+      fx_apply_h(L, L.fr, L.r, static_cast<const double*>(in), static_cast<double*>(out), dagger, c->st, var);
+    });
   } else if (var != APPLY_IL) {
     run(c, OV_KIND_LAYOUT, 1,
         [&] { pack_spinors<R>(static_cast<const double*>(in), L.r, nsrc, L.g.V, L.vs, c->st); });
@@ -2423,9 +2346,6 @@ int autotune_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   CK(cudaMemsetAsync(L.r, 0, sizeof(R) * nsrc * L.vs, c->st));
   CK(cudaMemsetAsync(L.s, 0, sizeof(R) * nsrc * L.vs, c->st));
   CK(cudaMemsetAsync(L.sc, 0, sizeof(SrcScal) * nsrc, c->st));
-  if constexpr (std::is_same<R, double>::value) {
-    fx_encode(L.r, L.fr, nsrc, L.g.V, L.vs, c->st);
-  }
   cudaEvent_t e0 = c->ev[6], e1 = c->ev[7];
   auto time_us = [&](auto&& launch) {
     launch();
@@ -2672,8 +2592,8 @@ int ov_tsl_sign(ov_context* c, const int32_t dims[4], const void* U, double mu, 
   if (!c || k < 2 || k > 4096) return OV_ERR_INVALID_ARG;
   if (info) std::memset(info, 0, sizeof(*info));
   return guarded([&] {
-    return c->opt.precision == OV_MIXED ? tsl_sign_impl<float>(c, dims, U, mu, m_w, nsrc, b, k, x, info, false)
-                                        : tsl_sign_impl<double>(c, dims, U, mu, m_w, nsrc, b, k, x, info, false);
+    return c->opt.precision == OV_MIXED ? tsl_sign_impl<float>(c, dims, U, mu, m_w, nsrc, b, k, x, info)
+                                        : tsl_sign_impl<double>(c, dims, U, mu, m_w, nsrc, b, k, x, info);
   });
 }
 
