@@ -16,7 +16,8 @@
 // with their own scale E: units of 2^(E - 2100), kept to some 2^-56 of the largest
 // contribution to the site, against 2^-53 per operation in FP64 arithmetic.
 // Infinities, NaN and magnitudes outside the window below mark a site (FX_BAD), and
-// every sum that meets a marked site or link is formed in FP64.
+// every sum that meets a marked site or link, or whose terms may leave FP64's range, is
+// formed in FP64.
 //
 // The Lanczos recurrence and its derivatives stay in FP64: see setup() in ov_api.cu.
 #pragma once
@@ -51,10 +52,6 @@ __device__ __forceinline__ fxll fx_sar(fxll v, int n) {
 __device__ __forceinline__ unsigned fx_mag(double d) { return (unsigned)__double2hiint(d) & 0x7fffffffu; }
 // 2^s as an FP64 number, |s| <= 1022
 __device__ __forceinline__ double fx_pow2(int s) { return __hiloint2double((s + 1023) * (1 << 20), 0); }
-// 2^s for any s an exponent sum can give (0 or infinity past the FP64 range)
-__device__ __forceinline__ double fx_pow2_wide(int s) {
-  return s < -1022 ? 0.0 : s > 1023 ? __longlong_as_double(0x7ff0000000000000ll) : fx_pow2(s);
-}
 
 // d 2^(1079 - e) to the nearest integer (|d| < 2^(e - 1022) gives 57 bits), in integer
 // operations: a conversion instruction runs at the FP64 rate
@@ -155,9 +152,11 @@ __device__ __forceinline__ void fx_zero(FxHalf& a, int E) {
   for (int i = 0; i < 6; ++i) a.v[i] = FxZ{0, 0};
   a.E = E;
 }
+// whether a sum's unit is a normal FP64 number (E includes FX_BAD's)
+__device__ __forceinline__ bool fx_scale_ok(int E) { return E >= FX_E_BIAS - 1022 && E <= FX_E_BIAS + 1023; }
 // the sum's FP64 values
 __device__ __forceinline__ void fx_double(const FxHalf& a, zd (&o)[6]) {
-  const double u = fx_pow2_wide(a.E - FX_E_BIAS);
+  const double u = fx_pow2(a.E - FX_E_BIAS);
 #pragma unroll
   for (int i = 0; i < 6; ++i) o[i] = mk(u * (double)a.v[i].re, u * (double)a.v[i].im);
 }

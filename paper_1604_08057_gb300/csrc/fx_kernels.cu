@@ -131,7 +131,7 @@ void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t v
 // ov_apply_H
 // ---------------------------------------------------------------------------
 // FP64 hop sum from the user's links [site][direction][3][3] (out of line: reached only where
-// a site or link is marked)
+// a site or link is marked or the products may under- or overflow)
 template <int NU>
 __device__ __forceinline__ void hops_fp64_dir(Spinor<double>& acc, const FxLoad& ld, const double2* u, const Geom& g,
                                               int64_t x, const int c[4], double ff, double fb) {
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(128, 4) k_fx_apply(const __grid_constant__ Lat
   FxHalf acc;
   FxExps ex;
   fx_zero(acc, fx_range(ex, f, L.fu, L.g, s, dagger));
-  const bool ok = acc.E < FX_BAD;
+  const bool ok = fx_scale_ok(acc.E);
   if (!ok) acc.E = FX_E_BIAS;
   fx_hops(acc, f, L.fu, L.g, s, ex, dagger, sp, S);
   zd a[6];

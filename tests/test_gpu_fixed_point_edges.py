@@ -146,3 +146,21 @@ def test_operator_returns_its_own_term_as_it_is(dims, nsrc):
         got = binding.apply_H(T(u), MU, M_W, T(psi), dagger=dagger).cpu().numpy()
         for s in range(nsrc):
             assert np.array_equal(got[s], dirac.apply_gamma5(psi[s]))
+
+
+@pytest.mark.parametrize("field,link", [(2.0 ** -700, 2.0 ** -300), (2.0 ** -800, 2.0 ** -200), (2.0 ** 700, 2.0 ** 400)])
+def test_operator_products_at_the_ends_of_the_range(field, link):
+    """One colour of one site, diagonal links: products below 2^-1000 are still normal numbers, and
+    where they overflow the other colours stay zero."""
+    rng = np.random.default_rng(48)
+    dims = (3, 4, 3, 5)
+    u = np.zeros(inputs.lattice_shape(dims) + (4, 3, 3), dtype=np.complex128)
+    i = np.arange(3)
+    u[..., i, i] = link * np.exp(0.3j * rng.standard_normal(u.shape[:5] + (3,)))
+    psi = np.zeros(inputs.lattice_shape(dims) + (4, 3), dtype=np.complex128)
+    psi[2, 1, 2, 1, :, 1] = field * (1.0 + 0.5j)
+    if field < 1.0:
+        return check_operator(u, psi, 64)   # FP64 sums
+    got = binding.apply_H(T(u), MU, M_W, T(psi)).cpu().numpy()
+    assert np.array_equal(got[..., ::2], np.zeros_like(got[..., ::2]))
+    assert not np.isfinite(got[..., 1]).all()
