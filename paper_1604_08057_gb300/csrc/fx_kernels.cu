@@ -224,12 +224,11 @@ __global__ void __launch_bounds__(128, 4) k_fx_apply(const __grid_constant__ Lat
 }
 void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, const double* aos, double* out, int dagger,
                 cudaStream_t st, int variant) {
-  // threads per block in x (two per site) and sources per block: variant v > 0 takes shape v
-  // of this table (modulo its length), 0 the rule below
-  static const int shapes[][2] = {{128, 1}, {64, 1}, {32, 1}, {64, 2}, {32, 2}, {32, 4}, {128, 1}};
+  // threads per block in x (two per site) and sources per block, or (variant 0) the rule below
+  static const int shapes[FX_APPLY_SHAPES][2] = {{64, 1}, {32, 1}, {64, 2}, {32, 2}, {32, 4}, {128, 1}};
   int sx, sy;
   if (variant > 0) {
-    const int* s = shapes[variant % 7];
+    const int* s = shapes[fx_apply_shape(variant) - 1];
     sx = s[0];
     sy = s[1];
   } else if (L.g.V * L.nsrc < 152 * 128) {

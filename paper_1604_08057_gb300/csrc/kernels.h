@@ -133,6 +133,10 @@ void fx_encode(const double* d, const FxField& f, int nsrc, int64_t V, int64_t v
 // in: the field in fixed point, d: its FP64 companion, site-major (read where a site is marked);
 // aos: the field as the user's array, with out in the same layout, or null: out site-major and all
 // of d set
+constexpr int FX_APPLY_SHAPES = 6;
+// the shape that a variant number stands for: 0 the rule, v > 0 one of 1 .. FX_APPLY_SHAPES
+// (the FP32 operator has more variants; the numbers above start again)
+inline int fx_apply_shape(int v) { return v > 0 ? (v - 1) % FX_APPLY_SHAPES + 1 : 0; }
 void fx_apply_h(const Lat<double>& L, const FxField& in, const double* d, const double* aos, double* out, int dagger,
                 cudaStream_t st, int variant);
 

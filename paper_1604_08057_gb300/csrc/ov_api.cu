@@ -2346,6 +2346,10 @@ int autotune_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   CK(cudaMemsetAsync(L.r, 0, sizeof(R) * nsrc * L.vs, c->st));
   CK(cudaMemsetAsync(L.s, 0, sizeof(R) * nsrc * L.vs, c->st));
   CK(cudaMemsetAsync(L.sc, 0, sizeof(SrcScal) * nsrc, c->st));
+  if constexpr (std::is_same<R, double>::value) {
+    CK(cudaMemsetAsync(L.q, 0, sizeof(R) * nsrc * L.vs, c->st));
+    fx_encode(L.r, L.fr, nsrc, L.g.V, L.vs, c->st);
+  }
   cudaEvent_t e0 = c->ev[6], e1 = c->ev[7];
   auto time_us = [&](auto&& launch) {
     launch();
@@ -2360,13 +2364,24 @@ int autotune_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   r.n_apply = apply_h_variants();
   r.n_pair = tsl_stencil_variants();
   int* aerr = wsT<int>(c, B_AERR, 1, true);
-  for (int v = 0; v < r.n_apply && v < 16; ++v)
-    r.apply_us[v] = time_us([&] {
-      if constexpr (std::is_same<R, float>::value) {
-        if (v == APPLY_IL) return apply_h_il(L, L.r, L.p, 0, c->st);   // same buffers, its own layout
+  int timed = 0;
+  for (int v = 0; v < r.n_apply && v < 16; ++v) {
+    if constexpr (std::is_same<R, double>::value) {
+      // as ov_apply_H launches it, from and to the user's layout (q and p stand in)
+      const int s = fx_apply_shape(v);
+      if (s != v) {
+        r.apply_us[v] = r.apply_us[s];
+        continue;
       }
-      apply_h(L, L.r, L.p, 0, c->st, v, aerr);
-    });
+      r.apply_us[v] = time_us([&] { fx_apply_h(L, L.fr, L.r, L.q, L.p, 0, c->st, v); });
+    } else {
+      r.apply_us[v] = time_us([&] {
+        if (v == APPLY_IL) return apply_h_il(L, L.r, L.p, 0, c->st);   // same buffers, its own layout
+        apply_h(L, L.r, L.p, 0, c->st, v, aerr);
+      });
+    }
+    ++timed;
+  }
   for (int v = 0; v < r.n_pair && v < 16; ++v)
     r.pair_us[v] = time_us([&] { tsl_stencil(L, 0, true, c->st, v); });
   // a variant replaces the current choice only when it is more than 2% faster: the
@@ -2382,7 +2397,7 @@ int autotune_impl(ov_context* c, const int32_t dims[4], const void* U, double mu
   if (herr & ERRB_TIMEOUT) return OV_ERR_TIMEOUT;
   c->tuned_apply[c->opt.precision] = r.apply_variant;
   c->tuned_pair[c->opt.precision] = r.pair_variant;
-  c->launches += 6 * (r.n_apply + r.n_pair);
+  c->launches += 6 * (timed + r.n_pair);
   if (rep) *rep = r;
   return OV_OK;
 }

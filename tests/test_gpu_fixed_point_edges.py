@@ -164,3 +164,22 @@ def test_operator_products_at_the_ends_of_the_range(field, link):
     got = binding.apply_H(T(u), MU, M_W, T(psi)).cpu().numpy()
     assert np.array_equal(got[..., ::2], np.zeros_like(got[..., ::2]))
     assert not np.isfinite(got[..., 1]).all()
+
+
+@pytest.mark.parametrize("nsrc", [1, 3, 16])
+def test_operator_shapes(nsrc):
+    """The FP64 operator has six launch shapes beside its rule; the variant numbers above them start
+    again (and are not timed again), and every shape gives the same bits."""
+    rng = np.random.default_rng(49)
+    dims = (6, 4, 5, 7)
+    u, psi = T(inputs.su3_links(dims, 0.3, rng)), T(inputs.gaussian_spinors(dims, nsrc, rng))
+    want = binding.apply_H(u, MU, M_W, psi)
+    rep = binding.autotune(u, MU, M_W, nsrc=nsrc)
+    us = rep["apply_us"]
+    assert min(us) > 0.0 and all(us[v] == us[(v - 1) % 6 + 1] for v in range(7, len(us)))
+    try:
+        for v in range(len(us)):
+            binding.set_stencil_variants(v, 0)
+            assert torch.equal(binding.apply_H(u, MU, M_W, psi), want), v
+    finally:
+        binding.set_stencil_variants(0, 0)
