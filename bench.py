@@ -3,10 +3,9 @@
 
 Workload (default): 14x14^3 lattice (V = 38416, n = 460992), SU(3) links
 U = expm(i 0.2 A), mu = 0.3, m_w = -2, one Gaussian source, k = 800, one
-Gaussian cotangent; FP64 throughout, the lattice vectors and links in 57- and
-59-bit block fixed point (at this point the k-step map amplifies rounding by
-~1e6 and FP32 basis vectors break the recurrence down; the mixed-precision
-path is reported separately), pair-periodic
+Gaussian cotangent; FP64 throughout (at this point the k-step map amplifies
+rounding by ~1e6 and FP32 basis vectors break the recurrence down; the
+mixed-precision path is reported separately), pair-periodic
 re-biorthogonalisation every 60 steps with one Gram-Schmidt pass (at this
 point x stays within 1e-9 and dU within 1e-4 of the result with
 re-biorthogonalisation at every step, for any period from 10 to 100, and the
@@ -187,7 +186,7 @@ H_FLOP_PER_SITE = 1368   # one Wilson H application on half spinors (8 hops + di
 
 
 def algorithmic_flops(kind, k, V, nsrc, period, passes):
-    """Algorithmic FP64 flops of one ov_tsl_sign_vjp call for the lattice kinds.
+    """Algorithmic FP64 flops of one ov_tsl_sign_vjp call for the ALU-bound kinds.
 
     Gram-Schmidt kinds: 4 FMA (8 flop) per complex element and basis vector.
     stencil_pair: the two H applications and the alpha dot of each step, once
@@ -295,23 +294,40 @@ def run_ours(args, rank, world, local_rank):
     gbs = bytes_dom / (prof[dom][1] / 1e3) / 1e9
     per_launch = {"launches": prof[dom][0], "avg_launch_us": round(1e3 * prof[dom][1] / max(1, prof[dom][0]), 2),
                   "algorithmic_bytes_per_launch": int(bytes_dom / max(1, prof[dom][0]))}
-    # FP64 calls run in block fixed point on the integer pipes (8 bytes per real, as in FP64),
-    # so the large kernels' lower bound is their bytes, not the FP64 units
-    roofline = {"bound": "hbm", "kernel": dom, "achieved": round(gbs, 1), "peak": hbm, "unit": "GB/s",
-                "frac": round(gbs / hbm, 3), "peak_source": peak_src, "traffic": None, **per_launch}
-    if args.precision == "fp64" and dom in TRAFFIC_RATIO:
-        roofline["traffic"] = int(TRAFFIC_RATIO[dom] * per_launch["algorithmic_bytes_per_launch"])
-        roofline["traffic_source"] = (f"ncu dram bytes at 14x14^3 ({TRAFFIC_RATIO[dom]} x the algorithmic bytes of "
-                                      "the captured launches), scaled to this launch average")
-    flops = algorithmic_flops(dom, k, V, nsrc, args.rebiorth, args.passes)
-    if args.precision == "fp64" and flops:
-        # the same work against the FP64 units, which it does not use: 152 SMs x 2 FMA per clock
-        achieved = flops * args.steps / (prof[dom][1] / 1e3) / 1e12
-        peak_alu = 152 * 4 * (clk.get("sm_mhz") or 2070.0) * 1e6 / 1e12
-        gemm = fp64_peak(dev) / 1e3
-        roofline["fp64_view"] = {"achieved_TFLOP_s": round(achieved, 3), "fp64_unit_peak": round(peak_alu, 4),
-                                 "ratio": round(achieved / peak_alu, 3), "fp64_gemm_measured": round(gemm, 3),
-                                 "ratio_to_fp64_gemm": round(achieved / gemm, 3)}
+    if args.precision == "fp64" and dom in ("proj_dots", "proj_update", "rev_stencil", "stencil_pair"):
+        flops = algorithmic_flops(dom, k, V, nsrc, args.rebiorth, args.passes) * args.steps
+        achieved = flops / (prof[dom][1] / 1e3) / 1e12
+        # FP64 ALU peak from unit counts and clock: 152 SMs x 2 FP64 FMA (4 flop) per
+        # SM per clock (1.25 TFLOP/s nominal at 2070 MHz), at the median SM clock sampled
+        sm_mhz = clk.get("sm_mhz") or 2070.0
+        peak_alu = 152 * 4 * sm_mhz * 1e6 / 1e12
+        roofline = {"bound": "alu", "kernel": dom, "achieved": round(achieved, 3), "peak": round(peak_alu, 4),
+                    "unit": "TFLOP/s", "frac": round(achieved / peak_alu, 3),
+                    "peak_source": f"derived: 152 SMs x 4 FP64 flop/clk x {sm_mhz:.0f} MHz (sampled)",
+                    "fp64_gemm_measured_tflops": round(fp64_peak(dev) / 1e3, 3),
+                    "frac_of_fp64_gemm": None,
+                    "hbm_view": {"achieved_GB_s": round(gbs, 1), "peak": hbm, "frac": round(gbs / hbm, 3)},
+                    **per_launch}
+        roofline["frac_of_fp64_gemm"] = round(achieved / roofline["fp64_gemm_measured_tflops"], 3)
+        if dom == "rev_stencil":
+            # ncu: DRAM bytes of k_rev_stencil launches at 14x14^3, k = 120 = 0.845 x their
+            # algorithmic bytes; launches differ only in how many fields they stream
+            roofline["traffic"] = int(REV_STENCIL_TRAFFIC_RATIO * per_launch["algorithmic_bytes_per_launch"])
+            roofline["traffic_source"] = ("ncu dram bytes of two k_rev_stencil launches at 14x14^3, k=120 "
+                                          f"(ratio {REV_STENCIL_TRAFFIC_RATIO} to algorithmic), scaled to this "
+                                          "launch average")
+        elif dom == "proj_dots":
+            # ncu: DRAM bytes of a two-sided k_proj_dots launch = 1.018 x its algorithmic
+            # bytes (14x14^3, k = 120, nb = 61); traffic grows with the fields streamed
+            roofline["traffic"] = int(PROJ_DOTS_TRAFFIC_RATIO * per_launch["algorithmic_bytes_per_launch"])
+            roofline["traffic_source"] = ("ncu dram bytes of one k_proj_dots launch at 14x14^3, k=120, nb=61 "
+                                          f"(ratio {PROJ_DOTS_TRAFFIC_RATIO} to algorithmic), scaled to this "
+                                          "launch average")
+        else:
+            roofline["traffic"] = None
+    else:
+        roofline = {"bound": "hbm", "kernel": dom, "achieved": round(gbs, 1), "peak": hbm, "unit": "GB/s",
+                    "frac": round(gbs / hbm, 3), "peak_source": peak_src, "traffic": None, **per_launch}
     kernels_ms = {kd: round(v[1], 3) for kd, v in prof_w.items() if v[0]}
 
     out = {"metric": METRIC, "value": round(value, 6), "unit": "s", "n_gpus": world, "steps": args.steps,
@@ -352,8 +368,8 @@ def run_ours(args, rank, world, local_rank):
     return out
 
 
-# DRAM bytes of a kind's launches over their algorithmic bytes, from ncu at 14x14^3
-TRAFFIC_RATIO = {"rev_stencil": 1.06}
+PROJ_DOTS_TRAFFIC_RATIO = 1.018
+REV_STENCIL_TRAFFIC_RATIO = 0.845
 
 
 def hbm_peak():
@@ -368,7 +384,7 @@ def hbm_peak():
 
 
 def fp64_peak(dev, n=4096, reps=3):
-    """cuBLAS float64 GEMM rate (context for the FP64 view of the roofline), GFLOP/s."""
+    """cuBLAS float64 GEMM rate (context for the FP64 ALU roofline), GFLOP/s."""
     import torch
     a = torch.randn(n, n, dtype=torch.float64, device=dev)
     b = torch.randn(n, n, dtype=torch.float64, device=dev)

@@ -54,9 +54,14 @@ extern "C" {
                                      diagnostics, or ov_overlap_solve within maxit */
 
 /* Precision of lattice vectors, links and stencil arithmetic.
- * OV_FP64 : FP64 accuracy throughout.  Lattice vectors and links are held as 57- and
- *           59-bit integers with an exponent per site or link (their products and sums
- *           run on the integer units), scalars and k x k matrices in FP64.
+ * OV_FP64 : everything in FP64 but the hop sums of the operator itself (ov_apply_H and the
+ *           eigen-solvers' applications of H).  These run on the integer units: field and
+ *           links as 57- and 59-bit integers with one exponent per site or link, so a
+ *           component 2^-n below its site's largest enters the sums with 57 - n bits (an
+ *           FP64 number has 53), and each component of (H psi)(x) is within 8 2^-53 of
+ *           |psi(x)| + |kappa| sum |U| |psi(neighbour)| (largest components).  psi(x)'s own
+ *           term is exact, and sums that meet non-finite values or sites below 2^-822 or
+ *           above 2^878 are formed in FP64.  ov_apply_H_noalloc is FP64 throughout.
  * OV_MIXED: links, basis vectors and stencils in FP32; dot products accumulated
  *           with compensated (Dot2) FP32 arithmetic per thread and FP64 across
  *           threads; recurrence coefficients, re-biorthogonalisation
