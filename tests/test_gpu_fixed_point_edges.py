@@ -1,5 +1,6 @@
-"""Edges of the fixed-point operator and recurrence: zero links, values outside the exponent
-windows, sources beside one another, components far below their site's largest.
+"""Edges of the fixed-point operator (zero links, values outside the exponent windows, products at
+the ends of FP64's range, components far below their site's largest), and what the calls around it
+have to keep: values that small in b and xbar, sources that do not depend on one another.
 
 Operator: per site against the numpy oracle in extended precision, in units of 2^-53 m(x),
 m(x) = |psi(x)| + |kappa| sum over the eight hops of |U|_max |psi(neighbour)| (largest components).
@@ -74,8 +75,8 @@ def tails(rng, dims):
     return f
 
 
-# b (and the cotangent) far below the fixed-point window on some sites, a link there too.  x and the
-# gradients are the oracle's to the bars of the parity tests at m_w = -1
+# b (and the cotangent) down to subnormals on some sites, a link of 1e-290.  x and the gradients are
+# the oracle's to the bars of the parity tests at m_w = -1
 @pytest.mark.parametrize("rebiorth,passes", [(1, 2), (10, 1)])
 def test_sites_and_links_below_the_window(rebiorth, passes):
     dims, k = (3, 4, 3, 5), 30
@@ -117,7 +118,7 @@ def test_operator_below_the_window():
     check_operator(u, psi, 64)
 
 
-# on either side of the rule that splits a small lattice's sites over warps, which counts the sources
+# V times the sources on either side of the number of warps that fill the GPU
 @pytest.mark.parametrize("dims,nsrc", [((8, 8, 8, 8), 4), ((6, 6, 6, 6), 8), ((6, 8, 4, 6), 9)])
 def test_a_source_does_not_depend_on_those_beside_it(dims, nsrc):
     rng = np.random.default_rng(45)
